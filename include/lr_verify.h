@@ -164,7 +164,7 @@ int lr_verify_attention(lr_plan *plan, const void *q_d, const void *k_pool_d, co
                         void *out_d, float *lse_d, float softmax_scale, void *stream);
 
 /* What lr_verify_attention will launch for this plan (host-side query, no device work).
- *   tensor_core_ok   1 when the shape allows the tcgen05 kernel (head_dim 128, tensor-map coordinates
+ *   tensor_core_ok   1 when the shape allows the tcgen05 kernel (tensor-map coordinates
  *                    within 32 bits, at most 254 branches per request, tails of at most 2047 pages)
  *   path             the current selection (0 automatic, 1 CUDA cores, 2 tensor cores)
  *   uses_tensor_core 1 when the next call would run the tcgen05 kernel

@@ -1,5 +1,5 @@
-// CUDA-core nested-prefix attention: the path for shapes whose packed query
-// count is too small to be a dense contraction (and an on-device cross-check of
+// CUDA-core nested-prefix attention: the path for shapes the tensor-core path does not take (more than 254 branches to a
+// request, tails past 2047 pages, pools past 2^31 key rows) and an on-device cross-check of
 // the tensor-core path).  One warp per (query row, query head); the warp walks
 // the spans the row may see -- prefix, segments 1..depth, its own tail up to and
 // including itself -- 32 keys at a time: each lane scores one key, the warp

@@ -1,4 +1,4 @@
-// Tensor-core nested-prefix attention for sm_100a (head_dim 128).
+// Tensor-core nested-prefix attention for sm_100a (head_dim 64 or 128).
 //
 // Work decomposition.  For one request the *extended chain* is the list of its
 // KV pages in the order prefix, segments 1..gamma, branch tails; 8 consecutive
@@ -26,8 +26,8 @@
 // softmax warpgroups with setmaxnreg):
 //   warp 8      TMA producer: the Q tiles of a piece (3-D boxes: 64 channels x G
 //               heads x T tokens, so that the rows land packed) and, per tile,
-//               8 + 8 bulk tensor copies (one 4 KB box per page, K and V) into a
-//               5-stage ring of 32 KB buffers.  A box is a 4-D view of the page,
+//               8 + 8 bulk tensor copies (one box per page, K and V: 4 KB, or 2 KB with
+//               head size 64) into a ring of five 32 KB (ten 16 KB) buffers.  A box is a 4-D view of the page,
 //               [8-key group][channel half][8 keys][64 channels], so a tile lies in
 //               shared memory as 1024-byte swizzle atoms, the two channel halves of
 //               an 8-key group side by side (groups 2048 bytes apart): the layout
@@ -49,6 +49,10 @@
 //               bf16 P written back over S.
 // Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 fp32 columns each; P_s
 // occupies the first 64 columns of S_s.
+//
+// Head size 64.  The same kernel with half as many channels (struct Shape).  The CUDA-core kernel served this size before
+// and keeps the shapes the page tables here cannot describe; on one request of 4 K tokens, 3 branches of 16 drafts, 32
+// query and 8 KV heads it takes 724 us, this kernel and its merge 17 us (B200; the bytes alone: 2.7 us).
 //
 // Visibility.  Tiles made only of full prefix pages need no mask.  In every other
 // tile each page carries (valid tokens, first and last node number that sees it,
@@ -73,20 +77,32 @@ namespace lr {
 
 namespace {
 
-constexpr int kD = 128;
-constexpr int kStages = 5;
-constexpr int kTileBytes = 32768;  // [2 halves of 64 channels][128 keys or rows][128 B]
-constexpr int kHalfBytes = 16384;
+constexpr int kHalfBytes = 16384;  // 128 rows or keys x 64 channels
 constexpr int kAtomBytes = 1024;   // K/V tiles: 8 keys x 64 channels, one 128-byte-swizzle atom
-constexpr int kGroupBytes = 2048;  // ... two atoms (the two channel halves) per 8-key group
+constexpr int kMaxStages = 10;
 constexpr int kThreads = 384;
+
+// What depends on the head size (64 or 128 channels).  Both rings hold 160 KB of K and V in flight.
+template <int kD>
+struct Shape {
+  static_assert(kD == 64 || kD == 128, "head sizes of the tensor-core path");
+  static constexpr int kHalves = kD / 64;                 // 64-channel halves of a row (one 128-byte swizzle line each)
+  static constexpr int kTileBytes = kHalves * kHalfBytes; // [halves][128 rows][128 B] for Q, [16 groups][halves][8 keys][128 B] for K/V
+  static constexpr int kGroupBytes = kHalves * kAtomBytes;  // the atoms of one 8-key group
+  static constexpr int kStages = kD == 128 ? 5 : 10;
+  static constexpr int kSmemBytes = 2 * kTileBytes + kStages * kTileBytes + 2048;  // tiles, then Ctrl; the base must be 1024-aligned
+  // Head size 64 sends the softmax weights to the tensor core as two bf16 terms (value and remainder: 2^-17 of a
+  // weight instead of 2^-9), as precise as the fp32 weights of the CUDA-core kernel that used to serve it.  The second
+  // product is affordable there: its N is 64, and the sweep waits for the softmax, not for the tensor pipe.
+  static constexpr bool kSplitP = kD == 64;
+};
 constexpr int kPagesPerTile = 8;
 constexpr uint64_t kDrainLimitNs = 50ull * 1000ull * 1000ull;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: the reference exponent follows the row maximum within 2^8
 constexpr float kRedoThreshold = 64.0f;    // log2 units: beyond this a tile is redone with its own maximum as reference
 
 struct __align__(8) Ctrl {
-  uint64_t kv_full[kStages], kv_empty[kStages];
+  uint64_t kv_full[kMaxStages], kv_empty[kMaxStages];
   uint64_t q_full, q_empty;
   uint64_t s_full[2][2], p_full[2][2], o_done[2];  // [stream][half]
   uint64_t epi_done, drain[2];
@@ -98,8 +114,7 @@ struct __align__(8) Ctrl {
 };
 constexpr int kCtrlBytes = 2048;
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "Ctrl must fit behind the tiles");
-constexpr int kSmemBytes = 2 * kTileBytes + kStages * kTileBytes + kCtrlBytes;  // tiles, then Ctrl; the base must be 1024-aligned
-static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
+static_assert(Shape<64>::kSmemBytes <= 227 * 1024 && Shape<128>::kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
 // ---- PTX wrappers ----------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -179,10 +194,11 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t addr, uint32_t lbo_bytes,
          (1ull << 46) | (2ull << 61);
 }
 // Instruction descriptors: D fp32, A and B bf16, M = 128 (bits 24-28 = M/16), N in bits 17-22 (= N/8).
-// QK: N = 64 keys of a half-tile, both operands K-major.  PV: N = 128 channels, bit 16 selects the N-major B operand.
+// QK: N = 64 keys of a half-tile, both operands K-major.  PV: N = head size, bit 16 selects the N-major B operand.
 constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
 constexpr uint32_t kIdescQK = kIdescBase | ((64u >> 3) << 17);
-constexpr uint32_t kIdescPV = kIdescBase | ((128u >> 3) << 17) | (1u << 16);
+template <int kD>
+constexpr uint32_t kIdescPV = kIdescBase | (((uint32_t)kD >> 3) << 17) | (1u << 16);
 
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
   asm volatile(
@@ -214,6 +230,11 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&r)[64]) {
 }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+               : "memory");
+}
+
+__device__ __forceinline__ void tmem_st64(uint32_t taddr, const uint32_t (&r)[64]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x64.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63, %64};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(r[32]), "r"(r[33]), "r"(r[34]), "r"(r[35]), "r"(r[36]), "r"(r[37]), "r"(r[38]), "r"(r[39]), "r"(r[40]), "r"(r[41]), "r"(r[42]), "r"(r[43]), "r"(r[44]), "r"(r[45]), "r"(r[46]), "r"(r[47]), "r"(r[48]), "r"(r[49]), "r"(r[50]), "r"(r[51]), "r"(r[52]), "r"(r[53]), "r"(r[54]), "r"(r[55]), "r"(r[56]), "r"(r[57]), "r"(r[58]), "r"(r[59]), "r"(r[60]), "r"(r[61]), "r"(r[62]), "r"(r[63])
                : "memory");
 }
 
@@ -361,8 +382,23 @@ __device__ __forceinline__ float max_half(const uint32_t (&v)[64]) {
   }
   return fmaxf(fmaxf(a, b), fmaxf(c, e));
 }
-// P = exp2(scale * s - m) for 64 scores -> 32 packed bf16 pairs; returns the fp32 sum
-__device__ __forceinline__ float exp_half(const uint32_t (&v)[64], uint32_t (&pk)[32], float scale_log2, float neg_m) {
+// Four weights -> two packed bf16 pairs at pk[at], pk[at + 1]; with kSplit also what bf16 leaves of them at pk[32 + at] ..
+template <bool kSplit>
+__device__ __forceinline__ void pack_weights(float2 y0, float2 y1, uint32_t (&pk)[kSplit ? 64 : 32], int at) {
+  pk[at] = pack_bf16(y0.x, y0.y);
+  pk[at + 1] = pack_bf16(y1.x, y1.y);
+  if constexpr (kSplit) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float2 y = i ? y1 : y0;
+      const uint32_t h = pk[at + i];
+      pk[32 + at + i] = pack_bf16(y.x - bits_f(h << 16), y.y - bits_f(h & 0xFFFF0000u));
+    }
+  }
+}
+// P = exp2(scale * s - m) for 64 scores -> packed bf16 pairs; returns the fp32 sum
+template <bool kSplit>
+__device__ __forceinline__ float exp_half(const uint32_t (&v)[64], uint32_t (&pk)[kSplit ? 64 : 32], float scale_log2, float neg_m) {
   const float2 sc = make_float2(scale_log2, scale_log2), nm = make_float2(neg_m, neg_m);
   float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -375,15 +411,15 @@ __device__ __forceinline__ float exp_half(const uint32_t (&v)[64], uint32_t (&pk
     y1.y = ex2(y1.y);
     acc0 = fadd2(acc0, y0);
     acc1 = fadd2(acc1, y1);
-    pk[i >> 1] = pack_bf16(y0.x, y0.y);
-    pk[(i >> 1) + 1] = pack_bf16(y1.x, y1.y);
+    pack_weights<kSplit>(y0, y1, pk, i >> 1);
   }
   acc0 = fadd2(acc0, acc1);
   return acc0.x + acc0.y;
 }
 
 // exp_half on v, and beside it (in the shadow of the MUFU) the maximum of the raw scores
-__device__ __forceinline__ float exp_half_max(const uint32_t (&v)[64], uint32_t (&pk)[32], float scale_log2, float neg_m,
+template <bool kSplit>
+__device__ __forceinline__ float exp_half_max(const uint32_t (&v)[64], uint32_t (&pk)[kSplit ? 64 : 32], float scale_log2, float neg_m,
                                               float &raw_max) {
   const float2 sc = make_float2(scale_log2, scale_log2), nm = make_float2(neg_m, neg_m);
   float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
@@ -400,8 +436,7 @@ __device__ __forceinline__ float exp_half_max(const uint32_t (&v)[64], uint32_t 
     y1.y = ex2(y1.y);
     acc0 = fadd2(acc0, y0);
     acc1 = fadd2(acc1, y1);
-    pk[i >> 1] = pack_bf16(y0.x, y0.y);
-    pk[(i >> 1) + 1] = pack_bf16(y1.x, y1.y);
+    pack_weights<kSplit>(y0, y1, pk, i >> 1);
   }
   raw_max = fmaxf(m0, m1);
   acc0 = fadd2(acc0, acc1);
@@ -411,6 +446,7 @@ __device__ __forceinline__ float exp_half_max(const uint32_t (&v)[64], uint32_t 
 // The store epilogue of a softmax thread: row r of the accumulator at o_addr (and, when the CTA's two streams worked on
 // the same rows, of the other stream's at o_other, weighted) goes out as bf16 (slot < 0) or as an fp32 partial.
 // Not inlined: its two 64-register row buffers must not weigh on the register allocation of the sweep.
+template <int kD>
 __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int slot, bool pair, float w_self, float w_other, float m_out,
                                         float l_out, int r, int64_t q_index, uint16_t *__restrict__ out, float *__restrict__ lse,
                                         float *__restrict__ partial_o, float *__restrict__ partial_ml) {
@@ -418,7 +454,7 @@ __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int s
           if (slot < 0) {
             const float inv = 1.0f / l_out, a = w_self * inv, b = w_other * inv;
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
+            for (int hf = 0; hf < kD / 64; ++hf) {
               uint32_t o[64];
               tmem_ld64(o_addr + hf * 64, o);
               tc_wait_ld();
@@ -445,7 +481,7 @@ __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int s
           } else {
             const int64_t prow = (int64_t)slot * 128 + r;
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
+            for (int hf = 0; hf < kD / 64; ++hf) {
               uint32_t o[64];
               tmem_ld64(o_addr + hf * 64, o);
               tc_wait_ld();
@@ -464,7 +500,7 @@ __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int s
               }
               if (q_index >= 0) {
                 // chunk-major: 16-byte chunk k of row r at [slot][k][r], so a warp's store is 512 contiguous bytes
-                uint4 *dst = reinterpret_cast<uint4 *>(partial_o) + ((int64_t)slot * 32 + hf * 16) * 128 + r;
+                uint4 *dst = reinterpret_cast<uint4 *>(partial_o) + ((int64_t)slot * (kD / 4) + hf * 16) * 128 + r;
 #pragma unroll
                 for (int jj = 0; jj < 16; ++jj) dst[jj * 128] = make_uint4(o[4 * jj], o[4 * jj + 1], o[4 * jj + 2], o[4 * jj + 3]);
               }
@@ -473,10 +509,13 @@ __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int s
           }
 }
 
+template <int kD>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map,
                const __grid_constant__ CUtensorMap q_map, DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out,
                float *__restrict__ lse, float scale_log2) {
+  using Sh = Shape<kD>;
+  constexpr int kTileBytes = Sh::kTileBytes, kGroupBytes = Sh::kGroupBytes, kStages = Sh::kStages, kHalves = Sh::kHalves;
   extern __shared__ __align__(1024) unsigned char smem[];
   if ((smem_u32(smem) & 1023u) != 0u) {  // the swizzled tiles need a 1024-byte aligned base
     if (threadIdx.x == 0) {
@@ -485,8 +524,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
     }
     return;
   }
-  unsigned char *q_smem = smem;                         // 2 x 32 KB
-  unsigned char *kv_smem = smem + 2 * kTileBytes;       // kStages x 32 KB
+  unsigned char *q_smem = smem;                         // two M-tiles
+  unsigned char *kv_smem = smem + 2 * kTileBytes;       // kStages tiles
   Ctrl *ctrl = reinterpret_cast<Ctrl *>(kv_smem + kStages * kTileBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -549,11 +588,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
       // Q tiles of the piece, once the MMAs of the previous piece no longer read the buffers
       ok = wait_bar(&ctrl->q_empty, (q_count & 1u) ^ 1u, ctrl, d.status, 205);
       if (!ok) break;
-      if (lane == 0) mbar_arrive_expect_tx(&ctrl->q_full, (uint32_t)pi.n_mt * 2u * q_box_bytes);
+      if (lane == 0) mbar_arrive_expect_tx(&ctrl->q_full, (uint32_t)(pi.n_mt * kHalves) * q_box_bytes);
       __syncwarp();
-      if (lane < 2 * pi.n_mt)
-        tma_load_3d(smem_u32(q_smem) + (lane >> 1) * kTileBytes + (lane & 1) * kHalfBytes, &q_map, (lane & 1) * 64, pi.kv_head * G,
-                    rq.q_row0 + (pi.mtile0 + (lane >> 1)) * T, &ctrl->q_full);
+      if (lane < kHalves * pi.n_mt)
+        tma_load_3d(smem_u32(q_smem) + lane * kHalfBytes, &q_map, (lane % kHalves) * 64, pi.kv_head * G,
+                    rq.q_row0 + (pi.mtile0 + lane / kHalves) * T, &ctrl->q_full);
       ++q_count;
       const RingOrder ord(n, pi.n_mt);
       // Page ids arrive 32 at a time (one per lane = 4 tiles) and one chunk ahead of their first use,
@@ -597,10 +636,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
         ok = wait_bar(&ctrl->kv_empty[stage], ((ring / kStages) & 1u) ^ 1u, ctrl, d.status, 210);
         if (!ok) break;
         if (lane == 0)
-          mbar_arrive_expect_tx(&ctrl->kv_full[stage], (uint32_t)npages * 4096u + ((blockIdx.x == 0 && ring == 0) ? tc.phantom_tx_bytes : 0u));
+          mbar_arrive_expect_tx(&ctrl->kv_full[stage], (uint32_t)(npages * 2 * kGroupBytes) + ((blockIdx.x == 0 && ring == 0) ? tc.phantom_tx_bytes : 0u));
         __syncwarp();
-        if (lane < 8 && page >= 0) {  // one 4 KB box per page: two 8-key groups x two d halves
-          const uint32_t dst = smem_u32(kv_smem + stage * kTileBytes) + lane * 4096;
+        if (lane < 8 && page >= 0) {  // one box per page: two 8-key groups, all channels
+          const uint32_t dst = smem_u32(kv_smem + stage * kTileBytes) + lane * (2 * kGroupBytes);
           tma_load_4d(dst, is_v ? &v_map : &k_map, 0, 0, 0, (int32_t)(((int64_t)page * d.n_kv_heads + pi.kv_head) * 2),
                       &ctrl->kv_full[stage]);
         }
@@ -633,7 +672,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
       const uint64_t a = qdesc0 + (uint64_t)(m * (kTileBytes >> 4)),
                      b = kdesc0 + (uint64_t)(stage * (kTileBytes >> 4) + half * (8 * kGroupBytes >> 4));
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+      for (int h = 0; h < kHalves; ++h)
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           mma_ss(s_tmem + half * 64, a + (uint64_t)(h * (kHalfBytes >> 4) + kk * 2), b + (uint64_t)(h * (kAtomBytes >> 4) + kk * 2),
@@ -643,7 +682,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
       const uint64_t b = vdesc0 + (uint64_t)(stage * (kTileBytes >> 4) + half * (8 * kGroupBytes >> 4));
 #pragma unroll
       for (int k4 = 0; k4 < 4; ++k4)
-        mma_ts(o_tmem, s_tmem + half * 64 + k4 * 8, b + (uint64_t)(k4 * (2 * kGroupBytes >> 4)), kIdescPV, acc || k4 != 0);
+        mma_ts(o_tmem, s_tmem + half * 64 + k4 * 8, b + (uint64_t)(k4 * (2 * kGroupBytes >> 4)), kIdescPV<kD>, acc || k4 != 0);
+      if constexpr (Sh::kSplitP)
+#pragma unroll
+        for (int k4 = 0; k4 < 4; ++k4)
+          mma_ts(o_tmem, s_tmem + half * 64 + 32 + k4 * 8, b + (uint64_t)(k4 * (2 * kGroupBytes >> 4)), kIdescPV<kD>, 1u);
     };
     for (int pc = piece0; pc < piece1 && ok; ++pc, ++pc_idx) {
       const TcPiece pi = pc == piece0 ? head->first : tc.pieces[pc];
@@ -705,8 +748,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
           const TcPage *pg = tc.pages + rq.page_off + (pi.tile_begin + t) * kPagesPerTile;
           for (int p = 0; p < kPagesPerTile; ++p) {
             const int valid = pg[p].meta & 31;
-            for (int idx = lane; idx < (kPage - valid) * 16; idx += 32) {
-              const int key = p * kPage + valid + (idx >> 4), h = (idx >> 3) & 1, ch = idx & 7;
+            for (int idx = lane; idx < (kPage - valid) * 8 * kHalves; idx += 32) {
+              const int key = p * kPage + valid + idx / (8 * kHalves), h = (idx >> 3) & (kHalves - 1), ch = idx & 7;
               *reinterpret_cast<uint4 *>(vs + (key >> 3) * kGroupBytes + h * kAtomBytes + (key & 7) * 128 + ch * 16) = make_uint4(0, 0, 0, 0);
             }
           }
@@ -791,7 +834,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
           if (!wait_bar(&ctrl->o_done[s], (done_needed - 1) & 1u, ctrl, d.status, 235 + s)) return false;
           tc_fence_after();
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
+          for (int ch = 0; ch < kD / 32; ++ch) {
             uint32_t o[32];
             tmem_ld32(o_addr + ch * 32, o);
             tc_wait_ld();
@@ -838,14 +881,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
               ok = rescale_o(alpha, g);
               if (!ok) break;
             }
-            uint32_t pk[32];
+            uint32_t pk[Sh::kSplitP ? 64 : 32];
             float sum = 0.f, mx;
             // Fast path: exponentials against the running reference exponent; the maximum of the 64 scores is
             // computed beside them and only checked afterwards.
             bool fast = __all_sync(0xFFFFFFFFu, m_used > -INFINITY);
             if (fast) {
               float raw;
-              sum = exp_half_max(v, pk, scale_log2, -m_used, raw);
+              sum = exp_half_max<Sh::kSplitP>(v, pk, scale_log2, -m_used, raw);
               mx = raw * scale_log2;
               if (__any_sync(0xFFFFFFFFu, mx > m_used + kRedoThreshold)) fast = false;  // could overflow: redo exactly
             } else {
@@ -866,13 +909,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
                   if (!ok) break;
                 }
               }
-              sum = exp_half(v, pk, scale_log2, (m_used == -INFINITY) ? 0.f : -m_used);
+              sum = exp_half<Sh::kSplitP>(v, pk, scale_log2, (m_used == -INFINITY) ? 0.f : -m_used);
             } else if (mx > m_used + kRescaleThreshold) {
               pend = true;
               m_new = mx;
             }
             l += sum;
-            tmem_st32(sh_addr, pk);
+            if constexpr (Sh::kSplitP) tmem_st64(sh_addr, pk);
+            else tmem_st32(sh_addr, pk);
             tc_wait_st();
             tc_fence_before();
             // Observe every completion of o_done in order (a parity wait must never fall two phases behind):
@@ -918,7 +962,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
         if (pair) ++x_cnt;
         if (ok && writer) {
           tc_fence_after();
-          store_rows(o_addr, lane_base + 256 + (1 - s) * 128, pi.slot[pair ? 0 : s], pair, w_self, w_other, m_out, l_out, r, ri.q_index, out,
+          store_rows<kD>(o_addr, lane_base + 256 + (1 - s) * 128, pi.slot[pair ? 0 : s], pair, w_self, w_other, m_out, l_out, r, ri.q_index, out,
                      lse, tc.partial_o, tc.partial_ml);
           tc_fence_before();
         }
@@ -941,13 +985,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
 
 // Merge of the partials of one M-tile: O = sum_j 2^(m_j - M) O_j / sum_j 2^(m_j - M) l_j.
 // One thread per (query row, 16-byte chunk of channels); a warp holds 32 consecutive rows of one chunk, which
-// is how the partials are laid out ([slot][chunk][row]).  Grid: targets x 16 CTAs of 256 threads.  The slots
-// are combined in a fixed order.
+// is how the partials are laid out ([slot][chunk][row]).  Grid: targets x (head size / 8) CTAs of 256 threads.  The
+// slots are combined in a fixed order.
+template <int kD>
 __global__ void __launch_bounds__(256)
 attn_tc_merge_kernel(DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out, float *__restrict__ lse) {
   const TcTarget g = tc.targets[blockIdx.x];
   const int T = tc.tokens_per_mtile, G = d.group;
-  const int item = blockIdx.y * 256 + threadIdx.x;  // 0 .. 4095
+  const int item = blockIdx.y * 256 + threadIdx.x;  // 0 .. kD / 4 * 128 - 1
   const int k = item >> 7, r = item & 127;           // chunk of 4 channels, row
   const int tok = g.mtile * T + r / G;
   const bool live = r < T * G && tok < g.n_q;
@@ -956,7 +1001,7 @@ attn_tc_merge_kernel(DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out, float
   if (!live) return;
   const int64_t qi = (int64_t)(g.q_row0 + tok) * d.n_q_heads + g.kv_head * G + r % G;
   const float2 *ml = reinterpret_cast<const float2 *>(tc.partial_ml) + (int64_t)g.slot_begin * 128 + r;
-  const float4 *po = reinterpret_cast<const float4 *>(tc.partial_o) + ((int64_t)g.slot_begin * 32 + k) * 128 + r;
+  const float4 *po = reinterpret_cast<const float4 *>(tc.partial_o) + ((int64_t)g.slot_begin * (kD / 4) + k) * 128 + r;
   // Eight slots at a time, the (exponent, sum) pairs and the partial outputs of a batch requested together: one
   // round trip to memory per batch.  The running maximum moves between batches (never within one), in slot order,
   // so the result depends on nothing but the partials.
@@ -969,7 +1014,7 @@ attn_tc_merge_kernel(DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out, float
     for (int jj = 0; jj < 8; ++jj)
       if (j0 + jj < g.n_slots) {
         v[jj] = ml[(int64_t)(j0 + jj) * 128];
-        o[jj] = po[(int64_t)(j0 + jj) * 32 * 128];
+        o[jj] = po[(int64_t)(j0 + jj) * (kD / 4) * 128];
       }
     float mb = M;
 #pragma unroll
@@ -1006,9 +1051,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// kind 0: a KV pool of n pages viewed as [8-key groups][2 channel halves][8 keys][64 channels]; box = one page of one
-//         KV head (4 KB), which lands in shared memory as two 8-key groups of two 1024-byte swizzle atoms each
-// kind 1: Q of n rows as [rows][q heads][128], box = 64 channels x G heads x T tokens
+// kind 0: a KV pool of n pages viewed as [8-key groups][channel halves][8 keys][64 channels]; box = one page of one
+//         KV head, which lands in shared memory as two 8-key groups of one or two 1024-byte swizzle atoms each
+// kind 1: Q of n rows as [rows][q heads][head size], box = 64 channels x G heads x T tokens
 int get_map(lr_ctx *ctx, int kind, const void *ptr, int64_t n, const CUtensorMap **out) {
   for (auto &e : ctx->tmaps)
     if (e.ptr == ptr && e.n == n && e.kind == kind) {
@@ -1032,12 +1077,13 @@ int get_map(lr_ctx *ctx, int kind, const void *ptr, int64_t n, const CUtensorMap
   ent.n = n;
   ent.kind = kind;
   const lr_model &m = ctx->model;
+  const int kD = m.head_dim, halves = kD / 64;
   CUresult r;
   if (kind == 0) {
-    // [8-key group][channel half][key in group][64 channels]: one box = one page of one KV head (4 KB)
-    cuuint64_t dims[4] = {64, 8, 2, (cuuint64_t)n * m.n_kv_heads * (kPage / 8)};
+    // [8-key group][channel half][key in group][64 channels]: one box = one page of one KV head
+    cuuint64_t dims[4] = {64, 8, (cuuint64_t)halves, (cuuint64_t)n * m.n_kv_heads * (kPage / 8)};
     cuuint64_t strides[3] = {(cuuint64_t)kD * 2, 128, (cuuint64_t)kD * 2 * 8};
-    cuuint32_t box[4] = {64, 8, 2, kPage / 8};
+    cuuint32_t box[4] = {64, 8, (cuuint32_t)halves, kPage / 8};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     r = reinterpret_cast<EncodeTiledFn>(ctx->tmap_encode)(
         reinterpret_cast<CUtensorMap *>(ent.map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(ptr), dims, strides, box,
@@ -1066,8 +1112,11 @@ int get_map(lr_ctx *ctx, int kind, const void *ptr, int64_t n, const CUtensorMap
 }  // namespace
 
 int init_attn_tc_kernel() {
-  return cuda_fail(cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes),
-                   "attn_tc_kernel shared-memory attribute");
+  if (int rc = cuda_fail(cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<128>::kSmemBytes),
+                         "attn_tc_kernel<128> shared-memory attribute"))
+    return rc;
+  return cuda_fail(cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<64>::kSmemBytes),
+                   "attn_tc_kernel<64> shared-memory attribute");
 }
 
 // ---- host planning -----------------------------------------------------------------
@@ -1079,7 +1128,7 @@ int tc_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
   out = TcHostPlan();
   const lr_model &m = ctx->model;
   const int G = m.n_q_heads / m.n_kv_heads;
-  if (m.head_dim != kD) return LR_OK;  // other head sizes take the CUDA-core path
+  if (m.head_dim != 64 && m.head_dim != 128) return LR_OK;
   if ((int64_t)b->n_pool_pages * m.n_kv_heads * kPage >= ((int64_t)1 << 31)) return LR_OK;  // tensor-map coordinates are 32-bit
   const int T = 128 / G;
   const int n_q_rows = b->cu_q[b->n_branch];
@@ -1295,7 +1344,7 @@ int tc_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
   out.o_targets = img.add(targets.data(), targets.size() * sizeof(TcTarget));
   out.s_ml = 0;
   out.s_o = ((size_t)n_slots * 128 * 2 * sizeof(float) + 255) / 256 * 256;
-  out.scratch_bytes = out.s_o + (size_t)n_slots * 128 * kD * sizeof(float);
+  out.scratch_bytes = out.s_o + (size_t)n_slots * 128 * m.head_dim * sizeof(float);
   out.scratch_zero_bytes = 0;
   return LR_OK;
 }
@@ -1327,6 +1376,20 @@ void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigne
   t.partial_o = reinterpret_cast<float *>(scratch_base + h.s_o);
 }
 
+template <int kD>
+static int launch_attn_tc_d(lr_plan *p, const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &qmap, uint16_t *out,
+                            float *lse, float scale_log2, cudaStream_t s) {
+  attn_tc_kernel<kD><<<p->tc.n_cta, kThreads, Shape<kD>::kSmemBytes, s>>>(kmap, vmap, qmap, p->dev, p->tc, out, lse, scale_log2);
+  p->ctx->launches++;
+  if (int rc = cuda_fail(cudaGetLastError(), "attn_tc_kernel launch")) return rc;
+  if (p->tc.n_targets > 0) {  // the merge grid is set up while the attention grid drains
+    p->ctx->launches++;
+    return cuda_fail(launch_dependent(attn_tc_merge_kernel<kD>, dim3((unsigned)p->tc.n_targets, kD / 8), dim3(256), 0, s, p->dev, p->tc, out, lse),
+                     "attn_tc_merge_kernel launch");
+  }
+  return LR_OK;
+}
+
 int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
                    cudaStream_t s) {
   const CUtensorMap *mp = nullptr;
@@ -1337,28 +1400,8 @@ int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void
   if (int rc = get_map(p->ctx, 1, q, p->dev.n_q_rows, &mp)) return rc;
   const CUtensorMap qmap = *mp;
   const float scale_log2 = scale * 1.4426950408889634f;
-  attn_tc_kernel<<<p->tc.n_cta, kThreads, kSmemBytes, s>>>(kmap, vmap, qmap, p->dev, p->tc, reinterpret_cast<uint16_t *>(out), lse,
-                                                            scale_log2);
-  p->ctx->launches++;
-  if (int rc = cuda_fail(cudaGetLastError(), "attn_tc_kernel launch")) return rc;
-  if (p->tc.n_targets > 0) {
-    // programmatic dependent launch: the merge grid is set up while the attention grid drains
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)p->tc.n_targets, 16, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, attn_tc_merge_kernel, p->dev, p->tc, reinterpret_cast<uint16_t *>(out), lse);
-    p->ctx->launches++;
-    if (int rc = cuda_fail(e, "attn_tc_merge_kernel launch")) return rc;
-  }
-  return LR_OK;
+  return (p->dev.head_dim == 128 ? launch_attn_tc_d<128> : launch_attn_tc_d<64>)(p, kmap, vmap, qmap, reinterpret_cast<uint16_t *>(out), lse,
+                                                                                scale_log2, s);
 }
 
 }  // namespace lr

@@ -1,0 +1,51 @@
+"""The tensor-core attention kernel at head size 64, named explicitly, against the fp64 oracle: one partial tile up to
+plans whose pieces hold two query tiles, chains and trees, split keys and unsplit ones."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import REL_LARGE, run_and_check_pass
+from lr_workloads import Model, make_config, make_random_small, make_random_tree
+from lr_workloads.gen import _finish
+from oracle import lr_oracle as O
+from paper_2506_19830_b200 import binding as B
+from paper_2506_19830_b200 import runner as R
+
+pytestmark = pytest.mark.gpu
+
+
+def _chain(seed, hq, hkv, P, gamma, L, n_req=1):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    reqs = [{"P": P + 37 * r, "segs": [int(v) for v in rng.integers(5, 70, size=gamma)], "branches": [(j, L, L, L) for j in range(gamma + 1)]}
+            for r in range(n_req)]
+    return _finish(f"chain64_{seed}", seed, Model(hq, hkv, 64, 1000), reqs, rng, 0.3, 0.6, True, True, "nan")
+
+
+@pytest.mark.parametrize("make", [lambda: make_config(1)] + [lambda s=s: make_random_small(4200 + s, head_dim=64) for s in range(6)]
+                         + [lambda s=s: make_random_tree(4300 + s, head_dim=64) for s in range(4)])
+def test_small(make):
+    run_and_check_pass(make(), path=B.PATH_TENSOR_CORE, rel_large=REL_LARGE)
+
+
+@pytest.mark.parametrize("args", [(1, 16, 4, 2500, 3, 16), (2, 5, 1, 6000, 4, 9), (3, 8, 8, 1111, 2, 7, 3), (4, 32, 8, 9000, 3, 16, 2)])
+def test_split_keys(args):
+    w = _chain(*args)
+    n = w.batch.n_branch
+    run_and_check_pass(w, path=B.PATH_TENSOR_CORE, check_rows_of_branches=sorted({0, n // 2, n - 1}))
+
+
+def test_weights_are_not_rounded_to_bf16():
+    """Two bf16 terms per weight leave 2^-17 of it, so the output's own rounding (at most 2^-9 of every value) is all
+    that is left to see in the 2-norm; bf16 weights alone would add 1.6e-3 to it."""
+    w = _chain(5, 16, 4, 1500, 3, 16)
+    b, t = w.batch, w.tensors
+    ctx = B.Context(b.model, 0)
+    plan = B.Plan(ctx, b)
+    assert plan.lr_plan_describe()["uses_tensor_core"] == 1  # the automatic choice
+    x, y = R.DeviceInputs(b, t), R.PassOutputs(b)
+    plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out)
+    assert plan.lr_poll_status() == 0
+    ref, _ = O.verify_attention(b, t.q, t.k_pool, t.v_pool)
+    got = y.out.to(torch.float64).cpu().numpy()
+    assert np.linalg.norm(got - ref) <= (2.0 ** -9 + 2.0 ** -15) * np.linalg.norm(ref)
+    ctx.close()
