@@ -1,8 +1,8 @@
 // Stochastic token-level acceptance (rejection sampling) for point-mass draft distributions.
 //
-// Two kernels.  accept_stats_kernel streams the bf16 logits once -- the HBM-bound part: grid (chunks of 8192
-// logits, rows); a CTA reduces its chunk to (raw maximum M_c, S_c = sum exp((x - M_c) / T)) and stores the pair.
-// accept_sample_kernel, one CTA per branch, combines the pairs of a row in chunk order into (m, Z), gets
+// Two kernels.  accept_stats_kernel streams the bf16 logits once -- the HBM-bound part: a warp takes one chunk of a row
+// at a time (2048 logits, or the next power-of-two multiple that leaves at most kMaxChunks chunks) and leaves the pair
+// (raw maximum M_c, S_c = sum exp((x - M_c) / T)).  accept_sample_kernel, one CTA per branch, combines the pairs of a row in chunk order into (m, Z), gets
 // P_i(d_i) = exp((x_d - m) / T) / Z for the drafts, walks the acceptance chain u_i < P_i(d_i), and draws the
 // final token by inverse CDF over the stop row with the rejected token removed: first over the chunk
 // weights S_c exp((M_c - m) / T) (no second pass over the row), then inside the one chunk that holds the
@@ -16,15 +16,12 @@ namespace lr {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kVec = 4;                       // 16-byte vectors per thread
-constexpr int kChunk = kThreads * kVec * 8;   // logits per chunk
+constexpr int kVec = 8;                       // 16-byte vectors a lane loads at a time
+constexpr int kStep = 32 * kVec * 8;          // logits a warp takes at a time
+constexpr int kMaxChunks = 160;               // per row: the pairs of kRowBatch rows must fit into 40 KB
+constexpr int kCtasPerSm = 4;
 constexpr int kRowBatch = 32;                 // rows of a branch handled at a time in the chain
 
-__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-  return v;
-}
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 __device__ __forceinline__ float ex2_approx(float x) {  // one MUFU operation; -inf gives 0
@@ -34,93 +31,106 @@ __device__ __forceinline__ float ex2_approx(float x) {  // one MUFU operation; -
 }
 __device__ __forceinline__ float denan(float x) { return fmaxf(x, -INFINITY); }  // NaN counts as -inf (max drops a NaN operand)
 
-// the 32 logits of thread `tid` in chunk `c` of a row: element e = c*kChunk + (k*kThreads + tid)*8 + j for the
-// striped layout (coalesced), or e = c*kChunk + tid*32 + k*8 + j for the blocked layout (contiguous per thread)
-template <bool kBlocked>
-__device__ __forceinline__ void load_chunk(const uint16_t *rp, int32_t vocab, int c, int tid, float (&x)[kVec * 8]) {
-  const int32_t n_vec = vocab >> 3;
+// the logits of vector vi of a row (-inf past its end)
+__device__ __forceinline__ void unpack(const uint4 &v, float *x) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int k = 0; k < kVec; ++k) {
-    const int32_t vi = c * (kChunk / 8) + (kBlocked ? tid * kVec + k : k * kThreads + tid);
-    if (vi < n_vec) {
-      const uint4 v = ld_stream(reinterpret_cast<const uint4 *>(rp) + vi);
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  for (int j = 0; j < 4; ++j) {
+    x[2 * j] = denan(bf_lo(w[j]));
+    x[2 * j + 1] = denan(bf_hi(w[j]));
+  }
+}
+__device__ __forceinline__ void load_tail(const uint16_t *rp, int32_t vocab, int32_t vi, float *x) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        x[k * 8 + 2 * j] = denan(bf_lo(w[j]));
-        x[k * 8 + 2 * j + 1] = denan(bf_hi(w[j]));
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {  // ragged end of the row (vocab not a multiple of 8), or beyond it
-        const int32_t e = vi * 8 + j;
-        x[k * 8 + j] = e < vocab ? denan(bf_lo((uint32_t)rp[e])) : -INFINITY;
-      }
-    }
+  for (int j = 0; j < 8; ++j) {  // ragged end of the row (vocab not a multiple of 8), or beyond it
+    const int32_t e = vi * 8 + j;
+    x[j] = e < vocab ? denan(bf_lo((uint32_t)rp[e])) : -INFINITY;
   }
 }
 
-__device__ __forceinline__ float block_reduce_max(float v, float *s_red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float r = s_red[0];
-#pragma unroll
-  for (int w = 1; w < kThreads / 32; ++w) r = fmaxf(r, s_red[w]);
-  __syncthreads();
+__device__ __forceinline__ uint32_t max_bf2(uint32_t x, uint32_t y) {  // a NaN operand loses
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
   return r;
 }
-__device__ __forceinline__ float block_reduce_sum(float v, float *s_red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float r = s_red[0];
-#pragma unroll
-  for (int w = 1; w < kThreads / 32; ++w) r += s_red[w];
-  __syncthreads();
-  return r;
+__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
 }
 
-__global__ void __launch_bounds__(kThreads)
-accept_stats_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2,
-                    float2 *__restrict__ stats) {
-  __shared__ float s_red[kThreads / 32];
-  const int c = blockIdx.x, row = blockIdx.y, n_chunks = gridDim.x;
+// One warp per chunk at a time, the grid's warps taking the chunks of all rows in turn: the 4 KB a warp has in flight come
+// back while the 31 others of its SM compute, and no warp ever waits for another.  617 rows of 152064 logits: 35.4 us,
+// 5.3 TB/s, bound by HBM and, close behind it, by the exponentials (21 us of the special-function units); one CTA per
+// chunk of 8192 with its loads in registers and two block reductions behind them took 54.8 us.
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+accept_stats_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, uint32_t n_chunks, int steps,
+                    uint32_t total, float2 *__restrict__ stats) {
+  const int lane = threadIdx.x & 31;
+  const int32_t n_vec = vocab >> 3, rem = vocab & 7;
+  constexpr uint32_t kNegInf2 = 0xFF80FF80u;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the logits may come from the kernel launched just before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  float x[kVec * 8];
-  load_chunk<false>(logits + (int64_t)row * row_stride, vocab, c, threadIdx.x, x);
-  float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;  // independent chains
+  for (uint32_t unit = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); unit < total; unit += gridDim.x * (kThreads / 32)) {
+    const uint32_t row = unit / n_chunks;
+    const uint16_t *rp = logits + (int64_t)row * row_stride;
+    int32_t v0 = (int32_t)(unit - row * n_chunks) * steps * (kStep / 8) + lane;
+    float m = -INFINITY, sum = 0.f;  // of this lane's share of the chunk
+    for (int st = 0; st < steps; ++st, v0 += kStep / 8) {
+      uint32_t x[kVec * 4];
 #pragma unroll
-  for (int i = 0; i < kVec * 8; i += 4) {
-    m0 = fmaxf(m0, x[i]);
-    m1 = fmaxf(m1, x[i + 1]);
-    m2 = fmaxf(m2, x[i + 2]);
-    m3 = fmaxf(m3, x[i + 3]);
-  }
-  const float M = block_reduce_max(fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)), s_red);
-  float sum = 0.f;
-  if (M > -INFINITY) {
-    const float off = -M * k_log2;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+      for (int k = 0; k < kVec; ++k) {
+        const int32_t vi = v0 + k * 32;
+        uint4 v = make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
+        if (vi < n_vec) v = ld_stream(reinterpret_cast<const uint4 *>(rp) + vi);
+        x[4 * k] = v.x;
+        x[4 * k + 1] = v.y;
+        x[4 * k + 2] = v.z;
+        x[4 * k + 3] = v.w;
+      }
+      if (rem != 0 && v0 <= n_vec && v0 + kStep / 8 > n_vec && ((n_vec - v0) & 31) == 0) {  // this lane has the ragged end of the row
 #pragma unroll
-    for (int i = 0; i < kVec * 8; i += 4) {
-      a0 += ex2_approx(fmaf(x[i], k_log2, off));
-      a1 += ex2_approx(fmaf(x[i + 1], k_log2, off));
-      a2 += ex2_approx(fmaf(x[i + 2], k_log2, off));
-      a3 += ex2_approx(fmaf(x[i + 3], k_log2, off));
+        for (int k = 0; k < kVec; ++k)
+          if (v0 + k * 32 == n_vec)
+#pragma unroll
+            for (int j = 0; j < 7; ++j)
+              if (j < rem) {
+                const uint32_t h = rp[(int64_t)n_vec * 8 + j];
+                x[4 * k + (j >> 1)] = (j & 1) ? ((x[4 * k + (j >> 1)] & 0xFFFFu) | (h << 16)) : ((x[4 * k + (j >> 1)] & 0xFFFF0000u) | h);
+              }
+      }
+      uint32_t mx = kNegInf2;
+#pragma unroll
+      for (int i = 0; i < kVec * 4; ++i) {
+        x[i] = max_bf2(x[i], kNegInf2);  // NaN counts as -inf
+        mx = max_bf2(mx, x[i]);
+      }
+      const float mn = fmaxf(m, fmaxf(bf_lo(mx), bf_hi(mx)));
+      const float off = mn > -INFINITY ? -mn * k_log2 : 0.f;
+      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+      for (int i = 0; i < kVec * 4; i += 2) {
+        a0 += ex2_approx(fmaf(bf_lo(x[i]), k_log2, off));
+        a1 += ex2_approx(fmaf(bf_hi(x[i]), k_log2, off));
+        a2 += ex2_approx(fmaf(bf_lo(x[i + 1]), k_log2, off));
+        a3 += ex2_approx(fmaf(bf_hi(x[i + 1]), k_log2, off));
+      }
+      sum = fmaf(sum, ex2_approx(fmaf(m, k_log2, off)), (a0 + a1) + (a2 + a3));
+      m = mn;
     }
-    sum = (a0 + a1) + (a2 + a3);
+    float M = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+    float S = sum * ex2_approx(fmaf(m, k_log2, M > -INFINITY ? -M * k_log2 : 0.f));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
+    if (lane == 0) stats[unit] = make_float2(M, S);
   }
-  const float S = block_reduce_sum(sum, s_red);
-  if (threadIdx.x == 0) stats[(int64_t)row * n_chunks + c] = make_float2(M, S);
 }
 
 __global__ void __launch_bounds__(kThreads)
 accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2,
-                     const float2 *__restrict__ stats, int n_chunks, const int32_t *__restrict__ draft_ids,
+                     const float2 *__restrict__ stats, int n_chunks, int chunk, const int32_t *__restrict__ draft_ids,
                      const int32_t *__restrict__ cu_draft, const float *__restrict__ u_accept,
                      const float *__restrict__ u_final, int32_t *__restrict__ n_accept, int32_t *__restrict__ final_id,
                      float *__restrict__ p_draft) {
@@ -212,7 +222,7 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   //      sums by shuffles, fixed order)
   if (warp == 0) {
     const float2 *st = s_st + kn * n_chunks;
-    const int dead_chunk = dead >= 0 ? dead / kChunk : -1;
+    const int dead_chunk = dead >= 0 ? dead / chunk : -1;
     auto weight = [&](int c) -> float {
       if (c >= n_chunks) return 0.f;
       const float2 v = st[c];
@@ -263,18 +273,25 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   }
   __syncthreads();
 
-  // ---- inside the chunk: thread t owns 32 consecutive logits; exclusive scan of the thread sums, then a
-  //      sequential walk in the one thread whose range holds the target
-  const int pc = s_pick_chunk;
+  // ---- inside the chunk: thread t owns chunk / kThreads consecutive logits (a multiple of 8); exclusive scan of the
+  //      thread sums, then a sequential walk in the one thread whose range holds the target
+  const int pc = s_pick_chunk, own = chunk / kThreads;
   const float remain = s_pick_before;
-  float x[kVec * 8];
-  load_chunk<true>(rp, vocab, pc, tid, x);
-  float w[kVec * 8], mine = 0.f;
+  const int32_t n_vec = vocab >> 3, e0 = pc * chunk + tid * own;
+  auto weights = [&](int i, float (&w)[8]) {  // of logits e0 + i .. e0 + i + 7
+    const int32_t vi = (e0 + i) >> 3;
+    float x[8];
+    if (vi < n_vec) unpack(__ldg(reinterpret_cast<const uint4 *>(rp) + vi), x);
+    else load_tail(rp, vocab, vi, x);
 #pragma unroll
-  for (int i = 0; i < kVec * 8; ++i) {
-    const int32_t e = pc * kChunk + tid * 32 + i;
-    w[i] = (e == dead || x[i] == -INFINITY) ? 0.f : exp2f((x[i] - m) * k_log2);
-    mine += w[i];
+    for (int j = 0; j < 8; ++j) w[j] = (e0 + i + j == dead || x[j] == -INFINITY) ? 0.f : exp2f((x[j] - m) * k_log2);
+  };
+  float mine = 0.f;
+  for (int i = 0; i < own; i += 8) {
+    float w[8];
+    weights(i, w);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mine += w[j];
   }
   float incl = mine;  // inclusive scan over the block, in thread order
 #pragma unroll
@@ -300,24 +317,34 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   if (tid == max(pt, 0)) {
     float cum = before;
     int pick = -1, last = 0;
+    for (int i = 0; i < own && pick < 0; i += 8) {
+      float w[8];
+      weights(i, w);
 #pragma unroll
-    for (int i = 0; i < kVec * 8; ++i) {
-      if (w[i] > 0.f) {
-        last = i;
-        if (pick < 0 && cum + w[i] > remain) pick = i;
-        cum += w[i];
-      }
+      for (int j = 0; j < 8; ++j)
+        if (w[j] > 0.f) {
+          last = i + j;
+          if (pick < 0 && cum + w[j] > remain) pick = i + j;
+          cum += w[j];
+        }
     }
     if (pick < 0) pick = last;
     n_accept[b] = n;
-    final_id[b] = pc * kChunk + tid * 32 + pick;
+    final_id[b] = e0 + pick;
   }
 }
 
 }  // namespace
 
+// steps of kStep logits per chunk
+static int chunk_steps(int32_t vocab) {
+  int steps = 1;
+  while ((vocab + (int64_t)steps * kStep - 1) / ((int64_t)steps * kStep) > kMaxChunks) steps *= 2;
+  return steps;
+}
+
 size_t accept_sample_scratch_bytes(int32_t vocab, int32_t n_rows) {
-  const size_t n_chunks = ((size_t)vocab + kChunk - 1) / kChunk;
+  const size_t chunk = (size_t)chunk_steps(vocab) * kStep, n_chunks = ((size_t)vocab + chunk - 1) / chunk;
   return std::max<size_t>(8, (size_t)n_rows * n_chunks * sizeof(float2));
 }
 
@@ -325,7 +352,7 @@ int launch_accept_sample(lr_ctx *ctx, const void *logits, int64_t stride, const 
                          int32_t n_branch, int32_t n_rows, float temperature, const float *u_accept, const float *u_final,
                          int32_t *n_accept, int32_t *final_id, float *p_draft, void *scratch, cudaStream_t s) {
   const int32_t vocab = ctx->model.vocab;
-  const int n_chunks = (vocab + kChunk - 1) / kChunk;
+  const int steps = chunk_steps(vocab), chunk = steps * kStep, n_chunks = (int)(((int64_t)vocab + chunk - 1) / chunk);
   if (n_rows > 65535) {
     set_error("lr_accept_sample: more than 65535 logits rows in one call");
     return LR_EUNSUPPORTED;
@@ -333,30 +360,17 @@ int launch_accept_sample(lr_ctx *ctx, const void *logits, int64_t stride, const 
   const float k_log2 = 1.4426950408889634f / temperature;
   auto *lg = reinterpret_cast<const uint16_t *>(logits);
   auto *st = reinterpret_cast<float2 *>(scratch);
-  accept_stats_kernel<<<dim3((unsigned)n_chunks, (unsigned)n_rows), kThreads, 0, s>>>(lg, stride, vocab, k_log2, st);
+  const uint32_t total = (uint32_t)n_rows * n_chunks;  // at most 65535 * kMaxChunks
+  const unsigned grid = std::min((total + kThreads / 32 - 1) / (kThreads / 32), (uint32_t)(ctx->sm_count * kCtasPerSm));
+  accept_stats_kernel<<<grid, kThreads, 0, s>>>(lg, stride, vocab, k_log2, (uint32_t)n_chunks, steps, total, st);
   ctx->launches++;
   if (int rc = cuda_fail(cudaGetLastError(), "accept_stats_kernel launch")) return rc;
-  const size_t smem = (size_t)kRowBatch * n_chunks * sizeof(float2);
-  if (smem > 40 * 1024) {
-    set_error("lr_accept_sample: vocabulary of %d entries needs %zu bytes of shared memory per branch (limit 40 KB)", vocab, smem);
-    return LR_EUNSUPPORTED;
-  }
   // programmatic dependent launch: the per-branch grid is set up while the streaming grid drains
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)n_branch, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, accept_sample_kernel, lg, stride, vocab, k_log2, (const float2 *)st, n_chunks, drafts,
-                                     cu_draft, u_accept, u_final, n_accept, final_id, p_draft);
   ctx->launches++;
-  return cuda_fail(e, "accept_sample_kernel launch");
+  return cuda_fail(launch_dependent(accept_sample_kernel, dim3((unsigned)n_branch), dim3(kThreads), (size_t)kRowBatch * n_chunks * sizeof(float2), s,
+                                    lg, stride, vocab, k_log2, st, n_chunks, chunk, drafts, cu_draft, u_accept, u_final, n_accept, final_id,
+                                    p_draft),
+                   "accept_sample_kernel launch");
 }
 
 }  // namespace lr

@@ -254,6 +254,7 @@ int init_kernels(lr_ctx *ctx);  // per-device function attributes; called by lr_
 int init_commit_kernel();
 int init_attn_tc_kernel();
 int init_attn_pair_kernel();
+
 int launch_attn_pair(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
                      cudaStream_t s);
 int launch_attn_generic(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
