@@ -3,25 +3,30 @@
 //
 // The filters keep a leading part of the ranking of a row's tokens by probability (descending; equal
 // probabilities in index order).  With bf16 logits the ranking is the ranking of a 16-bit ordered key (-0 and +0
-// sharing one), so the
-// kept set of a row is described by a cut: every token whose key is above cut_key, and of the tokens whose key
-// equals cut_key those with an index up to cut_idx.  filter_rows_kernel (one CTA per row) finds the cut:
-//   pass 0   row maximum m;
-//   pass 1   token counts per key over the window of the 8192 largest keys from m down (64 octaves: every positive
-//            logit when m > 0), one shared-memory atomic per token; the tokens below the window only add their
-//            mass to a per-thread sum.  Masses are w = exp2((x - m) log2(e) / T) as integers in units of 2^-40:
-//            all tokens of a key have the same mass, so a key's mass is count x w exactly, and integer sums do not
-//            depend on the order of the additions -- the result is the same on every run;
-//   scan     counts and masses of the window's keys from the top down: the key holding the last token top-k
-//            keeps, then, with W_k = mass of the top k, the key at which the mass reaches top_p W_k;
-//   more     if a cut lies below the window, the window moves down to the next key that occurs (one more pass
-//            each time) until it holds the cut; if top-p's cut lies above the window top-k ended in, the search
-//            starts again from the top;
-//   last     only when the cut splits a group of equal keys: the index of the last token kept in the group.
-// After pass 0 the row comes from L2.  accept_filtered_kernel (one CTA per branch) walks the acceptance chain
-// with P'(d) = w_d / Z' for kept tokens and 0 for the others, and draws the final token by inverse CDF over the
-// kept tokens of the stop row in index order, in the same integer masses (no rounding: the draw is exact given
-// the masses).
+// sharing one), so the kept set of a row is described by a cut: every token whose key is above cut_key, and of the
+// tokens whose key equals cut_key those with an index up to cut_idx.  Masses are w = exp2((x - m) log2(e) / T) as
+// integers in units of 2^-40 (m: the row maximum): integer sums do not depend on the order of the additions, so every
+// route below gives the same cut and the same draw.
+//
+// The cut of a row is found by one of two routes.
+//
+// Candidates (filter_scan_kernel, filter_cut_kernel): the logits are read once for the largest key of every group of 64
+// (or 8) tokens and, with top-k off, for the row's mass as an fp32 sum.  A CTA per row then finds the k_sel-th largest of the
+// group maxima, reads the few groups that reach it once more and ranks their tokens.  With top-k on that is all there is
+// to know.  With top-p alone the total mass is known to within kMassEps; the row is settled when both ends of that interval
+// give the same cut.
+//
+// Windows (filter_window_kernel): a cluster of CTAs holds the row in shared memory, counts tokens per key, merges the
+// counts through distributed shared memory and finds the cut in them, whatever the row looks like.  It takes the rows that
+// the candidates leave open -- a kept set larger than the candidates, many equal logits, a cut within rounding of a
+// step, no finite maximum -- and all rows of a call that cannot use the candidates or has few rows to settle by mass
+// (launch_accept_filtered has the rule).
+//
+// accept_filtered_kernel (per branch) walks the acceptance chain with P'(d) = w_d / Z' for kept tokens and 0 for
+// the others, and draws the final token by inverse CDF over the kept tokens of the stop row in index order: first over the
+// kept mass of every slice of the row, then inside one slice.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "lr_common.cuh"
@@ -30,20 +35,36 @@ namespace lr {
 
 namespace {
 
-constexpr int kFT = 1024;          // threads of filter_rows_kernel
-constexpr int kWin = 8192;         // keys per window
-constexpr int kPer = kWin / kFT;   // window positions per thread in the scan
-constexpr int kST = 1024;          // threads of accept_filtered_kernel
+constexpr int kT = 256;             // threads of every kernel but filter_window_kernel
+constexpr int kWarps = kT / 32;
+constexpr int kVec = 8;             // 16-byte vectors a lane of filter_scan_kernel takes at a time
+constexpr int kChunk = 32 * kVec * 8;  // logits a warp takes at a time
+constexpr int kScanCtasPerSm = 4;
+constexpr int kMaxGroups = 10240;   // group keys of a row that filter_cut_kernel can hold
+constexpr int kGroupCap = 512;      // groups it reads again
+constexpr int kListCap = 1024;      // candidates of a row
+constexpr int kSelMax = 256;        // largest top_k the candidates serve
+constexpr int kSelTopP = 128;       // leading tokens to look for when top-k is off
+constexpr int kWT = 512;            // threads of a CTA of filter_window_kernel
+constexpr int kWin = 8192;          // keys per window
+constexpr int kMaxSlices = 1024;    // slices of a row whose kept masses are written out
+constexpr size_t kWindowSmemMax = 200 * 1024;
+constexpr int kWindowRounds = 3;    // rounds of rows through the windows that a candidate pass has to spare
+// Relative distance between the fp32 sum of a row's masses and their integer sum: the argument of an exponential is
+// rounded at magnitude 40 (2^-19.4 absolute: 1e-6 of the mass), ex2.approx is good to 2^-22 on both sides, an fp32 sum of
+// 64 terms and some 30 further additions to 5e-6, rounding masses to 2^-40 of the largest to 1e-7; rounded up.
+constexpr double kMassEps = 2e-5;
 typedef unsigned long long u64;
 constexpr int32_t kNoKey = INT32_MIN;
 
-struct RowCut {  // what the second kernel needs to know about a row (32 bytes)
+struct RowCut {  // what the acceptance kernel needs to know about a row (32 bytes)
   float m;          // row maximum (finite: a row without a finite logit gets -3e38)
   int32_t cut_key;  // key32 of the last kept group of equal logits; kNoKey: everything is kept
   int32_t cut_idx;  // largest index kept inside that group
   int32_t n_kept;
   u64 z_fix;        // mass of the kept set
-  u64 reserved;
+  int32_t slices;   // 1: the kept mass of every slice of the row was written with the cut
+  int32_t pad;
 };
 
 // Order-preserving key of a bf16 value given as fp32 bits (low 16 bits zero): sign-magnitude turned into two's
@@ -58,116 +79,35 @@ __device__ __forceinline__ uint32_t f_of_key16(int32_t key16) {
   return key16 >= 0 ? (uint32_t)key16 << 16 : (0x8000u | (uint32_t)(-key16)) << 16;
 }
 // mass of a token in units of 2^-40 relative to the row maximum (at most 2^40): a subtraction, a multiply-add, one
-// exponential, one conversion.  The conversion turns NaN into 0.
+// exponential, one conversion.  The maximum turns NaN into 0 (the conversion alone would make it 2^63).
 __device__ __forceinline__ u64 wfix_of(uint32_t f, float m, float k_log2) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaf(__uint_as_float(f) - m, k_log2, 40.f)));
   u64 r;
-  asm("cvt.rni.u64.f32 %0, %1;" : "=l"(r) : "f"(y));
+  asm("cvt.rni.u64.f32 %0, %1;" : "=l"(r) : "f"(fmaxf(y, 0.f)));
   return r;
 }
 
-// f(e, bits) for every token e of the row (bits = the logit as fp32 bits), threads striding over 16-byte vectors
-template <int kT, class F>
-__device__ __forceinline__ void row_strided(const uint16_t *rp, int32_t vocab, F &&f) {
-  const int32_t n_vec = vocab >> 3;
-  const uint4 *vp = reinterpret_cast<const uint4 *>(rp);
-  for (int32_t v0 = 0; v0 < n_vec; v0 += 4 * kT) {
-    uint4 v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int32_t vi = v0 + k * kT + (int32_t)threadIdx.x;
-      if (vi < n_vec) v[k] = __ldg(vp + vi);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int32_t vi = v0 + k * kT + (int32_t)threadIdx.x;
-      if (vi < n_vec) {
-        const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          f(vi * 8 + 2 * j, w[j] << 16);
-          f(vi * 8 + 2 * j + 1, w[j] & 0xFFFF0000u);
-        }
-      }
-    }
-  }
-  const int32_t e = n_vec * 8 + (int32_t)threadIdx.x;  // vocab not a multiple of 8
-  if (e < vocab) f(e, (uint32_t)__ldg(rp + e) << 16);
+__device__ __forceinline__ bool is_kept(int32_t key, int32_t e, const RowCut &rc) {
+  return key > rc.cut_key || (key == rc.cut_key && e <= rc.cut_idx);
 }
 
-// the same with every thread owning a contiguous range of the row, ranges in thread order: visiting threads in
-// order and each thread's tokens in order is index order
-template <int kT, class F>
-__device__ __forceinline__ void row_blocked(const uint16_t *rp, int32_t vocab, F &&f) {
-  const int32_t n_vec = vocab >> 3, per = (n_vec + kT - 1) / kT;
-  const int32_t v_begin = min(n_vec, (int32_t)threadIdx.x * per), v_end = min(n_vec, v_begin + per);
-  const uint4 *vp = reinterpret_cast<const uint4 *>(rp);
-  for (int32_t v0 = v_begin; v0 < v_end; v0 += 4) {  // four loads in flight
-    uint4 v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (v0 + k < v_end) v[k] = __ldg(vp + v0 + k);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (v0 + k < v_end) {
-        const int32_t vi = v0 + k;
-        const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          f(vi * 8 + 2 * j, w[j] << 16);
-          f(vi * 8 + 2 * j + 1, w[j] & 0xFFFF0000u);
-        }
-      }
-    }
-  }
-  if (threadIdx.x == kT - 1)
-    for (int32_t e = n_vec * 8; e < vocab; ++e) f(e, (uint32_t)__ldg(rp + e) << 16);
+constexpr uint32_t kNegInf2 = 0xFF80FF80u;
+__device__ __forceinline__ uint32_t max_bf2(uint32_t x, uint32_t y) {  // a NaN operand loses
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
+  return r;
 }
-
-// maximum of a row, two bf16 at a time (max.bf16x2 returns the other operand when one is NaN); never below -3e38
-template <int kT>
-__device__ __forceinline__ float row_max(const uint16_t *rp, int32_t vocab, float *s_w, float &thread_max) {
-  const int32_t n_vec = vocab >> 3;
-  const uint4 *vp = reinterpret_cast<const uint4 *>(rp);
-  constexpr uint32_t kNegInf2 = 0xFF80FF80u;
-  uint32_t a = kNegInf2, b = kNegInf2;
-  auto mx = [](uint32_t x, uint32_t y) {
-    uint32_t r;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
-    return r;
-  };
-  for (int32_t v0 = 0; v0 < n_vec; v0 += 4 * kT) {
-    uint4 v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int32_t vi = v0 + k * kT + (int32_t)threadIdx.x;
-      v[k] = vi < n_vec ? __ldg(vp + vi) : make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      a = mx(a, mx(v[k].x, v[k].y));
-      b = mx(b, mx(v[k].z, v[k].w));
-    }
-  }
-  a = mx(a, b);
-  float m = fmaxf(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u));
-  const int32_t e = n_vec * 8 + (int32_t)threadIdx.x;
-  if (e < vocab) m = fmaxf(m, __uint_as_float((uint32_t)__ldg(rp + e) << 16));
-  thread_max = m;  // the largest logit among the tokens this thread looked at
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = m;
-  __syncthreads();
-  float r = s_w[0];
-#pragma unroll
-  for (int k = 1; k < kT / 32; ++k) r = fmaxf(r, s_w[k]);
-  __syncthreads();
-  return fmaxf(r, -3.0e38f);
+__device__ __forceinline__ float lo_f(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float hi_f(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // inclusive scan over the block in thread order; `total` receives the sum over the block
-template <int kT, class T>
+template <int kThreads, class T>
 __device__ __forceinline__ T block_scan(T v, T *s_w, T &total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -179,7 +119,7 @@ __device__ __forceinline__ T block_scan(T v, T *s_w, T &total) {
   __syncthreads();
   T base = 0, all = 0;
 #pragma unroll
-  for (int k = 0; k < kT / 32; ++k) {
+  for (int k = 0; k < kThreads / 32; ++k) {
     const T t = s_w[k];
     if (k < warp) base += t;
     all += t;
@@ -189,17 +129,326 @@ __device__ __forceinline__ T block_scan(T v, T *s_w, T &total) {
   return v + base;
 }
 
+// Candidates are ordered as 64-bit numbers: the key above, the complement of the index below, so that "larger" is
+// "ranked before".
+__device__ __forceinline__ u64 cand_of(uint32_t f, int32_t e) {
+  return ((u64)(uint32_t)((key32(f) >> 16) + 32768) << 32) | (uint32_t)~(uint32_t)e;
+}
+__device__ __forceinline__ int32_t cand_key16(u64 c) { return (int32_t)(c >> 32) - 32768; }
+__device__ __forceinline__ int32_t cand_idx(u64 c) { return (int32_t)~(uint32_t)c; }
+
+// the last vector of a row whose length is not a multiple of 8, padded with -inf
+__device__ __forceinline__ uint4 ragged_vec(const uint16_t *rp, int32_t n_vec, int32_t rem) {
+  uint32_t w[4] = {kNegInf2, kNegInf2, kNegInf2, kNegInf2};
+#pragma unroll
+  for (int j = 0; j < 7; ++j)
+    if (j < rem) {
+      const uint32_t h = rp[(int64_t)n_vec * 8 + j];
+      w[j >> 1] = (j & 1) ? ((w[j >> 1] & 0xFFFFu) | (h << 16)) : ((w[j >> 1] & 0xFFFF0000u) | h);
+    }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// ---- one read of the logits -------------------------------------------------------------------------------
+// A warp per chunk of 2048 logits at a time, no warp ever waiting for another.  A lane's kGV vectors of a chunk, 32 vectors
+// apart, are a group: the group's largest key goes out (2 bytes, biased by 32768), and with kSum the chunk's pair (largest
+// logit, sum of exp((x - largest) / T)).  Bound: HBM (kSum: and the special-function units close behind).
+template <bool kSum, int kGV>
+__global__ void __launch_bounds__(kT, kScanCtasPerSm)
+filter_scan_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, uint32_t n_chunks, uint32_t total,
+                   uint16_t *__restrict__ group_key, float2 *__restrict__ stats, int32_t *__restrict__ n_open) {
+  const int lane = threadIdx.x & 31;
+  const int32_t n_vec = vocab >> 3, rem = vocab & 7;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the logits may come from the kernel launched just before
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (blockIdx.x == 0 && threadIdx.x == 0) *n_open = 0;
+  for (uint32_t unit = blockIdx.x * kWarps + (threadIdx.x >> 5); unit < total; unit += gridDim.x * kWarps) {
+    const uint32_t row = unit / n_chunks;
+    const uint16_t *rp = logits + (int64_t)row * row_stride;
+    const int32_t v0 = (int32_t)(unit - row * n_chunks) * (kChunk / 8) + lane;
+    uint32_t x[kVec * 4];
+#pragma unroll
+    for (int k = 0; k < kVec; ++k) {
+      const int32_t vi = v0 + k * 32;
+      uint4 v = make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
+      if (vi < n_vec)
+        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(reinterpret_cast<const uint4 *>(rp) + vi));
+      x[4 * k] = v.x;
+      x[4 * k + 1] = v.y;
+      x[4 * k + 2] = v.z;
+      x[4 * k + 3] = v.w;
+    }
+    if (rem != 0 && v0 <= n_vec && v0 + kChunk / 8 > n_vec && ((n_vec - v0) & 31) == 0) {  // this lane has the ragged end of the row
+#pragma unroll
+      for (int k = 0; k < kVec; ++k)
+        if (v0 + k * 32 == n_vec) {
+          const uint4 v = ragged_vec(rp, n_vec, rem);
+          x[4 * k] = v.x;
+          x[4 * k + 1] = v.y;
+          x[4 * k + 2] = v.z;
+          x[4 * k + 3] = v.w;
+        }
+    }
+    float top = -INFINITY;
+#pragma unroll
+    for (int k0 = 0; k0 < kVec; k0 += kGV) {
+      uint32_t mx = kNegInf2;
+#pragma unroll
+      for (int i = 4 * k0; i < 4 * (k0 + kGV); ++i) {
+        if (kSum) x[i] = max_bf2(x[i], kNegInf2);  // NaN counts as -inf
+        mx = max_bf2(mx, x[i]);
+      }
+      const float g = fmaxf(lo_f(mx), hi_f(mx));
+      top = fmaxf(top, g);
+      group_key[(int64_t)unit * (32 * kVec / kGV) + (k0 / kGV) * 32 + lane] = (uint16_t)((key32(__float_as_uint(g)) >> 16) + 32768);
+    }
+    if (kSum) {
+      const float off = top > -INFINITY ? -top * k_log2 : 0.f;
+      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+      for (int i = 0; i < kVec * 4; i += 2) {
+        a0 += ex2_approx(fmaf(lo_f(x[i]), k_log2, off));
+        a1 += ex2_approx(fmaf(hi_f(x[i]), k_log2, off));
+        a2 += ex2_approx(fmaf(lo_f(x[i + 1]), k_log2, off));
+        a3 += ex2_approx(fmaf(hi_f(x[i + 1]), k_log2, off));
+      }
+      float M = top;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+      float S = ((a0 + a1) + (a2 + a3)) * ex2_approx(fmaf(top, k_log2, M > -INFINITY ? -M * k_log2 : 0.f));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
+      if (lane == 0) stats[unit] = make_float2(M, S);
+    }
+  }
+}
+
+// tokens of a CTA's share of a row in a cluster of n (a multiple of 8)
+__host__ __device__ __forceinline__ int32_t share_of(int32_t vocab, int n) { return ((vocab + 7) / 8 + n - 1) / n * 8; }
+// tokens of a slice (a multiple of 256; at most kMaxSlices of them)
+__host__ __device__ __forceinline__ int slice_len_of(int32_t vocab) { return 256 * ((vocab + 256 * kMaxSlices - 1) / (256 * kMaxSlices)); }
+
+// ---- the cut of a row from its candidates -----------------------------------------------------------------
+// T, the k_sel-th largest group maximum, is a lower bound of the k_sel-th largest logit (the maxima are logits of different
+// tokens), and only the k_sel groups that reach it (more with ties) hold tokens of at least T: they are read again.
+template <int kGV>
+__global__ void __launch_bounds__(kT)
+filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, int32_t top_k, float top_p, int k_sel,
+                  int n_chunks, const uint16_t *__restrict__ group_key, const float2 *__restrict__ stats, RowCut *__restrict__ cuts,
+                  u64 *__restrict__ slice_mass, int n_slices, int32_t *__restrict__ n_kept_out, int32_t *__restrict__ n_open,
+                  int32_t *__restrict__ open_rows) {
+  extern __shared__ __align__(16) uint32_t s_key2[];  // the row's group keys, two to a word
+  __shared__ __align__(16) u64 s_cand[kListCap];
+  __shared__ u64 s_sorted[kListCap], s_slice[kMaxSlices];
+  __shared__ u64 s_w[kWarps];
+  __shared__ double s_z;
+  __shared__ int s_grp[kGroupCap];
+  __shared__ int s_n, s_n_grp, s_r[2], s_cnt[2][kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t row = blockIdx.x;
+  constexpr int kPerChunk = 32 * kVec / kGV;
+  const int n_words = n_chunks * kPerChunk / 2;
+  if (tid == 0) {
+    s_n = s_n_grp = 0;
+    s_r[0] = s_r[1] = -1;
+  }
+  for (int i = tid; i < n_slices; i += kT) s_slice[i] = 0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the keys come from the kernel launched just before
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const uint4 *src = reinterpret_cast<const uint4 *>(group_key + row * n_chunks * kPerChunk);
+  for (int i = tid; i < n_words / 4; i += kT) reinterpret_cast<uint4 *>(s_key2)[i] = src[i];
+  __syncthreads();
+  uint32_t T = 0;  // bisection on the biased key
+#pragma unroll 1
+  for (int bit = 15; bit >= 0; --bit) {
+    const uint32_t u = T | (1u << bit);
+    int c = 0;
+    for (int i = tid; i < n_words; i += kT) {
+      const uint32_t w = s_key2[i];
+      c += ((w & 0xFFFFu) >= u ? 1 : 0) + ((w >> 16) >= u ? 1 : 0);
+    }
+    c = __reduce_add_sync(0xFFFFFFFFu, c);
+    if (lane == 0) s_cnt[bit & 1][warp] = c;
+    __syncthreads();
+    c = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) c += s_cnt[bit & 1][w];
+    if (c >= k_sel) T = u;
+  }
+  const uint32_t least = max(T, 129u);  // 128 is the key of -inf
+  for (int i = tid; i < n_words; i += kT) {
+    const uint32_t w = s_key2[i];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if ((h ? w >> 16 : w & 0xFFFFu) >= least) {
+        const int at = atomicAdd(&s_n_grp, 1);
+        if (at < kGroupCap) s_grp[at] = 2 * i + h;
+      }
+  }
+  __syncthreads();
+  const int n_grp = s_n_grp;
+  const uint16_t *rp = logits + row * row_stride;
+  if (n_grp <= kGroupCap) {
+    const int32_t n_vec = vocab >> 3, rem = vocab & 7;
+    for (int i = tid; i < n_grp * kGV; i += kT) {
+      const int g = s_grp[i / kGV];
+      const int32_t vi = (g / kPerChunk) * (kChunk / 8) + (g % kPerChunk) + (i % kGV) * 32;
+      if (vi > n_vec || (vi == n_vec && rem == 0)) continue;
+      const uint4 v = vi < n_vec ? __ldg(reinterpret_cast<const uint4 *>(rp) + vi) : ragged_vec(rp, n_vec, rem);
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
+        const float x = __uint_as_float(f);
+        if (x == x && (uint32_t)((key32(f) >> 16) + 32768) >= least) {
+          const int at = atomicAdd(&s_n, 1);
+          if (at < kListCap) s_cand[at] = cand_of(f, vi * 8 + j);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  const int n = s_n;
+  const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
+  bool ok = n_grp <= kGroupCap && n >= 1 && n <= kListCap && (!by_k || n >= top_k);
+  if (ok)
+    for (int i = tid; i < n; i += kT) {  // rank by counting: the candidates are all different
+      const u64 e = s_cand[i];
+      int before = 0;
+#pragma unroll 8
+      for (int j = 0; j < n; ++j) before += s_cand[j] > e ? 1 : 0;
+      s_sorted[before] = e;
+    }
+  __syncthreads();
+  float m = 0.f;
+  if (ok) {
+    m = __uint_as_float(f_of_key16(cand_key16(s_sorted[0])));
+    ok = fabsf(m) < INFINITY;
+  }
+  constexpr int kPer = kListCap / kT;
+  u64 w[kPer], mine = 0, all = 0, before = 0;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int r = tid * kPer + i;
+    w[i] = ok && r < n ? wfix_of(f_of_key16(cand_key16(s_sorted[r])), m, k_log2) : 0;
+    mine += w[i];
+  }
+  before = block_scan<kT, u64>(mine, s_w, all) - mine;
+  // the last rank kept: top_k - 1, or the first one at which the mass, itself included, reaches t = ceil(top_p W), where W
+  // is the mass of the leading top_k ranks, or -- to within kMassEps -- of the whole row
+  if (by_k) {
+    u64 cum = before;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      cum += w[i];
+      if (tid * kPer + i == top_k - 1) s_w[0] = cum;
+    }
+    if (tid == 0) s_r[0] = s_r[1] = top_k - 1;
+  } else if (warp == 0) {
+    double z = 0.0;
+    for (int i = lane; i < n_chunks; i += 32) {
+      const float2 h = stats[row * n_chunks + i];
+      z += (double)(h.y * ex2_approx((h.x - m) * k_log2));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+    if (lane == 0) s_z = z * 1099511627776.0;  // units of 2^-40
+  }
+  __syncthreads();
+  if (by_p && ok) {
+    u64 t[2];
+    if (by_k) {
+      const u64 w_k = s_w[0];
+      const double t_d = ceil((double)top_p * (double)w_k);
+      t[0] = t_d < 1.0 ? 1ull : (u64)t_d;
+      if (t[0] > w_k) t[0] = w_k;
+      t[1] = t[0];
+      ok = w_k > 0;
+    } else {
+      t[0] = (u64)((double)top_p * s_z * (1.0 - kMassEps));
+      t[1] = (u64)((double)top_p * s_z * (1.0 + kMassEps)) + 2;
+      ok = t[0] > 0 && t[1] <= all;  // else the cut may lie beyond the candidates
+    }
+    __syncthreads();
+    if (ok) {
+      u64 cum = before;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const u64 next = cum + w[i];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          if (cum < t[q] && t[q] <= next) s_r[q] = tid * kPer + i;
+        cum = next;
+      }
+    }
+    __syncthreads();
+  }
+  const int r = s_r[0];
+  ok = ok && r >= 0 && r == s_r[1];
+  if (!ok) {
+    if (tid == 0) open_rows[atomicAdd(n_open, 1)] = (int32_t)row;
+    return;
+  }
+  {
+    u64 cum = before;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int at = tid * kPer + i;
+      cum += w[i];
+      if (at <= r && w[i] > 0) atomicAdd(&s_slice[cand_idx(s_sorted[at]) / slice_len_of(vocab)], w[i]);
+      if (at == r) {
+        RowCut rc;
+        rc.m = m;
+        rc.cut_key = cand_key16(s_sorted[at]) * 65536;
+        rc.cut_idx = cand_idx(s_sorted[at]);
+        rc.n_kept = r + 1;
+        rc.z_fix = cum;
+        rc.slices = 1;
+        rc.pad = 0;
+        cuts[row] = rc;
+        if (n_kept_out != nullptr) n_kept_out[row] = r + 1;
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < n_slices; i += kT) slice_mass[row * n_slices + i] = s_slice[i];
+}
+
+// ---- the cut of a row from counts per key: a cluster of kC CTAs per row --------------------------------------
 struct KeyCut {  // the last token kept: a key, and how many of the tokens with that key
   int32_t key;         // key16
-  uint32_t j;          // tokens of the key that are kept (>= 1 when found)
+  uint32_t j;          // tokens of the key that are kept (0: not found here)
   uint32_t cnt_key;    // tokens of the key
   uint32_t cnt_above;  // tokens with a larger key
   u64 mass_above;      // their mass
   u64 w_key;           // mass of one token of the key
 };
 
-// A window of kWin consecutive keys, hi down to hi - kWin + 1: per-key token counts in shared memory (position d
-// is key hi - d; keys here are key16), and what lies above the window.
+struct Xch {  // what a CTA tells the others in one exchange
+  u64 mass;
+  uint32_t cnt;
+  int32_t key;
+  KeyCut cut;
+};
+
+struct WindowShared {
+  uint32_t cnt[kWin];  // counts of this CTA's tokens
+  Xch xch[2];          // one for even, one for odd exchanges: a slot is written again only after every CTA has left the
+                       // barrier of the exchange in between, hence has read it
+  u64 w64[kWT / 32];
+  uint32_t w32[kWT / 32];
+  int32_t wi[kWT / 32];
+};
+
+// Counts cover kWin keys at a time.  The usual ones are fixed: position 0 is the largest key below 2^12, position 4095
+// that of 2^-20, position 4096 zero, the rest -2^-20 down to -2^12 (its last key left out): one pass, with no branch that
+// tokens take both ways, and nothing to know in advance.  A row that holds other finite values is counted again over
+// windows of kWin consecutive keys, hi down to hi - kWin + 1, from the row maximum down (a NaN is never counted).
+constexpr uint32_t kMag0 = (127 - 20) << 7;  // bf16 bits of 2^-20
+__device__ __forceinline__ int32_t fixed_key16(int pos) {
+  return pos < 4096 ? (int32_t)kMag0 + 4095 - pos : pos == 4096 ? 0 : -((int32_t)kMag0 + pos - 4097);
+}
 struct Window {
   int32_t hi;
   int32_t next_hi;     // the largest key below the window that occurs in the row; kNoKey if none
@@ -209,304 +458,375 @@ struct Window {
   u64 mass;            // their mass
 };
 
-struct FilterShared {
-  uint32_t cnt[kWin];
-  u64 w64[kFT / 32];
-  uint32_t w32[kFT / 32];
-  float wf[kFT / 32];
-  int32_t wi[kFT / 32];
-  KeyCut cut;
-  int32_t cut_idx;
-};
-
-template <int kT>
-__device__ __forceinline__ int32_t block_max_i32(int32_t v, int32_t *s_w) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
-  __syncthreads();
-  int32_t r = s_w[0];
-#pragma unroll
-  for (int k = 1; k < kT / 32; ++k) r = max(r, s_w[k]);
-  __syncthreads();
-  return r;
-}
-
-// One pass over the row: counts of the keys inside the window starting at `hi`.  On the first window (kFirst) the
-// mass of everything below the window is summed too, so that the mass of the whole row is known.  Tokens whose
-// logit is below `floor_x` are left out altogether (-inf: none is; a NaN always is).
-template <bool kFirst>
-__device__ __forceinline__ void build_window(FilterShared &sh, const uint16_t *rp, int32_t vocab, float m, float k_log2,
-                                             float floor_x, int32_t hi, Window &win, u64 &mass_below) {
-  for (int i = threadIdx.x; i < kWin; i += kFT) sh.cnt[i] = 0;
-  __syncthreads();
-  int32_t nh = kNoKey;
-  u64 rest = 0;
-  const int32_t hi32 = hi * 65536;
-  row_strided<kFT>(rp, vocab, [&](int32_t, uint32_t f) {
-    if (!(__uint_as_float(f) >= floor_x)) return;
-    const int32_t k32 = key32(f);
-    if (k32 <= hi32) {  // keys above the window were counted by an earlier pass (a NaN beyond +inf: never)
-      const uint32_t d = ((uint32_t)hi32 - (uint32_t)k32) >> 16;
-      if (d < (uint32_t)kWin) {
-        atomicAdd(&sh.cnt[d], 1u);
-      } else {
-        nh = max(nh, k32);
-        if (kFirst) rest += wfix_of(f, m, k_log2);
-      }
-    }
-  });
-  __syncthreads();
-  win.hi = hi;
-  nh = block_max_i32<kFT>(nh, sh.wi);
-  win.next_hi = nh == kNoKey ? kNoKey : nh >> 16;
-  if (kFirst) {
-    u64 all;
-    block_scan<kFT, u64>(rest, sh.w64, all);
-    mass_below = all;
-  }
-}
-
-// Per-thread view of the window: thread t owns positions t kPer .. t kPer + kPer - 1 (keys descending)
-struct Mine {
-  uint32_t c_excl;  // tokens of the window before this thread's positions
-  u64 m_excl;       // their mass
-  uint32_t c_sum;
-  u64 m_sum;
-};
-
-__device__ __forceinline__ u64 w_of_pos(const Window &win, int pos, float m, float k_log2) {
-  return wfix_of(f_of_key16(win.hi - pos), m, k_log2);
-}
-
-__device__ __forceinline__ void scan_window(FilterShared &sh, Window &win, Mine &me, float m, float k_log2) {
-  me.c_sum = 0;
-  me.m_sum = 0;
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const uint32_t c = sh.cnt[threadIdx.x * kPer + i];
-    if (c != 0) {
-      me.c_sum += c;
-      me.m_sum += (u64)c * w_of_pos(win, threadIdx.x * kPer + i, m, k_log2);  // all tokens of a key weigh the same
-    }
-  }
-  me.c_excl = block_scan<kFT, uint32_t>(me.c_sum, sh.w32, win.cnt) - me.c_sum;
-  me.m_excl = block_scan<kFT, u64>(me.m_sum, sh.w64, win.mass) - me.m_sum;
-}
-
-// The key of the window at which the token count (from the top of the ranking) reaches k, or at which the mass
-// reaches t; the caller has made sure that it lies inside the window.  Every thread returns the same value.
-template <bool kByMass>
-__device__ __forceinline__ KeyCut locate(FilterShared &sh, const Window &win, const Mine &me, uint32_t k, u64 t, float m,
-                                         float k_log2) {
-  const uint32_t k_rel = k - win.cnt_above;
-  const u64 t_rel = t - win.mass_above;
-  const bool mine = kByMass ? (me.m_sum > 0 && me.m_excl < t_rel && t_rel <= me.m_excl + me.m_sum)
-                            : (me.c_excl < k_rel && k_rel <= me.c_excl + me.c_sum);
-  if (mine) {
-    uint32_t cnt = me.c_excl;
-    u64 mass = me.m_excl;
-    bool done = false;
-    for (int i = 0; i < kPer; ++i) {
-      const uint32_t c = sh.cnt[threadIdx.x * kPer + i];
-      if (c != 0 && !done) {
-        const int pos = threadIdx.x * kPer + i;
-        const u64 w = w_of_pos(win, pos, m, k_log2);
-        const bool here = kByMass ? (w > 0 && mass + (u64)c * w >= t_rel) : (cnt + c >= k_rel);
-        if (here) {
-          KeyCut r;
-          r.key = win.hi - pos;
-          r.cnt_key = c;
-          r.cnt_above = win.cnt_above + cnt;
-          r.mass_above = win.mass_above + mass;
-          r.w_key = w;
-          r.j = kByMass ? (uint32_t)((t_rel - mass + w - 1) / w) : (k_rel - cnt);
-          sh.cut = r;
-          done = true;
-        }
-        cnt += c;
-        mass += (u64)c * w;
-      }
-    }
-  }
-  __syncthreads();
-  const KeyCut r = sh.cut;
-  __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(kFT, 1)
-filter_rows_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, int32_t top_k,
-                   float top_p, RowCut *__restrict__ cuts, int32_t *__restrict__ n_kept_out) {
-  __shared__ FilterShared sh;
-  const int tid = threadIdx.x;
-  const int64_t row = blockIdx.x;
-  const uint16_t *rp = logits + row * row_stride;
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the logits may come from the kernel launched just before
+// The row is cut into kC contiguous shares, CTA rank order being index order; a share sits in shared memory when it fits
+// (cached != 0), else every pass reads it from L2.  All exchanged values are the same in every CTA, so every CTA takes the
+// same way through the cluster barriers.  Bound: the instructions of the count pass (about ten a token) and a chain of five
+// cluster barriers.
+template <int kC>
+__global__ void __launch_bounds__(kWT, 2)
+filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, int32_t top_k, float top_p,
+                     RowCut *__restrict__ cuts, int32_t *__restrict__ n_kept_out, const int32_t *__restrict__ n_open,
+                     const int32_t *__restrict__ open_rows, int n_all, int cached) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  WindowShared &sh = *reinterpret_cast<WindowShared *>(smem_raw);
+  uint16_t *s_row = reinterpret_cast<uint16_t *>(smem_raw + (sizeof(WindowShared) + 15) / 16 * 16);
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = (int)cluster.block_rank();
+  constexpr int kPW = kWin / kC, kPer = kPW / kWT;  // positions of this CTA and of one thread
+  const int32_t share = share_of(vocab, kC), e0 = min(vocab, rank * share), e1 = min(vocab, e0 + share);
+  const int32_t n_vec = (e1 - e0) >> 3, rem = (e1 - e0) & 7;
+  const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int n_rows = n_all > 0 ? n_all : *n_open;
+  int ph = 0;
 
-  // ---- pass 0: the row maximum
-  if (tid == 0) {
-    sh.cut_idx = INT32_MAX;
-    sh.cut.j = 0;
-  }
-  float thread_max;
-  const float m = row_max<kFT>(rp, vocab, sh.wf, thread_max);
-  const int32_t key_top = key32(__float_as_uint(m)) >> 16;
-
-  // ---- pass 1: the window that starts at the largest key, and the mass of the whole row
-  Window win;
-  Mine me;
-  u64 mass_below = 0;
-  win.cnt_above = 0;
-  win.mass_above = 0;
-  const uint32_t cnt_total = (uint32_t)vocab;
-  const bool by_k = top_k > 0 && (uint32_t)top_k < cnt_total;
-  const bool by_p = top_p < 1.f;
-  // With top-k on and k no larger than the number of threads, the k-th largest of the threads' own maxima (each is
-  // the logit of a different token) is a lower bound of the k-th largest logit of the row: tokens below it cannot be
-  // kept, and the passes that follow skip them after one comparison.
-  float floor_x = -INFINITY;
-  if (by_k && top_k <= kFT) {
-    for (int i = tid; i < kWin; i += kFT) sh.cnt[i] = 0;
+  auto peer = [&](int r) -> const Xch * { return cluster.map_shared_rank(&sh.xch[ph], r); };
+  auto block_max = [&](int32_t v) -> int32_t {
+    v = __reduce_max_sync(0xFFFFFFFFu, v);
+    if (lane == 0) sh.wi[warp] = v;
     __syncthreads();
-    const int32_t k32 = key32(__float_as_uint(thread_max));
-    const uint32_t d = ((uint32_t)(key_top * 65536) - (uint32_t)k32) >> 16;  // thread_max <= m
-    if (thread_max > -INFINITY && d < (uint32_t)kWin) atomicAdd(&sh.cnt[d], 1u);
+    const int32_t r = __reduce_max_sync(0xFFFFFFFFu, lane < kWT / 32 ? sh.wi[lane] : INT32_MIN);
     __syncthreads();
-    win.hi = key_top;
-    scan_window(sh, win, me, m, k_log2);
-    if ((uint32_t)top_k <= win.cnt) {
-      const KeyCut kc = locate<false>(sh, win, me, (uint32_t)top_k, 0, m, k_log2);
-      floor_x = __uint_as_float(f_of_key16(kc.key));
+    return r;
+  };
+  // key: maximum over the cluster; cnt, mass: sums over the cluster and over the CTAs of lower rank.  Lane q of every warp
+  // reads what CTA q says.
+  struct Sums { int32_t key; uint32_t cnt, cnt_before; u64 mass, mass_before; };
+  auto exchange = [&](int32_t key, uint32_t cnt, u64 mass) -> Sums {
+    if (tid == 0) {
+      sh.xch[ph].key = key;
+      sh.xch[ph].cnt = cnt;
+      sh.xch[ph].mass = mass;
     }
-    __syncthreads();
-  }
-  // the mass of the whole row is needed only when top-k does not cut: else the mass of the top k takes its place
-  if (by_k) build_window<false>(sh, rp, vocab, m, k_log2, floor_x, key_top, win, mass_below);
-  else build_window<true>(sh, rp, vocab, m, k_log2, floor_x, key_top, win, mass_below);
-  scan_window(sh, win, me, m, k_log2);
-  const u64 mass_total = win.mass + mass_below;
-
-  auto advance = [&]() -> bool {  // the next window down; false when nothing is left below
-    if (win.next_hi == kNoKey) return false;
-    win.cnt_above += win.cnt;
-    win.mass_above += win.mass;
-    u64 unused;
-    build_window<false>(sh, rp, vocab, m, k_log2, floor_x, win.next_hi, win, unused);
-    scan_window(sh, win, me, m, k_log2);
-    return true;
+    cluster.sync();
+    Sums r = {INT32_MIN, 0, 0, 0, 0};
+    if (lane < kC) {
+      const Xch *x = peer(lane);
+      r.key = x->key;
+      r.cnt = x->cnt;
+      r.mass = x->mass;
+    }
+    r.cnt_before = __reduce_add_sync(0xFFFFFFFFu, lane < rank ? r.cnt : 0u);
+    r.cnt = __reduce_add_sync(0xFFFFFFFFu, r.cnt);
+    r.key = __reduce_max_sync(0xFFFFFFFFu, r.key);
+    u64 all = 0;
+#pragma unroll
+    for (int q = 0; q < kC; ++q) {
+      if (q == rank) r.mass_before = all;
+      all += __shfl_sync(0xFFFFFFFFu, r.mass, q);
+    }
+    r.mass = all;
+    ph ^= 1;
+    return r;
+  };
+  auto clear_counts = [&]() {
+    for (int i = tid; i < kWin / 4; i += kWT) reinterpret_cast<uint4 *>(sh.cnt)[i] = make_uint4(0, 0, 0, 0);
   };
 
-  KeyCut cut;
-  bool have_cut = false;
-  u64 w_k = mass_total;  // mass of what top-k keeps
-  uint32_t n_all = cnt_total;
+  for (int at = (int)blockIdx.x / kC; at < n_rows; at += (int)gridDim.x / kC) {
+    const int64_t row = n_all > 0 ? at : open_rows[at];
+    const uint16_t *gp = logits + row * row_stride + e0;
+    const uint16_t *rp = cached ? s_row : gp;
 
-  if (by_k) {
-    const uint32_t k = (uint32_t)top_k;
-    bool ok = true;
-    while (ok && k > win.cnt_above + win.cnt) ok = advance();
-    if (ok) {
-      cut = locate<false>(sh, win, me, k, 0, m, k_log2);
-      have_cut = true;
-      w_k = cut.mass_above + (u64)cut.j * cut.w_key;
-    } else {  // fewer than k tokens that are numbers: every window was visited, nothing is cut
-      w_k = win.mass_above + win.mass;
-      n_all = win.cnt_above + win.cnt;
+    // ---- the share into shared memory; counts of the fixed keys; the row maximum
+    if (cached) {
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_row);
+      for (int32_t vi = tid; vi < n_vec; vi += kWT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + vi * 16), "l"(gp + (int64_t)vi * 8) : "memory");
+      if (tid < rem) s_row[n_vec * 8 + tid] = gp[n_vec * 8 + tid];
     }
-  }
-  if (by_p && w_k > 0) {
-    // rank r stays iff the mass ranked before it is below top_p W_k: the last one kept is the first rank at which
-    // the mass, itself included, reaches t
-    const double t_d = ceil((double)top_p * (double)w_k);
-    u64 t = t_d < 1.0 ? 1ull : (u64)t_d;
-    if (t > w_k) t = w_k;
-    bool ok = true;
-    if (t <= win.mass_above) {  // the top-k search went past it: start again from the top
-      win.cnt_above = 0;
-      win.mass_above = 0;
-      u64 unused;
-      build_window<false>(sh, rp, vocab, m, k_log2, floor_x, key_top, win, unused);
-      scan_window(sh, win, me, m, k_log2);
-    }
-    while (ok && t > win.mass_above + win.mass) ok = advance();
-    if (ok) {
-      KeyCut cp = locate<true>(sh, win, me, 0, t, m, k_log2);
-      if (have_cut && cp.key == cut.key) cp.j = min(cp.j, cut.j);  // (already implied by t <= W_k)
-      cut = cp;
-      have_cut = true;
-    }
-  }
-
-  // ---- last pass, only when the cut splits a group of equal keys: the index of the last one kept
-  if (have_cut && cut.j < cut.cnt_key) {
-    uint32_t mine = 0;
-    const int32_t cut32 = cut.key * 65536;
-    row_blocked<kFT>(rp, vocab, [&](int32_t, uint32_t f) { mine += key32(f) == cut32 ? 1u : 0u; });
-    uint32_t all;
-    const uint32_t before = block_scan<kFT, uint32_t>(mine, sh.w32, all) - mine;
-    if (before < cut.j && cut.j <= before + mine) {
-      uint32_t seen = before;
-      row_blocked<kFT>(rp, vocab, [&](int32_t e, uint32_t f) {
-        if (key32(f) == cut32 && ++seen == cut.j) sh.cut_idx = e;
-      });
-    }
+    clear_counts();
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-  }
-  if (tid == 0) {
-    RowCut rc;
-    rc.m = m;
-    rc.cut_key = have_cut ? cut.key * 65536 : kNoKey;
-    rc.cut_idx = sh.cut_idx;
-    rc.n_kept = have_cut ? (int32_t)(cut.cnt_above + cut.j) : (int32_t)n_all;
-    rc.z_fix = have_cut ? cut.mass_above + (u64)cut.j * cut.w_key : w_k;
-    rc.reserved = 0;
-    cuts[row] = rc;
-    if (n_kept_out != nullptr) n_kept_out[row] = rc.n_kept;
+    uint32_t mx = kNegInf2;
+    int odd = 0;  // finite values outside the fixed keys
+    auto count = [&](uint32_t u) {
+      const uint32_t mag = u & 0x7FFFu, t = mag - kMag0;
+      const bool neg = u > 0x7FFFu;
+      if (t < (neg ? 4095u : 4096u)) atomicAdd(&sh.cnt[neg ? 4097 + t : 4095 - t], 1u);
+      else if (mag == 0) atomicAdd(&sh.cnt[4096], 1u);
+      else odd |= (mag < 0x7F80u || u == 0x7F80u) ? 1 : 0;
+    };
+    for (int32_t vi = tid; vi < n_vec; vi += kWT) {
+      const uint4 v = reinterpret_cast<const uint4 *>(rp)[vi];
+      mx = max_bf2(mx, max_bf2(max_bf2(v.x, v.y), max_bf2(v.z, v.w)));
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        count(w[j] & 0xFFFFu);
+        count(w[j] >> 16);
+      }
+    }
+    float top = fmaxf(lo_f(mx), hi_f(mx));
+    if (tid < rem) {
+      const uint32_t u = rp[n_vec * 8 + tid];
+      count(u);
+      top = fmaxf(top, __uint_as_float(u << 16));
+    }
+    odd = __syncthreads_or(odd);
+    const Sums first = exchange(block_max(key32(__float_as_uint(top))), odd ? 1u : 0u, 0);
+    const float m = fmaxf(__uint_as_float(f_of_key16(first.key >> 16)), -3.0e38f);  // finite: a row without a finite logit
+    const int32_t key_top = key32(__float_as_uint(m)) >> 16;
+
+    // ---- the cut
+    KeyCut cut;
+    cut.j = 0;
+    bool have_cut = false;
+    uint32_t n_kept_all = (uint32_t)vocab;
+    u64 w_k = 0, t = 0;  // mass of what top-k keeps; the mass top-p's cut has to reach
+    // rank r stays iff the mass ranked before it is below top_p W_k: the last one kept is the first rank at which the
+    // mass, itself included, reaches t
+    auto target_of = [&](u64 w) -> u64 {
+      const double t_d = ceil((double)top_p * (double)w);
+      return min(t_d < 1.0 ? 1ull : (u64)t_d, w);
+    };
+    bool fixed = first.cnt == 0 && first.key > (-32640 * 65536);  // some finite logit, and all of them counted
+    bool counting = by_k;   // looking for the k-th token; after it, or without it, for the mass t
+    bool whole = !by_k;     // the first pass also gives the mass of the whole row
+    Window win;
+    win.hi = key_top;
+    win.next_hi = kNoKey;
+    win.cnt_above = 0;
+    win.mass_above = 0;
+    bool search = true;
+#pragma unroll 1
+    while (search) {
+      u64 mass_below = 0;
+      if (!fixed) {
+        clear_counts();
+        __syncthreads();
+        int32_t nh = kNoKey;
+        u64 rest = 0, rest_all = 0;
+        const int32_t hi32 = win.hi * 65536;
+        auto count_in = [&](uint32_t f) {
+          const int32_t k32 = key32(f);
+          const float x = __uint_as_float(f);
+          if (k32 <= hi32 && x == x) {  // keys above the window were counted by an earlier pass
+            const uint32_t d = ((uint32_t)hi32 - (uint32_t)k32) >> 16;
+            if (d < (uint32_t)kWin) {
+              atomicAdd(&sh.cnt[d], 1u);
+            } else {
+              nh = max(nh, k32);
+              if (whole) rest += wfix_of(f, m, k_log2);
+            }
+          }
+        };
+#pragma unroll 1
+        for (int32_t vi = tid; vi < n_vec; vi += kWT) {
+          const uint4 v = reinterpret_cast<const uint4 *>(rp)[vi];
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll 1
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t x = j == 0 ? w[0] : j == 1 ? w[1] : j == 2 ? w[2] : w[3];
+            count_in(x << 16);
+            count_in(x & 0xFFFF0000u);
+          }
+        }
+        if (tid < rem) count_in((uint32_t)rp[n_vec * 8 + tid] << 16);
+        if (whole) block_scan<kWT, u64>(rest, sh.w64, rest_all);
+        const Sums below = exchange(block_max(nh), 0, rest_all);  // (its barrier also makes the counts visible to the cluster)
+        win.next_hi = below.key == kNoKey ? kNoKey : below.key >> 16;
+        mass_below = below.mass;
+      }
+      // every CTA sums the kPW positions it is given over the cluster; this thread has kPer of them, from pos0
+      const int pos0 = rank * kPW + tid * kPer;
+      auto key_of = [&](int i) -> int32_t { return fixed ? fixed_key16(pos0 + i) : win.hi - (pos0 + i); };
+      auto w_of = [&](int i) -> u64 { return wfix_of(f_of_key16(key_of(i)), m, k_log2); };
+      uint32_t c[kPer], c_sum = 0, c_all;
+      u64 m_sum = 0, m_all;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) c[i] = 0;
+#pragma unroll
+      for (int q = 0; q < kC; ++q) {
+        const uint32_t *rc = cluster.map_shared_rank(sh.cnt, q) + pos0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) c[i] += rc[i];
+      }
+#pragma unroll
+      for (int i = 0; i < kPer; ++i)
+        if (c[i] != 0) {
+          c_sum += c[i];
+          m_sum += (u64)c[i] * w_of(i);  // all tokens of a key weigh the same
+        }
+      uint32_t c_excl = block_scan<kWT, uint32_t>(c_sum, sh.w32, c_all) - c_sum;
+      u64 m_excl = block_scan<kWT, u64>(m_sum, sh.w64, m_all) - m_sum;
+      const Sums sums = exchange(0, c_all, m_all);  // (after it the counts may be cleared again)
+      c_excl += sums.cnt_before;
+      m_excl += sums.mass_before;
+      win.cnt = sums.cnt;
+      win.mass = sums.mass;
+      if (whole) {
+        whole = false;
+        w_k = win.mass + mass_below;
+        t = target_of(w_k);
+        if (!by_p || w_k == 0) break;
+      }
+      if (fixed && counting && (uint32_t)top_k > win.cnt) {  // fewer finite logits than k
+        fixed = false;
+        continue;
+      }
+      // what lies here?  First the k-th token, then, perhaps in the same window, the mass t.
+#pragma unroll 1
+      for (;;) {
+        const bool hit = counting ? (uint32_t)top_k <= win.cnt_above + win.cnt : t <= win.mass_above + win.mass;
+        if (hit) {
+          if (tid == 0) sh.xch[ph].cut.j = 0;
+          __syncthreads();
+          const uint32_t k_rel = (uint32_t)top_k - win.cnt_above;
+          const u64 t_rel = t - win.mass_above;
+          if (counting ? (c_excl < k_rel && k_rel <= c_excl + c_sum) : (m_sum > 0 && m_excl < t_rel && t_rel <= m_excl + m_sum)) {
+            uint32_t cnt = c_excl;
+            u64 mass = m_excl;
+            bool done = false;
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+              if (c[i] != 0 && !done) {
+                const u64 w = w_of(i);
+                if (counting ? (cnt + c[i] >= k_rel) : (w > 0 && mass + (u64)c[i] * w >= t_rel)) {
+                  KeyCut r;
+                  r.key = key_of(i);
+                  r.cnt_key = c[i];
+                  r.cnt_above = win.cnt_above + cnt;
+                  r.mass_above = win.mass_above + mass;
+                  r.w_key = w;
+                  r.j = counting ? (k_rel - cnt) : (uint32_t)((t_rel - mass + w - 1) / w);
+                  sh.xch[ph].cut = r;
+                  done = true;
+                }
+                cnt += c[i];
+                mass += (u64)c[i] * w;
+              }
+          }
+          cluster.sync();
+          const unsigned has = __ballot_sync(0xFFFFFFFFu, lane < kC && peer(lane & (kC - 1))->cut.j != 0);
+          const KeyCut found = peer(has ? __ffs(has) - 1 : 0)->cut;  // (some CTA always has it)
+          const uint32_t j_k = have_cut && found.key == cut.key ? cut.j : found.j;
+          cut = found;
+          cut.j = min(cut.j, j_k);  // top-p keeps no more of a key than top-k did (implied by t <= W_k)
+          have_cut = true;
+          ph ^= 1;
+        }
+        if (counting && (hit || win.next_hi == kNoKey)) {
+          if (hit) {
+            w_k = cut.mass_above + (u64)cut.j * cut.w_key;
+          } else {  // fewer than k tokens that are numbers: every window was visited, nothing is cut
+            w_k = win.mass_above + win.mass;
+            n_kept_all = win.cnt_above + win.cnt;
+          }
+          counting = false;
+          search = by_p && w_k > 0;
+          t = target_of(w_k);
+          if (search && t > win.mass_above) continue;  // look for it in this window first
+          win.hi = key_top;  // the top-k search went past it: start again from the top
+          win.cnt_above = 0;
+          win.mass_above = 0;
+          break;
+        }
+        if (hit || win.next_hi == kNoKey) {
+          search = false;
+          break;
+        }
+        win.cnt_above += win.cnt;
+        win.mass_above += win.mass;
+        win.hi = win.next_hi;
+        break;
+      }
+    }
+    const bool split = have_cut && cut.j < cut.cnt_key;
+    if (rank == 0 && tid == 0) {
+      RowCut *rc = cuts + row;
+      rc->m = m;
+      rc->cut_key = have_cut ? cut.key * 65536 : kNoKey;
+      if (!split) rc->cut_idx = INT32_MAX;  // else whoever holds the last token kept of the group writes it
+      rc->n_kept = have_cut ? (int32_t)(cut.cnt_above + cut.j) : (int32_t)n_kept_all;
+      rc->z_fix = have_cut ? cut.mass_above + (u64)cut.j * cut.w_key : w_k;
+      rc->slices = 0;
+      if (n_kept_out != nullptr) n_kept_out[row] = have_cut ? (int32_t)(cut.cnt_above + cut.j) : (int32_t)n_kept_all;
+    }
+    // ---- only when the cut splits a group of equal keys (the usual thing with bf16): the index of the last one kept.
+    //      Threads own contiguous runs of vectors; equality of the values is equality of the keys.
+    if (split) {
+      const uint32_t cb = f_of_key16(cut.key) >> 16, pat = cb | (cb << 16);
+      const int32_t per = (n_vec + kWT - 1) / kWT, v0 = min(n_vec, tid * per), v1 = min(n_vec, v0 + per);
+      auto equal = [&](uint32_t w) -> uint32_t {
+        return __heq2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w), *reinterpret_cast<const __nv_bfloat162 *>(&pat));
+      };
+      uint32_t mine = 0, all;
+      for (int32_t vi = v0; vi < v1; ++vi) {
+        const uint4 v = reinterpret_cast<const uint4 *>(rp)[vi];
+        mine += __popc(equal(v.x)) + __popc(equal(v.y)) + __popc(equal(v.z)) + __popc(equal(v.w));
+      }
+      mine >>= 4;  // 16 bits to a value
+      if (tid == kWT - 1)
+        for (int j = 0; j < rem; ++j) mine += equal(rp[n_vec * 8 + j]) & 1u;
+      uint32_t before = block_scan<kWT, uint32_t>(mine, sh.w32, all) - mine;
+      before += exchange(0, all, 0).cnt_before;
+      if (before < cut.j && cut.j <= before + mine) {
+        uint32_t seen = before;
+        int32_t found = -1;
+#pragma unroll 1
+        for (int32_t i = v0 * 8; i < (tid == kWT - 1 ? n_vec * 8 + rem : v1 * 8) && found < 0; ++i)
+          if ((equal(rp[i]) & 1u) && ++seen == cut.j) found = e0 + i;
+        cuts[row].cut_idx = found;
+      }
+    }
+    cluster.sync();  // nobody leaves, or starts on the next row, while its shared memory is being read
   }
 }
 
-__device__ __forceinline__ bool is_kept(int32_t key, int32_t e, const RowCut &rc) {
-  return key > rc.cut_key || (key == rc.cut_key && e <= rc.cut_idx);
-}
-
-__global__ void __launch_bounds__(kST)
+// ---- acceptance: a cluster of kC CTAs per branch ----------------------------------------------------------
+// Every CTA walks the chain; the stop row's kept masses per slice come with the cut, or, when the cut came from the
+// windows, are summed here, each CTA taking a share of the row.
+template <int kC>
+__global__ void __launch_bounds__(kT)
 accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2,
-                       const RowCut *__restrict__ cuts, const int32_t *__restrict__ draft_ids,
-                       const int32_t *__restrict__ cu_draft, const float *__restrict__ u_accept,
-                       const float *__restrict__ u_final, int32_t *__restrict__ n_accept, int32_t *__restrict__ final_id,
-                       float *__restrict__ p_draft) {
-  __shared__ u64 s_w64[kST / 32];
-  __shared__ int s_n;
-  __shared__ int32_t s_final;
-  const int b = blockIdx.x, tid = threadIdx.x;
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the cuts come from the kernel launched just before
+                       const RowCut *__restrict__ cuts, const u64 *__restrict__ slice_mass, int n_slices,
+                       const int32_t *__restrict__ draft_ids, const int32_t *__restrict__ cu_draft,
+                       const float *__restrict__ u_accept, const float *__restrict__ u_final, int32_t *__restrict__ n_accept,
+                       int32_t *__restrict__ final_id, float *__restrict__ p_draft) {
+  __shared__ u64 s_mass[kMaxSlices], s_w64[kWarps];
+  __shared__ u64 s_before, s_total;
+  __shared__ int s_n, s_slice;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int b = blockIdx.x / kC, rank = kC == 1 ? 0 : (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the cuts come from the kernels launched just before
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int32_t d0 = cu_draft[b], L = cu_draft[b + 1] - d0, r0 = d0 + b;
+  const double u_fin = (double)u_final[b];
   if (tid == 0) {
     s_n = L;
-    s_final = 0;
+    s_slice = -1;
   }
   __syncthreads();
 
   // ---- acceptance chain: draft i passes iff u_i < P'_i(d_i); the first one that does not ends it
-  for (int i = tid; i < L; i += kST) {
+  for (int i = tid; i < L; i += kT) {
     const RowCut rc = cuts[r0 + i];
     const int32_t d = draft_ids[d0 + i];
+    const float u = u_accept[d0 + i];
     float p = 0.f;
     if (d >= 0 && d < vocab && rc.z_fix > 0) {
       const uint32_t f = (uint32_t)logits[(int64_t)(r0 + i) * row_stride + d] << 16;
       if (is_kept(key32(f), d, rc)) p = (float)wfix_of(f, rc.m, k_log2) / (float)rc.z_fix;
     }
-    if (p_draft != nullptr) p_draft[d0 + i] = p;
-    if (!(u_accept[d0 + i] < p)) atomicMin(&s_n, i);
+    if (p_draft != nullptr && rank == 0) p_draft[d0 + i] = p;
+    if (!(u < p)) atomicMin(&s_n, i);
   }
   __syncthreads();
   const int n = s_n;
+  if (rank == 0 && tid == 0) n_accept[b] = n;
 
   // ---- the final token: inverse CDF over the kept tokens of the stop row, the rejected one removed
   const RowCut rc = cuts[r0 + n];
+  const bool given = rc.slices != 0;  // every CTA of the cluster sees the same
+  if (given && rank != 0) return;
   const uint16_t *rp = logits + (int64_t)(r0 + n) * row_stride;
+  const int slice_len = slice_len_of(vocab);
+  const int spc = given ? n_slices : (n_slices + kC - 1) / kC, sl0 = min(n_slices, rank * spc), n_here = min(spc, n_slices - sl0);
   int32_t dead = -1;
   u64 w_dead = 0;
   if (n < L) {
@@ -519,39 +839,148 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
       }
     }
   }
-  const u64 total = rc.z_fix - w_dead;
-  // smallest v whose cumulative mass exceeds u * total; the masses are integers, so "exceeds floor(u * total)"
-  u64 target = (u64)((double)u_final[b] * (double)total);
-  if (total > 0 && target >= total) target = total - 1;
-  u64 mine = 0;
-  row_blocked<kST>(rp, vocab, [&](int32_t e, uint32_t bts) {
-    if (e != dead && is_kept(key32(bts), e, rc)) mine += wfix_of(bts, rc.m, k_log2);
-  });
-  u64 all;
-  const u64 before = block_scan<kST, u64>(mine, s_w64, all) - mine;
-  if (mine > 0 && before <= target && target < before + mine) {
-    u64 cum = before;
-    bool done = false;
-    row_blocked<kST>(rp, vocab, [&](int32_t e, uint32_t bts) {
-      if (!done && e != dead && is_kept(key32(bts), e, rc)) {
-        cum += wfix_of(bts, rc.m, k_log2);
-        if (cum > target) {
-          s_final = e;
-          done = true;
+  if (given) {
+    const u64 *sm = slice_mass + (int64_t)(r0 + n) * n_slices;
+    for (int i = tid; i < n_here; i += kT) s_mass[i] = sm[i];
+  } else {  // a warp per slice, a lane per vector
+    const float cut_x = rc.cut_key == kNoKey ? -INFINITY : __uint_as_float(f_of_key16(rc.cut_key >> 16));
+    for (int i = warp; i < n_here; i += kWarps) {
+      u64 mass = 0;
+      const int32_t s_end = min(vocab, (sl0 + i + 1) * slice_len);
+      for (int32_t e = (sl0 + i) * slice_len + lane * 8; e < s_end; e += 256) {
+        const uint4 v = e + 8 <= vocab ? __ldg(reinterpret_cast<const uint4 *>(rp + e)) : ragged_vec(rp, vocab >> 3, vocab & 7);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
+          const float x = __uint_as_float(f);
+          if (x > cut_x || (x == cut_x && e + j <= rc.cut_idx)) mass += wfix_of(f, rc.m, k_log2);
         }
       }
-    });
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mass += __shfl_xor_sync(0xFFFFFFFFu, mass, o);
+      if (lane == 0) s_mass[i] = mass;
+    }
   }
   __syncthreads();
-  if (tid == 0) {
-    n_accept[b] = n;
-    final_id[b] = s_final;
+  const u64 total = rc.z_fix - w_dead;
+  // smallest v whose cumulative mass exceeds u * total; the masses are integers, so "exceeds floor(u * total)"
+  u64 target = (u64)(u_fin * (double)total);
+  if (total > 0 && target >= total) target = total - 1;
+  const int spt = (n_here + kT - 1) / kT;  // slices per thread, consecutive
+  u64 w[kMaxSlices / kT], mine = 0, all, base = 0;
+#pragma unroll
+  for (int i = 0; i < kMaxSlices / kT; ++i) {
+    const int at = tid * spt + i;
+    w[i] = 0;
+    if (i < spt && at < n_here) {
+      w[i] = s_mass[at];
+      if (dead >= 0 && sl0 + at == dead / slice_len) w[i] -= w_dead;
+    }
+    mine += w[i];
   }
+  u64 cum = block_scan<kT, u64>(mine, s_w64, all) - mine;
+  if (kC > 1 && !given) {
+    if (tid == 0) s_total = all;
+    cluster.sync();
+    for (int q = 0; q < rank; ++q) base += *cluster.map_shared_rank(&s_total, q);
+  }
+  cum += base;
+#pragma unroll
+  for (int i = 0; i < kMaxSlices / kT; ++i) {
+    if (w[i] > 0 && cum <= target && target < cum + w[i]) {
+      s_slice = sl0 + tid * spt + i;
+      s_before = cum;
+    }
+    cum += w[i];
+  }
+  __syncthreads();
+  const int sl = s_slice;
+  if (sl >= 0) {  // inside the slice: one token per thread at a time
+    u64 upto0 = s_before;
+    for (int32_t x0 = sl * slice_len; x0 < min(vocab, (sl + 1) * slice_len); x0 += kT) {
+      const int32_t e = x0 + tid;
+      u64 x = 0;
+      if (e < vocab && e != dead) {
+        const uint32_t f = (uint32_t)rp[e] << 16;
+        if (is_kept(key32(f), e, rc)) x = wfix_of(f, rc.m, k_log2);
+      }
+      const u64 upto = upto0 + block_scan<kT, u64>(x, s_w64, all);
+      if (x > 0 && upto - x <= target && target < upto) final_id[b] = e;
+      upto0 += all;
+    }
+  }
+  if (total == 0 && rank == 0 && tid == 0) final_id[b] = 0;  // a row without mass
+  if (kC > 1 && !given) cluster.sync();  // nobody leaves while its total is being read
+}
+
+struct ScratchLayout {
+  size_t cuts, slices, keys, stats, open, bytes;
+  int n_chunks, n_slices;
+};
+ScratchLayout filter_layout(int32_t vocab, int32_t n_rows) {
+  ScratchLayout s;
+  s.n_chunks = (int)(((int64_t)vocab + kChunk - 1) / kChunk);
+  s.n_slices = (int)(((int64_t)vocab + slice_len_of(vocab) - 1) / slice_len_of(vocab));
+  size_t off = 0;
+  auto take = [&](size_t n) {
+    const size_t o = off;
+    off += (n + 15) / 16 * 16;
+    return o;
+  };
+  s.cuts = take((size_t)n_rows * sizeof(RowCut));
+  s.slices = take((size_t)n_rows * s.n_slices * sizeof(u64));
+  s.keys = take((size_t)n_rows * s.n_chunks * 32 * kVec * sizeof(uint16_t));
+  s.stats = take((size_t)n_rows * s.n_chunks * sizeof(float2));
+  s.open = take(((size_t)n_rows + 1) * sizeof(int32_t));
+  s.bytes = off + 16;  // the caller's scratch is 8-byte aligned, the keys are read 16 bytes at a time
+  return s;
+}
+
+struct WindowShape {
+  size_t smem;
+  bool cached;
+  int clusters;  // on the chip at a time
+};
+WindowShape window_shape(const lr_ctx *ctx, int cluster) {
+  WindowShape w;
+  const size_t fixed = (sizeof(WindowShared) + 15) / 16 * 16, share = (size_t)share_of(ctx->model.vocab, cluster) * 2;
+  w.cached = fixed + share <= kWindowSmemMax;
+  w.smem = fixed + (w.cached ? share : 0);
+  const int per_sm = 2 * (w.smem + 1024) <= 227 * 1024 ? 2 : 1;  // 64 registers a thread allow two
+  w.clusters = std::max(1, ctx->sm_count * per_sm / cluster);
+  return w;
+}
+
+template <class... KArgs, class... Args>
+cudaError_t launch_clusters(void (*kernel)(KArgs...), int kc, int clusters, int threads, size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(kc * clusters));
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)kc;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 }  // namespace
 
-size_t accept_filtered_scratch_bytes(int32_t n_rows) { return std::max<size_t>(32, (size_t)n_rows * sizeof(RowCut)); }
+int init_accept_filter_kernels() {
+  const int smem = (int)kWindowSmemMax;
+  cudaError_t e = cudaFuncSetAttribute(filter_window_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(filter_window_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(filter_window_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return cuda_fail(e, "filter_window_kernel shared-memory attribute");
+}
+
+size_t accept_filtered_scratch_bytes(int32_t vocab, int32_t n_rows) { return filter_layout(vocab, n_rows).bytes; }
 
 int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
                            int32_t n_branch, int32_t n_rows, float temperature, int32_t top_k, float top_p,
@@ -559,25 +988,62 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
                            int32_t *n_kept, void *scratch, cudaStream_t s) {
   const int32_t vocab = ctx->model.vocab;
   const float k_log2 = 1.4426950408889634f / temperature;
+  const ScratchLayout L = filter_layout(vocab, n_rows);
+  unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)scratch + 15) & ~(uintptr_t)15);
   auto *lg = reinterpret_cast<const uint16_t *>(logits);
-  auto *cuts = reinterpret_cast<RowCut *>(scratch);
-  filter_rows_kernel<<<(unsigned)n_rows, kFT, 0, s>>>(lg, stride, vocab, k_log2, top_k, top_p, cuts, n_kept);
+  auto *cuts = reinterpret_cast<RowCut *>(base + L.cuts);
+  auto *slices = reinterpret_cast<u64 *>(base + L.slices);
+  auto *keys = reinterpret_cast<uint16_t *>(base + L.keys);
+  auto *stats = reinterpret_cast<float2 *>(base + L.stats);
+  auto *n_open = reinterpret_cast<int32_t *>(base + L.open);
+  const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
+  // Cluster size when every row goes through the windows: the largest with room for all rows at a time, else the one with
+  // room for the most.
+  int kc = 8;
+  for (const int c : {4, 2}) {
+    const int have = window_shape(ctx, kc).clusters;
+    if (have < n_rows && window_shape(ctx, c).clusters > have) kc = c;
+  }
+  WindowShape w = window_shape(ctx, kc);
+  const int k_sel = by_k ? top_k : kSelTopP;
+  // Groups of 64 tokens when that makes many more of them than k_sel, else of 8
+  const bool wide = vocab / 64 >= 4 * (int64_t)k_sel;
+  const int64_t n_keys = (int64_t)L.n_chunks * 32 * (wide ? 1 : kVec);
+  // Can a few leading tokens decide a row?  With a top-k up to kSelMax always.  With top-p alone mostly, but then the rows
+  // they leave open go through the windows all the same, so the candidates pay only when they spare many rounds of those.
+  const bool candidates = n_keys <= kMaxGroups && (by_k ? top_k <= kSelMax : by_p && n_rows > kWindowRounds * w.clusters);
+  if (candidates) {
+    auto scan = by_k ? (wide ? filter_scan_kernel<false, kVec> : filter_scan_kernel<false, 1>)
+                     : (wide ? filter_scan_kernel<true, kVec> : filter_scan_kernel<true, 1>);
+    const uint32_t total = (uint32_t)n_rows * L.n_chunks;
+    const unsigned grid = std::min((total + kWarps - 1) / kWarps, (uint32_t)(ctx->sm_count * kScanCtasPerSm));
+    scan<<<grid, kT, 0, s>>>(lg, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, keys, stats, n_open);
+    ctx->launches++;
+    if (int rc = cuda_fail(cudaGetLastError(), "filter_scan_kernel launch")) return rc;
+    ctx->launches++;
+    if (int rc = cuda_fail(launch_dependent(wide ? filter_cut_kernel<kVec> : filter_cut_kernel<1>, dim3((unsigned)n_rows), dim3(kT),
+                                            (size_t)n_keys * 2, s, lg, stride, vocab, k_log2, top_k, top_p, k_sel, L.n_chunks, keys, stats, cuts,
+                                            slices, L.n_slices, n_kept, n_open, n_open + 1),
+                           "filter_cut_kernel launch"))
+      return rc;
+    kc = 8;  // few rows are left, as a rule: the most CTAs for each
+    w = window_shape(ctx, kc);
+  }
   ctx->launches++;
-  if (int rc = cuda_fail(cudaGetLastError(), "filter_rows_kernel launch")) return rc;
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)n_branch, 1, 1);
-  cfg.blockDim = dim3(kST, 1, 1);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, accept_filtered_kernel, lg, stride, vocab, k_log2, (const RowCut *)cuts, drafts, cu_draft,
-                                     u_accept, u_final, n_accept, final_id, p_draft);
+  auto window = kc == 8 ? filter_window_kernel<8> : kc == 4 ? filter_window_kernel<4> : filter_window_kernel<2>;
+  if (int rc = cuda_fail(launch_clusters(window, kc, candidates ? w.clusters : std::min(n_rows, w.clusters), kWT, w.smem, s, lg, stride, vocab,
+                                         k_log2, top_k, top_p, cuts, n_kept, n_open, n_open + 1, candidates ? 0 : n_rows, w.cached ? 1 : 0),
+                         "filter_window_kernel launch"))
+    return rc;
   ctx->launches++;
-  return cuda_fail(e, "accept_filtered_kernel launch");
+  // slices of a stop row to sum: always after the windows, hardly ever after the candidates of a top-k
+  if (candidates && by_k)
+    return cuda_fail(launch_dependent(accept_filtered_kernel<1>, dim3((unsigned)n_branch), dim3(kT), 0, s, lg, stride, vocab, k_log2, cuts, slices,
+                                      L.n_slices, drafts, cu_draft, u_accept, u_final, n_accept, final_id, p_draft),
+                     "accept_filtered_kernel launch");
+  return cuda_fail(launch_clusters(accept_filtered_kernel<8>, 8, n_branch, kT, 0, s, lg, stride, vocab, k_log2, cuts, slices, L.n_slices, drafts,
+                                   cu_draft, u_accept, u_final, n_accept, final_id, p_draft),
+                   "accept_filtered_kernel launch");
 }
 
 }  // namespace lr

@@ -282,6 +282,7 @@ extern "C" int lr_create(lr_ctx **out, const lr_model *m, int device) {
   if (int rc = init_commit_kernel()) { delete c; return rc; }
   if (int rc = init_attn_tc_kernel()) { delete c; return rc; }
   if (int rc = init_attn_pair_kernel()) { delete c; return rc; }
+  if (int rc = init_accept_filter_kernels()) { delete c; return rc; }
   *out = c;
   return LR_OK;
 }
@@ -664,7 +665,7 @@ extern "C" int lr_accept_sample_filtered_scratch_bytes(const lr_ctx *ctx, int32_
     set_error("lr_accept_sample_filtered_scratch_bytes: bad argument");
     return LR_EINVAL;
   }
-  *bytes_out = accept_filtered_scratch_bytes(n_rows);
+  *bytes_out = accept_filtered_scratch_bytes(ctx->model.vocab, n_rows);
   return LR_OK;
 }
 

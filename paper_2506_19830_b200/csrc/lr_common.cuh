@@ -254,6 +254,7 @@ int init_kernels(lr_ctx *ctx);  // per-device function attributes; called by lr_
 int init_commit_kernel();
 int init_attn_tc_kernel();
 int init_attn_pair_kernel();
+int init_accept_filter_kernels();
 
 int launch_attn_pair(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
                      cudaStream_t s);
@@ -271,7 +272,7 @@ size_t accept_sample_scratch_bytes(int32_t vocab, int32_t n_rows);
 int launch_accept_sample(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
                          int32_t n_branch, int32_t n_rows, float temperature, const float *u_accept, const float *u_final,
                          int32_t *n_accept, int32_t *final_id, float *p_draft, void *scratch, cudaStream_t s);
-size_t accept_filtered_scratch_bytes(int32_t n_rows);
+size_t accept_filtered_scratch_bytes(int32_t vocab, int32_t n_rows);
 int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
                            int32_t n_branch, int32_t n_rows, float temperature, int32_t top_k, float top_p,
                            const float *u_accept, const float *u_final, int32_t *n_accept, int32_t *final_id, float *p_draft,

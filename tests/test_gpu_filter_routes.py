@@ -1,0 +1,47 @@
+"""lr_accept_sample_filtered on both sides of every line its dispatch draws -- group sizes, candidates or windows, rows
+left over by the candidates, cluster sizes, rows in and out of shared memory -- by the rule of test_gpu_accept_filtered."""
+import numpy as np
+import pytest
+
+from lr_workloads import Model, bf16_round
+from test_gpu_accept_filtered import _check, _run
+
+pytestmark = pytest.mark.gpu
+
+# vocabulary, branches, drafts per branch, top_k, top_p
+ROUTES = [
+    (5, 3, 2, 2, 0.9), (300, 4, 3, 20, 0.95), (1023, 4, 3, 0, 0.9), (1025, 170, 2, 0, 0.9),  # fewer groups than leading tokens
+    (5119, 5, 3, 20, 0.95), (5120, 5, 3, 20, 0.95), (5121, 5, 3, 20, 1.0),                     # groups of 8, of 64
+    (4100, 5, 3, 256, 0.97), (65600, 5, 2, 256, 1.0), (65600, 5, 2, 257, 1.0),                 # the largest top_k of the candidates
+    (32771, 12, 2, 0, 0.95), (32771, 160, 2, 0, 0.95), (40009, 30, 4, 0, 0.6),                 # few rows by windows, many by candidates
+    (655361, 2, 1, 20, 0.95), (1700003, 1, 1, 0, 0.9), (9000, 2, 1, 0, 1.0),                   # too many groups; shares beyond shared memory
+]
+
+
+@pytest.mark.parametrize("vocab,nb,L,top_k,top_p", ROUTES)
+def test_routes(vocab, nb, L, top_k, top_p):
+    rng = np.random.default_rng(vocab + nb)
+    n_rows = nb * (L + 1)
+    x = (rng.standard_normal((n_rows, vocab), dtype=np.float32) * 1.5)
+    lead = rng.integers(0, vocab, (n_rows, 3))
+    for r in range(n_rows):  # peaked, flat, coarse (many ties), and rows with values outside the usual octaves
+        if r % 4 != 1:
+            x[r, lead[r]] = rng.uniform(6, 20, 3)
+        if r % 4 == 2:
+            x[r] = np.round(x[r] * 2) / 2
+        if r % 4 == 3:
+            x[r, : max(1, vocab // 100)] = 1e-9
+            x[r, vocab // 2] = -7000.0
+    x[::5, vocab // 3: vocab // 2] = -np.inf
+    bits = bf16_round(x)
+    bits[::3, -1] = 0x7FC0  # NaN counts as -inf
+    cu = (np.arange(nb + 1) * L).astype(np.int32)
+    drafts = lead.reshape(nb, L + 1, 3)[:, :L, 0].reshape(-1).astype(np.int32).copy()
+    ua, uf = rng.uniform(0, 1, len(drafts)), rng.uniform(0, 1, nb)
+    ua[::3] = 0.0
+    got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, 0.8, top_k, top_p, ua, uf)
+    rows = None if n_rows * vocab < 3e6 else sorted(set(rng.integers(0, n_rows, 12).tolist()))
+    # A flat row of 40009 tokens keeps some 2000 at top_p 0.6, the last with 1.5e-4 of their mass: above HEAVY, and within
+    # the checker's 4e-5 of the step in one row of four.  A branch looks at two rows or so, one in four of them flat, and
+    # draws differ on a few more: 0.4 of the branches leaves room for twice the expected number.
+    _check(bits, drafts, cu, 0.8, top_k, top_p, ua, uf, got, max_ambiguous_frac=0.4, rows_to_check=rows)
