@@ -23,8 +23,8 @@
 // (launch_accept_filtered has the rule).
 //
 // accept_filtered_kernel (per branch) walks the acceptance chain with P'(d) = w_d / Z' for kept tokens and 0 for
-// the others, and draws the final token by inverse CDF over the kept tokens of the stop row in index order: first over the
-// kept mass of every slice of the row, then inside one slice.
+// the others, and draws the final token by inverse CDF over the kept tokens of the stop row in index order: from the list of
+// them when the candidates settled the row, else first over the kept mass of every slice of the row, then inside one slice.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -40,14 +40,14 @@ constexpr int kWarps = kT / 32;
 constexpr int kVec = 8;             // 16-byte vectors a lane of filter_scan_kernel takes at a time
 constexpr int kChunk = 32 * kVec * 8;  // logits a warp takes at a time
 constexpr int kScanCtasPerSm = 4;
-constexpr int kMaxGroups = 10240;   // group keys of a row that filter_cut_kernel can hold
 constexpr int kGroupCap = 512;      // groups it reads again
-constexpr int kListCap = 1024;      // candidates of a row
+constexpr int kListCap = 512;       // candidates of a row
+constexpr int kKeyWords = 8;        // words of group maxima a thread of filter_cut_kernel keeps in registers
 constexpr int kSelMax = 256;        // largest top_k the candidates serve
 constexpr int kSelTopP = 128;       // leading tokens to look for when top-k is off
 constexpr int kWT = 512;            // threads of a CTA of filter_window_kernel
 constexpr int kWin = 8192;          // keys per window
-constexpr int kMaxSlices = 1024;    // slices of a row whose kept masses are written out
+constexpr int kMaxSlices = 1024;    // slices a row is cut into for the draw
 constexpr size_t kWindowSmemMax = 200 * 1024;
 constexpr int kWindowRounds = 3;    // rounds of rows through the windows that a candidate pass has to spare
 // Relative distance between the fp32 sum of a row's masses and their integer sum: the argument of an exponential is
@@ -63,7 +63,7 @@ struct RowCut {  // what the acceptance kernel needs to know about a row (32 byt
   int32_t cut_idx;  // largest index kept inside that group
   int32_t n_kept;
   u64 z_fix;        // mass of the kept set
-  int32_t slices;   // 1: the kept mass of every slice of the row was written with the cut
+  int32_t listed;   // 1: the kept tokens were written as a list
   int32_t pad;
 };
 
@@ -151,12 +151,12 @@ __device__ __forceinline__ uint4 ragged_vec(const uint16_t *rp, int32_t n_vec, i
 
 // ---- one read of the logits -------------------------------------------------------------------------------
 // A warp per chunk of 2048 logits at a time, no warp ever waiting for another.  A lane's kGV vectors of a chunk, 32 vectors
-// apart, are a group: the group's largest key goes out (2 bytes, biased by 32768), and with kSum the chunk's pair (largest
-// logit, sum of exp((x - largest) / T)).  Bound: HBM (kSum: and the special-function units close behind).
+// apart, are a group: the group's largest logit goes out, and with kSum the chunk's pair (largest logit, sum of
+// exp((x - largest) / T)).  Bound: HBM (kSum: and the special-function units close behind).
 template <bool kSum, int kGV>
 __global__ void __launch_bounds__(kT, kScanCtasPerSm)
 filter_scan_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, uint32_t n_chunks, uint32_t total,
-                   uint16_t *__restrict__ group_key, float2 *__restrict__ stats, int32_t *__restrict__ n_open) {
+                   uint16_t *__restrict__ group_max, float2 *__restrict__ stats, int32_t *__restrict__ n_open) {
   const int lane = threadIdx.x & 31;
   const int32_t n_vec = vocab >> 3, rem = vocab & 7;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the logits may come from the kernel launched just before
@@ -201,7 +201,7 @@ filter_scan_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int3
       }
       const float g = fmaxf(lo_f(mx), hi_f(mx));
       top = fmaxf(top, g);
-      group_key[(int64_t)unit * (32 * kVec / kGV) + (k0 / kGV) * 32 + lane] = (uint16_t)((key32(__float_as_uint(g)) >> 16) + 32768);
+      group_max[(int64_t)unit * (32 * kVec / kGV) + (k0 / kGV) * 32 + lane] = (uint16_t)(__float_as_uint(g) >> 16);
     }
     if (kSum) {
       const float off = top > -INFINITY ? -top * k_log2 : 0.f;
@@ -230,67 +230,98 @@ __host__ __device__ __forceinline__ int32_t share_of(int32_t vocab, int n) { ret
 __host__ __device__ __forceinline__ int slice_len_of(int32_t vocab) { return 256 * ((vocab + 256 * kMaxSlices - 1) / (256 * kMaxSlices)); }
 
 // ---- the cut of a row from its candidates -----------------------------------------------------------------
-// T, the k_sel-th largest group maximum, is a lower bound of the k_sel-th largest logit (the maxima are logits of different
-// tokens), and only the k_sel groups that reach it (more with ties) hold tokens of at least T: they are read again.
+// A lower bound of the k_sel-th largest logit is any value that k_sel group maxima reach (they are logits of different
+// tokens); it is raised by bisection on the key until little more than k_sel maxima reach it.  Only those groups hold tokens of at least that value: they are read again.  Bound: instructions, a few hundred per warp.
 template <int kGV>
 __global__ void __launch_bounds__(kT)
 filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, int32_t top_k, float top_p, int k_sel,
-                  int n_chunks, const uint16_t *__restrict__ group_key, const float2 *__restrict__ stats, RowCut *__restrict__ cuts,
-                  u64 *__restrict__ slice_mass, int n_slices, int32_t *__restrict__ n_kept_out, int32_t *__restrict__ n_open,
-                  int32_t *__restrict__ open_rows) {
-  extern __shared__ __align__(16) uint32_t s_key2[];  // the row's group keys, two to a word
-  __shared__ __align__(16) u64 s_cand[kListCap];
-  __shared__ u64 s_sorted[kListCap], s_slice[kMaxSlices];
-  __shared__ u64 s_w[kWarps];
-  __shared__ double s_z;
+                  int n_chunks, const uint16_t *__restrict__ group_max, const float2 *__restrict__ stats, RowCut *__restrict__ cuts,
+                  u64 *__restrict__ lists, int32_t *__restrict__ n_kept_out, int32_t *__restrict__ n_open, int32_t *__restrict__ open_rows) {
+  __shared__ u64 s_cand[kListCap], s_sorted[kListCap], s_cum[kListCap];
   __shared__ int s_grp[kGroupCap];
-  __shared__ int s_n, s_n_grp, s_r[2], s_cnt[2][kWarps];
+  __shared__ int s_n, s_n_grp, s_cnt[2][kWarps], s_kept;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t row = blockIdx.x;
   constexpr int kPerChunk = 32 * kVec / kGV;
   const int n_words = n_chunks * kPerChunk / 2;
-  if (tid == 0) {
-    s_n = s_n_grp = 0;
-    s_r[0] = s_r[1] = -1;
-  }
-  for (int i = tid; i < n_slices; i += kT) s_slice[i] = 0;
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the keys come from the kernel launched just before
+  const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
+  if (tid == 0) s_n = s_n_grp = 0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the maxima come from the kernel launched just before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const uint4 *src = reinterpret_cast<const uint4 *>(group_key + row * n_chunks * kPerChunk);
-  for (int i = tid; i < n_words / 4; i += kT) reinterpret_cast<uint4 *>(s_key2)[i] = src[i];
-  __syncthreads();
-  uint32_t T = 0;  // bisection on the biased key
+  const uint32_t *src = reinterpret_cast<const uint32_t *>(group_max + row * n_chunks * kPerChunk);
+  uint32_t g2[kKeyWords];  // word i of the thread is word i * kT + tid of the row
+#pragma unroll
+  for (int i = 0; i < kKeyWords; ++i) g2[i] = i * kT + tid < n_words ? __ldg(src + i * kT + tid) : kNegInf2;
+  // mass of the whole row (top-p alone), to within kMassEps: warp 0, while the others wait for it to bisect
+  float m_all = -INFINITY;
+  double z_all = 0.0;
+  if (!by_k && warp == 0) {
+    for (int i = lane; i < n_chunks; i += 32) m_all = fmaxf(m_all, stats[row * n_chunks + i].x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xFFFFFFFFu, m_all, o));
+    for (int i = lane; i < n_chunks; i += 32) {
+      const float2 h = stats[row * n_chunks + i];
+      z_all += (double)(h.y * ex2_approx((h.x - m_all) * k_log2));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) z_all += __shfl_xor_sync(0xFFFFFFFFu, z_all, o);
+  }
+  auto bf2_of = [](int32_t key16) -> __nv_bfloat162 {
+    const uint32_t u = f_of_key16(key16) >> 16, uu = u | (u << 16);
+    return *reinterpret_cast<const __nv_bfloat162 *>(&uu);
+  };
+  auto as_bf2 = [](const uint32_t &u) -> __nv_bfloat162 { return *reinterpret_cast<const __nv_bfloat162 *>(&u); };
+  int32_t least = -32639;  // key16 of the smallest finite logit: all groups with one
+  int reach = -1;          // groups that reach it
+  int buf = 0;
+  // keys from the largest finite one (32639) down to the smallest: 2^16 of them at most
 #pragma unroll 1
-  for (int bit = 15; bit >= 0; --bit) {
-    const uint32_t u = T | (1u << bit);
-    int c = 0;
-    for (int i = tid; i < n_words; i += kT) {
-      const uint32_t w = s_key2[i];
-      c += ((w & 0xFFFFu) >= u ? 1 : 0) + ((w >> 16) >= u ? 1 : 0);
+  for (int step = 32768; step > 0; step >>= 1) {
+    const int32_t u = least + step;
+    if (u > 32640) continue;  // the key of +inf
+    const __nv_bfloat162 t = bf2_of(u);
+    __nv_bfloat162 c2 = __floats2bfloat162_rn(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kKeyWords; ++i) c2 = __hadd2(c2, __hge2(as_bf2(g2[i]), t));
+    int c = (int)(__low2float(c2) + __high2float(c2));
+    for (int i = kKeyWords * kT + tid; i < n_words; i += kT) {  // more than 4096 groups
+      const uint32_t w = __ldg(src + i);
+      c += __popc(__hge2_mask(as_bf2(w), t)) >> 4;
     }
     c = __reduce_add_sync(0xFFFFFFFFu, c);
-    if (lane == 0) s_cnt[bit & 1][warp] = c;
+    if (lane == 0) s_cnt[buf][warp] = c;
     __syncthreads();
     c = 0;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) c += s_cnt[bit & 1][w];
-    if (c >= k_sel) T = u;
+    for (int w = 0; w < kWarps; ++w) c += s_cnt[buf][w];
+    buf ^= 1;
+    if (c >= k_sel) {
+      least = u;
+      reach = c;
+      if (c <= k_sel + k_sel / 4 + 4) break;
+    }
   }
-  const uint32_t least = max(T, 129u);  // 128 is the key of -inf
-  for (int i = tid; i < n_words; i += kT) {
-    const uint32_t w = s_key2[i];
+  auto note = [&](uint32_t w, int word) {
+    const uint32_t hit = __hge2_mask(as_bf2(w), bf2_of(least));
+    if (hit != 0)
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if ((h ? w >> 16 : w & 0xFFFFu) >= least) {
-        const int at = atomicAdd(&s_n_grp, 1);
-        if (at < kGroupCap) s_grp[at] = 2 * i + h;
-      }
+      for (int h = 0; h < 2; ++h)
+        if (hit & (h ? 0x10000u : 1u)) {
+          const int at = atomicAdd(&s_n_grp, 1);
+          if (at < kGroupCap) s_grp[at] = 2 * word + h;
+        }
+  };
+  if (reach <= kGroupCap) {
+#pragma unroll
+    for (int i = 0; i < kKeyWords; ++i) note(g2[i], i * kT + tid);
+    for (int i = kKeyWords * kT + tid; i < n_words; i += kT) note(__ldg(src + i), i);
   }
   __syncthreads();
   const int n_grp = s_n_grp;
   const uint16_t *rp = logits + row * row_stride;
   if (n_grp <= kGroupCap) {
     const int32_t n_vec = vocab >> 3, rem = vocab & 7;
+    const float least_x = __uint_as_float(f_of_key16(least));
     for (int i = tid; i < n_grp * kGV; i += kT) {
       const int g = s_grp[i / kGV];
       const int32_t vi = (g / kPerChunk) * (kChunk / 8) + (g % kPerChunk) + (i % kGV) * 32;
@@ -300,8 +331,7 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
-        const float x = __uint_as_float(f);
-        if (x == x && (uint32_t)((key32(f) >> 16) + 32768) >= least) {
+        if (__uint_as_float(f) >= least_x) {  // (a NaN is not)
           const int at = atomicAdd(&s_n, 1);
           if (at < kListCap) s_cand[at] = cand_of(f, vi * 8 + j);
         }
@@ -310,109 +340,81 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
   }
   __syncthreads();
   const int n = s_n;
-  const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
-  bool ok = n_grp <= kGroupCap && n >= 1 && n <= kListCap && (!by_k || n >= top_k);
-  if (ok)
+  const bool usable = n_grp <= kGroupCap && n >= 1 && n <= kListCap && (!by_k || n >= top_k);
+  if (usable)
     for (int i = tid; i < n; i += kT) {  // rank by counting: the candidates are all different
       const u64 e = s_cand[i];
       int before = 0;
-#pragma unroll 8
+#pragma unroll 4
       for (int j = 0; j < n; ++j) before += s_cand[j] > e ? 1 : 0;
       s_sorted[before] = e;
     }
   __syncthreads();
-  float m = 0.f;
-  if (ok) {
-    m = __uint_as_float(f_of_key16(cand_key16(s_sorted[0])));
-    ok = fabsf(m) < INFINITY;
-  }
-  constexpr int kPer = kListCap / kT;
-  u64 w[kPer], mine = 0, all = 0, before = 0;
+  // ---- warp 0: the last rank kept.  It is top_k - 1, or the first one at which the mass, itself included, reaches
+  //      t = ceil(top_p W), where W is the mass of the leading top_k ranks, or -- to within kMassEps -- of the whole row.
+  if (warp == 0) {
+    bool ok = usable;
+    const float m = ok ? __uint_as_float(f_of_key16(cand_key16(s_sorted[0]))) : 0.f;
+    ok = ok && fabsf(m) < INFINITY;
+    const int ranks = ok ? (by_k ? top_k : n) : 0;
+    u64 sum = 0;
+    for (int base = 0; base < ranks; base += 32) {
+      const int i = base + lane;
+      u64 c = i < ranks ? wfix_of(f_of_key16(cand_key16(s_sorted[i])), m, k_log2) : 0;
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int r = tid * kPer + i;
-    w[i] = ok && r < n ? wfix_of(f_of_key16(cand_key16(s_sorted[r])), m, k_log2) : 0;
-    mine += w[i];
-  }
-  before = block_scan<kT, u64>(mine, s_w, all) - mine;
-  // the last rank kept: top_k - 1, or the first one at which the mass, itself included, reaches t = ceil(top_p W), where W
-  // is the mass of the leading top_k ranks, or -- to within kMassEps -- of the whole row
-  if (by_k) {
-    u64 cum = before;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      cum += w[i];
-      if (tid * kPer + i == top_k - 1) s_w[0] = cum;
-    }
-    if (tid == 0) s_r[0] = s_r[1] = top_k - 1;
-  } else if (warp == 0) {
-    double z = 0.0;
-    for (int i = lane; i < n_chunks; i += 32) {
-      const float2 h = stats[row * n_chunks + i];
-      z += (double)(h.y * ex2_approx((h.x - m) * k_log2));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
-    if (lane == 0) s_z = z * 1099511627776.0;  // units of 2^-40
-  }
-  __syncthreads();
-  if (by_p && ok) {
-    u64 t[2];
-    if (by_k) {
-      const u64 w_k = s_w[0];
-      const double t_d = ceil((double)top_p * (double)w_k);
-      t[0] = t_d < 1.0 ? 1ull : (u64)t_d;
-      if (t[0] > w_k) t[0] = w_k;
-      t[1] = t[0];
-      ok = w_k > 0;
-    } else {
-      t[0] = (u64)((double)top_p * s_z * (1.0 - kMassEps));
-      t[1] = (u64)((double)top_p * s_z * (1.0 + kMassEps)) + 2;
-      ok = t[0] > 0 && t[1] <= all;  // else the cut may lie beyond the candidates
-    }
-    __syncthreads();
-    if (ok) {
-      u64 cum = before;
-#pragma unroll
-      for (int i = 0; i < kPer; ++i) {
-        const u64 next = cum + w[i];
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-          if (cum < t[q] && t[q] <= next) s_r[q] = tid * kPer + i;
-        cum = next;
+      for (int o = 1; o < 32; o <<= 1) {
+        const u64 y = __shfl_up_sync(0xFFFFFFFFu, c, o);
+        if (lane >= o) c += y;
       }
+      c += sum;
+      if (i < ranks) s_cum[i] = c;
+      sum = __shfl_sync(0xFFFFFFFFu, c, 31);
     }
-    __syncthreads();
-  }
-  const int r = s_r[0];
-  ok = ok && r >= 0 && r == s_r[1];
-  if (!ok) {
-    if (tid == 0) open_rows[atomicAdd(n_open, 1)] = (int32_t)row;
-    return;
-  }
-  {
-    u64 cum = before;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      const int at = tid * kPer + i;
-      cum += w[i];
-      if (at <= r && w[i] > 0) atomicAdd(&s_slice[cand_idx(s_sorted[at]) / slice_len_of(vocab)], w[i]);
-      if (at == r) {
+    int r = ranks - 1;
+    if (ok && by_p) {
+      u64 t0, t1;
+      if (by_k) {
+        const double t_d = ceil((double)top_p * (double)sum);
+        t0 = t_d < 1.0 ? 1ull : (u64)t_d;
+        if (t0 > sum) t0 = sum;
+        t1 = t0;
+        ok = sum > 0;
+      } else {
+        const double z = z_all * 1099511627776.0;  // units of 2^-40
+        t0 = (u64)((double)top_p * z * (1.0 - kMassEps));
+        t1 = (u64)((double)top_p * z * (1.0 + kMassEps)) + 2;
+        ok = t0 > 0 && t1 <= sum;  // else the cut may lie beyond the candidates
+      }
+      __syncwarp();
+      int lo = 0, below = 0;  // ranks whose cumulative mass stays below t0, t1
+      for (int i = lane; i < ranks; i += 32) {
+        lo += s_cum[i] < t0 ? 1 : 0;
+        below += s_cum[i] < t1 ? 1 : 0;
+      }
+      r = __reduce_add_sync(0xFFFFFFFFu, lo);
+      ok = ok && r == __reduce_add_sync(0xFFFFFFFFu, below);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      s_kept = ok ? r + 1 : 0;
+      if (ok) {
         RowCut rc;
         rc.m = m;
-        rc.cut_key = cand_key16(s_sorted[at]) * 65536;
-        rc.cut_idx = cand_idx(s_sorted[at]);
+        rc.cut_key = cand_key16(s_sorted[r]) * 65536;
+        rc.cut_idx = cand_idx(s_sorted[r]);
         rc.n_kept = r + 1;
-        rc.z_fix = cum;
-        rc.slices = 1;
+        rc.z_fix = s_cum[r];
+        rc.listed = 1;
         rc.pad = 0;
         cuts[row] = rc;
         if (n_kept_out != nullptr) n_kept_out[row] = r + 1;
+      } else {
+        open_rows[atomicAdd(n_open, 1)] = (int32_t)row;
       }
     }
   }
   __syncthreads();
-  for (int i = tid; i < n_slices; i += kT) slice_mass[row * n_slices + i] = s_slice[i];
+  for (int i = tid; i < s_kept; i += kT) lists[row * kListCap + i] = s_sorted[i];
 }
 
 // ---- the cut of a row from counts per key: a cluster of kC CTAs per row --------------------------------------
@@ -442,12 +444,12 @@ struct WindowShared {
 };
 
 // Counts cover kWin keys at a time.  The usual ones are fixed: position 0 is the largest key below 2^12, position 4095
-// that of 2^-20, position 4096 zero, the rest -2^-20 down to -2^12 (its last key left out): one pass, with no branch that
-// tokens take both ways, and nothing to know in advance.  A row that holds other finite values is counted again over
-// windows of kWin consecutive keys, hi down to hi - kWin + 1, from the row maximum down (a NaN is never counted).
+// that of 2^-20, then -2^-20 down to above -2^12: one pass without branches, about nine instructions a token, and nothing
+// to know in advance.  A row that holds other finite values is counted again over windows of kWin consecutive keys, hi
+// down to hi - kWin + 1, from the row maximum down (a NaN is never counted).
 constexpr uint32_t kMag0 = (127 - 20) << 7;  // bf16 bits of 2^-20
 __device__ __forceinline__ int32_t fixed_key16(int pos) {
-  return pos < 4096 ? (int32_t)kMag0 + 4095 - pos : pos == 4096 ? 0 : -((int32_t)kMag0 + pos - 4097);
+  return pos < 4096 ? (int32_t)kMag0 + 4095 - pos : -((int32_t)kMag0 + pos - 4096);
 }
 struct Window {
   int32_t hi;
@@ -542,13 +544,13 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     uint32_t mx = kNegInf2;
-    int odd = 0;  // finite values outside the fixed keys
-    auto count = [&](uint32_t u) {
-      const uint32_t mag = u & 0x7FFFu, t = mag - kMag0;
-      const bool neg = u > 0x7FFFu;
-      if (t < (neg ? 4095u : 4096u)) atomicAdd(&sh.cnt[neg ? 4097 + t : 4095 - t], 1u);
-      else if (mag == 0) atomicAdd(&sh.cnt[4096], 1u);
-      else odd |= (mag < 0x7F80u || u == 0x7F80u) ? 1 : 0;
+    uint32_t far = 0;  // largest distance from the first fixed magnitude: from 4096 on not among them
+    const uint32_t cnt_mid = (uint32_t)__cvta_generic_to_shared(sh.cnt) + 4096 * 4;
+    auto count = [&](uint32_t mag4, int32_t sign) {  // 4 x the magnitude's bits; 0 or -1
+      const uint32_t t4 = mag4 - 4 * kMag0;
+      const uint32_t at = cnt_mid + ((t4 ^ ~(uint32_t)sign) & ~3u);  // 4096 + t, or 4095 - t when positive
+      if (t4 < 4 * 4096u) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory");
+      far = max(far, t4);
     };
     for (int32_t vi = tid; vi < n_vec; vi += kWT) {
       const uint4 v = reinterpret_cast<const uint4 *>(rp)[vi];
@@ -556,17 +558,36 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        count(w[j] & 0xFFFFu);
-        count(w[j] >> 16);
+        count((w[j] << 2) & 0x1FFFCu, (int32_t)(w[j] << 16) >> 31);
+        count((w[j] >> 14) & 0x1FFFCu, (int32_t)w[j] >> 31);
       }
     }
     float top = fmaxf(lo_f(mx), hi_f(mx));
     if (tid < rem) {
       const uint32_t u = rp[n_vec * 8 + tid];
-      count(u);
+      count((u << 2) & 0x1FFFCu, (int32_t)(u << 16) >> 31);
       top = fmaxf(top, __uint_as_float(u << 16));
     }
-    odd = __syncthreads_or(odd);
+    int odd = far >= 4 * 4096u ? 1 : 0;
+    if (__syncthreads_or(odd)) {  // -inf and NaN do not matter (they have no mass), other values do
+      odd = 0;
+      auto look = [&](uint32_t u) {
+        const uint32_t mag = u & 0x7FFFu;
+        if (mag - kMag0 >= 4096u && (mag < 0x7F80u || u == 0x7F80u)) odd = 1;
+      };
+#pragma unroll 1
+      for (int32_t vi = tid; vi < n_vec; vi += kWT) {
+        const uint4 v = reinterpret_cast<const uint4 *>(rp)[vi];
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          look(w[j] & 0xFFFFu);
+          look(w[j] >> 16);
+        }
+      }
+      if (tid < rem) look(rp[n_vec * 8 + tid]);
+      odd = __syncthreads_or(odd);
+    }
     const Sums first = exchange(block_max(key32(__float_as_uint(top))), odd ? 1u : 0u, 0);
     const float m = fmaxf(__uint_as_float(f_of_key16(first.key >> 16)), -3.0e38f);  // finite: a row without a finite logit
     const int32_t key_top = key32(__float_as_uint(m)) >> 16;
@@ -743,7 +764,7 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       if (!split) rc->cut_idx = INT32_MAX;  // else whoever holds the last token kept of the group writes it
       rc->n_kept = have_cut ? (int32_t)(cut.cnt_above + cut.j) : (int32_t)n_kept_all;
       rc->z_fix = have_cut ? cut.mass_above + (u64)cut.j * cut.w_key : w_k;
-      rc->slices = 0;
+      rc->listed = 0;
       if (n_kept_out != nullptr) n_kept_out[row] = have_cut ? (int32_t)(cut.cnt_above + cut.j) : (int32_t)n_kept_all;
     }
     // ---- only when the cut splits a group of equal keys (the usual thing with bf16): the index of the last one kept.
@@ -778,16 +799,17 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
 }
 
 // ---- acceptance: a cluster of kC CTAs per branch ----------------------------------------------------------
-// Every CTA walks the chain; the stop row's kept masses per slice come with the cut, or, when the cut came from the
-// windows, are summed here, each CTA taking a share of the row.
+// Every CTA walks the chain.  When the stop row's kept tokens are listed, the first CTA draws from the list; else the kept
+// masses of the row's slices are summed first, each CTA taking a share of the row.
 template <int kC>
 __global__ void __launch_bounds__(kT)
 accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2,
-                       const RowCut *__restrict__ cuts, const u64 *__restrict__ slice_mass, int n_slices,
+                       const RowCut *__restrict__ cuts, const u64 *__restrict__ lists, int n_slices,
                        const int32_t *__restrict__ draft_ids, const int32_t *__restrict__ cu_draft,
                        const float *__restrict__ u_accept, const float *__restrict__ u_final, int32_t *__restrict__ n_accept,
                        int32_t *__restrict__ final_id, float *__restrict__ p_draft) {
   __shared__ u64 s_mass[kMaxSlices], s_w64[kWarps];
+  __shared__ int32_t s_idx[kListCap];
   __shared__ u64 s_before, s_total;
   __shared__ int s_n, s_slice;
   namespace cg = cooperative_groups;
@@ -822,11 +844,9 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
 
   // ---- the final token: inverse CDF over the kept tokens of the stop row, the rejected one removed
   const RowCut rc = cuts[r0 + n];
-  const bool given = rc.slices != 0;  // every CTA of the cluster sees the same
-  if (given && rank != 0) return;
+  const bool listed = rc.listed != 0;  // every CTA of the cluster sees the same
+  if (listed && rank != 0) return;
   const uint16_t *rp = logits + (int64_t)(r0 + n) * row_stride;
-  const int slice_len = slice_len_of(vocab);
-  const int spc = given ? n_slices : (n_slices + kC - 1) / kC, sl0 = min(n_slices, rank * spc), n_here = min(spc, n_slices - sl0);
   int32_t dead = -1;
   u64 w_dead = 0;
   if (n < L) {
@@ -839,34 +859,62 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
       }
     }
   }
-  if (given) {
-    const u64 *sm = slice_mass + (int64_t)(r0 + n) * n_slices;
-    for (int i = tid; i < n_here; i += kT) s_mass[i] = sm[i];
-  } else {  // a warp per slice, a lane per vector
-    const float cut_x = rc.cut_key == kNoKey ? -INFINITY : __uint_as_float(f_of_key16(rc.cut_key >> 16));
-    for (int i = warp; i < n_here; i += kWarps) {
-      u64 mass = 0;
-      const int32_t s_end = min(vocab, (sl0 + i + 1) * slice_len);
-      for (int32_t e = (sl0 + i) * slice_len + lane * 8; e < s_end; e += 256) {
-        const uint4 v = e + 8 <= vocab ? __ldg(reinterpret_cast<const uint4 *>(rp + e)) : ragged_vec(rp, vocab >> 3, vocab & 7);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
-          const float x = __uint_as_float(f);
-          if (x > cut_x || (x == cut_x && e + j <= rc.cut_idx)) mass += wfix_of(f, rc.m, k_log2);
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mass += __shfl_xor_sync(0xFFFFFFFFu, mass, o);
-      if (lane == 0) s_mass[i] = mass;
-    }
-  }
-  __syncthreads();
   const u64 total = rc.z_fix - w_dead;
   // smallest v whose cumulative mass exceeds u * total; the masses are integers, so "exceeds floor(u * total)"
   u64 target = (u64)(u_fin * (double)total);
   if (total > 0 && target >= total) target = total - 1;
+  if (listed) {
+    // the smallest index whose cumulative mass exceeds the target: every kept token sums those up to its own index
+    const u64 *list = lists + (int64_t)(r0 + n) * kListCap;
+    for (int i = tid; i < rc.n_kept; i += kT) {
+      const u64 e = list[i];
+      s_idx[i] = cand_idx(e);
+      s_mass[i] = s_idx[i] == dead ? 0 : wfix_of(f_of_key16(cand_key16(e)), rc.m, k_log2);
+    }
+    __syncthreads();
+    for (int i = tid; i < rc.n_kept; i += kT) {
+      u64 upto = 0;
+#pragma unroll 4
+      for (int j = 0; j < rc.n_kept; ++j) upto += s_idx[j] <= s_idx[i] ? s_mass[j] : 0;
+      if (s_mass[i] > 0 && upto - s_mass[i] <= target && target < upto) final_id[b] = s_idx[i];
+    }
+    if (total == 0 && tid == 0) final_id[b] = 0;  // a row without mass
+    return;
+  }
+  const int slice_len = slice_len_of(vocab);
+  const int spc = (n_slices + kC - 1) / kC, sl0 = min(n_slices, rank * spc), n_here = min(spc, n_slices - sl0);
+  const float cut_x = rc.cut_key == kNoKey ? -INFINITY : __uint_as_float(f_of_key16(rc.cut_key >> 16));
+  for (int i0 = warp; i0 < n_here; i0 += 4 * kWarps) {  // a warp per slice, a lane per vector, four slices in flight
+    u64 mass[4] = {0, 0, 0, 0};
+    for (int32_t off = lane * 8; off < slice_len; off += 256) {
+      uint4 v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int32_t e = (sl0 + i0 + q * kWarps) * slice_len + off;
+        v[q] = make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
+        if (i0 + q * kWarps < n_here && e < vocab)
+          v[q] = e + 8 <= vocab ? __ldg(reinterpret_cast<const uint4 *>(rp + e)) : ragged_vec(rp, vocab >> 3, vocab & 7);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int32_t e = (sl0 + i0 + q * kWarps) * slice_len + off;
+        const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
+          const float x = __uint_as_float(f);
+          if (x > cut_x || (x == cut_x && e + j <= rc.cut_idx)) mass[q] += wfix_of(f, rc.m, k_log2);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mass[q] += __shfl_xor_sync(0xFFFFFFFFu, mass[q], o);
+      if (lane == 0 && i0 + q * kWarps < n_here) s_mass[i0 + q * kWarps] = mass[q];
+    }
+  }
+  __syncthreads();
   const int spt = (n_here + kT - 1) / kT;  // slices per thread, consecutive
   u64 w[kMaxSlices / kT], mine = 0, all, base = 0;
 #pragma unroll
@@ -880,7 +928,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
     mine += w[i];
   }
   u64 cum = block_scan<kT, u64>(mine, s_w64, all) - mine;
-  if (kC > 1 && !given) {
+  if (kC > 1) {
     if (tid == 0) s_total = all;
     cluster.sync();
     for (int q = 0; q < rank; ++q) base += *cluster.map_shared_rank(&s_total, q);
@@ -911,11 +959,11 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
     }
   }
   if (total == 0 && rank == 0 && tid == 0) final_id[b] = 0;  // a row without mass
-  if (kC > 1 && !given) cluster.sync();  // nobody leaves while its total is being read
+  if (kC > 1) cluster.sync();  // nobody leaves while its total is being read
 }
 
 struct ScratchLayout {
-  size_t cuts, slices, keys, stats, open, bytes;
+  size_t cuts, lists, maxima, stats, open, bytes;
   int n_chunks, n_slices;
 };
 ScratchLayout filter_layout(int32_t vocab, int32_t n_rows) {
@@ -929,11 +977,11 @@ ScratchLayout filter_layout(int32_t vocab, int32_t n_rows) {
     return o;
   };
   s.cuts = take((size_t)n_rows * sizeof(RowCut));
-  s.slices = take((size_t)n_rows * s.n_slices * sizeof(u64));
-  s.keys = take((size_t)n_rows * s.n_chunks * 32 * kVec * sizeof(uint16_t));
+  s.lists = take((size_t)n_rows * kListCap * sizeof(u64));
+  s.maxima = take((size_t)n_rows * s.n_chunks * 32 * kVec * sizeof(uint16_t));
   s.stats = take((size_t)n_rows * s.n_chunks * sizeof(float2));
   s.open = take(((size_t)n_rows + 1) * sizeof(int32_t));
-  s.bytes = off + 16;  // the caller's scratch is 8-byte aligned, the keys are read 16 bytes at a time
+  s.bytes = off;
   return s;
 }
 
@@ -989,11 +1037,11 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
   const int32_t vocab = ctx->model.vocab;
   const float k_log2 = 1.4426950408889634f / temperature;
   const ScratchLayout L = filter_layout(vocab, n_rows);
-  unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)scratch + 15) & ~(uintptr_t)15);
+  unsigned char *base = reinterpret_cast<unsigned char *>(scratch);
   auto *lg = reinterpret_cast<const uint16_t *>(logits);
   auto *cuts = reinterpret_cast<RowCut *>(base + L.cuts);
-  auto *slices = reinterpret_cast<u64 *>(base + L.slices);
-  auto *keys = reinterpret_cast<uint16_t *>(base + L.keys);
+  auto *lists = reinterpret_cast<u64 *>(base + L.lists);
+  auto *maxima = reinterpret_cast<uint16_t *>(base + L.maxima);
   auto *stats = reinterpret_cast<float2 *>(base + L.stats);
   auto *n_open = reinterpret_cast<int32_t *>(base + L.open);
   const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
@@ -1008,22 +1056,21 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
   const int k_sel = by_k ? top_k : kSelTopP;
   // Groups of 64 tokens when that makes many more of them than k_sel, else of 8
   const bool wide = vocab / 64 >= 4 * (int64_t)k_sel;
-  const int64_t n_keys = (int64_t)L.n_chunks * 32 * (wide ? 1 : kVec);
   // Can a few leading tokens decide a row?  With a top-k up to kSelMax always.  With top-p alone mostly, but then the rows
   // they leave open go through the windows all the same, so the candidates pay only when they spare many rounds of those.
-  const bool candidates = n_keys <= kMaxGroups && (by_k ? top_k <= kSelMax : by_p && n_rows > kWindowRounds * w.clusters);
+  const bool candidates = by_k ? top_k <= kSelMax : by_p && n_rows > kWindowRounds * w.clusters;
   if (candidates) {
     auto scan = by_k ? (wide ? filter_scan_kernel<false, kVec> : filter_scan_kernel<false, 1>)
                      : (wide ? filter_scan_kernel<true, kVec> : filter_scan_kernel<true, 1>);
     const uint32_t total = (uint32_t)n_rows * L.n_chunks;
     const unsigned grid = std::min((total + kWarps - 1) / kWarps, (uint32_t)(ctx->sm_count * kScanCtasPerSm));
-    scan<<<grid, kT, 0, s>>>(lg, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, keys, stats, n_open);
+    scan<<<grid, kT, 0, s>>>(lg, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, maxima, stats, n_open);
     ctx->launches++;
     if (int rc = cuda_fail(cudaGetLastError(), "filter_scan_kernel launch")) return rc;
     ctx->launches++;
     if (int rc = cuda_fail(launch_dependent(wide ? filter_cut_kernel<kVec> : filter_cut_kernel<1>, dim3((unsigned)n_rows), dim3(kT),
-                                            (size_t)n_keys * 2, s, lg, stride, vocab, k_log2, top_k, top_p, k_sel, L.n_chunks, keys, stats, cuts,
-                                            slices, L.n_slices, n_kept, n_open, n_open + 1),
+                                            0, s, lg, stride, vocab, k_log2, top_k, top_p, k_sel, L.n_chunks, maxima, stats, cuts, lists, n_kept,
+                                            n_open, n_open + 1),
                            "filter_cut_kernel launch"))
       return rc;
     kc = 8;  // few rows are left, as a rule: the most CTAs for each
@@ -1036,12 +1083,12 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
                          "filter_window_kernel launch"))
     return rc;
   ctx->launches++;
-  // slices of a stop row to sum: always after the windows, hardly ever after the candidates of a top-k
+  // is there a stop row to walk?  Always after the windows, hardly ever after the candidates of a top-k
   if (candidates && by_k)
-    return cuda_fail(launch_dependent(accept_filtered_kernel<1>, dim3((unsigned)n_branch), dim3(kT), 0, s, lg, stride, vocab, k_log2, cuts, slices,
+    return cuda_fail(launch_dependent(accept_filtered_kernel<1>, dim3((unsigned)n_branch), dim3(kT), 0, s, lg, stride, vocab, k_log2, cuts, lists,
                                       L.n_slices, drafts, cu_draft, u_accept, u_final, n_accept, final_id, p_draft),
                      "accept_filtered_kernel launch");
-  return cuda_fail(launch_clusters(accept_filtered_kernel<8>, 8, n_branch, kT, 0, s, lg, stride, vocab, k_log2, cuts, slices, L.n_slices, drafts,
+  return cuda_fail(launch_clusters(accept_filtered_kernel<8>, 8, n_branch, kT, 0, s, lg, stride, vocab, k_log2, cuts, lists, L.n_slices, drafts,
                                    cu_draft, u_accept, u_final, n_accept, final_id, p_draft),
                    "accept_filtered_kernel launch");
 }
