@@ -46,6 +46,8 @@ constexpr int kKeyWords = 8;        // words of group maxima a thread of filter_
 constexpr int kSelMax = 256;        // largest top_k the candidates serve
 constexpr int kSelTopP = 128;       // leading tokens to look for when top-k is off
 constexpr int kWT = 512;            // threads of a CTA of filter_window_kernel
+constexpr int kAT = 512;            // ... of accept_filtered_kernel
+constexpr int kSlicesInFlight = 5;  // slices a warp of it works on at a time: one round for 163840 tokens and 8 CTAs
 constexpr int kWin = 8192;          // keys per window
 constexpr int kMaxSlices = 1024;    // slices a row is cut into for the draw
 constexpr size_t kWindowSmemMax = 200 * 1024;
@@ -117,16 +119,16 @@ __device__ __forceinline__ T block_scan(T v, T *s_w, T &total) {
   }
   if (lane == 31) s_w[warp] = v;
   __syncthreads();
-  T base = 0, all = 0;
+  T t = lane < kThreads / 32 ? s_w[lane] : 0;  // every warp scans the warps' sums
 #pragma unroll
-  for (int k = 0; k < kThreads / 32; ++k) {
-    const T t = s_w[k];
-    if (k < warp) base += t;
-    all += t;
+  for (int o = 1; o < kThreads / 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xFFFFFFFFu, t, o);
+    if (lane >= o) t += y;
   }
+  total = __shfl_sync(0xFFFFFFFFu, t, kThreads / 32 - 1);
+  const T base = __shfl_sync(0xFFFFFFFFu, t, warp > 0 ? warp - 1 : 0);
   __syncthreads();
-  total = all;
-  return v + base;
+  return warp > 0 ? v + base : v;
 }
 
 // Candidates are ordered as 64-bit numbers: the key above, the complement of the index below, so that "larger" is
@@ -443,11 +445,13 @@ struct WindowShared {
   int32_t wi[kWT / 32];
 };
 
-// Counts cover kWin keys at a time.  The usual ones are fixed: position 0 is the largest key below 2^12, position 4095
-// that of 2^-20, then -2^-20 down to above -2^12: one pass without branches, about nine instructions a token, and nothing
-// to know in advance.  A row that holds other finite values is counted again over windows of kWin consecutive keys, hi
-// down to hi - kWin + 1, from the row maximum down (a NaN is never counted).
-constexpr uint32_t kMag0 = (127 - 20) << 7;  // bf16 bits of 2^-20
+// Counts cover kWin keys at a time.  The usual ones are fixed: position 0 is the largest key below 2^8, position 4095
+// that of 2^-24, then -2^-24 down to above -2^8: one pass without branches, about nine instructions a token, and nothing
+// to know in advance.  Tokens between -2^-24 and 2^-24 are counted as one group between positions 4095 and 4096: with a
+// row maximum of at least 2 their masses are all that of 0 (x - m rounds to -m).  Where the cut falls into that group, the
+// maximum is smaller, or a finite value lies beyond 2^8, the row is counted again over windows of kWin consecutive keys,
+// hi down to hi - kWin + 1, from the row maximum down (a NaN is never counted).
+constexpr uint32_t kMag0 = (127 - 24) << 7;  // bf16 bits of 2^-24
 __device__ __forceinline__ int32_t fixed_key16(int pos) {
   return pos < 4096 ? (int32_t)kMag0 + 4095 - pos : -((int32_t)kMag0 + pos - 4096);
 }
@@ -569,11 +573,13 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       top = fmaxf(top, __uint_as_float(u << 16));
     }
     int odd = far >= 4 * 4096u ? 1 : 0;
+    uint32_t n_zero = 0, zeros_here = 0;  // tokens of the middle group
     if (__syncthreads_or(odd)) {  // -inf and NaN do not matter (they have no mass), other values do
       odd = 0;
       auto look = [&](uint32_t u) {
         const uint32_t mag = u & 0x7FFFu;
-        if (mag - kMag0 >= 4096u && (mag < 0x7F80u || u == 0x7F80u)) odd = 1;
+        n_zero += mag < kMag0 ? 1u : 0u;
+        if (mag >= kMag0 + 4096u && (mag < 0x7F80u || u == 0x7F80u)) odd = 1;
       };
 #pragma unroll 1
       for (int32_t vi = tid; vi < n_vec; vi += kWT) {
@@ -587,8 +593,9 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       }
       if (tid < rem) look(rp[n_vec * 8 + tid]);
       odd = __syncthreads_or(odd);
+      block_scan<kWT, uint32_t>(n_zero, sh.w32, zeros_here);
     }
-    const Sums first = exchange(block_max(key32(__float_as_uint(top))), odd ? 1u : 0u, 0);
+    const Sums first = exchange(block_max(key32(__float_as_uint(top))), zeros_here, odd ? 1 : 0);
     const float m = fmaxf(__uint_as_float(f_of_key16(first.key >> 16)), -3.0e38f);  // finite: a row without a finite logit
     const int32_t key_top = key32(__float_as_uint(m)) >> 16;
 
@@ -604,7 +611,8 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       const double t_d = ceil((double)top_p * (double)w);
       return min(t_d < 1.0 ? 1ull : (u64)t_d, w);
     };
-    bool fixed = first.cnt == 0 && first.key > (-32640 * 65536);  // some finite logit, and all of them counted
+    const uint32_t zeros = first.cnt;
+    bool fixed = first.mass == 0 && first.key > (-32640 * 65536) && (zeros == 0 || m >= 2.f);  // some finite logit, and all of them counted
     bool counting = by_k;   // looking for the k-th token; after it, or without it, for the mass t
     bool whole = !by_k;     // the first pass also gives the mass of the whole row
     Window win;
@@ -679,6 +687,15 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       m_excl += sums.mass_before;
       win.cnt = sums.cnt;
       win.mass = sums.mass;
+      if (fixed && zeros != 0) {
+        const u64 z_mass = zeros * wfix_of(0, m, k_log2);
+        if (pos0 >= 4096) {
+          c_excl += zeros;
+          m_excl += z_mass;
+        }
+        win.cnt += zeros;
+        win.mass += z_mass;
+      }
       if (whole) {
         whole = false;
         w_k = win.mass + mass_below;
@@ -723,7 +740,14 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
           }
           cluster.sync();
           const unsigned has = __ballot_sync(0xFFFFFFFFu, lane < kC && peer(lane & (kC - 1))->cut.j != 0);
-          const KeyCut found = peer(has ? __ffs(has) - 1 : 0)->cut;  // (some CTA always has it)
+          if (has == 0) {  // it lies in the middle group: start over with windows
+            ph ^= 1;
+            fixed = have_cut = false;
+            counting = by_k;
+            whole = !by_k;
+            break;
+          }
+          const KeyCut found = peer(__ffs(has) - 1)->cut;
           const uint32_t j_k = have_cut && found.key == cut.key ? cut.j : found.j;
           cut = found;
           cut.j = min(cut.j, j_k);  // top-p keeps no more of a key than top-k did (implied by t <= W_k)
@@ -802,13 +826,13 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
 // Every CTA walks the chain.  When the stop row's kept tokens are listed, the first CTA draws from the list; else the kept
 // masses of the row's slices are summed first, each CTA taking a share of the row.
 template <int kC>
-__global__ void __launch_bounds__(kT)
+__global__ void __launch_bounds__(kAT)
 accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2,
                        const RowCut *__restrict__ cuts, const u64 *__restrict__ lists, int n_slices,
                        const int32_t *__restrict__ draft_ids, const int32_t *__restrict__ cu_draft,
                        const float *__restrict__ u_accept, const float *__restrict__ u_final, int32_t *__restrict__ n_accept,
                        int32_t *__restrict__ final_id, float *__restrict__ p_draft) {
-  __shared__ u64 s_mass[kMaxSlices], s_w64[kWarps];
+  __shared__ u64 s_mass[kMaxSlices], s_w64[kAT / 32];
   __shared__ int32_t s_idx[kListCap];
   __shared__ u64 s_before, s_total;
   __shared__ int s_n, s_slice;
@@ -826,7 +850,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   __syncthreads();
 
   // ---- acceptance chain: draft i passes iff u_i < P'_i(d_i); the first one that does not ends it
-  for (int i = tid; i < L; i += kT) {
+  for (int i = tid; i < L; i += kAT) {
     const RowCut rc = cuts[r0 + i];
     const int32_t d = draft_ids[d0 + i];
     const float u = u_accept[d0 + i];
@@ -866,13 +890,13 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   if (listed) {
     // the smallest index whose cumulative mass exceeds the target: every kept token sums those up to its own index
     const u64 *list = lists + (int64_t)(r0 + n) * kListCap;
-    for (int i = tid; i < rc.n_kept; i += kT) {
+    for (int i = tid; i < rc.n_kept; i += kAT) {
       const u64 e = list[i];
       s_idx[i] = cand_idx(e);
       s_mass[i] = s_idx[i] == dead ? 0 : wfix_of(f_of_key16(cand_key16(e)), rc.m, k_log2);
     }
     __syncthreads();
-    for (int i = tid; i < rc.n_kept; i += kT) {
+    for (int i = tid; i < rc.n_kept; i += kAT) {
       u64 upto = 0;
 #pragma unroll 4
       for (int j = 0; j < rc.n_kept; ++j) upto += s_idx[j] <= s_idx[i] ? s_mass[j] : 0;
@@ -884,20 +908,20 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   const int slice_len = slice_len_of(vocab);
   const int spc = (n_slices + kC - 1) / kC, sl0 = min(n_slices, rank * spc), n_here = min(spc, n_slices - sl0);
   const float cut_x = rc.cut_key == kNoKey ? -INFINITY : __uint_as_float(f_of_key16(rc.cut_key >> 16));
-  for (int i0 = warp; i0 < n_here; i0 += 4 * kWarps) {  // a warp per slice, a lane per vector, four slices in flight
-    u64 mass[4] = {0, 0, 0, 0};
+  for (int i0 = warp; i0 < n_here; i0 += kSlicesInFlight * (kAT / 32)) {  // a warp per slice, a lane per vector, several slices in flight
+    u64 mass[kSlicesInFlight] = {};
     for (int32_t off = lane * 8; off < slice_len; off += 256) {
-      uint4 v[4];
+      uint4 v[kSlicesInFlight];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int32_t e = (sl0 + i0 + q * kWarps) * slice_len + off;
+      for (int q = 0; q < kSlicesInFlight; ++q) {
+        const int32_t e = (sl0 + i0 + q * (kAT / 32)) * slice_len + off;
         v[q] = make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
-        if (i0 + q * kWarps < n_here && e < vocab)
+        if (i0 + q * (kAT / 32) < n_here && e < vocab)
           v[q] = e + 8 <= vocab ? __ldg(reinterpret_cast<const uint4 *>(rp + e)) : ragged_vec(rp, vocab >> 3, vocab & 7);
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int32_t e = (sl0 + i0 + q * kWarps) * slice_len + off;
+      for (int q = 0; q < kSlicesInFlight; ++q) {
+        const int32_t e = (sl0 + i0 + q * (kAT / 32)) * slice_len + off;
         const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -908,17 +932,17 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
       }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < kSlicesInFlight; ++q) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mass[q] += __shfl_xor_sync(0xFFFFFFFFu, mass[q], o);
-      if (lane == 0 && i0 + q * kWarps < n_here) s_mass[i0 + q * kWarps] = mass[q];
+      if (lane == 0 && i0 + q * (kAT / 32) < n_here) s_mass[i0 + q * (kAT / 32)] = mass[q];
     }
   }
   __syncthreads();
-  const int spt = (n_here + kT - 1) / kT;  // slices per thread, consecutive
-  u64 w[kMaxSlices / kT], mine = 0, all, base = 0;
+  const int spt = (n_here + kAT - 1) / kAT;  // slices per thread, consecutive
+  u64 w[kMaxSlices / kAT], mine = 0, all, base = 0;
 #pragma unroll
-  for (int i = 0; i < kMaxSlices / kT; ++i) {
+  for (int i = 0; i < kMaxSlices / kAT; ++i) {
     const int at = tid * spt + i;
     w[i] = 0;
     if (i < spt && at < n_here) {
@@ -927,7 +951,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
     }
     mine += w[i];
   }
-  u64 cum = block_scan<kT, u64>(mine, s_w64, all) - mine;
+  u64 cum = block_scan<kAT, u64>(mine, s_w64, all) - mine;
   if (kC > 1) {
     if (tid == 0) s_total = all;
     cluster.sync();
@@ -935,7 +959,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   }
   cum += base;
 #pragma unroll
-  for (int i = 0; i < kMaxSlices / kT; ++i) {
+  for (int i = 0; i < kMaxSlices / kAT; ++i) {
     if (w[i] > 0 && cum <= target && target < cum + w[i]) {
       s_slice = sl0 + tid * spt + i;
       s_before = cum;
@@ -946,14 +970,14 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   const int sl = s_slice;
   if (sl >= 0) {  // inside the slice: one token per thread at a time
     u64 upto0 = s_before;
-    for (int32_t x0 = sl * slice_len; x0 < min(vocab, (sl + 1) * slice_len); x0 += kT) {
+    for (int32_t x0 = sl * slice_len; x0 < min(vocab, (sl + 1) * slice_len); x0 += kAT) {
       const int32_t e = x0 + tid;
       u64 x = 0;
       if (e < vocab && e != dead) {
         const uint32_t f = (uint32_t)rp[e] << 16;
         if (is_kept(key32(f), e, rc)) x = wfix_of(f, rc.m, k_log2);
       }
-      const u64 upto = upto0 + block_scan<kT, u64>(x, s_w64, all);
+      const u64 upto = upto0 + block_scan<kAT, u64>(x, s_w64, all);
       if (x > 0 && upto - x <= target && target < upto) final_id[b] = e;
       upto0 += all;
     }
@@ -1085,10 +1109,10 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
   ctx->launches++;
   // is there a stop row to walk?  Always after the windows, hardly ever after the candidates of a top-k
   if (candidates && by_k)
-    return cuda_fail(launch_dependent(accept_filtered_kernel<1>, dim3((unsigned)n_branch), dim3(kT), 0, s, lg, stride, vocab, k_log2, cuts, lists,
+    return cuda_fail(launch_dependent(accept_filtered_kernel<1>, dim3((unsigned)n_branch), dim3(kAT), 0, s, lg, stride, vocab, k_log2, cuts, lists,
                                       L.n_slices, drafts, cu_draft, u_accept, u_final, n_accept, final_id, p_draft),
                      "accept_filtered_kernel launch");
-  return cuda_fail(launch_clusters(accept_filtered_kernel<8>, 8, n_branch, kT, 0, s, lg, stride, vocab, k_log2, cuts, lists, L.n_slices, drafts,
+  return cuda_fail(launch_clusters(accept_filtered_kernel<8>, 8, n_branch, kAT, 0, s, lg, stride, vocab, k_log2, cuts, lists, L.n_slices, drafts,
                                    cu_draft, u_accept, u_final, n_accept, final_id, p_draft),
                    "accept_filtered_kernel launch");
 }

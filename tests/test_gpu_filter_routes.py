@@ -8,13 +8,13 @@ from test_gpu_accept_filtered import _check, _run
 
 pytestmark = pytest.mark.gpu
 
-# vocabulary, branches, drafts per branch, top_k, top_p
+# vocabulary, branches, drafts per branch, top_k, top_p (not 0.95 with 20 tokens of equal mass: 19 of them are a step of it)
 ROUTES = [
-    (5, 3, 2, 2, 0.9), (300, 4, 3, 20, 0.95), (1023, 4, 3, 0, 0.9), (1025, 170, 2, 0, 0.9),  # fewer groups than leading tokens
-    (5119, 5, 3, 20, 0.95), (5120, 5, 3, 20, 0.95), (5121, 5, 3, 20, 1.0),                     # groups of 8, of 64
+    (5, 3, 2, 2, 0.9), (300, 4, 3, 20, 0.93), (1023, 4, 3, 0, 0.9), (1025, 170, 2, 0, 0.9),  # fewer groups than leading tokens
+    (5119, 5, 3, 20, 0.93), (5120, 5, 3, 20, 0.93), (5121, 5, 3, 20, 1.0),                     # groups of 8, of 64
     (4100, 5, 3, 256, 0.97), (65600, 5, 2, 256, 1.0), (65600, 5, 2, 257, 1.0),                 # the largest top_k of the candidates
     (32771, 12, 2, 0, 0.95), (32771, 160, 2, 0, 0.95), (40009, 30, 4, 0, 0.6),                 # few rows by windows, many by candidates
-    (655361, 2, 1, 20, 0.95), (1700003, 1, 1, 0, 0.9), (9000, 2, 1, 0, 1.0),                   # too many groups; shares beyond shared memory
+    (655361, 2, 1, 20, 0.93), (1700003, 1, 1, 0, 0.9), (9000, 2, 1, 0, 1.0),                   # too many groups; shares beyond shared memory
 ]
 
 
@@ -33,6 +33,8 @@ def test_routes(vocab, nb, L, top_k, top_p):
             x[r, : max(1, vocab // 100)] = 1e-9
             x[r, vocab // 2] = -7000.0
     x[::5, vocab // 3: vocab // 2] = -np.inf
+    x[::6, vocab // 5: vocab // 4] = 1e-8  # with the ties of 0 in the coarse rows: the cut in, above and below the middle group
+    x[::9] = np.minimum(x[::9], -1.0)
     bits = bf16_round(x)
     bits[::3, -1] = 0x7FC0  # NaN counts as -inf
     cu = (np.arange(nb + 1) * L).astype(np.int32)
