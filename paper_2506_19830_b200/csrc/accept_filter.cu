@@ -40,18 +40,18 @@ constexpr int kWarps = kT / 32;
 constexpr int kVec = 8;             // 16-byte vectors a lane of filter_scan_kernel takes at a time
 constexpr int kChunk = 32 * kVec * 8;  // logits a warp takes at a time
 constexpr int kScanCtasPerSm = 4;
-constexpr int kGroupCap = 512;      // groups it reads again
-constexpr int kListCap = 512;       // candidates of a row
+constexpr int kGroupCap = 1344;     // groups filter_cut_kernel reads again (k_sel + k_sel / 4 + 4 at most, but for ties)
+constexpr int kListCap = 1408;      // candidates of a row
+constexpr int kListOut = 256;       // kept tokens that go out as a list
 constexpr int kKeyWords = 8;        // words of group maxima a thread of filter_cut_kernel keeps in registers
-constexpr int kSelMax = 256;        // largest top_k the candidates serve
+constexpr int kSelMax = 1024;       // largest top_k the candidates serve
 constexpr int kSelTopP = 128;       // leading tokens to look for when top-k is off
 constexpr int kWT = 512;            // threads of a CTA of filter_window_kernel
 constexpr int kAT = 512;            // ... of accept_filtered_kernel
 constexpr int kSlicesInFlight = 5;  // slices a warp of it works on at a time: one round for 163840 tokens and 8 CTAs
 constexpr int kWin = 8192;          // keys per window
 constexpr int kMaxSlices = 1024;    // slices a row is cut into for the draw
-constexpr size_t kWindowSmemMax = 200 * 1024;
-constexpr int kWindowRounds = 3;    // rounds of rows through the windows that a candidate pass has to spare
+constexpr size_t kWindowSmemMax = 112 * 1024;  // two CTAs per SM
 // Relative distance between the fp32 sum of a row's masses and their integer sum: the argument of an exponential is
 // rounded at magnitude 40 (2^-19.4 absolute: 1e-6 of the mass), ex2.approx is good to 2^-22 on both sides, an fp32 sum of
 // 64 terms and some 30 further additions to 5e-6, rounding masses to 2^-40 of the largest to 1e-7; rounded up.
@@ -406,7 +406,7 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
         rc.cut_idx = cand_idx(s_sorted[r]);
         rc.n_kept = r + 1;
         rc.z_fix = s_cum[r];
-        rc.listed = 1;
+        rc.listed = r < kListOut ? 1 : 0;
         rc.pad = 0;
         cuts[row] = rc;
         if (n_kept_out != nullptr) n_kept_out[row] = r + 1;
@@ -416,7 +416,7 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
     }
   }
   __syncthreads();
-  for (int i = tid; i < s_kept; i += kT) lists[row * kListCap + i] = s_sorted[i];
+  if (tid < s_kept && s_kept <= kListOut) lists[row * kListOut + tid] = s_sorted[tid];
 }
 
 // ---- the cut of a row from counts per key: a cluster of kC CTAs per row --------------------------------------
@@ -479,7 +479,11 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rank = (int)cluster.block_rank();
+  const int rank = kC == 1 ? 0 : (int)cluster.block_rank();
+  auto sync_all = [&]() {
+    if (kC == 1) __syncthreads();
+    else cluster.sync();
+  };
   constexpr int kPW = kWin / kC, kPer = kPW / kWT;  // positions of this CTA and of one thread
   const int32_t share = share_of(vocab, kC), e0 = min(vocab, rank * share), e1 = min(vocab, e0 + share);
   const int32_t n_vec = (e1 - e0) >> 3, rem = (e1 - e0) & 7;
@@ -489,7 +493,7 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   const int n_rows = n_all > 0 ? n_all : *n_open;
   int ph = 0;
 
-  auto peer = [&](int r) -> const Xch * { return cluster.map_shared_rank(&sh.xch[ph], r); };
+  auto peer = [&](int r) -> const Xch * { return kC == 1 ? &sh.xch[ph] : cluster.map_shared_rank(&sh.xch[ph], r); };
   auto block_max = [&](int32_t v) -> int32_t {
     v = __reduce_max_sync(0xFFFFFFFFu, v);
     if (lane == 0) sh.wi[warp] = v;
@@ -507,7 +511,7 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       sh.xch[ph].cnt = cnt;
       sh.xch[ph].mass = mass;
     }
-    cluster.sync();
+    sync_all();
     Sums r = {INT32_MIN, 0, 0, 0, 0};
     if (lane < kC) {
       const Xch *x = peer(lane);
@@ -556,15 +560,23 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       if (t4 < 4 * 4096u) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory");
       far = max(far, t4);
     };
-    for (int32_t vi = tid; vi < n_vec; vi += kWT) {
-      const uint4 v = reinterpret_cast<const uint4 *>(rp)[vi];
-      mx = max_bf2(mx, max_bf2(max_bf2(v.x, v.y), max_bf2(v.z, v.w)));
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    constexpr int kFly = kC >= 4 ? 1 : 4;  // loads in flight: the share of a small cluster may come from HBM here
+    for (int32_t v0 = tid; v0 < n_vec; v0 += kFly * kWT) {
+      uint4 v[kFly];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        count((w[j] << 2) & 0x1FFFCu, (int32_t)(w[j] << 16) >> 31);
-        count((w[j] >> 14) & 0x1FFFCu, (int32_t)w[j] >> 31);
-      }
+      for (int k = 0; k < kFly; ++k)
+        if (v0 + k * kWT < n_vec) v[k] = reinterpret_cast<const uint4 *>(rp)[v0 + k * kWT];
+#pragma unroll
+      for (int k = 0; k < kFly; ++k)
+        if (v0 + k * kWT < n_vec) {
+          mx = max_bf2(mx, max_bf2(max_bf2(v[k].x, v[k].y), max_bf2(v[k].z, v[k].w)));
+          const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            count((w[j] << 2) & 0x1FFFCu, (int32_t)(w[j] << 16) >> 31);
+            count((w[j] >> 14) & 0x1FFFCu, (int32_t)w[j] >> 31);
+          }
+        }
     }
     float top = fmaxf(lo_f(mx), hi_f(mx));
     if (tid < rem) {
@@ -670,7 +682,7 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       for (int i = 0; i < kPer; ++i) c[i] = 0;
 #pragma unroll
       for (int q = 0; q < kC; ++q) {
-        const uint32_t *rc = cluster.map_shared_rank(sh.cnt, q) + pos0;
+        const uint32_t *rc = (kC == 1 ? sh.cnt : cluster.map_shared_rank(sh.cnt, q)) + pos0;
 #pragma unroll
         for (int i = 0; i < kPer; ++i) c[i] += rc[i];
       }
@@ -738,7 +750,7 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
                 mass += (u64)c[i] * w;
               }
           }
-          cluster.sync();
+          sync_all();
           const unsigned has = __ballot_sync(0xFFFFFFFFu, lane < kC && peer(lane & (kC - 1))->cut.j != 0);
           if (has == 0) {  // it lies in the middle group: start over with windows
             ph ^= 1;
@@ -792,33 +804,51 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       if (n_kept_out != nullptr) n_kept_out[row] = have_cut ? (int32_t)(cut.cnt_above + cut.j) : (int32_t)n_kept_all;
     }
     // ---- only when the cut splits a group of equal keys (the usual thing with bf16): the index of the last one kept.
-    //      Threads own contiguous runs of vectors; equality of the values is equality of the keys.
+    //      Warps own contiguous runs of vectors (the last one the ragged end too); equality of the values is equality of
+    //      the keys.
     if (split) {
       const uint32_t cb = f_of_key16(cut.key) >> 16, pat = cb | (cb << 16);
-      const int32_t per = (n_vec + kWT - 1) / kWT, v0 = min(n_vec, tid * per), v1 = min(n_vec, v0 + per);
-      auto equal = [&](uint32_t w) -> uint32_t {
-        return __heq2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w), *reinterpret_cast<const __nv_bfloat162 *>(&pat));
+      const int32_t n_all_vec = n_vec + (rem ? 1 : 0), per = (n_all_vec + kWT / 32 - 1) / (kWT / 32);
+      const int32_t v0 = min(n_all_vec, warp * per), v1 = min(n_all_vec, v0 + per);
+      auto vec = [&](int32_t vi) -> uint4 {
+        return vi < n_vec ? reinterpret_cast<const uint4 *>(rp)[vi] : vi < n_all_vec ? ragged_vec(rp, n_vec, rem) : make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
       };
+      auto equal = [&](uint32_t x) -> uint32_t {  // 16 ones per value
+        return __heq2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&x), *reinterpret_cast<const __nv_bfloat162 *>(&pat));
+      };
+      auto equals = [&](const uint4 &v) -> uint32_t { return (__popc(equal(v.x)) + __popc(equal(v.y)) + __popc(equal(v.z)) + __popc(equal(v.w))) >> 4; };
       uint32_t mine = 0, all;
-      for (int32_t vi = v0; vi < v1; ++vi) {
-        const uint4 v = reinterpret_cast<const uint4 *>(rp)[vi];
-        mine += __popc(equal(v.x)) + __popc(equal(v.y)) + __popc(equal(v.z)) + __popc(equal(v.w));
-      }
-      mine >>= 4;  // 16 bits to a value
-      if (tid == kWT - 1)
-        for (int j = 0; j < rem; ++j) mine += equal(rp[n_vec * 8 + j]) & 1u;
-      uint32_t before = block_scan<kWT, uint32_t>(mine, sh.w32, all) - mine;
-      before += exchange(0, all, 0).cnt_before;
+#pragma unroll 4
+      for (int32_t vi = v0 + lane; vi < v1; vi += 32) mine += equals(vec(vi));
+      mine = __reduce_add_sync(0xFFFFFFFFu, mine);
+      uint32_t before = block_scan<kWT, uint32_t>(lane == 0 ? mine : 0, sh.w32, all);
+      before = __shfl_sync(0xFFFFFFFFu, before, 0) - mine;  // in the warps in front of this one ...
+      before += exchange(0, all, 0).cnt_before;             // ... and in the CTAs in front
       if (before < cut.j && cut.j <= before + mine) {
-        uint32_t seen = before;
-        int32_t found = -1;
 #pragma unroll 1
-        for (int32_t i = v0 * 8; i < (tid == kWT - 1 ? n_vec * 8 + rem : v1 * 8) && found < 0; ++i)
-          if ((equal(rp[i]) & 1u) && ++seen == cut.j) found = e0 + i;
-        cuts[row].cut_idx = found;
+        for (int32_t vi = v0 + lane; __any_sync(0xFFFFFFFFu, vi < v1); vi += 32) {
+          const uint4 v = vec(vi < v1 ? vi : n_all_vec);
+          const uint32_t c = equals(v);
+          uint32_t incl = c;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += y;
+          }
+          const uint32_t upto = before + incl;
+          if (upto - c < cut.j && cut.j <= upto) {
+            uint32_t seen = upto - c;
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if ((equal(w[j >> 1]) & ((j & 1) ? 0x10000u : 1u)) && ++seen == cut.j) cuts[row].cut_idx = e0 + vi * 8 + j;
+          }
+          before = __shfl_sync(0xFFFFFFFFu, upto, 31);
+          if (before >= cut.j) break;
+        }
       }
     }
-    cluster.sync();  // nobody leaves, or starts on the next row, while its shared memory is being read
+    sync_all();  // nobody leaves, or starts on the next row, while its shared memory is being read
   }
 }
 
@@ -833,7 +863,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
                        const float *__restrict__ u_accept, const float *__restrict__ u_final, int32_t *__restrict__ n_accept,
                        int32_t *__restrict__ final_id, float *__restrict__ p_draft) {
   __shared__ u64 s_mass[kMaxSlices], s_w64[kAT / 32];
-  __shared__ int32_t s_idx[kListCap];
+  __shared__ int32_t s_idx[kListOut];
   __shared__ u64 s_before, s_total;
   __shared__ int s_n, s_slice;
   namespace cg = cooperative_groups;
@@ -889,7 +919,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   if (total > 0 && target >= total) target = total - 1;
   if (listed) {
     // the smallest index whose cumulative mass exceeds the target: every kept token sums those up to its own index
-    const u64 *list = lists + (int64_t)(r0 + n) * kListCap;
+    const u64 *list = lists + (int64_t)(r0 + n) * kListOut;
     for (int i = tid; i < rc.n_kept; i += kAT) {
       const u64 e = list[i];
       s_idx[i] = cand_idx(e);
@@ -1001,7 +1031,7 @@ ScratchLayout filter_layout(int32_t vocab, int32_t n_rows) {
     return o;
   };
   s.cuts = take((size_t)n_rows * sizeof(RowCut));
-  s.lists = take((size_t)n_rows * kListCap * sizeof(u64));
+  s.lists = take((size_t)n_rows * kListOut * sizeof(u64));
   s.maxima = take((size_t)n_rows * s.n_chunks * 32 * kVec * sizeof(uint16_t));
   s.stats = take((size_t)n_rows * s.n_chunks * sizeof(float2));
   s.open = take(((size_t)n_rows + 1) * sizeof(int32_t));
@@ -1010,18 +1040,32 @@ ScratchLayout filter_layout(int32_t vocab, int32_t n_rows) {
 }
 
 struct WindowShape {
+  int cluster;
   size_t smem;
   bool cached;
-  int clusters;  // on the chip at a time
+  double us;  // estimated time
 };
-WindowShape window_shape(const lr_ctx *ctx, int cluster) {
-  WindowShape w;
-  const size_t fixed = (sizeof(WindowShared) + 15) / 16 * 16, share = (size_t)share_of(ctx->model.vocab, cluster) * 2;
-  w.cached = fixed + share <= kWindowSmemMax;
-  w.smem = fixed + (w.cached ? share : 0);
-  const int per_sm = 2 * (w.smem + 1024) <= 227 * 1024 ? 2 : 1;  // 64 registers a thread allow two
-  w.clusters = std::max(1, ctx->sm_count * per_sm / cluster);
-  return w;
+// Cluster size for n_rows rows through the windows: the one with the smallest estimate.  Two CTAs fit an SM.  The numbers
+// are us per CTA and per 1000 tokens of its share, fitted to measured rounds of rows with one CTA on every SM and with two
+// (rows of 152064 tokens: 14.5 us for 17 by clusters of eight, 27 for 51 by fours, 38 for 74 by fours, 59 for 136 by pairs, 80
+// for 296 by single CTAs, which have no cluster barriers; of 32000: 15 us for 68 by single CTAs, 23 by pairs, 21 for 296).
+WindowShape window_shape(const lr_ctx *ctx, int64_t n_rows) {
+  WindowShape best = {};
+  for (const int c : {8, 4, 2, 1}) {
+    const size_t fixed = (sizeof(WindowShared) + 15) / 16 * 16, share = (size_t)share_of(ctx->model.vocab, c) * 2;
+    WindowShape w;
+    w.cluster = c;
+    w.cached = fixed + share <= kWindowSmemMax;
+    w.smem = fixed + (w.cached ? share : 0);
+    const int64_t clusters = std::max(1, ctx->sm_count * 2 / c);
+    const double k = share_of(ctx->model.vocab, c) * 1e-3;
+    const double one = c == 1 ? 6 + 0.42 * k : c == 2 ? 19 + 0.22 * k : c == 4 ? 14 + 0.2 * k : 11 + 0.18 * k;
+    const double two = c == 1 ? 7 + 0.48 * k : c == 2 ? 22 + 0.5 * k : c == 4 ? 20 + 0.47 * k : 17 + 0.55 * k;
+    const double full = std::min(1.0, std::max(0.0, (double)(n_rows * c - ctx->sm_count) / ctx->sm_count));
+    w.us = (double)((n_rows + clusters - 1) / clusters) * (one + full * (two - one));
+    if (best.cluster == 0 || w.us < best.us) best = w;
+  }
+  return best;
 }
 
 template <class... KArgs, class... Args>
@@ -1045,11 +1089,11 @@ cudaError_t launch_clusters(void (*kernel)(KArgs...), int kc, int clusters, int 
 }  // namespace
 
 int init_accept_filter_kernels() {
-  const int smem = (int)kWindowSmemMax;
-  cudaError_t e = cudaFuncSetAttribute(filter_window_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(filter_window_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(filter_window_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return cuda_fail(e, "filter_window_kernel shared-memory attribute");
+  for (auto kernel : {filter_window_kernel<8>, filter_window_kernel<4>, filter_window_kernel<2>, filter_window_kernel<1>})
+    if (int rc = cuda_fail(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWindowSmemMax),
+                           "filter_window_kernel shared-memory attribute"))
+      return rc;
+  return LR_OK;
 }
 
 size_t accept_filtered_scratch_bytes(int32_t vocab, int32_t n_rows) { return filter_layout(vocab, n_rows).bytes; }
@@ -1069,20 +1113,21 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
   auto *stats = reinterpret_cast<float2 *>(base + L.stats);
   auto *n_open = reinterpret_cast<int32_t *>(base + L.open);
   const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
-  // Cluster size when every row goes through the windows: the largest with room for all rows at a time, else the one with
-  // room for the most.
-  int kc = 8;
-  for (const int c : {4, 2}) {
-    const int have = window_shape(ctx, kc).clusters;
-    if (have < n_rows && window_shape(ctx, c).clusters > have) kc = c;
-  }
-  WindowShape w = window_shape(ctx, kc);
   const int k_sel = by_k ? top_k : kSelTopP;
-  // Groups of 64 tokens when that makes many more of them than k_sel, else of 8
+  // Groups of 64 tokens when that makes many more of them than k_sel, else of 8.  With too few groups of 8 as well the
+  // bound is too low to be of use, unless the whole row fits the list of candidates.
   const bool wide = vocab / 64 >= 4 * (int64_t)k_sel;
-  // Can a few leading tokens decide a row?  With a top-k up to kSelMax always.  With top-p alone mostly, but then the rows
-  // they leave open go through the windows all the same, so the candidates pay only when they spare many rounds of those.
-  const bool candidates = by_k ? top_k <= kSelMax : by_p && n_rows > kWindowRounds * w.clusters;
+  const bool enough = vocab / 8 >= 4 * (int64_t)k_sel || vocab <= kListCap;
+  // Can a few leading tokens decide a row?  With a small top-k always: 17 us against 28 us through the windows for 51 rows
+  // of 152064 tokens and top-k 20, 46 against 213 for 612.  Reading and ranking the groups of a larger one costs about 0.1 us
+  // per k.  With top-p alone they mostly do, but the rows they leave open (taken to be one in five) go through the windows
+  // all the same: 137 us against 213 for 612 rows, 59 against 50 for 136.
+  WindowShape w = window_shape(ctx, n_rows);
+  const WindowShape w_open = window_shape(ctx, (n_rows + 4) / 5);
+  const double us_scan = (double)n_rows * vocab * 2 / 5.5e6;
+  const double us_candidates = by_k ? 12.0 + us_scan + (6.0 + 0.1 * top_k) * ((n_rows + 5 * ctx->sm_count - 1) / (5 * ctx->sm_count))
+                                    : 24.0 + us_scan + 0.02 * n_rows + w_open.us;
+  const bool candidates = enough && (by_k ? top_k <= kSelMax : by_p) && ((by_k && top_k <= 128) || us_candidates < w.us);
   if (candidates) {
     auto scan = by_k ? (wide ? filter_scan_kernel<false, kVec> : filter_scan_kernel<false, 1>)
                      : (wide ? filter_scan_kernel<true, kVec> : filter_scan_kernel<true, 1>);
@@ -1097,18 +1142,21 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
                                             n_open, n_open + 1),
                            "filter_cut_kernel launch"))
       return rc;
-    kc = 8;  // few rows are left, as a rule: the most CTAs for each
-    w = window_shape(ctx, kc);
+    w = by_k ? window_shape(ctx, 1) : w_open;  // after a top-k hardly ever a row is left
   }
   ctx->launches++;
-  auto window = kc == 8 ? filter_window_kernel<8> : kc == 4 ? filter_window_kernel<4> : filter_window_kernel<2>;
-  if (int rc = cuda_fail(launch_clusters(window, kc, candidates ? w.clusters : std::min(n_rows, w.clusters), kWT, w.smem, s, lg, stride, vocab,
+  auto window = w.cluster == 8   ? filter_window_kernel<8>
+                : w.cluster == 4 ? filter_window_kernel<4>
+                : w.cluster == 2 ? filter_window_kernel<2>
+                                 : filter_window_kernel<1>;
+  const int clusters = std::max(1, ctx->sm_count * 2 / w.cluster);
+  if (int rc = cuda_fail(launch_clusters(window, w.cluster, candidates ? clusters : std::min(n_rows, clusters), kWT, w.smem, s, lg, stride, vocab,
                                          k_log2, top_k, top_p, cuts, n_kept, n_open, n_open + 1, candidates ? 0 : n_rows, w.cached ? 1 : 0),
                          "filter_window_kernel launch"))
     return rc;
   ctx->launches++;
-  // is there a stop row to walk?  Always after the windows, hardly ever after the candidates of a top-k
-  if (candidates && by_k)
+  // one CTA per branch when there is no stop row to walk (hardly ever after the candidates of a small top-k) or it is short
+  if ((candidates && by_k && top_k <= kListOut) || vocab <= 16384)
     return cuda_fail(launch_dependent(accept_filtered_kernel<1>, dim3((unsigned)n_branch), dim3(kAT), 0, s, lg, stride, vocab, k_log2, cuts, lists,
                                       L.n_slices, drafts, cu_draft, u_accept, u_final, n_accept, final_id, p_draft),
                      "accept_filtered_kernel launch");

@@ -8,11 +8,15 @@ from test_gpu_accept_filtered import _check, _run
 
 pytestmark = pytest.mark.gpu
 
-# vocabulary, branches, drafts per branch, top_k, top_p (not 0.95 with 20 tokens of equal mass: 19 of them are a step of it)
+# vocabulary, branches, drafts per branch, top_k, top_p (not a multiple of 1 / top_k: with tokens of equal
+# mass the cut would lie on a step)
 ROUTES = [
     (5, 3, 2, 2, 0.9), (300, 4, 3, 20, 0.93), (1023, 4, 3, 0, 0.9), (1025, 170, 2, 0, 0.9),  # fewer groups than leading tokens
     (5119, 5, 3, 20, 0.93), (5120, 5, 3, 20, 0.93), (5121, 5, 3, 20, 1.0),                     # groups of 8, of 64
-    (4100, 5, 3, 256, 0.97), (65600, 5, 2, 256, 1.0), (65600, 5, 2, 257, 1.0),                 # the largest top_k of the candidates
+    (4100, 5, 3, 256, 0.97), (65600, 5, 2, 256, 1.0), (65600, 5, 2, 257, 1.0),                 # the longest list of kept tokens
+    (65600, 3, 2, 1024, 1.0), (65600, 3, 2, 1025, 0.9), (5000, 40, 2, 1024, 0.97),             # the largest top_k of the candidates
+    (20011, 150, 2, 3000, 0.9131), (160011, 60, 1, 2000, 0.9131), (160011, 150, 1, 2000, 0.9131),       # single CTAs, pairs, fours, eights
+    (90001, 4, 1, 2000, 0.9131), (600, 130, 1, 500, 0.9131),
     (32771, 12, 2, 0, 0.95), (32771, 160, 2, 0, 0.95), (40009, 30, 4, 0, 0.6),                 # few rows by windows, many by candidates
     (655361, 2, 1, 20, 0.93), (1700003, 1, 1, 0, 0.9), (9000, 2, 1, 0, 1.0),                   # too many groups; shares beyond shared memory
 ]
