@@ -66,6 +66,8 @@ class PassOutputs:
         self.keep_pages = torch.full((batch.n_page_slots,), -1, **i32)
         self.keep_valid = torch.full((batch.n_page_slots,), -1, **i32)
         self.free_pages = torch.full((batch.n_page_slots,), -1, **i32)
+        # one pass at a time writes these buffers, so the events that order its two streams are kept with them
+        self.fork, self.join = torch.cuda.Event(), torch.cuda.Event()
 
     def commit_dict(self):
         d = {k: getattr(self, k).cpu().numpy() for k in
@@ -93,14 +95,11 @@ def run_pass_overlapped(ctx: B.Context, plan: B.Plan, x: DeviceInputs, y: PassOu
     k_pool = x.k_pool if k_pool is None else k_pool
     v_pool = x.v_pool if v_pool is None else v_pool
     logits = x.logits if logits is None else logits
-    fork = torch.cuda.Event()
-    fork.record(main)
-    side.wait_event(fork)
-    with torch.cuda.stream(side):
-        ctx.lr_accept_greedy(logits, x.draft_ids, x.cu_draft, y.n_accept, y.bonus_id, y.scratch, None, None)
-        plan.lr_commit(x.verdict, y.n_accept, y.n_steps_accepted, y.survivor, y.committed_len, y.keep_off, y.keep_pages,
-                       y.keep_valid, y.free_off, y.free_pages, None)
-        join = torch.cuda.Event()
-        join.record(side)
-    plan.lr_verify_attention(x.q, k_pool, v_pool, y.out, None, 0.0, None)
-    main.wait_event(join)
+    y.fork.record(main)
+    side.wait_event(y.fork)
+    ctx.lr_accept_greedy(logits, x.draft_ids, x.cu_draft, y.n_accept, y.bonus_id, y.scratch, None, side)
+    plan.lr_commit(x.verdict, y.n_accept, y.n_steps_accepted, y.survivor, y.committed_len, y.keep_off, y.keep_pages,
+                   y.keep_valid, y.free_off, y.free_pages, side)
+    y.join.record(side)
+    plan.lr_verify_attention(x.q, k_pool, v_pool, y.out, None, 0.0, main)
+    main.wait_event(y.join)
