@@ -1031,7 +1031,7 @@ int init_attn_pair_kernel() {
 
 // ---- host planning -----------------------------------------------------------------
 int pair_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
-                         const int32_t *span_last, PairHostPlan &out, Image &img) {
+                         const int32_t *span_last, PairHostPlan &out, std::vector<unsigned char> &img) {
   out = PairHostPlan();
   const lr_model &m = ctx->model;
   const int G = m.n_q_heads / m.n_kv_heads;
@@ -1217,14 +1217,20 @@ int pair_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *re
       }
     }
   }
-  out.o_heads = img.add(heads.data(), heads.size() * sizeof(PrHead));
-  out.o_pages = img.add(pages.data(), pages.size() * sizeof(TcPage));
-  out.o_rows = img.add(rows.data(), rows.size() * sizeof(TcRow));
-  out.o_pieces = img.add(pieces.data(), pieces.size() * sizeof(PrPiece));
+  auto add = [&](const void *src, size_t n) -> size_t {
+    const size_t off = (img.size() + 255) / 256 * 256;
+    img.resize(off + n);
+    memcpy(img.data() + off, src, n);
+    return off;
+  };
+  out.o_heads = add(heads.data(), heads.size() * sizeof(PrHead));
+  out.o_pages = add(pages.data(), pages.size() * sizeof(TcPage));
+  out.o_rows = add(rows.data(), rows.size() * sizeof(TcRow));
+  out.o_pieces = add(pieces.data(), pieces.size() * sizeof(PrPiece));
   if (reqs.empty()) reqs.push_back(TcReq{});
-  out.o_reqs = img.add(reqs.data(), reqs.size() * sizeof(TcReq));
+  out.o_reqs = add(reqs.data(), reqs.size() * sizeof(TcReq));
   if (targets.empty()) targets.push_back(TcTarget{});  // keep the section non-empty
-  out.o_targets = img.add(targets.data(), targets.size() * sizeof(TcTarget));
+  out.o_targets = add(targets.data(), targets.size() * sizeof(TcTarget));
   // scratch behind the image: ticket counters (zeroed at upload, left zero by every launch), (exponent, sum) pairs,
   // fp32 partial outputs
   out.s_counters = 0;
@@ -1235,14 +1241,33 @@ int pair_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *re
   return LR_OK;
 }
 
+size_t pair_bytes_bound(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off) {
+  const lr_model &m = ctx->model;
+  if (m.head_dim != kD) return 0;
+  const int T = 128 / (m.n_q_heads / m.n_kv_heads);
+  int64_t lists = 0, pages = 0;
+  for (int r = 0; r < b->n_req; ++r) {
+    int64_t n_pg = 0;
+    for (int s = b->req_span_off[r]; s < b->req_span_off[r + 1]; ++s) n_pg += (b->span_len[s] + kPage - 1) / kPage;
+    for (int i = req_br_off[r]; i < req_br_off[r + 1]; ++i) n_pg += (b->br_own_len[i] + kPage - 1) / kPage;
+    const int n_mt = (b->cu_q[req_br_off[r + 1]] - b->cu_q[req_br_off[r]] + T - 1) / T;
+    lists += (n_mt + 1) / 2;
+    pages += (n_mt + 1) / 2 * (n_pg + kPagesPerTile);
+  }
+  // every pair beyond the first adds at most one piece; every piece at most two partial results
+  const int64_t groups = lists * m.n_kv_heads, pairs = std::max(1, ctx->sm_count / 2), pieces = groups + pairs;
+  const int64_t bytes[] = {pairs * (int64_t)sizeof(PrHead), pages * (int64_t)sizeof(TcPage), std::max(1, b->cu_q[b->n_branch]) * (int64_t)sizeof(TcRow),
+                           pieces * (int64_t)sizeof(PrPiece), (lists + 1) * (int64_t)sizeof(TcReq), (2 * groups + 1) * (int64_t)sizeof(TcTarget),
+                           (2 * groups + 1) * 4, 2 * pieces * 128 * 8, 2 * pieces * 128 * kD * 4};
+  size_t total = 0;
+  for (const int64_t n : bytes) total += (size_t)(n + 255) / 256 * 256;
+  return total;
+}
+
 void pair_bind_device_plan(const PairHostPlan &h, unsigned char *image_base, unsigned char *scratch_base, lr_plan *p) {
   p->pair_ok = h.ok;
   p->pr_pieces = h.n_pieces;
   p->pr_partial_slots = h.n_partial_slots;
-  p->o_pr_pages = h.o_pages;
-  p->o_pr_heads = h.o_heads;
-  p->n_pr_pages = h.ok ? h.n_pages : 0;
-  p->n_pr_heads = h.ok ? h.n_pairs : 0;
   memset(&p->pr, 0, sizeof(p->pr));
   if (!h.ok) return;
   DevPairPlan &t = p->pr;

@@ -1123,19 +1123,15 @@ int init_attn_tc_kernel() {
 // most CTAs worth using for a number of tiles (tiny problems: not one CTA per tile, their partial results cost more than they save)
 static int64_t max_ctas_for_tiles(int64_t tiles) { return tiles >= 64 ? tiles : tiles / 2; }
 
-int tc_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
-                       const int32_t *span_last, TcHostPlan &out, Image &img) {
+void tc_plan_structure(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
+                       const int32_t *span_last, TcHostPlan &out) {
   out = TcHostPlan();
   const lr_model &m = ctx->model;
   const int G = m.n_q_heads / m.n_kv_heads;
-  if (m.head_dim != 64 && m.head_dim != 128) return LR_OK;
-  if ((int64_t)b->n_pool_pages * m.n_kv_heads * kPage >= ((int64_t)1 << 31)) return LR_OK;  // tensor-map coordinates are 32-bit
+  if (m.head_dim != 64 && m.head_dim != 128) return;
+  if ((int64_t)b->n_pool_pages * m.n_kv_heads * kPage >= ((int64_t)1 << 31)) return;  // tensor-map coordinates are 32-bit
   const int T = 128 / G;
-  const int n_q_rows = b->cu_q[b->n_branch];
-  std::vector<TcPage> pages;
-  std::vector<TcRow> rows((size_t)std::max(1, n_q_rows));
-  std::vector<TcReq> reqs;  // one per page list (request x group of M-tiles); TcPiece.req indexes it
-  struct Grp { int req, kv, mtile0, n_mt, n_tiles, weight, first_piece, n_pieces; };
+  struct Grp { int list, mtile0, n_mt, n_tiles, n_dense, weight; };  // one per list; every KV head repeats it
   std::vector<Grp> grps;
   // Two M-tiles per group read every KV tile once for both, which is what a large pass needs.  A small pass --
   // a few tiles per SM -- is dominated by the partial results of its key split instead; there every M-tile is a
@@ -1160,67 +1156,56 @@ int tc_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
   // the tails of its own branches up to the last token one of its rows sees.  Pages no row of the group can see --
   // other branches' tails, segments off its paths through the tree -- are left out, so no tile of the sweep is fully
   // masked for everybody.  (The prefix pages appear in every list of the request: 8 bytes per page and list.)
-  reqs.clear();
+  std::vector<unsigned char> node_used;  // by depth-first number: a branch of the group continues it
+  std::vector<int> tail_limit;           // last tail token a row of the group sees, per branch
   for (int r = 0; r < b->n_req; ++r) {
     const int s0 = b->req_span_off[r], s1 = b->req_span_off[r + 1];
     const int br0 = req_br_off[r], br1 = req_br_off[r + 1];
     if (br1 == br0) continue;  // a request without branches has no query rows
-    if (br1 - br0 > 254) return LR_OK;
+    if (br1 - br0 > 254) return;
+    for (int i = br0; i < br1; ++i)
+      if ((b->br_own_len[i] + kPage - 1) / kPage > 2047) return;
     const int q_row0 = b->cu_q[br0], n_q = b->cu_q[br1] - b->cu_q[br0];
-    for (int i = br0; i < br1; ++i) {
-      const int tin = span_tin[s0 + b->br_depth[i]];
-      if ((b->br_own_len[i] + kPage - 1) / kPage > 2047) return LR_OK;
-      const int q_len = b->cu_q[i + 1] - b->cu_q[i];
-      for (int k = 0; k < q_len; ++k) {
-        TcRow &w = rows[(size_t)b->cu_q[i] + k];
-        w.depth_branch = tin | ((i - br0) << 16);
-        w.limit = b->br_own_len[i] - q_len + k;
-      }
-    }
     const int n_mtiles = (n_q + T - 1) / T;
     for (int m0 = 0; m0 < n_mtiles; m0 += m_step) {
       const int mts = std::min(m_step, n_mtiles - m0);
       const int row_lo = q_row0 + m0 * T, row_hi = q_row0 + std::min(n_q, (m0 + mts) * T);  // query rows of the group
-      TcReq rq;
-      memset(&rq, 0, sizeof(rq));
-      rq.page_off = (int)pages.size();
-      rq.q_row0 = q_row0;
-      rq.n_q = n_q;
-      std::vector<unsigned char> node_used((size_t)(s1 - s0), 0);  // by depth-first number: a branch of the group continues it
-      std::vector<int> tail_limit((size_t)(br1 - br0), -1);        // last tail token a row of the group sees, per branch
+      TcList list;
+      memset(&list, 0, sizeof(list));
+      list.rq.page_off = out.n_pages;
+      list.rq.q_row0 = q_row0;
+      list.rq.n_q = n_q;
+      list.rq.n_dense_tiles = (b->span_len[s0] / kPage) / kPagesPerTile;
+      list.run0 = (int)out.runs.size();
+      node_used.assign((size_t)(s1 - s0), 0);
+      tail_limit.assign((size_t)(br1 - br0), -1);
       for (int i = br0; i < br1; ++i) {
         const int lo = std::max(row_lo, b->cu_q[i]), hi = std::min(row_hi, b->cu_q[i + 1]);
         if (lo >= hi) continue;
         node_used[span_tin[s0 + b->br_depth[i]]] = 1;
-        tail_limit[i - br0] = rows[(size_t)hi - 1].limit;
+        tail_limit[i - br0] = b->br_own_len[i] - b->cu_q[i + 1] + hi - 1;
       }
-      auto add_span = [&](int slot, int len, int n_pg, int need, int last, int owner) {
-        for (int p = 0; p < n_pg; ++p) {
-          TcPage e;
-          e.page = b->page_ids[slot + p];
-          const uint32_t valid = (uint32_t)std::min(kPage, len - p * kPage);
-          e.meta = valid | ((uint32_t)need << 5) | ((uint32_t)owner << 13) | ((uint32_t)(owner ? p : last) << 21);
-          pages.push_back(e);
-        }
+      auto add = [&](int slot, int len, int n_pg, int need, int last, int owner) {
+        if (n_pg == 0) return;
+        out.runs.push_back(TcRun{slot, len, n_pg, ((uint32_t)need << 5) | ((uint32_t)owner << 13) | ((uint32_t)last << 21), owner != 0});
+        list.rq.n_pages += n_pg;
       };
-      add_span(b->span_slot[s0], b->span_len[s0], (b->span_len[s0] + kPage - 1) / kPage, 0, 255, 0);
-      rq.n_dense_tiles = (b->span_len[s0] / kPage) / kPagesPerTile;
+      add(b->span_slot[s0], b->span_len[s0], (b->span_len[s0] + kPage - 1) / kPage, 0, 255, 0);
       for (int c = 1; s0 + c < s1; ++c) {
         bool seen = false;
         for (int t = span_tin[s0 + c]; t <= span_last[s0 + c] && !seen; ++t) seen = node_used[t];
-        if (seen) add_span(b->span_slot[s0 + c], b->span_len[s0 + c], (b->span_len[s0 + c] + kPage - 1) / kPage, span_tin[s0 + c], span_last[s0 + c], 0);
+        if (seen) add(b->span_slot[s0 + c], b->span_len[s0 + c], (b->span_len[s0 + c] + kPage - 1) / kPage, span_tin[s0 + c], span_last[s0 + c], 0);
       }
       for (int i = br0; i < br1; ++i)
-        if (tail_limit[i - br0] >= 0) add_span(b->br_own_slot[i], b->br_own_len[i], tail_limit[i - br0] / kPage + 1, 0, 0, i - br0 + 1);
-      rq.n_pages = (int)pages.size() - rq.page_off;
-      while (pages.size() % kPagesPerTile) pages.push_back(TcPage{0, 0});  // absent pages of the last tile: nothing valid
-      const int n_tiles = (rq.n_pages + kPagesPerTile - 1) / kPagesPerTile;
-      const int list = (int)reqs.size();
-      reqs.push_back(rq);
-      for (int kv = 0; kv < m.n_kv_heads; ++kv) grps.push_back(Grp{list, kv, m0, mts, n_tiles, mts == 2 ? 16 : 10, 0, 0});
+        if (tail_limit[i - br0] >= 0) add(b->br_own_slot[i], b->br_own_len[i], tail_limit[i - br0] / kPage + 1, 0, 0, i - br0 + 1);
+      list.run1 = (int)out.runs.size();
+      const int n_tiles = (list.rq.n_pages + kPagesPerTile - 1) / kPagesPerTile;
+      out.n_pages += n_tiles * kPagesPerTile;  // absent pages of the last tile: nothing valid
+      grps.push_back(Grp{(int)out.lists.size(), m0, mts, n_tiles, std::min(n_tiles, list.rq.n_dense_tiles), mts == 2 ? 16 : 10});
+      out.lists.push_back(list);
     }
   }
-  if (grps.empty()) return LR_OK;
+  if (grps.empty()) return;
   // Contiguous partition of the tile sequence (groups in order, tiles in order) over at most max_cta CTAs that
   // minimises the largest CTA load.  A tile costs its group's weight (10 with one M-tile, 16 with two: per-CTA cycle
   // counts on the ragged serving workload gave 2360 and 3790 cycles a tile); every piece -- a CTA's share of one
@@ -1229,129 +1214,147 @@ int tc_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
   // CTAs possible; the smallest feasible L is found by bisection.  At most one CTA per two tiles: smaller shares
   // only add partial results to merge.
   constexpr int kPieceStartTiles = 2, kDense = 5, kMasked = 8;  // costs in fifths of a dense tile
-  auto tile_cost = [&](const Grp &g, int t) -> int64_t {
-    return (int64_t)g.weight * (t >= reqs[g.req].n_dense_tiles ? kMasked : kDense);
-  };
-  int64_t total_w = 0, total_tiles = 0, lo = 0;
+  const int n_kv = m.n_kv_heads;
+  int64_t total_w = 0, total_tiles = 0, most = 0;
   for (const Grp &g : grps) {
-    total_w += (int64_t)kPieceStartTiles * kDense * g.weight;
-    for (int t = 0; t < g.n_tiles; ++t) total_w += tile_cost(g, t);
-    total_tiles += g.n_tiles;
-    lo = std::max<int64_t>(lo, (int64_t)(kPieceStartTiles * kDense + kMasked) * g.weight);
+    total_w += (int64_t)n_kv * g.weight * (kPieceStartTiles * kDense + g.n_dense * kDense + (g.n_tiles - g.n_dense) * kMasked);
+    total_tiles += (int64_t)n_kv * g.n_tiles;
+    most = std::max<int64_t>(most, (int64_t)(kPieceStartTiles * kDense + kMasked) * g.weight);
   }
   const int64_t max_cta = std::min<int64_t>(ctx->sm_count, std::max<int64_t>(1, max_ctas_for_tiles(total_tiles)));
   // walks the partition for limit L; with `emit` it also records the pieces.  A group is a run of dense tiles
   // followed by a run of masked ones, each of uniform cost, so a walk takes O(CTAs + groups) steps.
-  std::vector<TcPiece> pieces;
-  std::vector<int32_t> cta_off;
+  struct Contrib { int first, n; };
+  std::vector<Contrib> contrib;  // the pieces of every (list, KV head), in that order of grps x heads
   auto walk = [&](int64_t L, bool emit) -> int64_t {
     int64_t n = 0, load = 0;
-    for (size_t gi = 0; gi < grps.size(); ++gi) {
-      Grp &g = grps[gi];
-      if (emit) g.first_piece = (int)pieces.size();
+    for (const Grp &g : grps) {
       const int64_t start = (int64_t)kPieceStartTiles * kDense * g.weight;
-      const int n_dense = std::min(g.n_tiles, reqs[g.req].n_dense_tiles);
-      bool new_piece = true;
-      int t = 0;
-      while (t < g.n_tiles) {
-        const int run_end = t < n_dense ? n_dense : g.n_tiles;
-        const int64_t cost = tile_cost(g, t);
-        if (n == 0 || load + cost + (new_piece ? start : 0) > L) {  // open the next CTA: its share of this group is a new piece
-          ++n;
-          load = 0;
-          new_piece = true;
-          if (emit) cta_off.push_back((int32_t)pieces.size());
-        }
-        if (new_piece) load += start;
-        const int k = (int)std::max<int64_t>(1, std::min<int64_t>(run_end - t, (L - load) / cost));
-        load += (int64_t)k * cost;
-        if (emit) {
-          if (new_piece) {
-            TcPiece p;
-            p.req = g.req; p.kv_head = g.kv; p.mtile0 = g.mtile0; p.n_mt = g.n_mt; p.tile_begin = t; p.tile_end = t + k;
-            p.slot[0] = p.slot[1] = -2;
-            pieces.push_back(p);
-          } else {
-            pieces.back().tile_end = t + k;
+      for (int kv = 0; kv < n_kv; ++kv) {
+        const int first = (int)out.pieces.size();
+        bool new_piece = true;
+        int t = 0;
+        while (t < g.n_tiles) {
+          const int run_end = t < g.n_dense ? g.n_dense : g.n_tiles;
+          const int64_t cost = (int64_t)g.weight * (t < g.n_dense ? kDense : kMasked);
+          if (n == 0 || load + cost + (new_piece ? start : 0) > L) {  // open the next CTA: its share of this group is a new piece
+            ++n;
+            load = 0;
+            new_piece = true;
+            if (emit) out.cta_piece_off.push_back((int32_t)out.pieces.size());
+            else if (n > max_cta) return n;
           }
+          if (new_piece) load += start;
+          const int k = (int)std::max<int64_t>(1, std::min<int64_t>(run_end - t, (L - load) / cost));
+          load += (int64_t)k * cost;
+          if (emit) {
+            if (new_piece) {
+              TcPiece p;
+              p.req = g.list; p.kv_head = kv; p.mtile0 = g.mtile0; p.n_mt = g.n_mt; p.tile_begin = t; p.tile_end = t + k;
+              p.slot[0] = p.slot[1] = -2;
+              out.pieces.push_back(p);
+            } else {
+              out.pieces.back().tile_end = t + k;
+            }
+          }
+          new_piece = false;
+          t += k;
         }
-        new_piece = false;
-        t += k;
+        if (emit) contrib.push_back({first, (int)out.pieces.size() - first});
       }
-      if (emit) g.n_pieces = (int)pieces.size() - g.first_piece;
     }
     return n;
   };
-  int64_t hi = total_w;  // one CTA takes everything
+  // No partition stays below the average load, and a greedy fill does not exceed it by more than a piece start and a tile
+  // per CTA, or nearly so: the bisection starts from there.
+  int64_t lo = std::max(most, (total_w + max_cta - 1) / max_cta), hi = lo + 2 * most;
+  if (walk(hi, false) > max_cta) hi = std::max(hi, total_w);  // one CTA takes everything
   while (lo < hi) {
     const int64_t mid = lo + (hi - lo) / 2;
     if (walk(mid, false) <= max_cta) hi = mid; else lo = mid + 1;
   }
-  const int n_cta = (int)walk(lo, true);
-  cta_off.push_back((int32_t)pieces.size());
-  // Targets (one M-tile of one group) and the streams that contribute to them, in piece order.
+  out.n_cta = (int)walk(lo, true);
+  out.cta_piece_off.push_back((int32_t)out.pieces.size());
+  // Targets (one M-tile of one group) and the streams that contribute to them, in piece order; the two streams of a
+  // one-M-tile piece are combined inside the CTA.
   int n_slots = 0;
-  std::vector<TcTarget> targets;
+  size_t at = 0;
   for (const Grp &g : grps)
-    for (int mt = 0; mt < g.n_mt; ++mt) {
-      std::vector<int32_t *> contrib;
-      for (int k = 0; k < g.n_pieces; ++k) {
-        TcPiece &p = pieces[g.first_piece + k];
-        if (g.n_mt == 2) contrib.push_back(&p.slot[mt]);
-        else contrib.push_back(&p.slot[0]);  // the two streams of a one-M-tile piece are combined inside the CTA
+    for (int kv = 0; kv < n_kv; ++kv, ++at)
+      for (int mt = 0; mt < g.n_mt; ++mt) {
+        const Contrib c = contrib[at];
+        if (c.n == 1) {
+          out.pieces[c.first].slot[mt] = -1;
+          continue;
+        }
+        TcTarget tg;
+        memset(&tg, 0, sizeof(tg));
+        tg.req = g.list; tg.kv_head = kv; tg.mtile = g.mtile0 + mt;
+        tg.slot_begin = n_slots; tg.n_slots = c.n;
+        tg.q_row0 = out.lists[g.list].rq.q_row0; tg.n_q = out.lists[g.list].rq.n_q;
+        for (int k = 0; k < c.n; ++k) out.pieces[c.first + k].slot[mt] = n_slots++;
+        out.targets.push_back(tg);
       }
-      if (contrib.size() == 1) { *contrib[0] = -1; continue; }
-      TcTarget tg;
-      memset(&tg, 0, sizeof(tg));
-      tg.req = g.req; tg.kv_head = g.kv; tg.mtile = g.mtile0 + mt;
-      tg.slot_begin = n_slots; tg.n_slots = (int)contrib.size();
-      tg.q_row0 = reqs[g.req].q_row0; tg.n_q = reqs[g.req].n_q;
-      for (int32_t *c : contrib) *c = n_slots++;
-      targets.push_back(tg);
-    }
   out.ok = true;
-  out.n_cta = n_cta;
-  out.n_pieces = (int)pieces.size();
-  out.n_targets = (int)targets.size();
   out.n_partial_slots = n_slots;
   out.tokens_per_mtile = T;
-  static_assert(sizeof(TcCtaHead) == 256, "one CTA head = 256 bytes");
-  std::vector<TcCtaHead> heads((size_t)n_cta);
-  for (int c = 0; c < n_cta; ++c) {
-    TcCtaHead &h = heads[c];
-    memset(&h, 0, sizeof(h));
-    h.piece0 = cta_off[c];
-    h.piece1 = cta_off[c + 1];
-    if (h.piece1 > h.piece0) {
-      h.first = pieces[h.piece0];
-      h.first_req = reqs[h.first.req];
-      const int c0 = h.first.tile_begin >> 2;
-      for (int k = 0; k < 32; ++k) {
-        const int idx = c0 * 32 + k;
-        h.first_pages[k] = idx < h.first_req.n_pages ? pages[(size_t)h.first_req.page_off + idx].page : -1;
-      }
-    }
-  }
-  out.o_heads = img.add(heads.data(), heads.size() * sizeof(TcCtaHead));
-  out.o_pages = img.add(pages.data(), pages.size() * sizeof(TcPage));
-  out.n_pages = (int)pages.size();
-  out.o_rows = img.add(rows.data(), rows.size() * sizeof(TcRow));
-  out.o_pieces = img.add(pieces.data(), pieces.size() * sizeof(TcPiece));
-  out.o_cta_piece_off = img.add(cta_off.data(), cta_off.size() * sizeof(int32_t));
-  if (reqs.empty()) reqs.push_back(TcReq{});
-  out.o_reqs = img.add(reqs.data(), reqs.size() * sizeof(TcReq));
-  if (targets.empty()) targets.push_back(TcTarget{});  // keep the section non-empty
-  out.o_targets = img.add(targets.data(), targets.size() * sizeof(TcTarget));
   out.s_ml = 0;
   out.s_o = ((size_t)n_slots * 128 * 2 * sizeof(float) + 255) / 256 * 256;
   out.scratch_bytes = out.s_o + (size_t)n_slots * 128 * m.head_dim * sizeof(float);
-  out.scratch_zero_bytes = 0;
-  return LR_OK;
+}
+
+void tc_plan_tables(const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin, TcHostPlan &h, Image &img) {
+  if (!h.ok) return;
+  static_assert(sizeof(TcCtaHead) == 256, "one CTA head = 256 bytes");
+  const int n_q_rows = b->cu_q[b->n_branch];
+  TcCtaHead *heads = img.add<TcCtaHead>((size_t)h.n_cta, h.o_heads);
+  TcPage *pages = img.add<TcPage>((size_t)h.n_pages, h.o_pages);
+  TcRow *rows = img.add<TcRow>((size_t)std::max(1, n_q_rows), h.o_rows);
+  h.o_pieces = img.copy(h.pieces.data(), h.pieces.size());
+  h.o_cta_piece_off = img.copy(h.cta_piece_off.data(), h.cta_piece_off.size());
+  TcReq *reqs = img.add<TcReq>(h.lists.size(), h.o_reqs);
+  TcTarget *targets = img.add<TcTarget>(std::max<size_t>(1, h.targets.size()), h.o_targets);
+  if (!img.base) return;
+  if (!h.targets.empty()) memcpy(targets, h.targets.data(), h.targets.size() * sizeof(TcTarget));
+  else memset(targets, 0, sizeof(TcTarget));  // keep the section non-empty
+  for (size_t l = 0; l < h.lists.size(); ++l) {
+    const TcList &list = h.lists[l];
+    reqs[l] = list.rq;
+    TcPage *e = pages + list.rq.page_off;
+    for (int i = list.run0; i < list.run1; ++i) {
+      const TcRun &run = h.runs[i];
+      const int full = std::min(run.n_pg, run.len / kPage);
+      const int32_t *ids = b->page_ids + run.slot;
+      const uint32_t step = run.tail ? 1u << 21 : 0u;
+      uint32_t meta = run.meta;
+      for (int p = 0; p < full; ++p, meta += step) *e++ = TcPage{ids[p], meta | (uint32_t)kPage};
+      if (full < run.n_pg) *e++ = TcPage{ids[full], meta | (uint32_t)(run.len - full * kPage)};
+    }
+    while ((e - pages) % kPagesPerTile) *e++ = TcPage{0, 0};
+  }
+  for (int r = 0; r < b->n_req; ++r)
+    for (int i = req_br_off[r]; i < req_br_off[r + 1]; ++i) {
+      const int depth_branch = span_tin[b->req_span_off[r] + b->br_depth[i]] | ((i - req_br_off[r]) << 16);
+      const int q0 = b->cu_q[i], q_len = b->cu_q[i + 1] - q0;
+      for (int k = 0; k < q_len; ++k) rows[q0 + k] = TcRow{depth_branch, b->br_own_len[i] - q_len + k};
+    }
+  memset(heads, 0, (size_t)h.n_cta * sizeof(TcCtaHead));
+  for (int c = 0; c < h.n_cta; ++c) {
+    TcCtaHead &hd = heads[c];
+    hd.piece0 = h.cta_piece_off[c];
+    hd.piece1 = h.cta_piece_off[c + 1];
+    if (hd.piece1 > hd.piece0) {
+      hd.first = h.pieces[hd.piece0];
+      hd.first_req = h.lists[hd.first.req].rq;
+      const int first = (hd.first.tile_begin >> 2) * 32;
+      for (int k = 0; k < 32; ++k) hd.first_pages[k] = first + k < hd.first_req.n_pages ? pages[hd.first_req.page_off + first + k].page : -1;
+    }
+  }
 }
 
 void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigned char *scratch_base, lr_plan *p) {
   p->tc_ok = h.ok;
-  p->tc_pieces = h.n_pieces;
+  p->tc_pieces = (int)h.pieces.size();
   p->o_tc_pages = h.o_pages;
   p->o_tc_heads = h.o_heads;
   p->n_tc_pages = h.ok ? h.n_pages : 0;
@@ -1368,7 +1371,7 @@ void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigne
   t.reqs = reinterpret_cast<const TcReq *>(image_base + h.o_reqs);
   t.targets = reinterpret_cast<const TcTarget *>(image_base + h.o_targets);
   t.n_cta = h.n_cta;
-  t.n_targets = h.n_targets;
+  t.n_targets = (int)h.targets.size();
   t.tokens_per_mtile = h.tokens_per_mtile;
   t.wait_limit_us = 1000000u;  // one second per wait
   t.phantom_tx_bytes = 0;

@@ -105,122 +105,125 @@ static int validate_batch(const lr_batch *b) {
 }
 
 // ---- plan image --------------------------------------------------------------
+// lr_plan_bytes needs the sizes only, lr_plan_create the sizes first (for the buffer) and then the tables: layout() works
+// out the structure of the plan once, sections() lays the image out and, given a buffer, fills it in place.
 struct Layout {
-  Image img;
   size_t o_req_span_off, o_span_len, o_span_slot, o_br_req, o_br_depth, o_br_own_len, o_br_own_slot, o_br_n_draft, o_cu_q,
       o_cu_draft, o_page_ids, o_req_br_off, o_span_req, o_status, o_slot_item, o_chain_pg, o_chain_tok, o_tail_pg, o_compact_stage_off,
       o_span_tin, o_span_last, o_child_off, o_child_list;
-  size_t compact_tokens;
-  std::vector<int32_t> cu_draft;
+  std::vector<int32_t> cu_draft, req_br_off, span_tin, span_last, child_off, child_list;
   TcHostPlan tc;
-  PairHostPlan pr;
-  size_t image_bytes, total_bytes, pair_scratch_off;
+  size_t image_bytes, region_bytes, total_bytes;
+  size_t compact_tokens;
 };
 
-static int build_layout(const lr_ctx *ctx, const lr_batch *b, Layout &L) {
+static void sections(const lr_batch *b, Layout &L, Image &g) {
+  L.o_req_span_off = g.copy(b->req_span_off, b->n_req + 1);
+  L.o_span_len = g.copy(b->span_len, b->n_span);
+  L.o_span_slot = g.copy(b->span_slot, b->n_span);
+  L.o_br_req = g.copy(b->br_req, b->n_branch);
+  L.o_br_depth = g.copy(b->br_depth, b->n_branch);
+  L.o_br_own_len = g.copy(b->br_own_len, b->n_branch);
+  L.o_br_own_slot = g.copy(b->br_own_slot, b->n_branch);
+  L.o_br_n_draft = g.copy(b->br_n_draft, b->n_branch);
+  L.o_cu_q = g.copy(b->cu_q, b->n_branch + 1);
+  L.o_cu_draft = g.copy(L.cu_draft.data(), L.cu_draft.size());
+  L.o_page_ids = g.copy(b->page_ids, b->n_page_slots);
+  L.o_req_br_off = g.copy(L.req_br_off.data(), L.req_br_off.size());
+  L.o_span_tin = g.copy(L.span_tin.data(), L.span_tin.size());
+  L.o_span_last = g.copy(L.span_last.data(), L.span_last.size());
+  L.o_child_off = g.copy(L.child_off.data(), L.child_off.size());
+  L.o_child_list = g.copy(L.child_list.data(), L.child_list.size());
+  int32_t *span_req = g.add<int32_t>(b->n_span, L.o_span_req);
+  int32_t *slot_item = g.add<int32_t>(b->n_page_slots, L.o_slot_item);
+  int32_t *chain_pg = g.add<int32_t>((size_t)b->n_span + b->n_req, L.o_chain_pg);
+  int32_t *chain_tok = g.add<int32_t>((size_t)b->n_span + b->n_req, L.o_chain_tok);
+  int32_t *tail_pg = g.add<int32_t>((size_t)b->n_branch + b->n_req, L.o_tail_pg);
+  int32_t *stage_off = g.add<int32_t>((size_t)b->n_req + 1, L.o_compact_stage_off);
+  int32_t *status = g.add<int32_t>(2, L.o_status);
+  if (g.base) {
+    status[0] = status[1] = 0;
+    std::fill(slot_item, slot_item + b->n_page_slots, -1);
+  }
+  // lr_compact: at most the segments and one tail of a request are displaced
+  size_t tokens = 0;
+  for (int r = 0; r < b->n_req; ++r) {
+    const int s0 = b->req_span_off[r], s1 = b->req_span_off[r + 1], base = s0 + r;
+    const int b0 = L.req_br_off[r], b1 = L.req_br_off[r + 1], tb = b0 + r;
+    size_t segs = 0, tail = 0;
+    for (int s = s0 + 1; s < s1; ++s) segs += (size_t)b->span_len[s];
+    for (int i = b0; i < b1; ++i) tail = std::max(tail, (size_t)b->br_own_len[i]);
+    if (g.base) {
+      stage_off[r] = (int32_t)tokens;
+      chain_pg[base] = chain_tok[base] = tail_pg[tb] = 0;
+      for (int s = s0; s < s1; ++s) {
+        const int npg = pages_of(b->span_len[s]);
+        span_req[s] = r;
+        chain_pg[base + (s - s0) + 1] = chain_pg[base + (s - s0)] + npg;
+        chain_tok[base + (s - s0) + 1] = chain_tok[base + (s - s0)] + b->span_len[s];
+        std::fill(slot_item + b->span_slot[s], slot_item + b->span_slot[s] + npg, s);
+      }
+      for (int i = b0; i < b1; ++i) {
+        const int npg = pages_of(b->br_own_len[i]);
+        tail_pg[tb + (i - b0) + 1] = tail_pg[tb + (i - b0)] + npg;
+        std::fill(slot_item + b->br_own_slot[i], slot_item + b->br_own_slot[i] + npg, b->n_span + i);
+      }
+    }
+    tokens += segs + tail;
+  }
+  if (g.base) stage_off[b->n_req] = (int32_t)tokens;
+  L.compact_tokens = tokens;
+  tc_plan_tables(b, L.req_br_off.data(), L.span_tin.data(), L.tc, g);
+}
+
+static int layout(const lr_ctx *ctx, const lr_batch *b, Layout &L) {
   if (!ctx) {
     set_error("null context");
     return LR_EINVAL;
   }
   if (int rc = validate_batch(b)) return rc;
-  const size_t I = sizeof(int32_t);
-  std::vector<int32_t> cu_draft(b->n_branch + 1, 0), req_br_off(b->n_req + 1, 0), span_req(b->n_span, 0);
+  L.cu_draft.assign(b->n_branch + 1, 0);
+  L.req_br_off.assign(b->n_req + 1, 0);
   for (int i = 0; i < b->n_branch; ++i) {
-    cu_draft[i + 1] = cu_draft[i] + b->br_n_draft[i];
-    req_br_off[b->br_req[i] + 1]++;
+    L.cu_draft[i + 1] = L.cu_draft[i] + b->br_n_draft[i];
+    L.req_br_off[b->br_req[i] + 1]++;
   }
-  for (int r = 0; r < b->n_req; ++r) {
-    req_br_off[r + 1] += req_br_off[r];
-    for (int s = b->req_span_off[r]; s < b->req_span_off[r + 1]; ++s) span_req[s] = r;
-  }
-  Image &g = L.img;
-  L.o_req_span_off = g.add(b->req_span_off, I * (b->n_req + 1));
-  L.o_span_len = g.add(b->span_len, I * b->n_span);
-  L.o_span_slot = g.add(b->span_slot, I * b->n_span);
-  L.o_br_req = g.add(b->br_req, I * b->n_branch);
-  L.o_br_depth = g.add(b->br_depth, I * b->n_branch);
-  L.o_br_own_len = g.add(b->br_own_len, I * b->n_branch);
-  L.o_br_own_slot = g.add(b->br_own_slot, I * b->n_branch);
-  L.o_br_n_draft = g.add(b->br_n_draft, I * b->n_branch);
-  L.o_cu_q = g.add(b->cu_q, I * (b->n_branch + 1));
-  L.o_cu_draft = g.add(cu_draft.data(), I * (b->n_branch + 1));
-  L.o_page_ids = g.add(b->page_ids, I * b->n_page_slots);
-  L.o_req_br_off = g.add(req_br_off.data(), I * (b->n_req + 1));
-  L.o_span_req = g.add(span_req.data(), I * b->n_span);
-  {
-    std::vector<int32_t> slot_item((size_t)b->n_page_slots, -1), chain_pg((size_t)b->n_span + b->n_req, 0),
-        chain_tok((size_t)b->n_span + b->n_req, 0), tail_pg((size_t)b->n_branch + b->n_req, 0);
-    for (int r = 0; r < b->n_req; ++r) {
-      const int s0 = b->req_span_off[r], s1 = b->req_span_off[r + 1], base = s0 + r;
-      for (int s = s0; s < s1; ++s) {
-        const int npg = pages_of(b->span_len[s]);
-        chain_pg[base + (s - s0) + 1] = chain_pg[base + (s - s0)] + npg;
-        chain_tok[base + (s - s0) + 1] = chain_tok[base + (s - s0)] + b->span_len[s];
-        for (int k = 0; k < npg; ++k) slot_item[b->span_slot[s] + k] = s;
-      }
-      const int b0 = req_br_off[r], b1 = req_br_off[r + 1], tb = b0 + r;
-      for (int i = b0; i < b1; ++i) {
-        const int npg = pages_of(b->br_own_len[i]);
-        tail_pg[tb + (i - b0) + 1] = tail_pg[tb + (i - b0)] + npg;
-        for (int k = 0; k < npg; ++k) slot_item[b->br_own_slot[i] + k] = b->n_span + i;
-      }
-    }
-    L.o_slot_item = g.add(slot_item.data(), I * slot_item.size());
-    L.o_chain_pg = g.add(chain_pg.data(), I * chain_pg.size());
-    L.o_chain_tok = g.add(chain_tok.data(), I * chain_tok.size());
-    L.o_tail_pg = g.add(tail_pg.data(), I * tail_pg.size());
-    // lr_compact: at most the segments and one tail of a request are displaced
-    std::vector<int32_t> stage_off((size_t)b->n_req + 1, 0);
-    size_t tokens = 0;
-    for (int r = 0; r < b->n_req; ++r) {
-      stage_off[r] = (int32_t)tokens;
-      size_t segs = 0, tail = 0;
-      for (int s = b->req_span_off[r] + 1; s < b->req_span_off[r + 1]; ++s) segs += (size_t)b->span_len[s];
-      for (int i = req_br_off[r]; i < req_br_off[r + 1]; ++i) tail = std::max(tail, (size_t)b->br_own_len[i]);
-      tokens += segs + tail;
-      stage_off[r + 1] = (int32_t)tokens;
-    }
-    L.compact_tokens = tokens;
-    L.o_compact_stage_off = g.add(stage_off.data(), I * stage_off.size());
-  }
+  for (int r = 0; r < b->n_req; ++r) L.req_br_off[r + 1] += L.req_br_off[r];
   // depth-first interval labels and child lists of the draft-step trees (a chain when seg_parent is absent)
-  std::vector<int32_t> span_tin((size_t)b->n_span, 0), span_last((size_t)b->n_span, 0), child_off((size_t)b->n_span + 1, 0),
-      child_list((size_t)b->n_span, 0);
+  L.span_tin.assign((size_t)b->n_span, 0);
+  L.span_last.assign((size_t)b->n_span, 0);
+  L.child_off.assign((size_t)b->n_span + 1, 0);
+  L.child_list.assign((size_t)b->n_span, 0);
+  std::vector<int> n_child, fill, size;
   for (int r = 0; r < b->n_req; ++r) {
     const int s0 = b->req_span_off[r], n = b->req_span_off[r + 1] - s0;
     auto parent_of = [&](int c) { return b->seg_parent ? b->seg_parent[s0 + c] : c - 1; };
-    std::vector<int> n_child((size_t)n, 0);
+    n_child.assign((size_t)n, 0);
     for (int c = 1; c < n; ++c) n_child[parent_of(c)]++;
-    for (int c = 0; c < n; ++c) child_off[s0 + c + 1] = child_off[s0 + c] + n_child[c];
-    std::vector<int> fill((size_t)n, 0);
+    for (int c = 0; c < n; ++c) L.child_off[s0 + c + 1] = L.child_off[s0 + c] + n_child[c];
+    fill.assign((size_t)n, 0);
     for (int c = 1; c < n; ++c) {  // increasing c: every list comes out sorted
       const int par = parent_of(c);
-      child_list[child_off[s0 + par] + fill[par]++] = c;
+      L.child_list[L.child_off[s0 + par] + fill[par]++] = c;
     }
-    std::vector<int> size((size_t)n, 1);  // subtree sizes: children have larger indices than parents
+    size.assign((size_t)n, 1);  // subtree sizes: children have larger indices than parents
     for (int c = n - 1; c >= 1; --c) size[parent_of(c)] += size[c];
     // pre-order numbers: a node's number is its parent's + 1 + the subtree sizes of its earlier siblings
     for (int c = 0; c < n; ++c) {
-      int next = span_tin[s0 + c] + 1;
-      for (int k = child_off[s0 + c]; k < child_off[s0 + c + 1]; ++k) {
-        span_tin[s0 + child_list[k]] = next;
-        next += size[child_list[k]];
+      int next = L.span_tin[s0 + c] + 1;
+      for (int k = L.child_off[s0 + c]; k < L.child_off[s0 + c + 1]; ++k) {
+        L.span_tin[s0 + L.child_list[k]] = next;
+        next += size[L.child_list[k]];
       }
-      span_last[s0 + c] = span_tin[s0 + c] + size[c] - 1;
+      L.span_last[s0 + c] = L.span_tin[s0 + c] + size[c] - 1;
     }
   }
-  L.o_span_tin = g.add(span_tin.data(), I * span_tin.size());
-  L.o_span_last = g.add(span_last.data(), I * span_last.size());
-  L.o_child_off = g.add(child_off.data(), I * child_off.size());
-  L.o_child_list = g.add(child_list.data(), I * child_list.size());
-  int32_t zero2[2] = {0, 0};
-  L.o_status = g.add(zero2, sizeof(zero2));
-  L.cu_draft = cu_draft;
-  if (int rc = tc_build_host_plan(ctx, b, req_br_off.data(), span_tin.data(), span_last.data(), L.tc, g)) return rc;
-  if (int rc = pair_build_host_plan(ctx, b, req_br_off.data(), span_tin.data(), span_last.data(), L.pr, g)) return rc;
-  L.image_bytes = align_up(g.bytes.size(), 256);
-  L.pair_scratch_off = L.image_bytes + align_up(L.tc.scratch_bytes, 256);
-  L.total_bytes = L.pair_scratch_off + align_up(L.pr.scratch_bytes, 256);
+  tc_plan_structure(ctx, b, L.req_br_off.data(), L.span_tin.data(), L.span_last.data(), L.tc);
+  Image sizes;
+  sections(b, L, sizes);
+  L.image_bytes = align_up(sizes.bytes, 256);
+  L.region_bytes = align_up(std::max(L.tc.scratch_bytes, pair_bytes_bound(ctx, b, L.req_br_off.data())), 256);
+  L.total_bytes = L.image_bytes + L.region_bytes;
   return LR_OK;
 }
 
@@ -265,10 +268,13 @@ extern "C" int lr_create(lr_ctx **out, const lr_model *m, int device) {
     set_error("lr_create: device %d not present (%d devices)", device, n_dev);
     return LR_EINVAL;
   }
-  cudaDeviceProp prop;
-  if (int rc = cuda_fail(cudaGetDeviceProperties(&prop, device), "cudaGetDeviceProperties")) return rc;
-  if (prop.major != 10) {
-    set_error("lr_create: device %d is sm_%d%d; this library is built for sm_100a only", device, prop.major, prop.minor);
+  int major = 0, minor = 0, sms = 0;  // (cudaGetDeviceProperties takes milliseconds)
+  cudaError_t e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  if (int rc = cuda_fail(e, "cudaDeviceGetAttribute")) return rc;
+  if (major != 10) {
+    set_error("lr_create: device %d is sm_%d%d; this library is built for sm_100a only", device, major, minor);
     return LR_EUNSUPPORTED;
   }
   if (int rc = cuda_fail(cudaSetDevice(device), "cudaSetDevice")) return rc;
@@ -276,7 +282,7 @@ extern "C" int lr_create(lr_ctx **out, const lr_model *m, int device) {
   if (!c) return LR_ENOMEM;
   c->model = *m;
   c->device = device;
-  c->sm_count = prop.multiProcessorCount;
+  c->sm_count = sms;
   c->launches = 0;
   c->tmap_encode = nullptr;
   if (int rc = init_commit_kernel()) { delete c; return rc; }
@@ -342,7 +348,7 @@ extern "C" int lr_plan_bytes(const lr_ctx *ctx, const lr_batch *b, size_t *bytes
     return LR_EINVAL;
   }
   Layout L;
-  if (int rc = build_layout(ctx, b, L)) return rc;
+  if (int rc = layout(ctx, b, L)) return rc;
   *bytes_out = L.total_bytes;
   return LR_OK;
 }
@@ -358,7 +364,7 @@ extern "C" int lr_plan_create(lr_ctx *ctx, const lr_batch *b, void *ws, size_t w
     return LR_EINVAL;
   }
   Layout L;
-  if (int rc = build_layout(ctx, b, L)) return rc;
+  if (int rc = layout(ctx, b, L)) return rc;
   if (ws_bytes < L.total_bytes) {
     set_error("lr_plan_create: workspace of %zu bytes, %zu needed", ws_bytes, L.total_bytes);
     return LR_ENOMEM;
@@ -375,12 +381,13 @@ extern "C" int lr_plan_create(lr_ctx *ctx, const lr_batch *b, void *ws, size_t w
   p->workspace_bytes = ws_bytes;
   p->attention_path = 0;
   p->o_page_ids = L.o_page_ids;
-  if (int rc = take_pinned(ctx, L.image_bytes, &p->pinned, &p->pinned_cap, &p->uploaded)) {
+  if (int rc = take_pinned(ctx, L.image_bytes + 64, &p->pinned, &p->pinned_cap, &p->uploaded)) {
     delete p;
     return rc;
   }
-  memset(p->pinned, 0, L.image_bytes);
-  memcpy(p->pinned, L.img.bytes.data(), L.img.bytes.size());
+  Image img;
+  img.base = reinterpret_cast<unsigned char *>(p->pinned);
+  sections(b, L, img);
   unsigned char *base = reinterpret_cast<unsigned char *>(ws);
   auto at = [&](size_t off) { return reinterpret_cast<const int32_t *>(base + off); };
   DevBatch &d = p->dev;
@@ -431,13 +438,25 @@ extern "C" int lr_plan_create(lr_ctx *ctx, const lr_batch *b, void *ws, size_t w
   p->n_rows_logits = p->n_drafts + b->n_branch;
   p->n_verdicts = b->n_span - b->n_req;
   tc_bind_device_plan(L.tc, base, base + L.image_bytes, p);
-  pair_bind_device_plan(L.pr, base, base + L.pair_scratch_off, p);
+  p->pair_ok = p->pair_built = p->pair_upload = false;
+  memset(&p->pr, 0, sizeof(p->pr));
+  p->pr.wait_limit_us = p->tc.wait_limit_us = 1000000u;  // one second per wait
+  p->region_off = L.image_bytes;
+  p->region_bytes = L.region_bytes;
+  p->o_req_span_off = L.o_req_span_off;
+  p->o_span_len = L.o_span_len;
+  p->o_span_slot = L.o_span_slot;
+  p->o_br_req = L.o_br_req;
+  p->o_br_depth = L.o_br_depth;
+  p->o_br_own_len = L.o_br_own_len;
+  p->o_br_own_slot = L.o_br_own_slot;
+  p->o_br_n_draft = L.o_br_n_draft;
+  p->o_cu_q = L.o_cu_q;
+  p->o_req_br_off = L.o_req_br_off;
+  p->o_span_tin = L.o_span_tin;
+  p->o_span_last = L.o_span_last;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemcpyAsync(ws, p->pinned, L.image_bytes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && L.tc.scratch_zero_bytes)
-    e = cudaMemsetAsync(base + L.image_bytes, 0, L.tc.scratch_zero_bytes, s);
-  if (e == cudaSuccess && L.pr.scratch_zero_bytes)
-    e = cudaMemsetAsync(base + L.pair_scratch_off, 0, L.pr.scratch_zero_bytes, s);
   if (e == cudaSuccess) e = cudaEventRecord(p->uploaded, s);
   if (e != cudaSuccess) {
     give_back_pinned(ctx, p->pinned, p->pinned_cap, p->uploaded);
@@ -456,10 +475,54 @@ extern "C" int lr_plan_destroy(lr_plan *p) {
   return LR_OK;
 }
 
+// Plans the CTA-pair path from the batch tables of the plan's host image.
+static int build_pair(lr_plan *p) {
+  const unsigned char *img = reinterpret_cast<const unsigned char *>(p->pinned);
+  auto at = [&](size_t off) { return reinterpret_cast<const int32_t *>(img + off); };
+  lr_batch b = {};
+  b.n_req = p->dev.n_req;
+  b.n_branch = p->dev.n_branch;
+  b.n_span = p->dev.n_span;
+  b.n_page_slots = p->dev.n_page_slots;
+  b.req_span_off = at(p->o_req_span_off);
+  b.span_len = at(p->o_span_len);
+  b.span_slot = at(p->o_span_slot);
+  b.br_req = at(p->o_br_req);
+  b.br_depth = at(p->o_br_depth);
+  b.br_own_len = at(p->o_br_own_len);
+  b.br_own_slot = at(p->o_br_own_slot);
+  b.br_n_draft = at(p->o_br_n_draft);
+  b.cu_q = at(p->o_cu_q);
+  b.page_ids = at(p->o_page_ids);
+  b.n_pool_pages = p->dev.n_pool_pages;
+  PairHostPlan h;
+  p->pr_image.clear();
+  if (int rc = pair_build_host_plan(p->ctx, &b, at(p->o_req_br_off), at(p->o_span_tin), at(p->o_span_last), h, p->pr_image)) return rc;
+  const size_t scratch = align_up(p->pr_image.size(), 256);
+  if (h.ok && scratch + h.scratch_bytes > p->region_bytes) {
+    set_error("lr_plan_set_attention_path: the CTA-pair plan needs %zu bytes of workspace, %zu are set aside", scratch + h.scratch_bytes, p->region_bytes);
+    return LR_ENOMEM;
+  }
+  unsigned char *region = reinterpret_cast<unsigned char *>(p->workspace_d) + p->region_off;
+  const uint32_t wait_limit_us = p->pr.wait_limit_us, phantom = p->pr.phantom_tx_bytes;
+  pair_bind_device_plan(h, region, region + scratch, p);
+  p->pr.wait_limit_us = wait_limit_us;
+  p->pr.phantom_tx_bytes = phantom;
+  p->pr_zero_off = scratch + h.s_counters;
+  p->pr_zero_bytes = h.scratch_zero_bytes;
+  p->pair_built = true;
+  return LR_OK;
+}
+
 extern "C" int lr_plan_set_attention_path(lr_plan *p, int path) {
   if (!p || path < 0 || path > 3) {
     set_error("lr_plan_set_attention_path: bad argument");
     return LR_EINVAL;
+  }
+  if (path == 3) {
+    if (!p->pair_built)
+      if (int rc = build_pair(p)) return rc;
+    p->pair_upload = true;  // another path may have used the region meanwhile
   }
   p->attention_path = path;
   return LR_OK;
@@ -533,13 +596,10 @@ extern "C" int lr_plan_debug_set_page(lr_plan *p, int32_t page_slot, int32_t new
   for (int c = 0; c < p->n_tc_heads; ++c)
     for (int k = 0; k < 32; ++k)
       if (heads[c].first_pages[k] == old_id && heads[c].piece1 > heads[c].piece0) heads[c].first_pages[k] = new_id;
-  TcPage *ppages = reinterpret_cast<TcPage *>(img + p->o_pr_pages);
-  for (int i = 0; i < p->n_pr_pages; ++i)
-    if (ppages[i].page == old_id && (ppages[i].meta & 31u) != 0u) ppages[i].page = new_id;
-  PrHead *pheads = reinterpret_cast<PrHead *>(img + p->o_pr_heads);
-  for (int c = 0; c < p->n_pr_heads; ++c)
-    for (int k = 0; k < 32; ++k)
-      if (pheads[c].first_pages[k] == old_id && pheads[c].piece1 > pheads[c].piece0) pheads[c].first_pages[k] = new_id;
+  if (p->pair_built) {
+    if (int rc = build_pair(p)) return rc;
+    p->pair_upload = true;
+  }
   cudaError_t e = cudaMemcpyAsync(p->workspace_d, p->pinned, p->image_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaEventRecord(p->uploaded, s);
   return cuda_fail(e, "lr_plan_debug_set_page upload");
@@ -562,6 +622,13 @@ extern "C" int lr_verify_attention(lr_plan *p, const void *q, const void *k, con
     if (!p->pair_ok) {
       set_error("lr_verify_attention: the CTA-pair tensor-core path does not support this shape");
       return LR_EUNSUPPORTED;
+    }
+    if (p->pair_upload) {
+      unsigned char *region = reinterpret_cast<unsigned char *>(p->workspace_d) + p->region_off;
+      cudaError_t e = cudaMemcpyAsync(region, p->pr_image.data(), p->pr_image.size(), cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaMemsetAsync(region + p->pr_zero_off, 0, p->pr_zero_bytes, s);
+      if (e != cudaSuccess) return cuda_fail(e, "CTA-pair plan upload");
+      p->pair_upload = false;
     }
     return launch_attn_pair(p, q, k, v, out, lse, scale, s);
   }
@@ -738,13 +805,14 @@ extern "C" int lr_poll_status(lr_plan *p, void *stream, int32_t *detail) {
     return LR_EINVAL;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  int32_t st[2] = {0, 0};
-  cudaError_t e = cudaMemcpyAsync(st, p->dev.status, sizeof(st), cudaMemcpyDeviceToHost, s);
+  // the last 64 bytes of the pinned buffer are for this (pageable memory would be staged by the driver)
+  volatile int32_t *st = reinterpret_cast<int32_t *>(reinterpret_cast<unsigned char *>(p->pinned) + p->pinned_cap - 64);
+  cudaError_t e = cudaMemcpyAsync(const_cast<int32_t *>(st), p->dev.status, 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "lr_poll_status");
   if (detail) *detail = st[1];
   if (st[0] == kDevOk) return LR_OK;
-  e = cudaMemsetAsync(p->dev.status, 0, sizeof(st), s);
+  e = cudaMemsetAsync(p->dev.status, 0, 8, s);
   if (e != cudaSuccess) return cuda_fail(e, "lr_poll_status clear");
   if (st[0] == kDevTimeout) {
     set_error("device wait expired (detail %d)", st[1]);

@@ -167,16 +167,21 @@ struct lr_plan {
   lr::DevTcPlan tc;
   lr::DevPairPlan pr;
   bool tc_ok;             // shape allows the tensor-core path
-  bool pair_ok;           // shape allows the CTA-pair tensor-core path
+  // The CTA-pair plan is built when its path is selected.  Its image and scratch lie over the single-CTA path's scratch
+  // (the two never run at the same time), so every selection uploads the image again.
+  bool pair_ok;           // shape allows the CTA-pair tensor-core path (known once built)
+  bool pair_built, pair_upload;  // ... upload before the next launch
   int pr_pieces, pr_partial_slots;
-  size_t o_pr_pages, o_pr_heads;
-  int n_pr_pages, n_pr_heads;
+  size_t pr_zero_off, pr_zero_bytes;  // ticket counters, relative to the region
+  std::vector<unsigned char> pr_image;
+  size_t region_off, region_bytes;    // behind the image in the workspace
+  size_t o_req_span_off, o_span_len, o_span_slot, o_br_req, o_br_depth, o_br_own_len, o_br_own_slot, o_br_n_draft, o_cu_q, o_req_br_off,
+      o_span_tin, o_span_last;        // batch tables in the image
   int attention_path;     // 0 auto, 1 generic, 2 tensor core (single CTA), 3 tensor core (CTA pairs)
   int tc_pieces, tc_partial_slots;  // for lr_plan_describe
   // where the physical page ids sit in the image (lr_plan_debug_set_page)
   size_t o_page_ids, o_tc_pages, o_tc_heads;
   int n_tc_pages, n_tc_heads;
-  std::vector<unsigned char> staging;  // host copy of the uploaded image (kept alive for the async copy)
   void *pinned;           // pinned host image
   size_t pinned_cap;
   void *results_pinned;   // pinned bounce buffer for the integer results of lr_verify_pass_host (allocated on first use)
@@ -193,28 +198,53 @@ struct lr_plan {
 
 namespace lr {
 
-// Byte image of everything lr_plan_create uploads; sections are 256-byte aligned.
+// Byte image of everything lr_plan_create uploads; sections are 256-byte aligned.  Without a buffer only sizes and offsets
+// are worked out, so that one function lays out and fills.
 struct Image {
-  std::vector<unsigned char> bytes;
-  size_t add(const void *src, size_t n) {
-    size_t off = (bytes.size() + 255) / 256 * 256;
-    bytes.resize(off + n);
-    if (src && n) memcpy(bytes.data() + off, src, n);
+  unsigned char *base = nullptr;
+  size_t bytes = 0;
+  template <class T>
+  T *add(size_t n, size_t &off) {  // n elements to be filled in by the caller; null without a buffer
+    off = (bytes + 255) / 256 * 256;
+    if (base) memset(base + bytes, 0, off - bytes);
+    bytes = off + n * sizeof(T);
+    return base ? reinterpret_cast<T *>(base + off) : nullptr;
+  }
+  template <class T>
+  size_t copy(const T *src, size_t n) {
+    size_t off;
+    if (T *dst = add<T>(n, off); dst && n) memcpy(dst, src, n * sizeof(T));
     return off;
   }
 };
 
-// Host-side result of planning the tensor-core attention for one batch.
+// Host-side plan of the tensor-core attention for one batch: first the structure (page lists as runs of page slots, the
+// work partition), from which all sizes follow, then the tables.
+struct TcRun {         // consecutive page slots of one span in a page list
+  int slot, len, n_pg; // first slot, tokens of the span, pages listed
+  uint32_t meta;       // TcPage.meta without the valid count (tails: and without the page number)
+  bool tail;
+};
+struct TcList {        // the page list of one (request, group of M-tiles)
+  TcReq rq;
+  int run0, run1;
+};
 struct TcHostPlan {
   bool ok = false;  // shape supported by the tensor-core path
+  std::vector<TcRun> runs;
+  std::vector<TcList> lists;
+  std::vector<TcPiece> pieces;
+  std::vector<int32_t> cta_piece_off;
+  std::vector<TcTarget> targets;
   size_t o_heads = 0, o_pages = 0, o_rows = 0, o_pieces = 0, o_cta_piece_off = 0, o_reqs = 0, o_targets = 0;  // image offsets
-  int n_cta = 0, n_targets = 0, n_pieces = 0, n_partial_slots = 0, tokens_per_mtile = 0, n_pages = 0;
+  int n_cta = 0, n_partial_slots = 0, tokens_per_mtile = 0, n_pages = 0;
   // scratch region behind the image: (exponent, sum) pairs, then fp32 partial outputs
-  size_t s_ml = 0, s_o = 0, scratch_bytes = 0, scratch_zero_bytes = 0;
+  size_t s_ml = 0, s_o = 0, scratch_bytes = 0;
 };
 // span_tin / span_last: depth-first interval labels of the spans ([n_span] each, see DevBatch)
-int tc_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
-                       const int32_t *span_last, TcHostPlan &out, Image &img);
+void tc_plan_structure(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
+                       const int32_t *span_last, TcHostPlan &out);
+void tc_plan_tables(const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin, TcHostPlan &h, Image &img);
 void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigned char *scratch_base, lr_plan *p);
 
 // Host-side result of planning the CTA-pair attention for one batch.
@@ -225,8 +255,11 @@ struct PairHostPlan {
   // scratch region behind the image: ticket counters, (exponent, sum) pairs, fp32 partial outputs
   size_t s_counters = 0, s_ml = 0, s_o = 0, scratch_bytes = 0, scratch_zero_bytes = 0;
 };
+// Builds the plan and its image (a vector: the pair path is planned only when it is selected).
 int pair_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
-                         const int32_t *span_last, PairHostPlan &out, Image &img);
+                         const int32_t *span_last, PairHostPlan &out, std::vector<unsigned char> &img);
+// An upper bound of the image and scratch bytes of that plan, from the batch's counts alone.
+size_t pair_bytes_bound(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off);
 void pair_bind_device_plan(const PairHostPlan &h, unsigned char *image_base, unsigned char *scratch_base, lr_plan *p);
 
 void set_error(const char *fmt, ...);
