@@ -1,17 +1,16 @@
 // Greedy token-level acceptance: one streaming pass over the bf16 logits.
 //
-// The logits are cut into equal contiguous ranges of 16-byte vectors, one per CTA
-// of a fixed grid (a few CTAs per SM), whatever the row boundaries; a range that
-// spans several rows is handled row segment by row segment.  Each segment is
-// reduced to (max value, lowest index) and published with one 64-bit atomicMax
-// on the row's key; a CTA then takes a ticket, and the one holding the last
-// ticket turns the row keys into n_accept / bonus per branch and zeroes the
-// scratch again.
+// The rows are cut into chunks of 2048 logits, which the warps of a fixed grid take
+// in turn; a warp reduces a chunk to (max value, lowest index) and publishes it
+// with one 64-bit atomicMax on the row's key.  Warps never wait for one another.
+// A CTA then takes a ticket, and the one holding the last ticket turns the row
+// keys into n_accept / bonus per branch and zeroes the scratch again.
 //
 // The work is bound by HBM reads: 2 bytes per logit, read once, 16-byte loads,
 // eight independent loads in flight per thread.  The maximum is taken with
 // packed bf16x2 max instructions on whole 16-byte vectors (about one
 // instruction per logit); the index is resolved only inside the winning vector.
+// Small passes are bound by the chain load - atomic - ticket - last CTA.
 #include <algorithm>
 
 #include "lr_common.cuh"
@@ -22,6 +21,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kVecPerThread = 8;                          // 16-byte vectors in flight per thread
+constexpr int kChunkVecs = 32 * kVecPerThread;            // vectors a warp takes at a time
 constexpr int kCtasPerSm = 4;
 
 // Monotone map of a float (already NaN-free, -0 folded to +0) to an unsigned key.
@@ -86,98 +86,57 @@ __device__ __forceinline__ Best better(Best a, Best b) {
 __global__ void __launch_bounds__(kThreads)
 accept_greedy_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab,
                      const int32_t *__restrict__ draft_ids, const int32_t *__restrict__ cu_draft, int32_t n_branch,
-                     int32_t n_rows, int32_t *__restrict__ n_accept, int32_t *__restrict__ bonus_id,
+                     int32_t n_rows, uint32_t n_chunks, uint32_t total, int32_t *__restrict__ n_accept, int32_t *__restrict__ bonus_id,
                      int32_t *__restrict__ row_argmax, unsigned long long *scratch) {
   unsigned int *counter = reinterpret_cast<unsigned int *>(scratch);
   unsigned long long *row_key = scratch + 1;
-  const int tid = threadIdx.x;
-  const int32_t n_vec = vocab >> 3;  // whole 16-byte vectors in a row
-  // A row is n_vec vector units plus one unit for its ragged end (vocab not a multiple of 8).
-  const int64_t upr = (int64_t)n_vec + 1, total = upr * n_rows;
-  const int64_t per = (total + gridDim.x - 1) / gridDim.x;
-  int64_t pos = (int64_t)blockIdx.x * per;
-  const int64_t end = min(total, pos + per);
-  __shared__ float s_v[kThreads / 32];
-  __shared__ int32_t s_i[kThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int32_t n_vec = vocab >> 3, rem = vocab & 7;
   __shared__ int s_last;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the logits may come from the kernel launched just before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // lr_commit's grid may be set up meanwhile
 
-  while (pos < end) {
-    const int row = (int)(pos / upr);
-    const int32_t u0 = (int32_t)(pos - (int64_t)row * upr);
-    const int32_t u1 = (int32_t)min(upr, (int64_t)u0 + (end - pos));
-    const int32_t v_end = min(u1, n_vec);
+  for (uint32_t unit = blockIdx.x * (kThreads / 32) + (tid >> 5); unit < total; unit += gridDim.x * (kThreads / 32)) {
+    const uint32_t row = unit / n_chunks, c = unit - row * n_chunks;
     const uint16_t *rp = logits + (int64_t)row * row_stride;
     const uint4 *vp = reinterpret_cast<const uint4 *>(rp);
-    // Per thread: vectors are visited in increasing index order and only a strictly
+    const int32_t v0 = (int32_t)c * kChunkVecs + lane;
+    uint4 v[kVecPerThread];
+#pragma unroll
+    for (int k = 0; k < kVecPerThread; ++k)
+      if (v0 + k * 32 < n_vec) v[k] = ld_stream(vp + v0 + k * 32);
+    // Per lane: vectors are visited in increasing index order and only a strictly
     // greater maximum replaces the current one, so the earliest maximum is kept.
     Best best;
     best.v = -INFINITY;
     best.i = 0x7FFFFFFF;  // "owns no element": loses every tie
     uint4 bv = make_uint4(0, 0, 0, 0);
     int32_t bvi = -1;
-    for (int32_t base = u0; base < v_end; base += kThreads * kVecPerThread) {
-      uint4 v[kVecPerThread];
 #pragma unroll
-      for (int k = 0; k < kVecPerThread; ++k) {
-        const int32_t vi = base + k * kThreads + tid;
-        if (vi < v_end) v[k] = ld_stream(vp + vi);
-      }
-#pragma unroll
-      for (int k = 0; k < kVecPerThread; ++k) {
-        const int32_t vi = base + k * kThreads + tid;
-        if (vi < v_end) {
-          const float m = denan(vec_max(v[k]));
-          if (m > best.v || bvi < 0) {
-            best.v = m;
-            bv = v[k];
-            bvi = vi;
-          }
+    for (int k = 0; k < kVecPerThread; ++k) {
+      const int32_t vi = v0 + k * 32;
+      if (vi < n_vec) {
+        const float m = denan(vec_max(v[k]));
+        if (m > best.v || bvi < 0) {
+          best.v = m;
+          bv = v[k];
+          bvi = vi;
         }
       }
     }
     // a maximum of -inf means every element is -inf or NaN: the first one wins
     if (bvi >= 0) best.i = bvi * 8 + (best.v == -INFINITY ? 0 : first_equal(bv, best.v));
-    // ragged end of the row: up to 7 single elements
-    if (u1 == (int32_t)upr) {
-      const int32_t e = n_vec * 8 + tid;
-      if (e < vocab) {
-        Best t;
-        t.v = denan(bf_lo((uint32_t)rp[e]));
-        t.i = e;
-        best = better(best, t);
-      }
+    if (c == n_chunks - 1 && lane < rem) {  // ragged end of the row: up to 7 single elements
+      Best t;
+      t.v = denan(bf_lo((uint32_t)rp[n_vec * 8 + lane]));
+      t.i = n_vec * 8 + lane;
+      best = better(best, t);
     }
-    // warp, then block reduction
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      Best o;
-      o.v = __shfl_down_sync(0xFFFFFFFFu, best.v, off);
-      o.i = __shfl_down_sync(0xFFFFFFFFu, best.i, off);
-      best = better(best, o);
-    }
-    if ((tid & 31) == 0) {
-      s_v[tid >> 5] = best.v;
-      s_i[tid >> 5] = best.i;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      for (int w = 1; w < kThreads / 32; ++w) {
-        Best o;
-        o.v = s_v[w];
-        o.i = s_i[w];
-        best = better(best, o);
-      }
-      if (best.i != 0x7FFFFFFF) {
-        unsigned long long key =
-            ((unsigned long long)order_key(best.v) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)best.i);
-        atomicMax(row_key + row, key);
-      }
-    }
-    __syncthreads();
-    pos += u1 - u0;
+    const uint32_t key = order_key(best.v), top = __reduce_max_sync(0xFFFFFFFFu, key);
+    const uint32_t first = __reduce_min_sync(0xFFFFFFFFu, key == top ? (uint32_t)best.i : 0x7FFFFFFFu);
+    if (lane == 0 && first != 0x7FFFFFFFu) atomicMax(row_key + row, ((unsigned long long)top << 32) | (unsigned long long)(0xFFFFFFFFu - first));
   }
+  __syncthreads();
   if (tid == 0) {
     __threadfence();
     unsigned int t = atomicAdd(counter, 1u);
@@ -278,12 +237,11 @@ int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t
                   int32_t n_branch, int32_t n_rows, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,
                   void *scratch, cudaStream_t s) {
   const int32_t vocab = ctx->model.vocab;
-  // equal ranges of at least one full round of loads per CTA, at most kCtasPerSm CTAs per SM
-  const int64_t total = ((int64_t)(vocab >> 3) + 1) * n_rows;
-  int64_t grid = (total + kThreads * kVecPerThread - 1) / (kThreads * kVecPerThread);
-  grid = std::max<int64_t>(1, std::min<int64_t>(grid, (int64_t)ctx->sm_count * kCtasPerSm));
-  accept_greedy_kernel<<<(unsigned)grid, kThreads, 0, s>>>(reinterpret_cast<const uint16_t *>(logits), stride, vocab, drafts,
-                                                            cu_draft, n_branch, n_rows, n_accept, bonus, row_argmax,
+  // a chunk per warp at least, at most kCtasPerSm CTAs per SM
+  const uint32_t n_chunks = std::max(1, ((vocab >> 3) + kChunkVecs - 1) / kChunkVecs), total = n_chunks * (uint32_t)n_rows;
+  const unsigned grid = std::min((total + kThreads / 32 - 1) / (kThreads / 32), (uint32_t)(ctx->sm_count * kCtasPerSm));
+  accept_greedy_kernel<<<grid, kThreads, 0, s>>>(reinterpret_cast<const uint16_t *>(logits), stride, vocab, drafts,
+                                                            cu_draft, n_branch, n_rows, n_chunks, total, n_accept, bonus, row_argmax,
                                                             reinterpret_cast<unsigned long long *>(scratch));
   ctx->launches++;
   return cuda_fail(cudaGetLastError(), "accept_greedy_kernel launch");
