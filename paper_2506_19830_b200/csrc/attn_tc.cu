@@ -40,13 +40,16 @@
 //               O += P V (P read from tensor memory, V from shared memory as the
 //               N-major operand).  Issue blocks while the tensor pipe is full, so
 //               one issuer per stream lets the waits of one overlap the MMAs of
-//               the other.
+//               the other.  The elected lane comes from elect.sync, so that operands stay in
+//               uniform registers (against lane 0: a single 4 K-token request 20.4 -> 19.9 us, 19.3 -> 18.0 with head size 64, nothing on long ones).
 //   warps 0-3   softmax of stream 0, one thread per query row: tcgen05.ld gives a
 //   warps 4-7   softmax of stream 1  thread its whole row of S in registers, so
 //               row max and row sum need no cross-lane traffic.  One sweep:
 //               max (3-input max), lazy rescale of O in tensor memory only when
 //               the maximum grew by more than 2^8, exp2 with packed fp32 FMA/ADD,
-//               bf16 P written back over S.
+//               bf16 P written back over S.  A barrier test costs a warp over 100 cycles
+//               even when it succeeds, so the sweep makes one per 64 keys, under the
+//               exponentials (with two, in line: 85 us against 81 for four 16 K-token requests).
 // Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 fp32 columns each; P_s
 // occupies the first 64 columns of S_s.
 //
@@ -213,6 +216,14 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
       "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc)
       : "memory");
+}
+
+// One lane of a converged warp, always the same one.  The compiler keeps what the elected lane does in uniform registers,
+// which is where the operands of tcgen05.mma have to be.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
 
 // tcgen05.ld / tcgen05.st, shape 32x32b: thread i of the warp owns lane (base + i), consecutive columns.
@@ -574,8 +585,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
   if (warp >= 8) {
    // service warpgroup: needs few registers; the softmax threads hold a whole row of scores in theirs
    // setmaxnreg.inc blocks until its request fits into what the CTA was launched with (168 registers x 384
-   // threads), so the totals after the moves must not exceed that: 72 x 128 + 216 x 256 = 168 x 384.
-   asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+   // threads), so the totals after the moves must not exceed that: 72 x 128 + 216 x 256 = 168 x 384 (head size 64) and
+   // 120 x 128 + 192 x 256 = 168 x 384 (head size 128, whose issuers keep more descriptors).
+   if constexpr (kD == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 120;");
+   else asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
    if (warp == 8) {
     // ======================= TMA producer ==========================================
     uint32_t ring = 0, q_count = 0;
@@ -660,11 +673,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
     // consumed by its MMAs (released by a tcgen05.commit), one it does not use (the other
     // stream's tiles in the even/odd split) is released with a plain arrive once it has landed.
     // So neither issuer nor the producer can get a whole ring ahead of the other.
-    const int s = warp - 9;
+    const int s = __shfl_sync(0xFFFFFFFFu, warp, 0) - 9;
     uint32_t ring_base = 0, waited = 0, p_cnt = 0, pc_idx = 0;
     bool ok = true;
     const uint32_t q_addr = smem_u32(q_smem), kv_addr = smem_u32(kv_smem);
-    const uint32_t s_tmem = tmem + s * 128, o_tmem = tmem + 256 + s * 128;
+    const uint32_t tmem_u = __shfl_sync(0xFFFFFFFFu, tmem, 0);
+    const uint32_t s_tmem = tmem_u + s * 128, o_tmem = tmem_u + 256 + s * 128;
     // Descriptors differ from a base only in the start-address field (units of 16 bytes).
     const uint64_t qdesc0 = make_desc(q_addr, 16, 1024), kdesc0 = make_desc(kv_addr, 16, kGroupBytes),
                    vdesc0 = make_desc(kv_addr, kAtomBytes, kGroupBytes);
@@ -700,7 +714,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
       auto need = [&](uint32_t pos, int code) -> bool {
         while (waited <= pos) {
           if (!wait_bar(&ctrl->kv_full[waited % kStages], (waited / kStages) & 1u, ctrl, d.status, code)) return false;
-          if (waited < pos && lane == 0) mbar_arrive(&ctrl->kv_empty[waited % kStages]);
+          if (waited < pos && elect_one()) mbar_arrive(&ctrl->kv_empty[waited % kStages]);
           ++waited;
         }
         return true;
@@ -714,7 +728,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
         ok = need(pos, 221);
         if (!ok) break;
         tc_fence_after();
-        if (lane == 0) {
+        if (elect_one()) {
           issue_qk(m_tile, pos % kStages, 0);
           tc_commit(&ctrl->s_full[s][0]);
           issue_qk(m_tile, pos % kStages, 1);
@@ -724,7 +738,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
         }
         __syncwarp();
       } else {
-        if (lane == 0) mbar_arrive(&ctrl->q_empty);
+        if (elect_one()) mbar_arrive(&ctrl->q_empty);
         // nothing to issue in this piece: still observe the previous piece's epilogue phase, so that the parity
         // wait of a later piece never finds this issuer two phases behind
         if (pc_idx > 0) {
@@ -773,7 +787,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
           ok = wait_bar(&ctrl->p_full[s][half], p_cnt & 1u, ctrl, d.status, 224 + s);
           if (!ok) break;
           tc_fence_after();
-          if (lane == 0) {
+          if (elect_one()) {
             issue_pv(sV, half, (j | half) != 0);
             tc_commit(&ctrl->o_done[s]);
             if (half == 1) release(pos_v);
@@ -796,7 +810,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
       if (waited < ring_base) {
         ok = need(ring_base - 1, 227);
         if (!ok) break;
-        if (lane == 0) mbar_arrive(&ctrl->kv_empty[(ring_base - 1) % kStages]);
+        if (elect_one()) mbar_arrive(&ctrl->kv_empty[(ring_base - 1) % kStages]);
       }
     }
     if (!ok && lane == 0) {
@@ -809,7 +823,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
     __syncwarp();
    }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+    if constexpr (kD == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
     // ======================= softmax warpgroups ======================================
     const int s = warp >> 2;                       // stream
     const int quarter = warp & 3;                  // tensor-memory lane quarter this warp may access
@@ -827,9 +842,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
       if (ok && my_units > 0) {
         const RowInfo ri = row_info(d, tc, rq, T, mode == 2 ? pi.mtile0 + s : pi.mtile0, r, pi.kv_head);
         float m_used = -INFINITY, l = 0.f, m_new = 0.f;
-        bool pend = false;
+        bool pend = false, s_ready = false;
         // O *= alpha.  The PV product of the previous half-unit must have retired first; the one before
-        // it has (its commit precedes the s_full this thread has just seen).
+        // it has (its commit precedes the s_full this thread has just seen), so o_done has completed done_needed or
+        // done_needed - 1 phases and the parity says which, whether or not this thread has looked at the earlier ones.
         auto rescale_o = [&](float alpha, uint32_t done_needed) -> bool {
           if (!wait_bar(&ctrl->o_done[s], (done_needed - 1) & 1u, ctrl, d.status, 235 + s)) return false;
           tc_fence_after();
@@ -863,12 +879,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
             const uint32_t sh_addr = s_addr + half * 64;
             const uint32_t g = o_cnt + (uint32_t)(2 * j + half);  // half-units of this stream before this one
             const bool first = (j | half) == 0;
-            ok = wait_bar(&ctrl->s_full[s][half], s_cnt & 1u, ctrl, d.status, 230 + s);
-            if (!ok) break;
+            if (!s_ready) {
+              ok = wait_bar(&ctrl->s_full[s][half], s_cnt & 1u, ctrl, d.status, 230 + s);
+              if (!ok) break;
+            }
             tc_fence_after();
             uint32_t v[64];
             tmem_ld64(sh_addr, v);
             tc_wait_ld();
+            // the scores after these are looked for under the exponentials: a test costs over 100 cycles even when it succeeds
+            const uint32_t next_ready = mbar_test_wait(&ctrl->s_full[s][half ^ 1], (s_cnt + (uint32_t)half) & 1u);
             if (masked) mask_half(v, n_ok + 4 * half);
             // A growth of the maximum noticed in an earlier half-unit is applied now.
             if (__any_sync(0xFFFFFFFFu, pend)) {
@@ -919,10 +939,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
             else tmem_st32(sh_addr, pk);
             tc_wait_st();
             tc_fence_before();
-            // Observe every completion of o_done in order (a parity wait must never fall two phases behind):
-            // the PV product of the previous half-unit has long retired by now.  Before the arrive below,
-            // because the PV product of this half-unit can only be issued after it.
-            if (g > 0) {
+            s_ready = __all_sync(0xFFFFFFFFu, next_ready) != 0;
+            // The wait at the end must not find o_done two phases back (one parity for both): the last arrive comes
+            // after the product before has been seen to retire.
+            if (half == 1 && j + 1 == my_units) {
               ok = wait_bar(&ctrl->o_done[s], (g - 1) & 1u, ctrl, d.status, 237 + s);
               if (!ok) break;
             }
