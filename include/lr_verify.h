@@ -391,8 +391,9 @@ typedef struct lr_pass_host_io {
 int lr_pass_staging_bytes(const lr_plan *plan, size_t *bytes_out);
 
 /* One whole pass from host buffers: copies Q, logits, draft ids and verdicts to
- * the device staging buffer, runs the three steps, copies every result back and
- * WAITS for the stream.  staging_d: caller-owned device memory of
+ * the device staging buffer (the logits on a stream of the context, ordered after
+ * what `stream` holds, beside attention), runs the three steps, copies every
+ * result back and WAITS for the stream.  staging_d: caller-owned device memory of
  * lr_pass_staging_bytes, zero-filled before its first use.  Returns the device
  * status like lr_poll_status. */
 int lr_verify_pass_host(lr_plan *plan, const lr_pass_host_io *io, const void *k_pool_d, const void *v_pool_d,

@@ -151,9 +151,11 @@ accept_greedy_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   // One thread per branch, so that hundreds of branches cost one pass: the bounds of its draft range with two loads in
   // flight, then its rows eight at a time -- keys and drafts of a chunk are loaded together, so a chunk costs one
   // round trip to L2 whatever the branch count -- and the scan stops at the first mismatch.
+  // The branches may be a run of a larger batch's: drafts are indexed from the batch's first one, rows from the run's.
+  const int32_t first_draft = cu_draft[0];
   for (int b = tid; b < n_branch; b += kThreads) {
     const int32_t d0 = cu_draft[b], L = cu_draft[b + 1] - d0;
-    const int32_t r0 = d0 + b;
+    const int32_t r0 = d0 - first_draft + b;
     int32_t n = L, bonus = 0;
     bool found = false;
     for (int32_t i0 = 0; i0 <= L && !found; i0 += 8) {

@@ -159,6 +159,9 @@ struct lr_ctx {
   // far more than building a plan.  `uploaded` is recorded after the buffer's last upload; a new user waits on it.
   struct PinnedBuf { void *ptr; size_t cap; cudaEvent_t uploaded; };
   std::vector<PinnedBuf> pinned_free;
+  // lr_verify_pass_host uploads the logits here, beside the caller's stream (made on first use; idle between calls)
+  cudaStream_t copy_stream;
+  cudaEvent_t copy_fork, copy_part, copy_join;
 };
 
 struct lr_plan {
@@ -184,8 +187,9 @@ struct lr_plan {
   int n_tc_pages, n_tc_heads;
   void *pinned;           // pinned host image
   size_t pinned_cap;
-  void *results_pinned;   // pinned bounce buffer for the integer results of lr_verify_pass_host (allocated on first use)
+  void *results_pinned;   // pinned bounce buffer for the integer results of lr_verify_pass_host (taken on first use)
   size_t results_pinned_cap;
+  cudaEvent_t results_copied;
   cudaEvent_t uploaded;   // recorded after the image's upload
   size_t image_bytes;
   void *workspace_d;
