@@ -723,6 +723,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
       auto release = [&](uint32_t pos) { tc_commit(&ctrl->kv_empty[pos % kStages]); };
       ok = wait_bar(&ctrl->q_full, pc_idx & 1u, ctrl, d.status, 220);
       if (!ok) break;
+      // The box of a last M-tile brought queries of the next request along.  As zeros these rows cost the tensor core less
+      // power (their scores, and with them their weights, are zeros too), and power is what bounds long runs of this kernel:
+      // at the 1000 W limit, back to back, 16 ragged requests (30 % of the rows padding) 148.9 -> 143.8 us, four of 16 K
+      // tokens (38 %) 95.5 -> 92.7.  Where the clock is not limited it costs nothing measurable.
+      const int live = min(T, rq.n_q - (pi.mtile0 + m_tile) * T) * d.group;
+      if (my_units > 0 && live < T * d.group) {
+        unsigned char *qs = q_smem + m_tile * kTileBytes;
+        for (int idx = lane; idx < (128 - live) * 8; idx += 32)
+#pragma unroll
+          for (int h = 0; h < kHalves; ++h) *reinterpret_cast<uint4 *>(qs + h * kHalfBytes + live * 128 + idx * 16) = make_uint4(0, 0, 0, 0);
+        fence_proxy_async();
+        __syncwarp();
+      }
       if (my_units > 0) {
         const uint32_t pos = ring_base + ord.pos_k(mode == 2 ? 0 : s);
         ok = need(pos, 221);
@@ -861,7 +874,18 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
           tc_wait_st();
           return true;
         };
-        for (int j = 0; j < my_units && ok; ++j) {
+        // A warp whose 32 rows are all padding only keeps the barriers' counts: what it leaves as weights multiplies into rows
+        // of O that nobody reads.  (Head size 64 does not wait for the exponentials; the branch alone cost it 3 %.)
+        const bool idle = kD == 128 && __all_sync(0xFFFFFFFFu, ri.q_index < 0);
+        if (idle) {
+          for (int u = 0; u < 2 * my_units && ok; ++u) {
+            ok = wait_bar(&ctrl->s_full[s][u & 1], (s_cnt + (uint32_t)(u >> 1)) & 1u, ctrl, d.status, 230 + s);
+            if (ok && u + 1 == 2 * my_units) ok = wait_bar(&ctrl->o_done[s], (o_cnt + (uint32_t)u - 1) & 1u, ctrl, d.status, 237 + s);
+            if (ok) mbar_arrive(&ctrl->p_full[s][u & 1]);
+          }
+          s_cnt += (uint32_t)my_units;
+        }
+        for (int j = 0; j < my_units && ok && !idle; ++j) {
           const int t = pi.tile_begin + (mode == 2 ? j : 2 * j + s);
           const bool masked = t >= rq.n_dense_tiles;
           int n_ok[kPagesPerTile];
@@ -980,7 +1004,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
           }
         }
         if (pair) ++x_cnt;
-        if (ok && writer) {
+        if (ok && writer && !idle) {
           tc_fence_after();
           store_rows<kD>(o_addr, lane_base + 256 + (1 - s) * 128, pi.slot[pair ? 0 : s], pair, w_self, w_other, m_out, l_out, r, ri.q_index, out,
                      lse, tc.partial_o, tc.partial_ml);
