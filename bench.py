@@ -521,10 +521,10 @@ def extras(M):
         partial = np.flatnonzero(v[:-1] != 16)
         if len(partial):
             displaced += int(v[partial[0] + 1:].sum())
-    cmp_bytes = displaced * 2 * b.model.n_kv_heads * b.model.head_dim * 2 * 4  # K and V, read and written, twice
+    cmp_bytes = displaced * 2 * b.model.n_kv_heads * b.model.head_dim * 2 * 2  # K and V, read and written
     out["lr_compact"] = {"us": us, "displaced_tokens": displaced, "bytes_moved": cmp_bytes,
                          "case": "all steps accepted, whole last draft kept",
-                         "note": "three dependent launches, latency-bound; not part of the timed step"}
+                         "note": "one launch, latency-bound; not part of the timed step"}
     return out
 
 

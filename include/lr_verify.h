@@ -359,7 +359,7 @@ int lr_commit(lr_plan *plan, const uint8_t *verdict_d, const int32_t *n_accept_d
  * request's first partly filled kept page are not touched.  Bytes of the kept
  * pages beyond the sequence are unspecified afterwards; no other page is written.
  * scratch_d: lr_compact_scratch_bytes bytes, 256-byte aligned, no initial
- * contents needed.  Three launches on `stream`; a page id outside the pools sets
+ * contents needed.  One launch on `stream`; a page id outside the pools sets
  * the plan's status word (LR_EBOUNDS) instead of being dereferenced.  The batch
  * must be the one the plan and the keep lists were made for.  At most
  * LR_COMPACT_MAX_REQUESTS requests per pass (LR_EUNSUPPORTED beyond, before

@@ -1,16 +1,16 @@
 // Compaction of the committed KV after lr_commit: token k of a request's committed sequence goes to slot
 // k % 16 of its kept page number k / 16.
 //
-// The moves are in place in the caller's pools and overlap (a page is both a source and a destination), so
-// they go through a staging area in two stream-ordered phases: every displaced token is first copied out
-// (gather), then copied to its place (scatter).  Tokens in front of the first partly filled page of a request
-// stay where they are.  Three small kernels:
-//   compact_scan_kernel     one CTA per request: exclusive scan of the valid counts of its kept pages
-//                           (token offset of every page), the new length, the first displaced page;
-//   compact_move_kernel<0>  a fixed grid over the displaced pages: tokens -> staging[token index]      (gather);
-//   compact_move_kernel<1>  the same walk: staging -> destination page and slot                      (scatter).
-// Bytes moved: 2 (K, V) x H_kv x D x 2 B per displaced token, read and written twice; the work is bound by
-// the latency of three dependent launches, not by bandwidth.
+// The moves are in place in the caller's pools.  Counted along the keep list (list index x 16 + slot), a token only ever
+// moves towards the front, so a CTA that owns some columns of a request (one KV head of K or V, or a slice of its
+// channels) can sweep them in order without a staging area: it loads a round of rows into registers, meets at a
+// barrier, and stores them; what a round overwrites lies in front of everything a later round still has to read.
+// Different CTAs never touch the same bytes.  Every CTA scans its request's valid counts itself (a few hundred to a few
+// thousand integers, in L2 after the first reader); tokens in front of the first partly filled page stay where they are.
+//
+// Bytes moved: 2 (K, V) x H_kv x D x 2 B per displaced token, read and written once.  Bound by the chain of dependent
+// reads (list bounds, counts, page ids, data), not by bandwidth.  One launch; as three (scan, gather to a staging area,
+// scatter) with the bytes read and written twice, one layer of 8 ragged requests took 16.3 us on a B200, this takes 4.1.
 #include <algorithm>
 
 #include "lr_common.cuh"
@@ -20,172 +20,144 @@ namespace lr {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kMaxReq = LR_COMPACT_MAX_REQUESTS;  // the move kernels keep one prefix sum per request in shared memory
+constexpr int kMaxReq = LR_COMPACT_MAX_REQUESTS;
+constexpr int kPerThread = 4;                  // pages per thread and step of the scan
+constexpr int kScan = kThreads * kPerThread;   // pages per step
+constexpr int kRows = 8;                       // 16-byte vectors a thread holds per round
 
+// blockIdx.x: (KV head, K or V, slice of the row); blockIdx.y: request.  1 << shift 16-byte vectors per slice.
 __global__ void __launch_bounds__(kThreads)
-compact_scan_kernel(const int32_t *__restrict__ keep_off, const int32_t *__restrict__ keep_valid, int32_t *__restrict__ tok_off,
-                    int32_t *__restrict__ first_moved, int32_t *__restrict__ new_len, int32_t *__restrict__ n_pages_kept) {
-  __shared__ int32_t warp_sum[kThreads / 32];
-  __shared__ int32_t s_carry, s_first;
-  const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+compact_kernel(DevBatch d, const int32_t *__restrict__ keep_off, const int32_t *__restrict__ keep_pages,
+               const int32_t *__restrict__ keep_valid, int shift, uint4 *k_pool, uint4 *v_pool, int32_t *__restrict__ new_len,
+               int32_t *__restrict__ n_pages_kept) {
+  __shared__ int32_t s_off[kScan + 1];  // tokens of the request in front of each page of the step
+  __shared__ int32_t warp_sum[kThreads / 32], warp_first[kThreads / 32];
+  const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int vec_per_row = d.head_dim / 8, slices = vec_per_row >> shift;
+  const int slice = blockIdx.x % slices, h = blockIdx.x / slices >> 1;
+  uint4 *pool = (blockIdx.x / slices) & 1 ? v_pool : k_pool;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the keep list comes from the kernel launched just before
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the next layer's grid may be set up meanwhile
   const int i0 = keep_off[r], i1 = keep_off[r + 1];
-  if (tid == 0) {
-    s_carry = 0;
-    s_first = i1;  // "no page is displaced"
+  if (i0 < 0 || i1 > d.n_page_slots) {  // keep lists that do not come from lr_commit
+    if (tid == 0) {
+      d.status[0] = kDevBounds;
+      d.status[1] = 402;
+    }
+    return;
   }
-  __syncthreads();
-  for (int base = i0; base < i1; base += kThreads) {
-    const int i = base + tid;
-    const int32_t x = i < i1 ? keep_valid[i] : 0;
-    int32_t inc = x;
+  int32_t carry = 0;
+  bool moved = false;  // a page of an earlier step was displaced, hence every page of this one
+  for (int base = i0; base < i1; base += kScan) {
+    const int n_here = min(kScan, i1 - base);
+    int32_t x[kPerThread], sum = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) warp_sum[wid] = inc;
-    __syncthreads();
-    int32_t wbase = 0;
-    for (int w = 0; w < wid; ++w) wbase += warp_sum[w];
-    const int32_t carry = s_carry;
-    const int32_t off = carry + wbase + inc - x;  // tokens of the request in front of page i
-    if (i < i1) {
-      tok_off[i] = off;
-      if (off != (i - i0) * kPage) atomicMin(&s_first, i);  // displaced: an earlier page was not full
-    }
-    __syncthreads();
-    if (tid == kThreads - 1) s_carry = carry + wbase + inc;
-    __syncthreads();
-  }
-  if (tid == 0) {
-    first_moved[r] = s_first;
-    new_len[r] = s_carry;
-    n_pages_kept[r] = (s_carry + kPage - 1) / kPage;
-  }
-}
-
-// kScatter = false: pools -> staging; true: staging -> pools.  A fixed grid walks the displaced entries of the keep
-// lists only: request r has keep_off[r+1] - first_moved[r] of them (none when nothing of it moves); every CTA builds
-// the prefix sums of those counts in shared memory and takes the work items blockIdx.x, blockIdx.x + gridDim.x, ...
-template <bool kScatter>
-__global__ void __launch_bounds__(kThreads)
-compact_move_kernel(DevBatch d, const int32_t *__restrict__ keep_off, const int32_t *__restrict__ keep_pages,
-                    const int32_t *__restrict__ keep_valid, const int32_t *__restrict__ tok_off,
-                    const int32_t *__restrict__ first_moved, const int32_t *__restrict__ stage_off, uint4 *__restrict__ k_pool,
-                    uint4 *__restrict__ v_pool, uint4 *__restrict__ staging) {
-  extern __shared__ int32_t s_off[];  // [n_req + 1] displaced entries in front of request r
-  __shared__ int32_t warp_sum[kThreads / 32];
-  __shared__ int32_t s_carry;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (tid == 0) s_carry = 0;
-  __syncthreads();
-  for (int base = 0; base < d.n_req; base += kThreads) {
-    const int r = base + tid;
-    const int32_t x = r < d.n_req ? min(d.n_page_slots, max(0, keep_off[r + 1] - first_moved[r])) : 0;
-    int32_t inc = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) warp_sum[wid] = inc;
-    __syncthreads();
-    int32_t wbase = 0;
-    for (int w = 0; w < wid; ++w) wbase += warp_sum[w];
-    const int32_t carry = s_carry;
-    if (r < d.n_req) s_off[r] = carry + wbase + inc - x;
-    __syncthreads();
-    if (tid == kThreads - 1) s_carry = carry + wbase + inc;
-    __syncthreads();
-  }
-  const int32_t total = s_carry;
-  if (tid == 0) s_off[d.n_req] = total;
-  __syncthreads();
-  const int vec_per_row = d.head_dim / 8;          // 16-byte vectors per (token, head)
-  const int per_tok = d.n_kv_heads * vec_per_row;  // per pool
-  // a work item is one KV head of one displaced page (8 KB of K and V): enough items to spread a few hundred pages
-  for (int64_t item = blockIdx.x; item < (int64_t)total * d.n_kv_heads; item += gridDim.x) {
-    const int32_t w = (int32_t)(item / d.n_kv_heads);
-    const int h = (int)(item - (int64_t)w * d.n_kv_heads);
-    int lo = 0, hi = d.n_req - 1;  // request of page w: largest r with s_off[r] <= w (requests without items are skipped)
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (s_off[mid] <= w) lo = mid; else hi = mid - 1;
-    }
-    const int r = lo;
-    const int f = first_moved[r], i = f + (w - s_off[r]);
-    if (f < 0 || i < 0 || i >= d.n_page_slots) {  // keep lists that do not come from lr_commit
-      if (tid == 0) {
-        d.status[0] = kDevBounds;
-        d.status[1] = 402;
-      }
-      continue;
-    }
-    const int valid = keep_valid[i];
-    const int64_t src_page = keep_pages[i];
-    const int m0 = tok_off[i] - tok_off[f];  // index among the request's displaced tokens
-    if (src_page < 0 || src_page >= d.n_pool_pages || valid < 0 || valid > kPage ||
-        m0 + valid > stage_off[r + 1] - stage_off[r]) {  // never touch memory outside the pools or the staging area
-      if (tid == 0) {
+    for (int j = 0; j < kPerThread; ++j) {
+      const int p = tid * kPerThread + j;
+      x[j] = p < n_here ? keep_valid[base + p] : 0;
+      if ((uint32_t)x[j] > kPage) {  // not from lr_commit
         d.status[0] = kDevBounds;
         d.status[1] = 400;
       }
-      continue;
     }
-    const int i0 = keep_off[r];
-    const int k0 = tok_off[i];  // committed-sequence index of the page's first token
-    for (int idx = tid; idx < valid * vec_per_row; idx += kThreads) {
-      const int t = idx / vec_per_row, c = idx - t * vec_per_row, rem = h * vec_per_row + c;
-      const int64_t s_idx = ((int64_t)(stage_off[r] + m0 + t) * 2) * per_tok + rem;  // [token][K, V][head][vector]
-      if (!kScatter) {
-        const int64_t src = ((src_page * d.n_kv_heads + h) * kPage + t) * vec_per_row + c;
-        staging[s_idx] = k_pool[src];
-        staging[s_idx + per_tok] = v_pool[src];
-      } else {
-        const int k = k0 + t;
-        const int64_t dst_page = keep_pages[i0 + k / kPage];
-        if (dst_page < 0 || dst_page >= d.n_pool_pages) {
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j) sum += x[j];
+    int32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) warp_sum[wid] = inc;
+    __syncthreads();
+    int32_t off = carry + inc - sum;
+    for (int w = 0; w < wid; ++w) off += warp_sum[w];
+    int32_t first = kScan;  // first page of the step with a page that is not full somewhere in front of it
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j) {
+      const int p = tid * kPerThread + j;
+      s_off[p] = off;
+      if (p < n_here && off != (base + p - i0) * kPage) first = min(first, p);
+      off += x[j];
+    }
+    if (tid == kThreads - 1) s_off[kScan] = off;
+    first = __reduce_min_sync(0xFFFFFFFFu, first);
+    if (lane == 0) warp_first[wid] = first;
+    __syncthreads();
+    carry = s_off[kScan];
+    if (moved) {
+      first = 0;
+    } else {
+      for (int w = 0; w < kThreads / 32; ++w) first = min(first, warp_first[w]);
+    }
+    moved = moved || first < n_here;
+    // rounds of kThreads * kRows vectors, in token order
+    const int total = ((n_here - first) * kPage) << shift;
+    for (int at = 0; at < total; at += kThreads * kRows) {
+      uint4 v[kRows];
+      int64_t to[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const int item = at + u * kThreads + tid, p = first + (item >> shift) / kPage, t = (item >> shift) % kPage;
+        const int c = (slice << shift) + (item & ((1 << shift) - 1));
+        to[u] = -1;
+        if (item >= total) continue;
+        const int32_t k0 = s_off[p], valid = s_off[p + 1] - k0, k = k0 + t;
+        if (t >= valid) continue;
+        const int32_t dst_entry = k / kPage;
+        // never touch memory outside the pools, nor a page behind the token's own
+        int code = 0;
+        int64_t src_page = 0, dst_page = 0;
+        if (valid > kPage || k0 < 0 || dst_entry > base + p - i0) {
+          code = 400;
+        } else {
+          src_page = keep_pages[base + p];
+          dst_page = keep_pages[i0 + dst_entry];
+          if (src_page < 0 || src_page >= d.n_pool_pages) code = 400;
+          else if (dst_page < 0 || dst_page >= d.n_pool_pages) code = 401;
+        }
+        if (code != 0) {
           d.status[0] = kDevBounds;
-          d.status[1] = 401;
+          d.status[1] = code;
           continue;
         }
-        const int64_t dst = ((dst_page * d.n_kv_heads + h) * kPage + (k % kPage)) * vec_per_row + c;
-        k_pool[dst] = staging[s_idx];
-        v_pool[dst] = staging[s_idx + per_tok];
+        v[u] = pool[((src_page * d.n_kv_heads + h) * kPage + t) * vec_per_row + c];
+        to[u] = ((dst_page * d.n_kv_heads + h) * kPage + k % kPage) * vec_per_row + c;
       }
+      __syncthreads();  // the round is in registers
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+        if (to[u] >= 0) pool[to[u]] = v[u];
     }
+    __syncthreads();  // s_off is free again
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    new_len[r] = carry;
+    n_pages_kept[r] = (carry + kPage - 1) / kPage;
   }
 }
 
 }  // namespace
 
 int launch_compact(lr_plan *p, const int32_t *keep_off, const int32_t *keep_pages, const int32_t *keep_valid, void *k_pool,
-                   void *v_pool, int32_t *new_len, int32_t *n_pages_kept, void *scratch, cudaStream_t s) {
+                   void *v_pool, int32_t *new_len, int32_t *n_pages_kept, cudaStream_t s) {
   const DevBatch &d = p->dev;
-  unsigned char *base = reinterpret_cast<unsigned char *>(scratch);
-  int32_t *tok_off = reinterpret_cast<int32_t *>(base + p->compact.o_tok_off);
-  int32_t *first_moved = reinterpret_cast<int32_t *>(base + p->compact.o_first_moved);
-  const int32_t *stage_off = d.compact_stage_off;  // per-request offsets into the staging area, fixed by the batch
-  uint4 *staging = reinterpret_cast<uint4 *>(base + p->compact.o_staging);
   if (d.n_req > kMaxReq) {
     set_error("lr_compact: more than %d requests in one pass", kMaxReq);
     return LR_EUNSUPPORTED;
   }
-  compact_scan_kernel<<<d.n_req, kThreads, 0, s>>>(keep_off, keep_valid, tok_off, first_moved, new_len, n_pages_kept);
+  // Rows are sliced while that gives idle SMs something to do: down to 64 bytes until there are two CTAs per SM (8 KV heads
+  // of 128 channels, whole rows and sliced: one request with 360 displaced tokens 10.8 and 5.5 us, 16 with 160 each 7.6 and
+  // 7.0, but sliced in four 8.8), down to one sector for half a CTA per SM (one request 5.5 and 4.5, with 4000 tokens 26 and
+  // 17; four requests 4.2 and 5.1).
+  int shift = d.head_dim == 128 ? 4 : 3;
+  const int64_t rows = (int64_t)d.n_req * d.n_kv_heads * 2;
+  while (shift > 1 && rows * (d.head_dim / 8 >> shift) < (shift > 2 ? 2 * p->ctx->sm_count : p->ctx->sm_count / 2)) --shift;
+  const dim3 grid((unsigned)(d.n_kv_heads * 2 * (d.head_dim / 8 >> shift)), (unsigned)d.n_req);
   p->ctx->launches++;
-  if (int rc = cuda_fail(cudaGetLastError(), "compact_scan_kernel launch")) return rc;
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)d.n_page_slots * d.n_kv_heads, p->ctx->sm_count * 4));
-  const size_t smem = sizeof(int32_t) * ((size_t)d.n_req + 1);
-  compact_move_kernel<false><<<grid, kThreads, smem, s>>>(d, keep_off, keep_pages, keep_valid, tok_off, first_moved, stage_off,
-                                                      reinterpret_cast<uint4 *>(k_pool), reinterpret_cast<uint4 *>(v_pool), staging);
-  p->ctx->launches++;
-  if (int rc = cuda_fail(cudaGetLastError(), "compact gather launch")) return rc;
-  compact_move_kernel<true><<<grid, kThreads, smem, s>>>(d, keep_off, keep_pages, keep_valid, tok_off, first_moved, stage_off,
-                                                     reinterpret_cast<uint4 *>(k_pool), reinterpret_cast<uint4 *>(v_pool), staging);
-  p->ctx->launches++;
-  return cuda_fail(cudaGetLastError(), "compact scatter launch");
+  return cuda_fail(launch_dependent(compact_kernel, grid, dim3(kThreads), 0, s, d, keep_off, keep_pages, keep_valid, shift,
+                                    reinterpret_cast<uint4 *>(k_pool), reinterpret_cast<uint4 *>(v_pool), new_len, n_pages_kept),
+                   "compact_kernel launch");
 }
 
 }  // namespace lr

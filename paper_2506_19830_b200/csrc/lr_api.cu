@@ -109,12 +109,11 @@ static int validate_batch(const lr_batch *b) {
 // out the structure of the plan once, sections() lays the image out and, given a buffer, fills it in place.
 struct Layout {
   size_t o_req_span_off, o_span_len, o_span_slot, o_br_req, o_br_depth, o_br_own_len, o_br_own_slot, o_br_n_draft, o_cu_q,
-      o_cu_draft, o_page_ids, o_req_br_off, o_span_req, o_status, o_slot_item, o_chain_pg, o_chain_tok, o_tail_pg, o_compact_stage_off,
+      o_cu_draft, o_page_ids, o_req_br_off, o_span_req, o_status, o_slot_item, o_chain_pg, o_chain_tok, o_tail_pg,
       o_span_tin, o_span_last, o_child_off, o_child_list;
   std::vector<int32_t> cu_draft, req_br_off, span_tin, span_last, child_off, child_list;
   TcHostPlan tc;
   size_t image_bytes, region_bytes, total_bytes;
-  size_t compact_tokens;
 };
 
 static void sections(const lr_batch *b, Layout &L, Image &g) {
@@ -139,22 +138,13 @@ static void sections(const lr_batch *b, Layout &L, Image &g) {
   int32_t *chain_pg = g.add<int32_t>((size_t)b->n_span + b->n_req, L.o_chain_pg);
   int32_t *chain_tok = g.add<int32_t>((size_t)b->n_span + b->n_req, L.o_chain_tok);
   int32_t *tail_pg = g.add<int32_t>((size_t)b->n_branch + b->n_req, L.o_tail_pg);
-  int32_t *stage_off = g.add<int32_t>((size_t)b->n_req + 1, L.o_compact_stage_off);
   int32_t *status = g.add<int32_t>(2, L.o_status);
   if (g.base) {
     status[0] = status[1] = 0;
     std::fill(slot_item, slot_item + b->n_page_slots, -1);
-  }
-  // lr_compact: at most the segments and one tail of a request are displaced
-  size_t tokens = 0;
-  for (int r = 0; r < b->n_req; ++r) {
-    const int s0 = b->req_span_off[r], s1 = b->req_span_off[r + 1], base = s0 + r;
-    const int b0 = L.req_br_off[r], b1 = L.req_br_off[r + 1], tb = b0 + r;
-    size_t segs = 0, tail = 0;
-    for (int s = s0 + 1; s < s1; ++s) segs += (size_t)b->span_len[s];
-    for (int i = b0; i < b1; ++i) tail = std::max(tail, (size_t)b->br_own_len[i]);
-    if (g.base) {
-      stage_off[r] = (int32_t)tokens;
+    for (int r = 0; r < b->n_req; ++r) {
+      const int s0 = b->req_span_off[r], s1 = b->req_span_off[r + 1], base = s0 + r;
+      const int b0 = L.req_br_off[r], b1 = L.req_br_off[r + 1], tb = b0 + r;
       chain_pg[base] = chain_tok[base] = tail_pg[tb] = 0;
       for (int s = s0; s < s1; ++s) {
         const int npg = pages_of(b->span_len[s]);
@@ -169,10 +159,7 @@ static void sections(const lr_batch *b, Layout &L, Image &g) {
         std::fill(slot_item + b->br_own_slot[i], slot_item + b->br_own_slot[i] + npg, b->n_span + i);
       }
     }
-    tokens += segs + tail;
   }
-  if (g.base) stage_off[b->n_req] = (int32_t)tokens;
-  L.compact_tokens = tokens;
   tc_plan_tables(b, L.req_br_off.data(), L.span_tin.data(), L.tc, g);
 }
 
@@ -413,20 +400,11 @@ extern "C" int lr_plan_create(lr_ctx *ctx, const lr_batch *b, void *ws, size_t w
   d.chain_pg = at(L.o_chain_pg);
   d.chain_tok = at(L.o_chain_tok);
   d.tail_pg = at(L.o_tail_pg);
-  d.compact_stage_off = at(L.o_compact_stage_off);
   d.span_tin = at(L.o_span_tin);
   d.span_last = at(L.o_span_last);
   d.child_off = at(L.o_child_off);
   d.child_list = at(L.o_child_list);
   d.tree = b->seg_parent ? 1 : 0;
-  {
-    size_t off = 0;
-    auto take = [&](size_t n) { size_t o = off; off = align_up(off + n, 256); return o; };
-    p->compact.o_tok_off = take(sizeof(int32_t) * (size_t)b->n_page_slots);
-    p->compact.o_first_moved = take(sizeof(int32_t) * (size_t)b->n_req);
-    p->compact.o_staging = take(L.compact_tokens * 2 * (size_t)ctx->model.n_kv_heads * ctx->model.head_dim * 2);
-    p->compact.bytes = std::max<size_t>(off, 256);
-  }
   d.status = reinterpret_cast<int32_t *>(base + L.o_status);
   d.n_req = b->n_req;
   d.n_branch = b->n_branch;
@@ -785,7 +763,7 @@ extern "C" int lr_compact_scratch_bytes(const lr_plan *p, size_t *bytes_out) {
     set_error("lr_compact_scratch_bytes: null argument");
     return LR_EINVAL;
   }
-  *bytes_out = p->compact.bytes;
+  *bytes_out = 256;  // the tokens move in place; the argument stays in the interface
   return LR_OK;
 }
 
@@ -799,7 +777,7 @@ extern "C" int lr_compact(lr_plan *p, const int32_t *keep_off, const int32_t *ke
     set_error("lr_compact: pools must be 16-byte aligned and the scratch 256-byte aligned");
     return LR_EINVAL;
   }
-  return launch_compact(p, keep_off, keep_pages, keep_valid, k_pool, v_pool, new_len, n_pages_kept, scratch,
+  return launch_compact(p, keep_off, keep_pages, keep_valid, k_pool, v_pool, new_len, n_pages_kept,
                         reinterpret_cast<cudaStream_t>(stream));
 }
 

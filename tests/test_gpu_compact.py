@@ -3,7 +3,8 @@ import numpy as np
 import pytest
 import torch
 
-from lr_workloads import make_config, make_random_small
+from lr_workloads import Model, make_config, make_random_small
+from lr_workloads.gen import _finish
 from oracle import lr_oracle as O
 from paper_2506_19830_b200 import binding as B
 from paper_2506_19830_b200 import runner as R
@@ -61,3 +62,16 @@ def test_configs(cfg):
     rng = np.random.default_rng(cfg)
     n_accept = np.array([rng.integers(0, L + 1) for L in w.batch.br_n_draft], dtype=np.int32)
     _run_and_check(w, n_accept)
+
+
+# (requests, KV heads, head size, prefix, segments): displaced pages behind more than one step of the scan (1024 pages), a
+# first partly filled page on both sides of that line, more displaced tokens than one round holds, rows in one slice to four
+@pytest.mark.parametrize("n_req,heads,head_dim,prefix,segs", [
+    (1, 8, 128, 16384 - 5, [300, 17, 200]), (1, 1, 64, 16384, [3, 40]), (2, 1, 64, 16384 - 16, [16, 5, 700]), (1, 2, 128, 17003, [1, 1, 1]),
+    (3, 8, 64, 31, [520, 16, 16]), (20, 8, 128, 90, [33, 7]), (1, 1, 128, 3, [2100, 900])])
+def test_long_lists_and_rounds(n_req, heads, head_dim, prefix, segs):
+    rng = np.random.Generator(np.random.PCG64(prefix))
+    reqs = [{"P": prefix + 3 * r, "segs": segs, "branches": [(n, 9, 9, 8) for n in range(1, len(segs) + 1)]} for r in range(n_req)]
+    w = _finish("compact", 6, Model(heads, heads, head_dim, 16), reqs, rng, 0.5, 1.0, False, True, "nan")
+    w.tensors.verdict[:] = 1
+    _run_and_check(w, np.asarray(w.batch.br_n_draft, dtype=np.int32) - 1)
