@@ -138,6 +138,16 @@ int lr_plan_bytes(const lr_ctx *ctx, const lr_batch *batch_h, size_t *bytes_out)
  * the same plan must not overlap on the device (they share the workspace). */
 int lr_plan_create(lr_ctx *ctx, const lr_batch *batch_h, void *workspace_d, size_t workspace_bytes,
                    void *stream, lr_plan **out);
+
+/* The same in two steps, which works the plan out once where lr_plan_bytes and
+ * lr_plan_create each do it: begin validates the batch and says how large the
+ * workspace must be, finish builds and uploads the tables.  The arrays of batch_h
+ * must stay as they are until finish, which destroys the draft whatever it
+ * returns; drop destroys one that is not to be finished. */
+typedef struct lr_plan_draft lr_plan_draft;
+int lr_plan_begin(lr_ctx *ctx, const lr_batch *batch_h, size_t *bytes_out, lr_plan_draft **out);
+int lr_plan_finish(lr_plan_draft *draft, void *workspace_d, size_t workspace_bytes, void *stream, lr_plan **out);
+int lr_plan_drop(lr_plan_draft *draft);
 /* Releases the plan (not the workspace, which is the caller's).  The plan's pinned host buffer goes back to its
  * context for the next plan, so destroy every plan before its context.  Contexts and their plans are not
  * thread-safe: one thread at a time per context. */

@@ -79,6 +79,9 @@ def lib() -> C.CDLL:
             "lr_destroy": [vp],
             "lr_plan_bytes": [vp, C.POINTER(lr_batch), C.POINTER(sz)],
             "lr_plan_create": [vp, C.POINTER(lr_batch), vp, sz, vp, C.POINTER(vp)],
+            "lr_plan_begin": [vp, C.POINTER(lr_batch), C.POINTER(sz), C.POINTER(vp)],
+            "lr_plan_finish": [vp, vp, sz, vp, C.POINTER(vp)],
+            "lr_plan_drop": [vp],
             "lr_plan_destroy": [vp],
             "lr_plan_set_attention_path": [vp, C.c_int],
             "lr_plan_describe": [vp, C.POINTER(lr_plan_info)],
@@ -269,15 +272,18 @@ class Plan:
     def __init__(self, ctx: Context, batch, stream=None):
         self.ctx = ctx
         self.host = HostBatch(batch)
-        n = C.c_size_t()
-        _check(lib().lr_plan_bytes(ctx.handle, C.byref(self.host.c), C.byref(n)), "lr_plan_bytes")
-        self.workspace_bytes = n.value
-        self.workspace = torch.empty(n.value + 256, dtype=torch.uint8, device=f"cuda:{ctx.device}")
-        off = (-self.workspace.data_ptr()) % 256
-        self._ws_ptr = self.workspace.data_ptr() + off
-        h = C.c_void_p()
-        _check(lib().lr_plan_create(ctx.handle, C.byref(self.host.c), self._ws_ptr, n.value, _stream_ptr(stream), C.byref(h)),
-               "lr_plan_create")
+        n, draft, h = C.c_size_t(), C.c_void_p(), C.c_void_p()
+        _check(lib().lr_plan_begin(ctx.handle, C.byref(self.host.c), C.byref(n), C.byref(draft)), "lr_plan_begin")
+        try:
+            self.workspace_bytes = n.value
+            self.workspace = torch.empty(n.value + 256, dtype=torch.uint8, device=ctx.device)
+            start = self.workspace.data_ptr()
+            self._ws_ptr = start + (-start) % 256
+            stream = _stream_ptr(stream)
+        except BaseException:
+            lib().lr_plan_drop(draft)
+            raise
+        _check(lib().lr_plan_finish(draft, self._ws_ptr, n.value, stream, C.byref(h)), "lr_plan_finish")
         self.handle = h
         ctx._plans.add(self)
         self.n_req = self.host.c.n_req

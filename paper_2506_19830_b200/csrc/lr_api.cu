@@ -345,7 +345,39 @@ extern "C" int lr_plan_bytes(const lr_ctx *ctx, const lr_batch *b, size_t *bytes
   return LR_OK;
 }
 
-extern "C" int lr_plan_create(lr_ctx *ctx, const lr_batch *b, void *ws, size_t ws_bytes, void *stream, lr_plan **out) {
+struct lr_plan_draft {
+  lr_ctx *ctx;
+  lr_batch batch;
+  Layout layout;
+};
+
+extern "C" int lr_plan_begin(lr_ctx *ctx, const lr_batch *b, size_t *bytes_out, lr_plan_draft **out) {
+  if (!bytes_out || !out) {
+    set_error("lr_plan_begin: null argument");
+    return LR_EINVAL;
+  }
+  *out = nullptr;
+  lr_plan_draft *draft = new (std::nothrow) lr_plan_draft();
+  if (!draft) return LR_ENOMEM;
+  if (int rc = layout(ctx, b, draft->layout)) {
+    delete draft;
+    return rc;
+  }
+  draft->ctx = ctx;
+  draft->batch = *b;
+  *bytes_out = draft->layout.total_bytes;
+  *out = draft;
+  return LR_OK;
+}
+
+extern "C" int lr_plan_drop(lr_plan_draft *draft) {
+  delete draft;
+  return LR_OK;
+}
+
+static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_t ws_bytes, void *stream, lr_plan **out);
+
+static int check_workspace(const void *ws, lr_plan **out) {
   if (!out || !ws) {
     set_error("lr_plan_create: null argument");
     return LR_EINVAL;
@@ -355,8 +387,28 @@ extern "C" int lr_plan_create(lr_ctx *ctx, const lr_batch *b, void *ws, size_t w
     set_error("lr_plan_create: workspace must be 256-byte aligned");
     return LR_EINVAL;
   }
+  return LR_OK;
+}
+
+extern "C" int lr_plan_finish(lr_plan_draft *draft, void *ws, size_t ws_bytes, void *stream, lr_plan **out) {
+  if (!draft) {
+    set_error("lr_plan_finish: null draft");
+    return LR_EINVAL;
+  }
+  int rc = check_workspace(ws, out);
+  if (rc == LR_OK) rc = plan_build(draft->ctx, &draft->batch, draft->layout, ws, ws_bytes, stream, out);
+  delete draft;
+  return rc;
+}
+
+extern "C" int lr_plan_create(lr_ctx *ctx, const lr_batch *b, void *ws, size_t ws_bytes, void *stream, lr_plan **out) {
+  if (int rc = check_workspace(ws, out)) return rc;
   Layout L;
   if (int rc = layout(ctx, b, L)) return rc;
+  return plan_build(ctx, b, L, ws, ws_bytes, stream, out);
+}
+
+static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_t ws_bytes, void *stream, lr_plan **out) {
   if (ws_bytes < L.total_bytes) {
     set_error("lr_plan_create: workspace of %zu bytes, %zu needed", ws_bytes, L.total_bytes);
     return LR_ENOMEM;
