@@ -117,7 +117,7 @@ int lr_validate_batch(const lr_model *model, const lr_batch *batch_h);
 /* ---- context ------------------------------------------------------------ */
 
 /* Creates a context on CUDA device `device` (must be compute capability 10.x).
- * Allocates only host memory.  LR_EUNSUPPORTED for geometry outside the list
+ * Allocates only host memory, and a stream.  LR_EUNSUPPORTED for geometry outside the list
  * above or a non-sm_100 device. */
 int lr_create(lr_ctx **out, const lr_model *model, int device);
 int lr_destroy(lr_ctx *ctx);
@@ -379,6 +379,29 @@ int lr_commit(lr_plan *plan, const uint8_t *verdict_d, const int32_t *n_accept_d
 int lr_compact_scratch_bytes(const lr_plan *plan, size_t *bytes_out);
 int lr_compact(lr_plan *plan, const int32_t *keep_off_d, const int32_t *keep_pages_d, const int32_t *keep_valid_d,
                void *k_pool_d, void *v_pool_d, int32_t *new_len_d, int32_t *n_pages_kept_d, void *scratch_d, void *stream);
+
+/* ---- whole pass with device buffers --------------------------------------- */
+
+/* The device buffers of one pass, as the three steps take them. */
+typedef struct lr_pass_io {
+  const void *q_d, *k_pool_d, *v_pool_d;
+  void *out_d;
+  float *lse_d;                  /* nullable */
+  const void *logits_d;
+  const int32_t *draft_ids_d, *cu_draft_d;
+  int32_t *n_accept_d, *bonus_id_d;
+  int32_t *row_argmax_d;         /* nullable */
+  void *accept_scratch_d;
+  const uint8_t *verdict_d;
+  int32_t *n_steps_accepted_d, *survivor_d, *committed_len_d, *keep_off_d, *keep_pages_d, *keep_valid_d, *free_off_d, *free_pages_d;
+  int64_t logits_stride, n_rows;
+} lr_pass_io;
+
+/* lr_verify_attention, lr_accept_greedy and lr_commit in one call: everything they
+ * write is ready in the order of `stream`.  Acceptance and commit need nothing
+ * from attention and may run beside it, on side_stream if one is given, else on
+ * a stream of the plan. */
+int lr_verify_pass(lr_ctx *ctx, lr_plan *plan, const lr_pass_io *io, float softmax_scale, void *side_stream, void *stream);
 
 /* ---- whole pass with host buffers ---------------------------------------- */
 

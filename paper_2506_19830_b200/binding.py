@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 import weakref
 from typing import Optional
 
@@ -104,6 +105,7 @@ def lib() -> C.CDLL:
             "lr_compact_scratch_bytes": [vp, C.POINTER(sz)],
             "lr_compact": [vp] * 10,
             "lr_pass_staging_bytes": [vp, C.POINTER(sz)],
+            "lr_verify_pass": [vp, vp, C.c_char_p, f32, vp, vp],
             "lr_verify_pass_host": [vp, C.POINTER(lr_pass_host_io), vp, vp, vp, sz, f32, vp],
             "lr_poll_status": [vp, vp, C.POINTER(i32)],
         }
@@ -156,6 +158,9 @@ class HostBatch:
         if parent is not None:
             self.arrays["seg_parent"] = _i32(parent)
             self.c.seg_parent = _addr(self.arrays["seg_parent"])
+
+
+_PASS_IO = struct.Struct("23q").pack  # lr_pass_io
 
 
 def _model_struct(model) -> lr_model:
@@ -350,6 +355,19 @@ class Plan:
         _check(lib().lr_pass_staging_bytes(self.handle, C.byref(n)), "lr_pass_staging_bytes")
         t = torch.zeros(n.value + 256, dtype=torch.uint8, device=f"cuda:{self.ctx.device}")
         return t
+
+    def lr_verify_pass(self, ctx: Context, q, k_pool, v_pool, out, lse, logits, draft_ids, cu_draft, n_accept, bonus_id, row_argmax, accept_scratch,
+                       verdict, n_steps_accepted, survivor, committed_len, keep_off, keep_pages, keep_valid, free_off, free_pages,
+                       softmax_scale: float = 0.0, side=None, stream=None) -> None:
+        """Attention, greedy acceptance and commit in one call; ``side`` is a stream for the latter two."""
+        io = _PASS_IO(q.data_ptr(), k_pool.data_ptr(), v_pool.data_ptr(), out.data_ptr(), 0 if lse is None else lse.data_ptr(),
+                      logits.data_ptr(), draft_ids.data_ptr(), cu_draft.data_ptr(), n_accept.data_ptr(), bonus_id.data_ptr(),
+                      0 if row_argmax is None else row_argmax.data_ptr(), accept_scratch.data_ptr(), verdict.data_ptr(),
+                      n_steps_accepted.data_ptr(), survivor.data_ptr(), committed_len.data_ptr(), keep_off.data_ptr(),
+                      keep_pages.data_ptr(), keep_valid.data_ptr(), free_off.data_ptr(), free_pages.data_ptr(), logits.stride(0),
+                      logits.shape[0])
+        _check(lib().lr_verify_pass(ctx.handle, self.handle, io, softmax_scale, 0 if side is None else side.cuda_stream, _stream_ptr(stream)),
+               "lr_verify_pass")
 
     def lr_verify_pass_host(self, io: lr_pass_host_io, k_pool, v_pool, staging: torch.Tensor, softmax_scale: float = 0.0,
                             stream=None) -> None:

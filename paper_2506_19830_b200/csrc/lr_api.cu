@@ -241,6 +241,33 @@ extern "C" int lr_validate_batch(const lr_model *m, const lr_batch *b) {
   return validate_batch(b);
 }
 
+static void destroy_side(const SideStream &side) {
+  for (cudaEvent_t ev : {side.fork, side.part, side.join})
+    if (ev) cudaEventDestroy(ev);
+  if (side.s) cudaStreamDestroy(side.s);
+}
+
+static int make_side(SideStream &side) {
+  side = SideStream{};
+  cudaError_t e = cudaStreamCreateWithFlags(&side.s, cudaStreamNonBlocking);
+  for (cudaEvent_t *ev : {&side.fork, &side.part, &side.join})
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) return LR_OK;
+  destroy_side(side);
+  side = SideStream{};
+  return cuda_fail(e, "side stream");
+}
+
+// The plan's side stream: the one the context was made with, that of an earlier plan, or a new one (about 90 us).
+static int take_side(lr_plan *p) {
+  if (p->side.s) return LR_OK;
+  std::vector<SideStream> &idle = p->ctx->side_free;
+  if (idle.empty()) return make_side(p->side);
+  p->side = idle.back();
+  idle.pop_back();
+  return LR_OK;
+}
+
 // ---- context -------------------------------------------------------------------
 extern "C" int lr_create(lr_ctx **out, const lr_model *m, int device) {
   if (!out || !m) {
@@ -272,14 +299,21 @@ extern "C" int lr_create(lr_ctx **out, const lr_model *m, int device) {
   c->sm_count = sms;
   c->launches = 0;
   c->tmap_encode = nullptr;
-  c->copy_stream = nullptr;
-  c->copy_fork = c->copy_part = c->copy_join = nullptr;
   if (int rc = init_commit_kernel()) { delete c; return rc; }
   if (int rc = init_attn_tc_kernel()) { delete c; return rc; }
   if (int rc = init_attn_pair_kernel()) { delete c; return rc; }
   if (int rc = init_accept_filter_kernels()) { delete c; return rc; }
+  SideStream side;
+  if (int rc = make_side(side)) { delete c; return rc; }
+  c->side_free.push_back(side);
   *out = c;
   return LR_OK;
+}
+
+static void give_back_side(lr_plan *p) {
+  if (!p->side.s) return;
+  if (p->ctx->side_free.size() < 8) p->ctx->side_free.push_back(p->side);
+  else destroy_side(p->side);  // work still queued on it is finished all the same
 }
 
 extern "C" int lr_destroy(lr_ctx *ctx) {
@@ -289,9 +323,7 @@ extern "C" int lr_destroy(lr_ctx *ctx) {
       cudaEventDestroy(pb.uploaded);
       cudaFreeHost(pb.ptr);
     }
-    for (cudaEvent_t ev : {ctx->copy_fork, ctx->copy_part, ctx->copy_join})
-      if (ev) cudaEventDestroy(ev);
-    if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+    for (auto &side : ctx->side_free) destroy_side(side);
   }
   delete ctx;
   return LR_OK;
@@ -420,6 +452,7 @@ static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_
   p->pinned = nullptr;
   p->results_pinned = nullptr;
   p->results_pinned_cap = 0;
+  p->side = SideStream{};
   p->image_bytes = L.image_bytes;
   p->workspace_d = ws;
   p->workspace_bytes = ws_bytes;
@@ -505,6 +538,7 @@ static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_
 extern "C" int lr_plan_destroy(lr_plan *p) {
   if (!p) return LR_OK;
   if (p->pinned) give_back_pinned(p->ctx, p->pinned, p->pinned_cap, p->uploaded);
+  give_back_side(p);
   if (p->results_pinned) give_back_pinned(p->ctx, p->results_pinned, p->results_pinned_cap, p->results_copied);
   delete p;
   return LR_OK;
@@ -857,6 +891,47 @@ extern "C" int lr_poll_status(lr_plan *p, void *stream, int32_t *detail) {
   return LR_EBOUNDS;
 }
 
+// ---- whole pass on device buffers ----------------------------------------------------
+static int pass_accept_commit(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, void *stream) {
+  if (int rc = lr_accept_greedy(ctx, io->logits_d, io->logits_stride, io->draft_ids_d, io->cu_draft_d, p->dev.n_branch, io->n_rows,
+                                io->n_accept_d, io->bonus_id_d, io->row_argmax_d, io->accept_scratch_d, stream))
+    return rc;
+  return lr_commit(p, io->verdict_d, io->n_accept_d, io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d,
+                   io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d, stream);
+}
+
+extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, float scale, void *side_stream, void *stream) {
+  if (!ctx || !p || !io) {
+    set_error("lr_verify_pass: null argument");
+    return LR_EINVAL;
+  }
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), side = reinterpret_cast<cudaStream_t>(side_stream);
+  bool beside = true;
+  if (!p->side.s) {
+    // a stream cannot be made while the caller's is being captured: such a first pass stays on one stream
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (int rc = cuda_fail(cudaStreamIsCapturing(s, &capture), "cudaStreamIsCapturing")) return rc;
+    beside = capture == cudaStreamCaptureStatusNone;
+    if (beside)
+      if (int rc = take_side(p)) return rc;
+  }
+  // Attention, then acceptance and commit beside it: they fill the SMs while its last CTAs, the merge of its partial results
+  // and the gaps between launches leave them idle.  (Which of the two comes first makes no difference.)  One after another
+  // and so: the smallest request 22.6 and 19.0 us, one of 4 K tokens 36.9 and 27.2 (head size 64: 28.9 and 22.8), of 32 K
+  // 87.7 and 80.2, four of 16 K 102.4 and 91.7, trees 597 and 592.
+  cudaError_t e = beside ? cudaEventRecord(p->side.fork, s) : cudaSuccess;
+  if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
+  if (int rc = lr_verify_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, stream)) return rc;
+  if (!beside) return pass_accept_commit(ctx, p, io, stream);
+  if (!side) side = p->side.s;
+  e = cudaStreamWaitEvent(side, p->side.fork, 0);
+  if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
+  const int rc = pass_accept_commit(ctx, p, io, side);
+  e = cudaEventRecord(p->side.join, side);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->side.join, 0);
+  return rc != LR_OK ? rc : cuda_fail(e, "lr_verify_pass: join");
+}
+
 // ---- whole pass from host buffers --------------------------------------------------
 namespace {
 struct Staging {
@@ -908,17 +983,8 @@ extern "C" int lr_pass_staging_bytes(const lr_plan *p, size_t *bytes_out) {
 // 248 MB 4725 and 4685; 3 MB 126 and 131.
 constexpr size_t kAcceptInPartsBytes = 64 << 20;
 
-static int make_copy_stream(lr_ctx *ctx) {
-  if (ctx->copy_join) return LR_OK;
-  cudaError_t e = cudaSuccess;
-  if (!ctx->copy_stream) e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking);
-  for (cudaEvent_t *ev : {&ctx->copy_fork, &ctx->copy_part, &ctx->copy_join})
-    if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
-  return cuda_fail(e, "lr_verify_pass_host: copy stream");
-}
-
 // Queues the whole pass.  The logits are nearly all of what crosses the host link (188 MB against 5 MB of queries for 16
-// ragged requests), so they are uploaded on the context's copy stream while attention runs and its output goes back on the
+// ragged requests), so they are uploaded on the plan's side stream while attention runs and its output goes back on the
 // caller's.  All on one stream and so: that batch 3815 and 3570 us (the upload alone 3.5 ms), one 4 K-token request with
 // 16 MB of logits 375 and 346, with 0.2 MB 94 and 90, the smallest request 62 to 70 and 62.
 static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_pool, const void *v_pool, unsigned char *b, const Staging &L,
@@ -927,7 +993,7 @@ static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_
   const DevBatch &d = p->dev;
   const int vocab = ctx->model.vocab;
   const size_t qo = (size_t)d.n_q_rows * d.n_q_heads * d.head_dim * 2, row_bytes = (size_t)vocab * 2, logit_bytes = p->n_rows_logits * row_bytes;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), c = ctx->copy_stream;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), c = p->side.s;
   auto I = [&](size_t off) { return reinterpret_cast<int32_t *>(b + off); };
   // branches of the first part of the acceptance
   int b_part = 0;
@@ -938,13 +1004,13 @@ static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_
   cudaError_t e = cudaMemcpyAsync(b + L.q, io->q_h, qo, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && p->n_drafts) e = cudaMemcpyAsync(b + L.drafts, io->draft_ids_h, (size_t)p->n_drafts * 4, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && p->n_verdicts) e = cudaMemcpyAsync(b + L.verdict, io->verdict_h, (size_t)p->n_verdicts, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_fork, s);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(c, ctx->copy_fork, 0);
+  if (e == cudaSuccess) e = cudaEventRecord(p->side.fork, s);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(c, p->side.fork, 0);
   const unsigned char *logits_h = reinterpret_cast<const unsigned char *>(io->logits_h);
   if (e == cudaSuccess && part_bytes) e = cudaMemcpyAsync(b + L.logits, logits_h, part_bytes, cudaMemcpyHostToDevice, c);
-  if (e == cudaSuccess && part_bytes) e = cudaEventRecord(ctx->copy_part, c);
+  if (e == cudaSuccess && part_bytes) e = cudaEventRecord(p->side.part, c);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b + L.logits + part_bytes, logits_h + part_bytes, logit_bytes - part_bytes, cudaMemcpyHostToDevice, c);
-  if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_join, c);
+  if (e == cudaSuccess) e = cudaEventRecord(p->side.join, c);
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass_host: host-to-device copies");
 
   if (int rc = lr_verify_attention(p, b + L.q, k_pool, v_pool, b + L.out, nullptr, scale, stream)) return rc;
@@ -956,10 +1022,10 @@ static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_
                             I(L.n_accept) + b0, I(L.bonus) + b0, nullptr, b + L.scratch, stream);
   };
   if (part_bytes) {
-    if (int rc = cuda_fail(cudaStreamWaitEvent(s, ctx->copy_part, 0), "cudaStreamWaitEvent")) return rc;
+    if (int rc = cuda_fail(cudaStreamWaitEvent(s, p->side.part, 0), "cudaStreamWaitEvent")) return rc;
     if (int rc = accept(0, b_part, 0, part_rows)) return rc;
   }
-  if (int rc = cuda_fail(cudaStreamWaitEvent(s, ctx->copy_join, 0), "cudaStreamWaitEvent")) return rc;
+  if (int rc = cuda_fail(cudaStreamWaitEvent(s, p->side.join, 0), "cudaStreamWaitEvent")) return rc;
   if (int rc = accept(b_part, d.n_branch, part_rows, p->n_rows_logits - part_rows)) return rc;
   if (int rc = lr_commit(p, b + L.verdict, I(L.n_accept), I(L.n_steps), I(L.survivor), I(L.committed), I(L.keep_off),
                          I(L.keep_pages), I(L.keep_valid), I(L.free_off), I(L.free_pages), stream))
@@ -997,11 +1063,11 @@ extern "C" int lr_verify_pass_host(lr_plan *p, const lr_pass_host_io *io, const 
   const size_t small_bytes = L.scratch - L.n_accept;
   if (p->results_pinned_cap < small_bytes)
     if (int rc = take_pinned(p->ctx, small_bytes, &p->results_pinned, &p->results_pinned_cap, &p->results_copied)) return rc;
-  if (int rc = make_copy_stream(p->ctx)) return rc;
+  if (int rc = take_side(p)) return rc;
   if (int issued = issue_pass_host(p, io, k_pool, v_pool, b, L, scale, stream)) {
     // whatever was queued beside the caller's stream still comes before what the caller does next
-    cudaEventRecord(p->ctx->copy_join, p->ctx->copy_stream);
-    cudaStreamWaitEvent(reinterpret_cast<cudaStream_t>(stream), p->ctx->copy_join, 0);
+    cudaEventRecord(p->side.join, p->side.s);
+    cudaStreamWaitEvent(reinterpret_cast<cudaStream_t>(stream), p->side.join, 0);
     return issued;
   }
   const int rc = lr_poll_status(p, stream, nullptr);  // waits for the stream

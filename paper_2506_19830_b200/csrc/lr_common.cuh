@@ -146,6 +146,15 @@ struct DevPairPlan {
 
 }  // namespace lr
 
+namespace lr {
+// A second stream beside the caller's and the events that order the two.  One per plan (whose passes never overlap), so
+// that passes of different plans on different streams do not wait for one another.
+struct SideStream {
+  cudaStream_t s;
+  cudaEvent_t fork, part, join;
+};
+}  // namespace lr
+
 struct lr_ctx {
   lr_model model;
   int device;
@@ -158,9 +167,7 @@ struct lr_ctx {
   // far more than building a plan.  `uploaded` is recorded after the buffer's last upload; a new user waits on it.
   struct PinnedBuf { void *ptr; size_t cap; cudaEvent_t uploaded; };
   std::vector<PinnedBuf> pinned_free;
-  // lr_verify_pass_host uploads the logits here, beside the caller's stream (made on first use; idle between calls)
-  cudaStream_t copy_stream;
-  cudaEvent_t copy_fork, copy_part, copy_join;
+  std::vector<lr::SideStream> side_free;  // of destroyed plans, kept for the next one
 };
 
 struct lr_plan {
@@ -189,6 +196,7 @@ struct lr_plan {
   void *results_pinned;   // pinned bounce buffer for the integer results of lr_verify_pass_host (taken on first use)
   size_t results_pinned_cap;
   cudaEvent_t results_copied;
+  lr::SideStream side;    // taken on the first pass that needs one
   cudaEvent_t uploaded;   // recorded after the image's upload
   size_t image_bytes;
   void *workspace_d;

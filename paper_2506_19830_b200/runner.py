@@ -66,8 +66,6 @@ class PassOutputs:
         self.keep_pages = torch.full((batch.n_page_slots,), -1, **i32)
         self.keep_valid = torch.full((batch.n_page_slots,), -1, **i32)
         self.free_pages = torch.full((batch.n_page_slots,), -1, **i32)
-        # one pass at a time writes these buffers, so the events that order its two streams are kept with them
-        self.fork, self.join = torch.cuda.Event(), torch.cuda.Event()
 
     def commit_dict(self):
         d = {k: getattr(self, k).cpu().numpy() for k in
@@ -78,12 +76,10 @@ class PassOutputs:
 
 
 def run_pass(ctx: B.Context, plan: B.Plan, x: DeviceInputs, y: PassOutputs, stream=None, want_lse=True, want_row_argmax=True):
-    """One whole verify pass on device-resident inputs (three kernel launches)."""
-    plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out, y.lse if want_lse else None, 0.0, stream)
-    ctx.lr_accept_greedy(x.logits, x.draft_ids, x.cu_draft, y.n_accept, y.bonus_id, y.scratch,
-                         y.row_argmax if want_row_argmax else None, stream)
-    plan.lr_commit(x.verdict, y.n_accept, y.n_steps_accepted, y.survivor, y.committed_len, y.keep_off, y.keep_pages,
-                   y.keep_valid, y.free_off, y.free_pages, stream)
+    """One whole verify pass on device-resident inputs; its results are ready in the order of ``stream``."""
+    plan.lr_verify_pass(ctx, x.q, x.k_pool, x.v_pool, y.out, y.lse if want_lse else None, x.logits, x.draft_ids, x.cu_draft, y.n_accept,
+                        y.bonus_id, y.row_argmax if want_row_argmax else None, y.scratch, x.verdict, y.n_steps_accepted, y.survivor,
+                        y.committed_len, y.keep_off, y.keep_pages, y.keep_valid, y.free_off, y.free_pages, 0.0, None, stream)
 
 
 def run_pass_overlapped(ctx: B.Context, plan: B.Plan, x: DeviceInputs, y: PassOutputs, side: torch.cuda.Stream,
@@ -91,15 +87,7 @@ def run_pass_overlapped(ctx: B.Context, plan: B.Plan, x: DeviceInputs, y: PassOu
     """One whole verify pass with the two independent chains on two streams: attention on the current
     stream, acceptance -> commit (which need nothing from attention) on ``side``; both are joined back
     into the current stream.  Works under CUDA-graph capture (fork/join through events)."""
-    main = torch.cuda.current_stream()
-    k_pool = x.k_pool if k_pool is None else k_pool
-    v_pool = x.v_pool if v_pool is None else v_pool
-    logits = x.logits if logits is None else logits
-    y.fork.record(main)
-    side.wait_event(y.fork)
-    ctx.lr_accept_greedy(logits, x.draft_ids, x.cu_draft, y.n_accept, y.bonus_id, y.scratch, None, side)
-    plan.lr_commit(x.verdict, y.n_accept, y.n_steps_accepted, y.survivor, y.committed_len, y.keep_off, y.keep_pages,
-                   y.keep_valid, y.free_off, y.free_pages, side)
-    y.join.record(side)
-    plan.lr_verify_attention(x.q, k_pool, v_pool, y.out, None, 0.0, main)
-    main.wait_event(y.join)
+    plan.lr_verify_pass(ctx, x.q, x.k_pool if k_pool is None else k_pool, x.v_pool if v_pool is None else v_pool, y.out, None,
+                        x.logits if logits is None else logits, x.draft_ids, x.cu_draft, y.n_accept, y.bonus_id, None, y.scratch,
+                        x.verdict, y.n_steps_accepted, y.survivor, y.committed_len, y.keep_off, y.keep_pages, y.keep_valid, y.free_off,
+                        y.free_pages, 0.0, side, None)
