@@ -2,11 +2,14 @@
 //
 // Two kernels.  accept_stats_kernel streams the bf16 logits once -- the HBM-bound part: a warp takes one chunk of a row
 // at a time (2048 logits, or the next power-of-two multiple that leaves at most kMaxChunks chunks) and leaves the pair
-// (raw maximum M_c, S_c = sum exp((x - M_c) / T)).  accept_sample_kernel, one CTA per branch, combines the pairs of a row in chunk order into (m, Z), gets
-// P_i(d_i) = exp((x_d - m) / T) / Z for the drafts, walks the acceptance chain u_i < P_i(d_i), and draws the
-// final token by inverse CDF over the stop row with the rejected token removed: first over the chunk
-// weights S_c exp((M_c - m) / T) (no second pass over the row), then inside the one chunk that holds the
-// target, which is read again and prefix-summed.  Every reduction has a fixed order: same inputs, same output.
+// (raw maximum M_c, S_c = sum exp((x - M_c) / T)).  accept_sample_kernel, one CTA per branch, combines the pairs of a row
+// into (m, Z), gets P_i(d_i) = exp((x_d - m) / T) / Z for the drafts, walks the acceptance chain u_i < P_i(d_i), and draws
+// the final token by inverse CDF over the stop row with the rejected token removed: first over the chunk weights
+// S_c exp((M_c - m) / T) (no second pass over the row), then inside the one chunk that holds the target, which is read
+// again and prefix-summed.  Every reduction has a fixed order: same inputs, same output.  The second kernel is a chain of
+// latencies (about 10 us behind the first, half of it instruction fetch); what does not depend on the statistics it reads
+// while the first one drains, one butterfly sums a row and one scan finds the chunk: 617 rows, both and the commit 51.7 ->
+// 49.9 us.
 #include <algorithm>
 
 #include "lr_common.cuh"
@@ -142,9 +145,10 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   __shared__ int s_pick_chunk, s_pick_thread;
   __shared__ float s_pick_before;
   const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the statistics come from the kernel launched just before
+  // Only the statistics come from the kernel launched just before, and that kernel let this one start when everything older
+  // had finished: all else is fetched while it drains.
   const int32_t d0 = cu_draft[b], L = cu_draft[b + 1] - d0, r0 = d0 + b;
-  const float u_fin = u_final[b];  // fetched early: needed only after the chain
+  const float u_fin = u_final[b];
   static_assert(kRowBatch == 32, "the chain uses one lane per row of a batch");
 
   // ---- acceptance chain, kRowBatch rows at a time.  Everything a batch needs from global memory (the chunk
@@ -157,8 +161,6 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   for (;; i0 += kRowBatch) {
     const int rows = min(kRowBatch, L + 1 - i0);
     __syncthreads();
-    const float2 *src = stats + (int64_t)(r0 + i0) * n_chunks;  // consecutive rows are contiguous
-    for (int idx = tid; idx < rows * n_chunks; idx += kThreads) s_st[idx] = src[idx];
     if (tid < rows) {
       const int i = i0 + tid;
       int32_t dtok = -1;
@@ -173,6 +175,10 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       s_xd[tid] = xd;
       s_u[tid] = u;
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // lr_commit's grid may be set up meanwhile
+    const float2 *src = stats + (int64_t)(r0 + i0) * n_chunks;  // consecutive rows are contiguous
+    for (int idx = tid; idx < rows * n_chunks; idx += kThreads) s_st[idx] = src[idx];
     __syncthreads();
     for (int k = warp; k < rows; k += kThreads / 32) {  // one warp per row combines the row's chunk pairs in order
       const float2 *st = s_st + k * n_chunks;
@@ -181,17 +187,12 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
       float z = 0.f;
-      for (int c0 = 0; c0 < n_chunks; c0 += 32) {  // chunk order: 32 at a time, butterfly inside
-        const int c = c0 + lane;
-        float t = 0.f;
-        if (c < n_chunks) {
-          const float2 v = st[c];
-          if (v.y > 0.f) t = v.y * exp2f((v.x - m) * k_log2);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-        z += t;
+      for (int c = lane; c < n_chunks; c += 32) {
+        const float2 v = st[c];
+        if (v.y > 0.f) z += v.y * exp2f((v.x - m) * k_log2);
       }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
       if (lane == 0) {
         const float p = (s_tok[k] >= 0 && z > 0.f) ? exp2f((s_xd[k] - m) * k_log2) / z : 0.f;
         if (p_draft != nullptr && i0 + k < L) p_draft[d0 + i0 + k] = p;
@@ -230,37 +231,37 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
       if (c == dead_chunk) w = fmaxf(w - w_dead, 0.f);
       return w;
     };
-    float total = 0.f;
-    for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-      float t = weight(c0 + lane);
+    constexpr int kSteps = kMaxChunks / 32;
+    float w[kSteps], t[kSteps], total = 0.f;  // of the chunks c0 + lane: weight, inclusive sum over all chunks so far
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float y = __shfl_up_sync(0xFFFFFFFFu, t, o);
-        if (lane >= o) t += y;
+    for (int k = 0; k < kSteps; ++k) t[k] = w[k] = weight(k * 32 + lane);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+      for (int k = 0; k < kSteps; ++k) {
+        const float y = __shfl_up_sync(0xFFFFFFFFu, t[k], o);
+        if (lane >= o) t[k] += y;
       }
-      total += __shfl_sync(0xFFFFFFFFu, t, 31);
+    }
+#pragma unroll
+    for (int k = 0; k < kSteps; ++k) {
+      const float base = total;
+      total += __shfl_sync(0xFFFFFFFFu, t[k], 31);
+      t[k] += base;
     }
     const float target = u_fin * total;
-    float base = 0.f;
     int pick = -1, last_nonzero = 0;
     float before = 0.f;
-    for (int c0 = 0; c0 < n_chunks && pick < 0; c0 += 32) {
-      const float w = weight(c0 + lane);
-      float t = w;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float y = __shfl_up_sync(0xFFFFFFFFu, t, o);
-        if (lane >= o) t += y;
-      }
-      const unsigned nz = __ballot_sync(0xFFFFFFFFu, w > 0.f);
-      if (nz != 0u) last_nonzero = c0 + 31 - __clz(nz);
-      const unsigned hit = __ballot_sync(0xFFFFFFFFu, w > 0.f && base + t > target);
-      if (hit != 0u) {
+    for (int k = 0; k < kSteps; ++k) {
+      const unsigned nz = __ballot_sync(0xFFFFFFFFu, w[k] > 0.f), hit = __ballot_sync(0xFFFFFFFFu, w[k] > 0.f && t[k] > target);
+      if (nz != 0u) last_nonzero = k * 32 + 31 - __clz(nz);
+      const float less = t[k] - w[k];
+      if (hit != 0u && pick < 0) {
         const int l = __ffs(hit) - 1;
-        pick = c0 + l;
-        before = base + __shfl_sync(0xFFFFFFFFu, t - w, l);
+        pick = k * 32 + l;
+        before = __shfl_sync(0xFFFFFFFFu, less, l);
       }
-      base += __shfl_sync(0xFFFFFFFFu, t, 31);
     }
     if (pick < 0) {  // rounding pushed the target past the last chunk: take the last chunk with any weight
       pick = last_nonzero;
