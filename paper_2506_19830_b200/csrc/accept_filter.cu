@@ -46,6 +46,7 @@ constexpr int kListOut = 256;       // kept tokens that go out as a list
 constexpr int kKeyWords = 8;        // words of group maxima a thread of filter_cut_kernel keeps in registers
 constexpr int kSelMax = 1024;       // largest top_k the candidates serve
 constexpr int kSelTopP = 128;       // leading tokens to look for when top-k is off
+constexpr int kProbeRows = 16;      // rows the candidates are tried on first when top-k is off
 constexpr int kWT = 512;            // threads of a CTA of filter_window_kernel
 constexpr int kAT = 512;            // ... of accept_filtered_kernel
 constexpr int kSlicesInFlight = 5;  // slices a warp of it works on at a time: one round for 163840 tokens and 8 CTAs
@@ -158,12 +159,18 @@ __device__ __forceinline__ uint4 ragged_vec(const uint16_t *rp, int32_t n_vec, i
 template <bool kSum, int kGV>
 __global__ void __launch_bounds__(kT, kScanCtasPerSm)
 filter_scan_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, uint32_t n_chunks, uint32_t total,
-                   uint16_t *__restrict__ group_max, float2 *__restrict__ stats, int32_t *__restrict__ n_open) {
+                   uint16_t *__restrict__ group_max, float2 *__restrict__ stats, int32_t *n_open, int n_probe, int32_t *__restrict__ gave_up) {
   const int lane = threadIdx.x & 31;
   const int32_t n_vec = vocab >> 3, rem = vocab & 7;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the logits may come from the kernel launched just before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (blockIdx.x == 0 && threadIdx.x == 0) *n_open = 0;
+  if (gave_up == nullptr) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_open = 0;
+  } else {  // the rows behind the probe: not worth reading when it left most of its rows open
+    const bool skip = 2 * *n_open > n_probe;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *gave_up = skip;
+    if (skip) return;
+  }
   for (uint32_t unit = blockIdx.x * kWarps + (threadIdx.x >> 5); unit < total; unit += gridDim.x * kWarps) {
     const uint32_t row = unit / n_chunks;
     const uint16_t *rp = logits + (int64_t)row * row_stride;
@@ -238,18 +245,23 @@ template <int kGV>
 __global__ void __launch_bounds__(kT)
 filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, int32_t top_k, float top_p, int k_sel,
                   int n_chunks, const uint16_t *__restrict__ group_max, const float2 *__restrict__ stats, RowCut *__restrict__ cuts,
-                  u64 *__restrict__ lists, int32_t *__restrict__ n_kept_out, int32_t *__restrict__ n_open, int32_t *__restrict__ open_rows) {
+                  u64 *__restrict__ lists, int32_t *__restrict__ n_kept_out, int32_t *__restrict__ n_open, int32_t *__restrict__ open_rows,
+                  int row0, const int32_t *__restrict__ gave_up) {
   __shared__ u64 s_cand[kListCap], s_sorted[kListCap], s_cum[kListCap];
   __shared__ int s_grp[kGroupCap];
   __shared__ int s_n, s_n_grp, s_cnt[2][kWarps], s_kept;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t row = blockIdx.x;
+  const int64_t row = row0 + (int)blockIdx.x;
   constexpr int kPerChunk = 32 * kVec / kGV;
   const int n_words = n_chunks * kPerChunk / 2;
   const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
   if (tid == 0) s_n = s_n_grp = 0;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the maxima come from the kernel launched just before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (gave_up != nullptr && *gave_up != 0) {
+    if (tid == 0) open_rows[atomicAdd(n_open, 1)] = (int32_t)row;
+    return;
+  }
   const uint32_t *src = reinterpret_cast<const uint32_t *>(group_max + row * n_chunks * kPerChunk);
   uint32_t g2[kKeyWords];  // word i of the thread is word i * kT + tid of the row
 #pragma unroll
@@ -472,7 +484,7 @@ template <int kC>
 __global__ void __launch_bounds__(kWT, 2)
 filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, int32_t top_k, float top_p,
                      RowCut *__restrict__ cuts, int32_t *__restrict__ n_kept_out, const int32_t *__restrict__ n_open,
-                     const int32_t *__restrict__ open_rows, int n_all, int cached) {
+                     const int32_t *__restrict__ open_rows, int n_all, int cached, int n_min, int n_max) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   WindowShared &sh = *reinterpret_cast<WindowShared *>(smem_raw);
   uint16_t *s_row = reinterpret_cast<uint16_t *>(smem_raw + (sizeof(WindowShared) + 15) / 16 * 16);
@@ -491,6 +503,7 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int n_rows = n_all > 0 ? n_all : *n_open;
+  if (n_rows < n_min || n_rows > n_max) return;  // another cluster size takes this many rows
   int ph = 0;
 
   auto peer = [&](int r) -> const Xch * { return kC == 1 ? &sh.xch[ph] : cluster.map_shared_rank(&sh.xch[ph], r); };
@@ -1034,7 +1047,7 @@ ScratchLayout filter_layout(int32_t vocab, int32_t n_rows) {
   s.lists = take((size_t)n_rows * kListOut * sizeof(u64));
   s.maxima = take((size_t)n_rows * s.n_chunks * 32 * kVec * sizeof(uint16_t));
   s.stats = take((size_t)n_rows * s.n_chunks * sizeof(float2));
-  s.open = take(((size_t)n_rows + 1) * sizeof(int32_t));
+  s.open = take(((size_t)n_rows + 2) * sizeof(int32_t));  // how many, which, and whether the probe gave up
   s.bytes = off;
   return s;
 }
@@ -1049,6 +1062,14 @@ struct WindowShape {
 // are us per CTA and per 1000 tokens of its share, fitted to measured rounds of rows with one CTA on every SM and with two
 // (rows of 152064 tokens: 14.5 us for 17 by clusters of eight, 27 for 51 by fours, 38 for 74 by fours, 59 for 136 by pairs, 80
 // for 296 by single CTAs, which have no cluster barriers; of 32000: 15 us for 68 by single CTAs, 23 by pairs, 21 for 296).
+double window_us(const lr_ctx *ctx, int c, int64_t n_rows) {
+  const int64_t clusters = std::max(1, ctx->sm_count * 2 / c);
+  const double k = share_of(ctx->model.vocab, c) * 1e-3;
+  const double one = c == 1 ? 6 + 0.42 * k : c == 2 ? 19 + 0.22 * k : c == 4 ? 14 + 0.2 * k : 11 + 0.18 * k;
+  const double two = c == 1 ? 7 + 0.48 * k : c == 2 ? 22 + 0.5 * k : c == 4 ? 20 + 0.47 * k : 17 + 0.55 * k;
+  const double full = std::min(1.0, std::max(0.0, (double)(n_rows * c - ctx->sm_count) / ctx->sm_count));
+  return (double)((n_rows + clusters - 1) / clusters) * (one + full * (two - one));
+}
 WindowShape window_shape(const lr_ctx *ctx, int64_t n_rows) {
   WindowShape best = {};
   for (const int c : {8, 4, 2, 1}) {
@@ -1057,12 +1078,7 @@ WindowShape window_shape(const lr_ctx *ctx, int64_t n_rows) {
     w.cluster = c;
     w.cached = fixed + share <= kWindowSmemMax;
     w.smem = fixed + (w.cached ? share : 0);
-    const int64_t clusters = std::max(1, ctx->sm_count * 2 / c);
-    const double k = share_of(ctx->model.vocab, c) * 1e-3;
-    const double one = c == 1 ? 6 + 0.42 * k : c == 2 ? 19 + 0.22 * k : c == 4 ? 14 + 0.2 * k : 11 + 0.18 * k;
-    const double two = c == 1 ? 7 + 0.48 * k : c == 2 ? 22 + 0.5 * k : c == 4 ? 20 + 0.47 * k : 17 + 0.55 * k;
-    const double full = std::min(1.0, std::max(0.0, (double)(n_rows * c - ctx->sm_count) / ctx->sm_count));
-    w.us = (double)((n_rows + clusters - 1) / clusters) * (one + full * (two - one));
+    w.us = window_us(ctx, c, n_rows);
     if (best.cluster == 0 || w.us < best.us) best = w;
   }
   return best;
@@ -1121,39 +1137,74 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
   // Can a few leading tokens decide a row?  With a small top-k always: 17 us against 28 us through the windows for 51 rows
   // of 152064 tokens and top-k 20, 46 against 213 for 612.  Reading and ranking the groups of a larger one costs about 0.1 us
   // per k.  With top-p alone they mostly do, but the rows they leave open (taken to be one in five) go through the windows
-  // all the same: 137 us against 213 for 612 rows, 59 against 50 for 136.
+  // all the same, and when a kept set is half the vocabulary that is every row.  So they are tried on a few rows first and,
+  // if most of those stay open, on no more.  Rows of 152064 tokens, peaked, as a language model's, flat: 408 of them 89,
+  // 152 and 191 us (tried on all at once 61, 122 and 231; windows alone about 175), 612 of them 105, 175 and 281 (75, 142 and
+  // 340), 136 of them 50, 61 and 62 (42, 61 and 156).
   WindowShape w = window_shape(ctx, n_rows);
   const WindowShape w_open = window_shape(ctx, (n_rows + 4) / 5);
   const double us_scan = (double)n_rows * vocab * 2 / 5.5e6;
+  const int n_probe = !by_k && n_rows >= 4 * kProbeRows ? kProbeRows : 0;
   const double us_candidates = by_k ? 12.0 + us_scan + (6.0 + 0.1 * top_k) * ((n_rows + 5 * ctx->sm_count - 1) / (5 * ctx->sm_count))
-                                    : 24.0 + us_scan + 0.02 * n_rows + w_open.us;
+                                    : 24.0 + (n_probe ? 12.0 : 0.0) + us_scan + 0.02 * n_rows + w_open.us;
   const bool candidates = enough && (by_k ? top_k <= kSelMax : by_p) && ((by_k && top_k <= 128) || us_candidates < w.us);
+  // The open rows are few or all of them; only the device knows.  Up to n_few rows take the shape for a few.
+  WindowShape few = w;
+  int n_few = n_rows;
   if (candidates) {
     auto scan = by_k ? (wide ? filter_scan_kernel<false, kVec> : filter_scan_kernel<false, 1>)
                      : (wide ? filter_scan_kernel<true, kVec> : filter_scan_kernel<true, 1>);
-    const uint32_t total = (uint32_t)n_rows * L.n_chunks;
-    const unsigned grid = std::min((total + kWarps - 1) / kWarps, (uint32_t)(ctx->sm_count * kScanCtasPerSm));
-    scan<<<grid, kT, 0, s>>>(lg, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, maxima, stats, n_open);
-    ctx->launches++;
-    if (int rc = cuda_fail(cudaGetLastError(), "filter_scan_kernel launch")) return rc;
-    ctx->launches++;
-    if (int rc = cuda_fail(launch_dependent(wide ? filter_cut_kernel<kVec> : filter_cut_kernel<1>, dim3((unsigned)n_rows), dim3(kT),
-                                            0, s, lg, stride, vocab, k_log2, top_k, top_p, k_sel, L.n_chunks, maxima, stats, cuts, lists, n_kept,
-                                            n_open, n_open + 1),
-                           "filter_cut_kernel launch"))
-      return rc;
-    w = by_k ? window_shape(ctx, 1) : w_open;  // after a top-k hardly ever a row is left
+    auto cut = wide ? filter_cut_kernel<kVec> : filter_cut_kernel<1>;
+    int32_t *gave_up = n_open + 1 + n_rows;
+    const int64_t maxima_per_row = (int64_t)L.n_chunks * 32 * kVec / (wide ? kVec : 1);
+    auto settle = [&](int r0, int n, int32_t *verdict) -> int {
+      const uint32_t total = (uint32_t)n * L.n_chunks;
+      const unsigned grid = std::min((total + kWarps - 1) / kWarps, (uint32_t)(ctx->sm_count * kScanCtasPerSm));
+      ctx->launches += 2;
+      const uint16_t *from = lg + (int64_t)r0 * stride;
+      uint16_t *to = maxima + r0 * maxima_per_row;
+      float2 *to_stats = stats + (int64_t)r0 * L.n_chunks;
+      if (verdict) {
+        if (int rc = cuda_fail(launch_dependent(scan, dim3(grid), dim3(kT), 0, s, from, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, to,
+                                                to_stats, n_open, kProbeRows, verdict),
+                               "filter_scan_kernel launch"))
+          return rc;
+      } else {
+        scan<<<grid, kT, 0, s>>>(from, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, to, to_stats, n_open, kProbeRows, verdict);
+        if (int rc = cuda_fail(cudaGetLastError(), "filter_scan_kernel launch")) return rc;
+      }
+      return cuda_fail(launch_dependent(cut, dim3((unsigned)n), dim3(kT), 0, s, lg, stride, vocab, k_log2, top_k, top_p, k_sel, L.n_chunks, maxima,
+                                        stats, cuts, lists, n_kept, n_open, n_open + 1, r0, (const int32_t *)verdict),
+                       "filter_cut_kernel launch");
+    };
+    if (n_probe)
+      if (int rc = settle(0, n_probe, nullptr)) return rc;
+    if (int rc = settle(n_probe, n_rows - n_probe, n_probe ? gave_up : nullptr)) return rc;
+    few = by_k ? window_shape(ctx, 1) : w_open;  // after a top-k hardly ever a row is left
+    if (n_probe && few.cluster != w.cluster) {
+      int lo = (n_rows + 4) / 5, hi = n_rows;  // `few` is the better one at lo, w at hi
+      while (hi - lo > 1) {
+        const int mid = lo + (hi - lo) / 2;
+        if (window_us(ctx, few.cluster, mid) <= window_us(ctx, w.cluster, mid)) lo = mid;
+        else hi = mid;
+      }
+      n_few = lo;
+    }
   }
-  ctx->launches++;
-  auto window = w.cluster == 8   ? filter_window_kernel<8>
-                : w.cluster == 4 ? filter_window_kernel<4>
-                : w.cluster == 2 ? filter_window_kernel<2>
-                                 : filter_window_kernel<1>;
-  const int clusters = std::max(1, ctx->sm_count * 2 / w.cluster);
-  if (int rc = cuda_fail(launch_clusters(window, w.cluster, candidates ? clusters : std::min(n_rows, clusters), kWT, w.smem, s, lg, stride, vocab,
-                                         k_log2, top_k, top_p, cuts, n_kept, n_open, n_open + 1, candidates ? 0 : n_rows, w.cached ? 1 : 0),
-                         "filter_window_kernel launch"))
-    return rc;
+  auto windows = [&](const WindowShape &shape, int n_min, int n_max) -> int {
+    auto kernel = shape.cluster == 8   ? filter_window_kernel<8>
+                  : shape.cluster == 4 ? filter_window_kernel<4>
+                  : shape.cluster == 2 ? filter_window_kernel<2>
+                                       : filter_window_kernel<1>;
+    const int clusters = std::max(1, ctx->sm_count * 2 / shape.cluster);
+    ctx->launches++;
+    return cuda_fail(launch_clusters(kernel, shape.cluster, candidates ? clusters : std::min(n_rows, clusters), kWT, shape.smem, s, lg, stride, vocab,
+                                     k_log2, top_k, top_p, cuts, n_kept, n_open, n_open + 1, candidates ? 0 : n_rows, shape.cached ? 1 : 0, n_min, n_max),
+                     "filter_window_kernel launch");
+  };
+  if (int rc = windows(few, 0, n_few)) return rc;
+  if (n_few < n_rows)
+    if (int rc = windows(w, n_few + 1, n_rows)) return rc;
   ctx->launches++;
   // one CTA per branch when there is no stop row to walk (hardly ever after the candidates of a small top-k) or it is short
   if ((candidates && by_k && top_k <= kListOut) || vocab <= 16384)

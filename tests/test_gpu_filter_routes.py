@@ -51,3 +51,27 @@ def test_routes(vocab, nb, L, top_k, top_p):
     # the checker's 4e-5 of the step in one row of four.  A branch looks at two rows or so, one in four of them flat, and
     # draws differ on a few more: 0.4 of the branches leaves room for twice the expected number.
     _check(bits, drafts, cu, 0.8, top_k, top_p, ua, uf, got, max_ambiguous_frac=0.4, rows_to_check=rows)
+
+
+# Top-p alone over many rows: the candidates are tried on 16 of them first.  Which rows are flat -- none, all, those tried
+# only, those behind only -- decides whether the rest is tried and by which windows the open rows go.
+@pytest.mark.parametrize("flat", ["none", "all", "first", "rest", "mixed"])
+def test_probe(flat):
+    vocab, nb, L = 40009, 150, 3
+    n_rows = nb * (L + 1)
+    rng = np.random.default_rng(len(flat))
+    x = rng.standard_normal((n_rows, vocab), dtype=np.float32)
+    lead = rng.integers(0, vocab, n_rows)
+    r = np.arange(n_rows)
+    peaked = {"none": r >= 0, "all": r < 0, "first": r >= 16, "rest": r < 16, "mixed": r % 2 == 0}[flat]
+    x[r[peaked], lead[peaked]] = 18.0
+    bits = bf16_round(x)
+    cu = (np.arange(nb + 1) * L).astype(np.int32)
+    drafts = lead.reshape(nb, L + 1)[:, :L].reshape(-1).astype(np.int32).copy()
+    ua, uf = rng.uniform(0, 1, len(drafts)), rng.uniform(0, 1, nb)
+    ua[::3] = 0.0
+    got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, 0.8, 0, 0.93, ua, uf)
+    rows = sorted({0, 15, 16, 17, n_rows - 1} | set(rng.integers(0, n_rows, 12).tolist()))
+    # A flat row keeps some 25000 tokens, the last one with 1e-5 of their mass: nearly every draw from one lies within the
+    # checker's 4e-5 of a step, so that all branches may be undecided by it; the kept counts and masses are checked all the same.
+    _check(bits, drafts, cu, 0.8, 0, 0.93, ua, uf, got, max_ambiguous_frac=1.0, rows_to_check=rows)
