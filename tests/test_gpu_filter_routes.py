@@ -48,7 +48,7 @@ def test_routes(vocab, nb, L, top_k, top_p):
     got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, 0.8, top_k, top_p, ua, uf)
     rows = None if n_rows * vocab < 3e6 else sorted(set(rng.integers(0, n_rows, 12).tolist()))
     # A flat row of 40009 tokens keeps some 2000 at top_p 0.6, the last with 1.5e-4 of their mass: above HEAVY, and within
-    # the checker's 4e-5 of the step in one row of four.  A branch looks at two rows or so, one in four of them flat, and
+    # the rule's 4e-5 of the step in one row of four.  A branch looks at two rows or so, one in four of them flat, and
     # draws differ on a few more: 0.4 of the branches leaves room for twice the expected number.
     _check(bits, drafts, cu, 0.8, top_k, top_p, ua, uf, got, max_ambiguous_frac=0.4, rows_to_check=rows)
 
@@ -73,5 +73,5 @@ def test_probe(flat):
     got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, 0.8, 0, 0.93, ua, uf)
     rows = sorted({0, 15, 16, 17, n_rows - 1} | set(rng.integers(0, n_rows, 12).tolist()))
     # A flat row keeps some 25000 tokens, the last one with 1e-5 of their mass: nearly every draw from one lies within the
-    # checker's 4e-5 of a step, so that all branches may be undecided by it; the kept counts and masses are checked all the same.
+    # rule's 4e-5 of a step, so that all branches may be undecided by it; the kept counts and masses are checked all the same.
     _check(bits, drafts, cu, 0.8, 0, 0.93, ua, uf, got, max_ambiguous_frac=1.0, rows_to_check=rows)
