@@ -50,12 +50,13 @@
 //               bf16 P written back over S.  A barrier test costs a warp over 100 cycles
 //               even when it succeeds, so the sweep makes one per 64 keys, under the
 //               exponentials (with two, in line: 85 us against 81 for four 16 K-token requests).
-// Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 fp32 columns each; P_s
-// occupies the first 64 columns of S_s.
+// Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 fp32 columns each.  The
+// weights of a 64-key half take the first 32 of the 64 columns its scores held
+// (head size 64: all 64 for two terms; the third lies behind O, which needs 64).
 //
 // Head size 64.  The same kernel with half as many channels (struct Shape).  The CUDA-core kernel served this size before
 // and keeps the shapes the page tables here cannot describe; on one request of 4 K tokens, 3 branches of 16 drafts, 32
-// query and 8 KV heads it takes 724 us, this kernel and its merge 17 us (B200; the bytes alone: 2.7 us).
+// query and 8 KV heads it takes 724 us, this kernel and its merge 18.5 us (B200; the bytes alone: 2.7 us).
 //
 // Visibility.  Tiles made only of full prefix pages need no mask.  In every other
 // tile each page carries (valid tokens, first and last node number that sees it,
@@ -94,10 +95,12 @@ struct Shape {
   static constexpr int kGroupBytes = kHalves * kAtomBytes;  // the atoms of one 8-key group
   static constexpr int kStages = kD == 128 ? 5 : 10;
   static constexpr int kSmemBytes = 2 * kTileBytes + kStages * kTileBytes + 2048;  // tiles, then Ctrl; the base must be 1024-aligned
-  // Head size 64 sends the softmax weights to the tensor core as two bf16 terms (value and remainder: 2^-17 of a
-  // weight instead of 2^-9), as precise as the fp32 weights of the CUDA-core kernel that used to serve it.  The second
-  // product is affordable there: its N is 64, and the sweep waits for the softmax, not for the tensor pipe.
-  static constexpr bool kSplitP = kD == 64;
+  // Head size 64 sends the softmax weights to the tensor core as three bf16 terms, whose sum is the fp32 weight itself:
+  // as precise as the CUDA-core kernel that used to serve it.  The two further products are affordable there: their N is
+  // 64.  Two terms (2^-17 of a weight lost) put four times as many outputs on the other side of a rounding step as fp32
+  // weights do, 0.2 % against 0.05 %; they took 16.6 us where three take 18.5 (one request of 4 K tokens), 67.6 and 75.8 (of
+  // 32 K), 119 and 137 (16 ragged requests).
+  static constexpr int kTermsP = kD == 64 ? 3 : 1;
 };
 constexpr int kPagesPerTile = 8;
 constexpr uint64_t kDrainLimitNs = 50ull * 1000ull * 1000ull;
@@ -244,8 +247,8 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_st64(uint32_t taddr, const uint32_t (&r)[64]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x64.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63, %64};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(r[32]), "r"(r[33]), "r"(r[34]), "r"(r[35]), "r"(r[36]), "r"(r[37]), "r"(r[38]), "r"(r[39]), "r"(r[40]), "r"(r[41]), "r"(r[42]), "r"(r[43]), "r"(r[44]), "r"(r[45]), "r"(r[46]), "r"(r[47]), "r"(r[48]), "r"(r[49]), "r"(r[50]), "r"(r[51]), "r"(r[52]), "r"(r[53]), "r"(r[54]), "r"(r[55]), "r"(r[56]), "r"(r[57]), "r"(r[58]), "r"(r[59]), "r"(r[60]), "r"(r[61]), "r"(r[62]), "r"(r[63])
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
                : "memory");
 }
 
@@ -393,45 +396,35 @@ __device__ __forceinline__ float max_half(const uint32_t (&v)[64]) {
   }
   return fmaxf(fmaxf(a, b), fmaxf(c, e));
 }
-// Four weights -> two packed bf16 pairs at pk[at], pk[at + 1]; with kSplit also what bf16 leaves of them at pk[32 + at] ..
-template <bool kSplit>
-__device__ __forceinline__ void pack_weights(float2 y0, float2 y1, uint32_t (&pk)[kSplit ? 64 : 32], int at) {
-  pk[at] = pack_bf16(y0.x, y0.y);
-  pk[at + 1] = pack_bf16(y1.x, y1.y);
-  if constexpr (kSplit) {
+// The weights of a half as they go to tensor memory, 16 columns (32 weights) at a time, so that no more than these sit in
+// registers beside the scores (which a redo needs again).  Column c of a term holds the weights 2c and 2c + 1.  With three
+// terms each is the leading eight bits of what the terms before it leave: cut off, not rounded, which takes one
+// instruction for two weights, and the third has nothing left to cut.
+template <int kTerms>
+struct WeightOut {
+  uint32_t pk[kTerms][16];
+  uint32_t addr[kTerms];
+  __device__ __forceinline__ void add(float2 y, int c) {
+    if constexpr (kTerms == 1) {
+      pk[0][c & 15] = pack_bf16(y.x, y.y);
+    } else {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const float2 y = i ? y1 : y0;
-      const uint32_t h = pk[at + i];
-      pk[32 + at + i] = pack_bf16(y.x - bits_f(h << 16), y.y - bits_f(h & 0xFFFF0000u));
+      for (int t = 0; t < kTerms; ++t) {
+        const uint32_t x0 = __float_as_uint(y.x), x1 = __float_as_uint(y.y);
+        pk[t][c & 15] = __byte_perm(x0, x1, 0x7632);
+        if (t + 1 < kTerms) y = fadd2(y, make_float2(-bits_f(x0 & 0xFFFF0000u), -bits_f(x1 & 0xFFFF0000u)));
+      }
     }
-  }
-}
-// P = exp2(scale * s - m) for 64 scores -> packed bf16 pairs; returns the fp32 sum
-template <bool kSplit>
-__device__ __forceinline__ float exp_half(const uint32_t (&v)[64], uint32_t (&pk)[kSplit ? 64 : 32], float scale_log2, float neg_m) {
-  const float2 sc = make_float2(scale_log2, scale_log2), nm = make_float2(neg_m, neg_m);
-  float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+    if ((c & 15) == 15)
 #pragma unroll
-  for (int i = 0; i < 64; i += 4) {
-    float2 y0 = ffma2(make_float2(bits_f(v[i]), bits_f(v[i + 1])), sc, nm);
-    float2 y1 = ffma2(make_float2(bits_f(v[i + 2]), bits_f(v[i + 3])), sc, nm);
-    y0.x = ex2(y0.x);
-    y0.y = ex2(y0.y);
-    y1.x = ex2(y1.x);
-    y1.y = ex2(y1.y);
-    acc0 = fadd2(acc0, y0);
-    acc1 = fadd2(acc1, y1);
-    pack_weights<kSplit>(y0, y1, pk, i >> 1);
+      for (int t = 0; t < kTerms; ++t) tmem_st16(addr[t] + (c & 16), pk[t]);
   }
-  acc0 = fadd2(acc0, acc1);
-  return acc0.x + acc0.y;
-}
+};
 
-// exp_half on v, and beside it (in the shadow of the MUFU) the maximum of the raw scores
-template <bool kSplit>
-__device__ __forceinline__ float exp_half_max(const uint32_t (&v)[64], uint32_t (&pk)[kSplit ? 64 : 32], float scale_log2, float neg_m,
-                                              float &raw_max) {
+// P = exp2(scale * s - m) for 64 scores, out to tensor memory; returns the fp32 sum.  With kMax also (in the shadow of the
+// MUFU) the maximum of the raw scores.
+template <int kTerms, bool kMax>
+__device__ __forceinline__ float exp_half(const uint32_t (&v)[64], WeightOut<kTerms> &out, float scale_log2, float neg_m, float &raw_max) {
   const float2 sc = make_float2(scale_log2, scale_log2), nm = make_float2(neg_m, neg_m);
   float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
   float m0 = -INFINITY, m1 = -INFINITY;
@@ -439,17 +432,18 @@ __device__ __forceinline__ float exp_half_max(const uint32_t (&v)[64], uint32_t 
   for (int i = 0; i < 64; i += 4) {
     float2 y0 = ffma2(make_float2(bits_f(v[i]), bits_f(v[i + 1])), sc, nm);
     float2 y1 = ffma2(make_float2(bits_f(v[i + 2]), bits_f(v[i + 3])), sc, nm);
-    m0 = max3(m0, bits_f(v[i]), bits_f(v[i + 1]));
+    if (kMax) m0 = max3(m0, bits_f(v[i]), bits_f(v[i + 1]));
     y0.x = ex2(y0.x);
     y0.y = ex2(y0.y);
-    m1 = max3(m1, bits_f(v[i + 2]), bits_f(v[i + 3]));
+    if (kMax) m1 = max3(m1, bits_f(v[i + 2]), bits_f(v[i + 3]));
     y1.x = ex2(y1.x);
     y1.y = ex2(y1.y);
     acc0 = fadd2(acc0, y0);
     acc1 = fadd2(acc1, y1);
-    pack_weights<kSplit>(y0, y1, pk, i >> 1);
+    out.add(y0, i >> 1);
+    out.add(y1, (i >> 1) + 1);
   }
-  raw_max = fmaxf(m0, m1);
+  if (kMax) raw_max = fmaxf(m0, m1);
   acc0 = fadd2(acc0, acc1);
   return acc0.x + acc0.y;
 }
@@ -697,10 +691,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
 #pragma unroll
       for (int k4 = 0; k4 < 4; ++k4)
         mma_ts(o_tmem, s_tmem + half * 64 + k4 * 8, b + (uint64_t)(k4 * (2 * kGroupBytes >> 4)), kIdescPV<kD>, acc || k4 != 0);
-      if constexpr (Sh::kSplitP)
+#pragma unroll
+      for (int term = 1; term < Sh::kTermsP; ++term)
 #pragma unroll
         for (int k4 = 0; k4 < 4; ++k4)
-          mma_ts(o_tmem, s_tmem + half * 64 + 32 + k4 * 8, b + (uint64_t)(k4 * (2 * kGroupBytes >> 4)), kIdescPV<kD>, 1u);
+          mma_ts(o_tmem, (term == 1 ? s_tmem + half * 64 + 32 : o_tmem + 64 + half * 32) + k4 * 8, b + (uint64_t)(k4 * (2 * kGroupBytes >> 4)),
+                 kIdescPV<kD>, 1u);
     };
     for (int pc = piece0; pc < piece1 && ok; ++pc, ++pc_idx) {
       const TcPiece pi = pc == piece0 ? head->first : tc.pieces[pc];
@@ -925,14 +921,18 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
               ok = rescale_o(alpha, g);
               if (!ok) break;
             }
-            uint32_t pk[Sh::kSplitP ? 64 : 32];
-            float sum = 0.f, mx;
+            WeightOut<Sh::kTermsP> weights;
+            weights.addr[0] = sh_addr;
+            if constexpr (Sh::kTermsP == 3) {
+              weights.addr[1] = sh_addr + 32;
+              weights.addr[2] = o_addr + 64 + half * 32;
+            }
+            float sum = 0.f, mx, raw;
             // Fast path: exponentials against the running reference exponent; the maximum of the 64 scores is
             // computed beside them and only checked afterwards.
             bool fast = __all_sync(0xFFFFFFFFu, m_used > -INFINITY);
             if (fast) {
-              float raw;
-              sum = exp_half_max<Sh::kSplitP>(v, pk, scale_log2, -m_used, raw);
+              sum = exp_half<Sh::kTermsP, true>(v, weights, scale_log2, -m_used, raw);
               mx = raw * scale_log2;
               if (__any_sync(0xFFFFFFFFu, mx > m_used + kRedoThreshold)) fast = false;  // could overflow: redo exactly
             } else {
@@ -953,14 +953,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
                   if (!ok) break;
                 }
               }
-              sum = exp_half<Sh::kSplitP>(v, pk, scale_log2, (m_used == -INFINITY) ? 0.f : -m_used);
+              tc_wait_st();
+              sum = exp_half<Sh::kTermsP, false>(v, weights, scale_log2, (m_used == -INFINITY) ? 0.f : -m_used, raw);
             } else if (mx > m_used + kRescaleThreshold) {
               pend = true;
               m_new = mx;
             }
             l += sum;
-            if constexpr (Sh::kSplitP) tmem_st64(sh_addr, pk);
-            else tmem_st32(sh_addr, pk);
             tc_wait_st();
             tc_fence_before();
             s_ready = __all_sync(0xFFFFFFFFu, next_ready) != 0;

@@ -35,8 +35,8 @@ def test_split_keys(args):
 
 
 def test_weights_are_not_rounded_to_bf16():
-    """Two bf16 terms per weight leave 2^-17 of it, so the output's own rounding (at most 2^-9 of every value) is all
-    that is left to see in the 2-norm; bf16 weights alone would add 1.6e-3 to it."""
+    """Several bf16 terms per weight leave at most 2^-17 of it, so the output's own rounding (at most 2^-9 of every value) is
+    all that is left to see in the 2-norm; bf16 weights alone would add 1.6e-3 to it."""
     w = _chain(5, 16, 4, 1500, 3, 16)
     b, t = w.batch, w.tensors
     ctx = B.Context(b.model, 0)
@@ -49,3 +49,26 @@ def test_weights_are_not_rounded_to_bf16():
     got = y.out.to(torch.float64).cpu().numpy()
     assert np.linalg.norm(got - ref) <= (2.0 ** -9 + 2.0 ** -15) * np.linalg.norm(ref)
     ctx.close()
+
+
+def test_weights_keep_their_fp32_bits():
+    """The weights go to the tensor core as three bf16 terms that add up to the fp32 weight, so the kernel's only errors are
+    those of fp32 sums (some 2^-21 of a value) and the rounding of the output.  An output is not the closest bf16 when
+    the former carry it over the middle between two neighbours: twice 2^-21 / 2^-9, 5e-4 of them.  Two terms would leave
+    2^-17 of a weight and 2e-3 of the outputs."""
+    off, total = 0, 0
+    for args in [(1, 16, 4, 2500, 3, 16), (2, 5, 1, 600, 4, 9), (3, 8, 8, 111, 2, 7, 3), (4, 32, 8, 256, 3, 16, 2)]:
+        w = _chain(*args)
+        b, t = w.batch, w.tensors
+        ctx = B.Context(b.model, 0)
+        plan = B.Plan(ctx, b)
+        assert plan.lr_plan_describe()["uses_tensor_core"] == 1  # the automatic choice
+        x, y = R.DeviceInputs(b, t), R.PassOutputs(b)
+        plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out)
+        assert plan.lr_poll_status() == 0
+        ref, _ = O.verify_attention(b, t.q, t.k_pool, t.v_pool)
+        got = y.out.to(torch.float64).cpu().numpy()
+        closest = torch.from_numpy(ref).to(torch.bfloat16).to(torch.float64).numpy()
+        off, total = off + int((closest != got).sum()), total + got.size
+        ctx.close()
+    assert off <= 1e-3 * total, off / total
