@@ -53,9 +53,12 @@ constexpr int kSlicesInFlight = 5;  // slices a warp of it works on at a time: o
 constexpr int kWin = 8192;          // keys per window
 constexpr int kMaxSlices = 1024;    // slices a row is cut into for the draw
 constexpr size_t kWindowSmemMax = 112 * 1024;  // two CTAs per SM
-// Relative distance between the fp32 sum of a row's masses and their integer sum: the argument of an exponential is
-// rounded at magnitude 40 (2^-19.4 absolute: 1e-6 of the mass), ex2.approx is good to 2^-22 on both sides, an fp32 sum of
-// 64 terms and some 30 further additions to 5e-6, rounding masses to 2^-40 of the largest to 1e-7; rounded up.
+// Relative distance between the fp32 sum of a row's masses and their integer sum.  A token below the 2^-40th of the row's
+// largest mass has none, so every argument that matters lies within 40 of 0, whatever the logits and the temperature: it is
+// a difference scaled, rounded twice (2^-18.7 absolute, 1.7e-6 of the mass), on the way from the lane to its chunk and from
+// there to the row twice more, and once in the integer masses (5.1e-6 together); ex2.approx is good to 2^-22 each time
+// (1e-6), an fp32 sum of 64 terms and some 30 further additions to 5e-6, rounding masses to 2^-40 of the largest to 1e-7;
+// rounded up.
 constexpr double kMassEps = 2e-5;
 typedef unsigned long long u64;
 constexpr int32_t kNoKey = INT32_MIN;
@@ -213,19 +216,20 @@ filter_scan_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int3
       group_max[(int64_t)unit * (32 * kVec / kGV) + (k0 / kGV) * 32 + lane] = (uint16_t)(__float_as_uint(g) >> 16);
     }
     if (kSum) {
-      const float off = top > -INFINITY ? -top * k_log2 : 0.f;
+      // subtracted before it is scaled: top * k_log2 would be rounded at its own magnitude, for all terms alike
+      const float ref = top > -INFINITY ? top : 0.f;
       float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
       for (int i = 0; i < kVec * 4; i += 2) {
-        a0 += ex2_approx(fmaf(lo_f(x[i]), k_log2, off));
-        a1 += ex2_approx(fmaf(hi_f(x[i]), k_log2, off));
-        a2 += ex2_approx(fmaf(lo_f(x[i + 1]), k_log2, off));
-        a3 += ex2_approx(fmaf(hi_f(x[i + 1]), k_log2, off));
+        a0 += ex2_approx((lo_f(x[i]) - ref) * k_log2);
+        a1 += ex2_approx((hi_f(x[i]) - ref) * k_log2);
+        a2 += ex2_approx((lo_f(x[i + 1]) - ref) * k_log2);
+        a3 += ex2_approx((hi_f(x[i + 1]) - ref) * k_log2);
       }
       float M = top;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
-      float S = ((a0 + a1) + (a2 + a3)) * ex2_approx(fmaf(top, k_log2, M > -INFINITY ? -M * k_log2 : 0.f));
+      float S = ((a0 + a1) + (a2 + a3)) * ex2_approx((top - (M > -INFINITY ? M : 0.f)) * k_log2);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
       if (lane == 0) stats[unit] = make_float2(M, S);

@@ -2,8 +2,11 @@
 left over by the candidates, cluster sizes, rows in and out of shared memory -- by the rule of test_gpu_accept_filtered."""
 import numpy as np
 import pytest
+import torch
 
 from lr_workloads import Model, bf16_round
+from paper_2506_19830_b200 import binding as B
+from paper_2506_19830_b200 import runner as R
 from test_gpu_accept_filtered import _check, _run
 
 pytestmark = pytest.mark.gpu
@@ -75,3 +78,44 @@ def test_probe(flat):
     # A flat row keeps some 25000 tokens, the last one with 1e-5 of their mass: nearly every draw from one lies within the
     # rule's 4e-5 of a step, so that all branches may be undecided by it; the kept counts and masses are checked all the same.
     _check(bits, drafts, cu, 0.8, 0, 0.93, ua, uf, got, max_ambiguous_frac=1.0, rows_to_check=rows)
+
+
+# Which route a row takes depends on how many rows the call has; what comes out must not.  Low temperatures and offsets make
+# the scaled logits large, equal leaders put top_p next to a step of the cumulative mass (0.94999 of 20 equal tokens: 19
+# are kept, by a margin of 1e-5).
+@pytest.mark.parametrize("T,offset,top_p", [(0.05, 0.0, 0.94999), (0.1, 0.0, 0.94999), (0.1, 0.0, 0.9), (0.6, 0.0, 0.94999), (0.6, 250.0, 0.94999),
+                                            (0.6, -1000.0, 0.94999), (1.0, 1000.0, 0.94999)])
+def test_routes_agree(T, offset, top_p):
+    vocab, nb, L, part = 152064, 102, 3, 3
+    n_rows = nb * (L + 1)
+    rng = np.random.default_rng(int(abs(offset) + 100 * T))
+    x = rng.standard_normal((n_rows, vocab), dtype=np.float32) * np.float32(1.5 * min(T, 0.6) / 0.6)
+    lead = rng.integers(0, vocab // 20, n_rows)
+    for r in range(n_rows):
+        n = (20, 1, 20, 4, 20, 19)[r % 6]
+        x[r, lead[r] + vocab // 20 * np.arange(n)] = rng.uniform(18, 60)
+    bits = bf16_round(x + np.float32(offset))
+    cu = (np.arange(nb + 1) * L).astype(np.int32)
+    drafts = lead.reshape(nb, L + 1)[:, :L].reshape(-1).astype(np.int32).copy()
+    ua, uf = rng.uniform(0, 1, len(drafts)), rng.uniform(0, 1, nb)
+    ua[::3] = 0.0
+    lg = R.bf16_tensor(bits, "cuda:0")
+    ctx = B.Context(Model(1, 1, 64, vocab), 0)
+
+    def call(b0, b1):
+        r, d = slice(b0 * (L + 1), b1 * (L + 1)), slice(b0 * L, b1 * L)
+        t = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a, dtype=dt)).to("cuda:0")  # noqa: E731
+        out = [torch.full((n,), -7, dtype=dt, device="cuda:0") for n, dt in ((b1 - b0, torch.int32), (b1 - b0, torch.int32), ((b1 - b0) * L, torch.float32),
+                                                                           ((b1 - b0) * (L + 1), torch.int32))]
+        before = ctx.launch_count
+        ctx.lr_accept_sample_filtered(lg[r], t(drafts[d], np.int32), t(cu[: b1 - b0 + 1], np.int32), T, 0, top_p, t(ua[d], np.float32),
+                                      t(uf[b0:b1], np.float32), out[0], out[1], ctx.accept_sample_filtered_scratch((b1 - b0) * (L + 1)), out[2], out[3])
+        return [o.cpu().numpy() for o in out], ctx.launch_count - before
+
+    many, n_many = call(0, nb)
+    for b in range(0, nb, part):
+        few, n_few = call(b, b + part)
+        assert n_few < n_many  # windows alone
+        for name, a, e, size in zip(("n_accept", "final_id", "p_draft", "n_kept"), many, few, (1, 1, L, L + 1)):
+            assert np.array_equal(a[b * size: (b + part) * size], e), (name, b)
+    ctx.close()
