@@ -190,8 +190,10 @@ int lr_plan_describe(const lr_plan *plan, lr_plan_info *info_out);
 
 /* Selects the attention implementation for later lr_verify_attention calls on
  * this plan: 0 = automatic (tensor-core path when the shape allows it), 1 =
- * force the CUDA-core path (every shape), 2 = force the tensor-core path
- * (LR_EUNSUPPORTED later if the shape does not allow it).  For testing. */
+ * force the CUDA-core path (every shape), 2 = force the tensor-core path, 3 =
+ * force the CTA-pair tensor-core path (LR_EUNSUPPORTED later if the shape does
+ * not allow it).  The first selection of 3 on a plan uploads that path's tables
+ * and waits for them.  For testing. */
 int lr_plan_set_attention_path(lr_plan *plan, int path);
 
 /* Test hook for the device-side bounds checks: overwrites the physical page id of page slot `page_slot`

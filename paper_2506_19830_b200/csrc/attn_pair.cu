@@ -1231,19 +1231,17 @@ int pair_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *re
   out.o_reqs = add(reqs.data(), reqs.size() * sizeof(TcReq));
   if (targets.empty()) targets.push_back(TcTarget{});  // keep the section non-empty
   out.o_targets = add(targets.data(), targets.size() * sizeof(TcTarget));
-  // scratch behind the image: ticket counters (zeroed at upload, left zero by every launch), (exponent, sum) pairs,
-  // fp32 partial outputs
-  out.s_counters = 0;
-  out.scratch_zero_bytes = ((size_t)std::max(1, out.n_targets) * sizeof(uint32_t) + 255) / 256 * 256;
-  out.s_ml = out.scratch_zero_bytes;
-  out.s_o = out.s_ml + ((size_t)n_slots * 128 * 2 * sizeof(float) + 255) / 256 * 256;
+  const std::vector<uint32_t> zeros((size_t)std::max(1, out.n_targets), 0u);
+  out.o_counters = add(zeros.data(), zeros.size() * sizeof(uint32_t));
+  out.s_ml = 0;
+  out.s_o = ((size_t)n_slots * 128 * 2 * sizeof(float) + 255) / 256 * 256;
   out.scratch_bytes = out.s_o + (size_t)n_slots * 128 * kD * sizeof(float);
   return LR_OK;
 }
 
-size_t pair_bytes_bound(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off) {
+PairBytes pair_bytes_bound(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off) {
   const lr_model &m = ctx->model;
-  if (m.head_dim != kD) return 0;
+  if (m.head_dim != kD) return {0, 0};
   const int T = 128 / (m.n_q_heads / m.n_kv_heads);
   int64_t lists = 0, pages = 0;
   for (int r = 0; r < b->n_req; ++r) {
@@ -1256,12 +1254,15 @@ size_t pair_bytes_bound(const lr_ctx *ctx, const lr_batch *b, const int32_t *req
   }
   // every pair beyond the first adds at most one piece; every piece at most two partial results
   const int64_t groups = lists * m.n_kv_heads, pairs = std::max(1, ctx->sm_count / 2), pieces = groups + pairs;
-  const int64_t bytes[] = {pairs * (int64_t)sizeof(PrHead), pages * (int64_t)sizeof(TcPage), std::max(1, b->cu_q[b->n_branch]) * (int64_t)sizeof(TcRow),
-                           pieces * (int64_t)sizeof(PrPiece), (lists + 1) * (int64_t)sizeof(TcReq), (2 * groups + 1) * (int64_t)sizeof(TcTarget),
-                           (2 * groups + 1) * 4, 2 * pieces * 128 * 8, 2 * pieces * 128 * kD * 4};
-  size_t total = 0;
-  for (const int64_t n : bytes) total += (size_t)(n + 255) / 256 * 256;
-  return total;
+  auto total = [](std::initializer_list<int64_t> sections) {
+    size_t sum = 0;
+    for (const int64_t n : sections) sum += (size_t)(n + 255) / 256 * 256;
+    return sum;
+  };
+  return {total({pairs * (int64_t)sizeof(PrHead), pages * (int64_t)sizeof(TcPage), std::max(1, b->cu_q[b->n_branch]) * (int64_t)sizeof(TcRow),
+                 pieces * (int64_t)sizeof(PrPiece), (lists + 1) * (int64_t)sizeof(TcReq), (2 * groups + 1) * (int64_t)sizeof(TcTarget),
+                 (2 * groups + 1) * (int64_t)sizeof(uint32_t)}),
+          total({2 * pieces * 128 * 2 * (int64_t)sizeof(float), 2 * pieces * 128 * kD * (int64_t)sizeof(float)})};
 }
 
 void pair_bind_device_plan(const PairHostPlan &h, unsigned char *image_base, unsigned char *scratch_base, lr_plan *p) {
@@ -1282,7 +1283,7 @@ void pair_bind_device_plan(const PairHostPlan &h, unsigned char *image_base, uns
   t.tokens_per_mtile = h.tokens_per_mtile;
   t.wait_limit_us = 1000000u;  // one second per wait, measured on the global timer
   t.phantom_tx_bytes = 0;
-  t.counters = reinterpret_cast<uint32_t *>(scratch_base + h.s_counters);
+  t.counters = reinterpret_cast<uint32_t *>(image_base + h.o_counters);
   t.partial_ml = reinterpret_cast<float *>(scratch_base + h.s_ml);
   t.partial_o = reinterpret_cast<float *>(scratch_base + h.s_o);
 }

@@ -113,7 +113,7 @@ struct Layout {
       o_span_tin, o_span_last, o_child_off, o_child_list;
   std::vector<int32_t> cu_draft, req_br_off, span_tin, span_last, child_off, child_list;
   TcHostPlan tc;
-  size_t image_bytes, region_bytes, total_bytes;
+  size_t image_bytes, pair_cap, scratch_cap, total_bytes;
 };
 
 static void sections(const lr_batch *b, Layout &L, Image &g) {
@@ -209,8 +209,10 @@ static int layout(const lr_ctx *ctx, const lr_batch *b, Layout &L) {
   Image sizes;
   sections(b, L, sizes);
   L.image_bytes = align_up(sizes.bytes, 256);
-  L.region_bytes = align_up(std::max(L.tc.scratch_bytes, pair_bytes_bound(ctx, b, L.req_br_off.data())), 256);
-  L.total_bytes = L.image_bytes + L.region_bytes;
+  const PairBytes pair = pair_bytes_bound(ctx, b, L.req_br_off.data());
+  L.pair_cap = align_up(pair.image, 256);
+  L.scratch_cap = align_up(std::max(L.tc.scratch_bytes, pair.scratch), 256);
+  L.total_bytes = L.image_bytes + L.pair_cap + L.scratch_cap;
   return LR_OK;
 }
 
@@ -408,6 +410,8 @@ extern "C" int lr_plan_drop(lr_plan_draft *draft) {
 }
 
 static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_t ws_bytes, void *stream, lr_plan **out);
+static int build_pair(lr_plan *p);
+static cudaError_t queue_pair_upload(lr_plan *p, cudaStream_t s);
 
 static int check_workspace(const void *ws, lr_plan **out) {
   if (!out || !ws) {
@@ -505,12 +509,14 @@ static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_
   p->n_drafts = L.cu_draft[b->n_branch];
   p->n_rows_logits = p->n_drafts + b->n_branch;
   p->n_verdicts = b->n_span - b->n_req;
-  tc_bind_device_plan(L.tc, base, base + L.image_bytes, p);
-  p->pair_ok = p->pair_built = p->pair_upload = false;
+  p->pair_off = L.image_bytes;
+  p->pair_cap = L.pair_cap;
+  p->scratch_off = L.image_bytes + L.pair_cap;
+  p->scratch_cap = L.scratch_cap;
+  tc_bind_device_plan(L.tc, base, base + p->scratch_off, p);
+  p->pair_ok = p->pair_built = false;
   memset(&p->pr, 0, sizeof(p->pr));
   p->pr.wait_limit_us = p->tc.wait_limit_us = 1000000u;  // one second per wait
-  p->region_off = L.image_bytes;
-  p->region_bytes = L.region_bytes;
   p->o_req_span_off = L.o_req_span_off;
   p->o_span_len = L.o_span_len;
   p->o_span_slot = L.o_span_slot;
@@ -526,6 +532,13 @@ static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemcpyAsync(ws, p->pinned, L.image_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaEventRecord(p->uploaded, s);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (e == cudaSuccess) e = cudaStreamIsCapturing(s, &capture);
+  // a captured upload has to bring the CTA-pair tables along: nothing tells when it will have run
+  if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone && build_pair(p) == LR_OK) {
+    if (p->pair_ok) e = queue_pair_upload(p, s);
+    p->pair_built = true;
+  }
   if (e != cudaSuccess) {
     give_back_pinned(ctx, p->pinned, p->pinned_cap, p->uploaded);
     delete p;
@@ -567,20 +580,36 @@ static int build_pair(lr_plan *p) {
   PairHostPlan h;
   p->pr_image.clear();
   if (int rc = pair_build_host_plan(p->ctx, &b, at(p->o_req_br_off), at(p->o_span_tin), at(p->o_span_last), h, p->pr_image)) return rc;
-  const size_t scratch = align_up(p->pr_image.size(), 256);
-  if (h.ok && scratch + h.scratch_bytes > p->region_bytes) {
-    set_error("lr_plan_set_attention_path: the CTA-pair plan needs %zu bytes of workspace, %zu are set aside", scratch + h.scratch_bytes, p->region_bytes);
+  if (h.ok && (p->pr_image.size() > p->pair_cap || h.scratch_bytes > p->scratch_cap)) {
+    set_error("lr_plan_set_attention_path: the CTA-pair plan needs %zu and %zu bytes of workspace, %zu and %zu are set aside", p->pr_image.size(),
+              h.scratch_bytes, p->pair_cap, p->scratch_cap);
     return LR_ENOMEM;
   }
-  unsigned char *region = reinterpret_cast<unsigned char *>(p->workspace_d) + p->region_off;
+  unsigned char *ws = reinterpret_cast<unsigned char *>(p->workspace_d);
   const uint32_t wait_limit_us = p->pr.wait_limit_us, phantom = p->pr.phantom_tx_bytes;
-  pair_bind_device_plan(h, region, region + scratch, p);
+  pair_bind_device_plan(h, ws + p->pair_off, ws + p->scratch_off, p);
   p->pr.wait_limit_us = wait_limit_us;
   p->pr.phantom_tx_bytes = phantom;
-  p->pr_zero_off = scratch + h.s_counters;
-  p->pr_zero_bytes = h.scratch_zero_bytes;
-  p->pair_built = true;
   return LR_OK;
+}
+
+static cudaError_t queue_pair_upload(lr_plan *p, cudaStream_t s) {
+  return cudaMemcpyAsync(reinterpret_cast<unsigned char *>(p->workspace_d) + p->pair_off, p->pr_image.data(), p->pr_image.size(), cudaMemcpyHostToDevice, s);
+}
+
+// Uploads the tables on a stream of their own, behind the plan's image (before which the workspace may still be another's), and
+// waits: whatever launches the path later, on whichever stream and captured or not, finds them.
+static int upload_pair(lr_plan *p) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // the caller may be capturing: none of this is part of it
+  if (int rc = cuda_fail(cudaThreadExchangeStreamCaptureMode(&mode), "cudaThreadExchangeStreamCaptureMode")) return rc;
+  int rc = cuda_fail(cudaEventSynchronize(p->uploaded), "cudaEventSynchronize(plan image)");
+  cudaStream_t own = nullptr;
+  if (rc == LR_OK) rc = cuda_fail(cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking), "cudaStreamCreate");
+  if (rc == LR_OK) rc = cuda_fail(queue_pair_upload(p, own), "CTA-pair plan upload");
+  if (rc == LR_OK) rc = cuda_fail(cudaStreamSynchronize(own), "CTA-pair plan upload");
+  if (own) cudaStreamDestroy(own);
+  const cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  return rc != LR_OK ? rc : cuda_fail(e, "cudaThreadExchangeStreamCaptureMode");
 }
 
 extern "C" int lr_plan_set_attention_path(lr_plan *p, int path) {
@@ -588,10 +617,11 @@ extern "C" int lr_plan_set_attention_path(lr_plan *p, int path) {
     set_error("lr_plan_set_attention_path: bad argument");
     return LR_EINVAL;
   }
-  if (path == 3) {
-    if (!p->pair_built)
-      if (int rc = build_pair(p)) return rc;
-    p->pair_upload = true;  // another path may have used the region meanwhile
+  if (path == 3 && !p->pair_built) {
+    if (int rc = build_pair(p)) return rc;
+    if (p->pair_ok)
+      if (int rc = upload_pair(p)) return rc;
+    p->pair_built = true;
   }
   p->attention_path = path;
   return LR_OK;
@@ -665,11 +695,11 @@ extern "C" int lr_plan_debug_set_page(lr_plan *p, int32_t page_slot, int32_t new
   for (int c = 0; c < p->n_tc_heads; ++c)
     for (int k = 0; k < 32; ++k)
       if (heads[c].first_pages[k] == old_id && heads[c].piece1 > heads[c].piece0) heads[c].first_pages[k] = new_id;
+  cudaError_t e = cudaMemcpyAsync(p->workspace_d, p->pinned, p->image_bytes, cudaMemcpyHostToDevice, s);
   if (p->pair_built) {
     if (int rc = build_pair(p)) return rc;
-    p->pair_upload = true;
+    if (e == cudaSuccess && p->pair_ok) e = queue_pair_upload(p, s);
   }
-  cudaError_t e = cudaMemcpyAsync(p->workspace_d, p->pinned, p->image_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaEventRecord(p->uploaded, s);
   return cuda_fail(e, "lr_plan_debug_set_page upload");
 }
@@ -691,13 +721,6 @@ extern "C" int lr_verify_attention(lr_plan *p, const void *q, const void *k, con
     if (!p->pair_ok) {
       set_error("lr_verify_attention: the CTA-pair tensor-core path does not support this shape");
       return LR_EUNSUPPORTED;
-    }
-    if (p->pair_upload) {
-      unsigned char *region = reinterpret_cast<unsigned char *>(p->workspace_d) + p->region_off;
-      cudaError_t e = cudaMemcpyAsync(region, p->pr_image.data(), p->pr_image.size(), cudaMemcpyHostToDevice, s);
-      if (e == cudaSuccess) e = cudaMemsetAsync(region + p->pr_zero_off, 0, p->pr_zero_bytes, s);
-      if (e != cudaSuccess) return cuda_fail(e, "CTA-pair plan upload");
-      p->pair_upload = false;
     }
     return launch_attn_pair(p, q, k, v, out, lse, scale, s);
   }

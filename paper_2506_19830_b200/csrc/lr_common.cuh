@@ -176,14 +176,14 @@ struct lr_plan {
   lr::DevTcPlan tc;
   lr::DevPairPlan pr;
   bool tc_ok;             // shape allows the tensor-core path
-  // The CTA-pair plan is built when its path is selected.  Its image and scratch lie over the single-CTA path's scratch
-  // (the two never run at the same time), so every selection uploads the image again.
+  // The CTA-pair plan is built and uploaded when its path is first selected.  Its tables have a part of the workspace to
+  // themselves, so that launches that were captured or queued find them whatever has run since; partial results share
+  // theirs with the single-CTA path's (the two never run at the same time).
   bool pair_ok;           // shape allows the CTA-pair tensor-core path (known once built)
-  bool pair_built, pair_upload;  // ... upload before the next launch
+  bool pair_built;        // ... and uploaded
   int pr_pieces, pr_partial_slots;
-  size_t pr_zero_off, pr_zero_bytes;  // ticket counters, relative to the region
   std::vector<unsigned char> pr_image;
-  size_t region_off, region_bytes;    // behind the image in the workspace
+  size_t pair_off, pair_cap, scratch_off, scratch_cap;  // behind the image in the workspace: those tables, partial results
   size_t o_req_span_off, o_span_len, o_span_slot, o_br_req, o_br_depth, o_br_own_len, o_br_own_slot, o_br_n_draft, o_cu_q, o_req_br_off,
       o_span_tin, o_span_last;        // batch tables in the image
   int attention_path;     // 0 auto, 1 generic, 2 tensor core (single CTA), 3 tensor core (CTA pairs)
@@ -262,14 +262,16 @@ struct PairHostPlan {
   bool ok = false;
   size_t o_heads = 0, o_pages = 0, o_rows = 0, o_pieces = 0, o_reqs = 0, o_targets = 0;  // image offsets
   int n_pairs = 0, n_targets = 0, n_pieces = 0, n_partial_slots = 0, tokens_per_mtile = 0, n_pages = 0;
-  // scratch region behind the image: ticket counters, (exponent, sum) pairs, fp32 partial outputs
-  size_t s_counters = 0, s_ml = 0, s_o = 0, scratch_bytes = 0, scratch_zero_bytes = 0;
+  size_t o_counters = 0;  // in the image as zeros, left zero by every launch
+  // scratch region: (exponent, sum) pairs, fp32 partial outputs
+  size_t s_ml = 0, s_o = 0, scratch_bytes = 0;
 };
 // Builds the plan and its image (a vector: the pair path is planned only when it is selected).
 int pair_build_host_plan(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
                          const int32_t *span_last, PairHostPlan &out, std::vector<unsigned char> &img);
-// An upper bound of the image and scratch bytes of that plan, from the batch's counts alone.
-size_t pair_bytes_bound(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off);
+// Upper bounds of the image and scratch bytes of that plan, from the batch's counts alone.
+struct PairBytes { size_t image, scratch; };
+PairBytes pair_bytes_bound(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off);
 void pair_bind_device_plan(const PairHostPlan &h, unsigned char *image_base, unsigned char *scratch_base, lr_plan *p);
 
 void set_error(const char *fmt, ...);
