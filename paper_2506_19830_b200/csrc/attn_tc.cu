@@ -822,8 +822,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
         if (elect_one()) mbar_arrive(&ctrl->kv_empty[(ring_base - 1) % kStages]);
       }
     }
-    if (!ok && lane == 0) {
-      // let every MMA already issued retire before tensor memory is released
+    if (!ok && elect_one()) {
+      // let every MMA already issued retire before tensor memory is released (a commit covers what its own thread issued)
       tc_commit(&ctrl->drain[s]);
       const uint64_t t0 = global_ns();
       while (!mbar_try_wait(&ctrl->drain[s], 0))

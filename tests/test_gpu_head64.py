@@ -72,3 +72,27 @@ def test_weights_keep_their_fp32_bits():
         off, total = off + int((closest != got).sum()), total + got.size
         ctx.close()
     assert off <= 1e-3 * total, off / total
+
+
+def test_a_wait_that_runs_out():
+    """As in test_gpu_errors, at this head size: the issuers' drain commits from the lane that issued the products."""
+    w = _chain(6, 16, 4, 1500, 3, 16)
+    b, t = w.batch, w.tensors
+    ctx = B.Context(b.model, 0)
+    plan = B.Plan(ctx, b)
+    x, y = R.DeviceInputs(b, t), R.PassOutputs(b)
+    plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out)
+    want = y.out.clone()
+    plan.lr_plan_debug_set_wait_limit(3000)
+    plan.lr_plan_debug_set_phantom_bytes(4096)
+    plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out)
+    with pytest.raises(B.LrError) as e:
+        plan.lr_poll_status()
+    assert e.value.status == -4, e.value  # LR_ETIMEOUT
+    plan.lr_plan_debug_set_phantom_bytes(0)
+    plan.lr_plan_debug_set_wait_limit(1_000_000)
+    for _ in range(2):
+        plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out)
+        assert plan.lr_poll_status() == 0
+        assert torch.equal(y.out, want)
+    ctx.close()
