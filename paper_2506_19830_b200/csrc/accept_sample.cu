@@ -78,7 +78,10 @@ accept_stats_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int
     const uint32_t row = unit / n_chunks;
     const uint16_t *rp = logits + (int64_t)row * row_stride;
     int32_t v0 = (int32_t)(unit - row * n_chunks) * steps * (kStep / 8) + lane;
-    float m = -INFINITY, sum = 0.f;  // of this lane's share of the chunk
+    // Of this lane's share of the chunk: the maximum, an exponent near -m * k_log2 and the sum of 2^(x * k_log2 + off).  `off` is
+    // rounded at its own magnitude, which for large logits or low temperatures is far above that of the differences:
+    // whatever goes from one lane or step to another is scaled by what `off` really is, not by what it stands for.
+    float m = -INFINITY, off = 0.f, sum = 0.f;
     for (int st = 0; st < steps; ++st, v0 += kStep / 8) {
       uint32_t x[kVec * 4];
 #pragma unroll
@@ -109,7 +112,8 @@ accept_stats_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int
         mx = max_bf2(mx, x[i]);
       }
       const float mn = fmaxf(m, fmaxf(bf_lo(mx), bf_hi(mx)));
-      const float off = mn > -INFINITY ? -mn * k_log2 : 0.f;
+      const float off_before = off;
+      off = mn > -INFINITY ? -mn * k_log2 : 0.f;
       float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
       for (int i = 0; i < kVec * 4; i += 2) {
@@ -118,13 +122,13 @@ accept_stats_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int
         a2 += ex2_approx(fmaf(bf_lo(x[i + 1]), k_log2, off));
         a3 += ex2_approx(fmaf(bf_hi(x[i + 1]), k_log2, off));
       }
-      sum = fmaf(sum, ex2_approx(fmaf(m, k_log2, off)), (a0 + a1) + (a2 + a3));
+      sum = fmaf(sum, m > -INFINITY ? ex2_approx(off - off_before) : 0.f, (a0 + a1) + (a2 + a3));
       m = mn;
     }
     float M = m;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
-    float S = sum * ex2_approx(fmaf(m, k_log2, M > -INFINITY ? -M * k_log2 : 0.f));
+    float S = m > -INFINITY ? sum * ex2_approx(-fmaf(M, k_log2, off)) : 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
     if (lane == 0) stats[unit] = make_float2(M, S);

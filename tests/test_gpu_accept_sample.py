@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 import torch
 
-from lr_workloads import Model, bf16_round, make_config, make_random_small
+from lr_workloads import Model, bf16_round, bf16_to_f32, make_config, make_random_small
 from oracle import lr_oracle as O
 from paper_2506_19830_b200 import binding as B
 from paper_2506_19830_b200 import runner as R
@@ -113,3 +113,27 @@ def test_flat_rows_special_values_and_long_chains():
     got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, 1.0, ua, uf)
     _check(bits, drafts, cu, 1.0, ua, uf, got, max_ambiguous_frac=0.4)
     assert got[0][2] == L and got[0][0] == 5
+
+
+@pytest.mark.parametrize("T,offset", [(0.6, 0.0), (0.6, 100.0), (0.6, -1000.0), (0.1, 0.0), (0.05, 0.0), (0.05, 100.0)])
+@pytest.mark.parametrize("vocab", [5003, 400003])  # chunks of one step and of two
+def test_probabilities_of_large_scaled_logits(vocab, T, offset):
+    """P(draft) depends on differences of logits, however large the logits over the temperature are.  The arguments of the
+    exponentials that matter here lie within 20 of 0 (base 2) and are rounded twice, three times over: 6 * 20 * 2^-24 * ln 2 =
+    5e-6, with 1e-6 for the exponentials and the sums."""
+    rng = np.random.default_rng(int(1000 * T) + int(abs(offset)))
+    L, nb = 3, 8
+    n_rows = nb * (L + 1)
+    x = np.full((n_rows, vocab), -64.0, dtype=np.float32)
+    lead = rng.integers(0, vocab // 8, n_rows)
+    for r in range(n_rows):
+        x[r, lead[r] + vocab // 8 * np.arange(8)] = 24.0 - T * rng.uniform(0, 6, 8)
+    bits = bf16_round(x + np.float32(offset))
+    cu = (np.arange(nb + 1) * L).astype(np.int32)
+    drafts = lead.reshape(nb, L + 1)[:, :L].reshape(-1).astype(np.int32).copy()
+    got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, T, np.zeros(nb * L), rng.uniform(0, 1, nb))
+    z = bf16_to_f32(bits).astype(np.float64) / float(np.float32(T))
+    P = np.exp(z - z.max(axis=1, keepdims=True))
+    P /= P.sum(axis=1, keepdims=True)
+    want = np.array([P[b * (L + 1) + i, drafts[b * L + i]] for b in range(nb) for i in range(L)])
+    assert np.abs(got[2] / want - 1).max() <= 6e-6
