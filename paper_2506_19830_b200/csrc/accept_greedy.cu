@@ -86,7 +86,7 @@ __device__ __forceinline__ Best better(Best a, Best b) {
 __global__ void __launch_bounds__(kThreads)
 accept_greedy_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab,
                      const int32_t *__restrict__ draft_ids, const int32_t *__restrict__ cu_draft, int32_t n_branch,
-                     int32_t n_rows, uint32_t n_chunks, uint32_t total, int32_t *__restrict__ n_accept, int32_t *__restrict__ bonus_id,
+                     int32_t n_rows, int32_t first_draft, uint32_t n_chunks, uint32_t total, int32_t *__restrict__ n_accept, int32_t *__restrict__ bonus_id,
                      int32_t *__restrict__ row_argmax, unsigned long long *scratch) {
   unsigned int *counter = reinterpret_cast<unsigned int *>(scratch);
   unsigned long long *row_key = scratch + 1;
@@ -151,8 +151,7 @@ accept_greedy_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   // One thread per branch, so that hundreds of branches cost one pass: the bounds of its draft range with two loads in
   // flight, then its rows eight at a time -- keys and drafts of a chunk are loaded together, so a chunk costs one
   // round trip to L2 whatever the branch count -- and the scan stops at the first mismatch.
-  // The branches may be a run of a larger batch's: drafts are indexed from the batch's first one, rows from the run's.
-  const int32_t first_draft = cu_draft[0];
+  // Branch b's rows start at cu_draft[b] - first_draft + b.
   for (int b = tid; b < n_branch; b += kThreads) {
     const int32_t d0 = cu_draft[b], L = cu_draft[b + 1] - d0;
     const int32_t r0 = d0 - first_draft + b;
@@ -227,7 +226,7 @@ int launch_accept_static(lr_ctx *ctx, const void *logits, int64_t stride, const 
   }
   // Every call shares the array and it keeps what the last call left: start from zero regardless.
   if (rc == LR_OK) rc = cuda_fail(cudaMemsetAsync(ptr, 0, 8 * ((size_t)n_rows + 1), s), "cudaMemsetAsync(static scratch)");
-  if (rc == LR_OK) rc = launch_accept(ctx, logits, stride, drafts, cu_draft, n_branch, n_rows, n_accept, bonus, row_argmax, ptr, s);
+  if (rc == LR_OK) rc = launch_accept(ctx, logits, stride, drafts, cu_draft, n_branch, n_rows, 0, n_accept, bonus, row_argmax, ptr, s);
   if (prev_device != ctx->device) {
     const cudaError_t e = cudaSetDevice(prev_device);
     if (rc == LR_OK) rc = cuda_fail(e, "cudaSetDevice(restore)");
@@ -236,14 +235,14 @@ int launch_accept_static(lr_ctx *ctx, const void *logits, int64_t stride, const 
 }
 
 int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
-                  int32_t n_branch, int32_t n_rows, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,
+                  int32_t n_branch, int32_t n_rows, int32_t first_draft, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,
                   void *scratch, cudaStream_t s) {
   const int32_t vocab = ctx->model.vocab;
   // a chunk per warp at least, at most kCtasPerSm CTAs per SM
   const uint32_t n_chunks = std::max(1, ((vocab >> 3) + kChunkVecs - 1) / kChunkVecs), total = n_chunks * (uint32_t)n_rows;
   const unsigned grid = std::min((total + kThreads / 32 - 1) / (kThreads / 32), (uint32_t)(ctx->sm_count * kCtasPerSm));
   accept_greedy_kernel<<<grid, kThreads, 0, s>>>(reinterpret_cast<const uint16_t *>(logits), stride, vocab, drafts,
-                                                            cu_draft, n_branch, n_rows, n_chunks, total, n_accept, bonus, row_argmax,
+                                                            cu_draft, n_branch, n_rows, first_draft, n_chunks, total, n_accept, bonus, row_argmax,
                                                             reinterpret_cast<unsigned long long *>(scratch));
   ctx->launches++;
   return cuda_fail(cudaGetLastError(), "accept_greedy_kernel launch");

@@ -760,7 +760,7 @@ extern "C" int lr_accept_greedy(lr_ctx *ctx, const void *logits, int64_t stride,
     return LR_EINVAL;
   }
   if (n_branch == 0) return LR_OK;
-  return launch_accept(ctx, logits, stride, drafts, cu_draft, n_branch, n_rows, n_accept, bonus, row_argmax, scratch,
+  return launch_accept(ctx, logits, stride, drafts, cu_draft, n_branch, n_rows, 0, n_accept, bonus, row_argmax, scratch,
                        reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -1041,8 +1041,8 @@ static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass_host: device-to-host copy of the output");
   // rows and branches of a part are counted from its first branch, drafts from the batch's first one
   auto accept = [&](int b0, int b1, size_t row0, size_t n_rows) {
-    return lr_accept_greedy(ctx, b + L.logits + row0 * row_bytes, vocab, I(L.drafts), d.cu_draft + b0, b1 - b0, (int32_t)n_rows,
-                            I(L.n_accept) + b0, I(L.bonus) + b0, nullptr, b + L.scratch, stream);
+    return launch_accept(ctx, b + L.logits + row0 * row_bytes, vocab, I(L.drafts), d.cu_draft + b0, b1 - b0, (int32_t)n_rows,
+                         p->cu_draft_h[b0], I(L.n_accept) + b0, I(L.bonus) + b0, nullptr, b + L.scratch, s);
   };
   if (part_bytes) {
     if (int rc = cuda_fail(cudaStreamWaitEvent(s, p->side.part, 0), "cudaStreamWaitEvent")) return rc;

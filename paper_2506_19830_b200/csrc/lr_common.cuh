@@ -307,8 +307,9 @@ int launch_attn_generic(lr_plan *p, const void *q, const void *k, const void *v,
                         cudaStream_t s);
 int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
                    cudaStream_t s);
+// first_draft: what cu_draft counts in front of the first branch's rows (a later part of a batch whose rows are given alone)
 int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
-                  int32_t n_branch, int32_t n_rows, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,
+                  int32_t n_branch, int32_t n_rows, int32_t first_draft, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,
                   void *scratch, cudaStream_t s);
 int launch_accept_static(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
                          int32_t n_branch, int32_t n_rows, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,

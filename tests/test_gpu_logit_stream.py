@@ -59,3 +59,25 @@ def test_sample(vocab, nb, L):
         drafts = np.zeros(1, np.int32)
     got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, 0.7, ua, uf)
     _check(bits, drafts, cu, 0.7, ua, uf, got)
+
+
+@pytest.mark.parametrize("static", [False, True])
+@pytest.mark.parametrize("b0", [0, 1, 20])
+def test_greedy_on_the_later_branches_of_a_batch(b0, static):
+    """Branch b's rows start at cu_draft[b] + b, also where cu_draft does not start at 0."""
+    vocab, nb, L = 2049, 30, 5
+    _, bits, ref, cu, drafts = _make(vocab, nb, L, 7)
+    n_ref, b_ref, _ = O.accept_greedy(bits, drafts, cu)
+    padded = np.full((len(bits), 2056), 0x7F80, dtype=np.uint16)
+    padded[:, :vocab] = bits
+    ctx = B.Context(Model(1, 1, 64, vocab), 0)
+    i32 = dict(dtype=torch.int32, device="cuda:0")
+    n, rows = nb - b0, len(bits) - b0
+    n_acc, bonus, arg = torch.empty(n, **i32), torch.empty(n, **i32), torch.empty(rows, **i32)
+    lg, d, c = R.bf16_tensor(padded, "cuda:0")[b0:, :vocab], torch.from_numpy(drafts).to("cuda:0"), torch.from_numpy(cu[b0:].copy()).to("cuda:0")
+    if static:
+        ctx.lr_accept_greedy_static(lg, d, c, n_acc, bonus, arg)
+    else:
+        ctx.lr_accept_greedy(lg, d, c, n_acc, bonus, B.Context.accept_scratch(rows, "cuda:0"), arg)
+    assert np.array_equal(arg.cpu().numpy(), ref[b0:]) and np.array_equal(n_acc.cpu().numpy(), n_ref[b0:]) and np.array_equal(bonus.cpu().numpy(), b_ref[b0:])
+    ctx.close()
