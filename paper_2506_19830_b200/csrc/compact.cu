@@ -25,17 +25,18 @@ constexpr int kPerThread = 4;                  // pages per thread and step of t
 constexpr int kScan = kThreads * kPerThread;   // pages per step
 constexpr int kRows = 8;                       // 16-byte vectors a thread holds per round
 
-// blockIdx.x: (KV head, K or V, slice of the row); blockIdx.y: request.  1 << shift 16-byte vectors per slice.
+// blockIdx.x: (KV head, K or V, slice of the row); blockIdx.y: request.  1 << shift 16-byte vectors per slice.  sides: 2, or 1
+// when K and V are the same pool, whose bytes one CTA has to own as well.
 __global__ void __launch_bounds__(kThreads)
 compact_kernel(DevBatch d, const int32_t *__restrict__ keep_off, const int32_t *__restrict__ keep_pages,
-               const int32_t *__restrict__ keep_valid, int shift, uint4 *k_pool, uint4 *v_pool, int32_t *__restrict__ new_len,
+               const int32_t *__restrict__ keep_valid, int shift, int sides, uint4 *k_pool, uint4 *v_pool, int32_t *__restrict__ new_len,
                int32_t *__restrict__ n_pages_kept) {
   __shared__ int32_t s_off[kScan + 1];  // tokens of the request in front of each page of the step
   __shared__ int32_t warp_sum[kThreads / 32], warp_first[kThreads / 32];
   const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int vec_per_row = d.head_dim / 8, slices = vec_per_row >> shift;
-  const int slice = blockIdx.x % slices, h = blockIdx.x / slices >> 1;
-  uint4 *pool = (blockIdx.x / slices) & 1 ? v_pool : k_pool;
+  const int slice = blockIdx.x % slices, h = blockIdx.x / slices / sides;
+  uint4 *pool = blockIdx.x / slices % sides ? v_pool : k_pool;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the keep list comes from the kernel launched just before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the next layer's grid may be set up meanwhile
   const int i0 = keep_off[r], i1 = keep_off[r + 1];
@@ -151,11 +152,12 @@ int launch_compact(lr_plan *p, const int32_t *keep_off, const int32_t *keep_page
   // 7.0, but sliced in four 8.8), down to one sector for half a CTA per SM (one request 5.5 and 4.5, with 4000 tokens 26 and
   // 17; four requests 4.2 and 5.1).
   int shift = d.head_dim == 128 ? 4 : 3;
-  const int64_t rows = (int64_t)d.n_req * d.n_kv_heads * 2;
+  const int sides = k_pool == v_pool ? 1 : 2;
+  const int64_t rows = (int64_t)d.n_req * d.n_kv_heads * sides;
   while (shift > 1 && rows * (d.head_dim / 8 >> shift) < (shift > 2 ? 2 * p->ctx->sm_count : p->ctx->sm_count / 2)) --shift;
-  const dim3 grid((unsigned)(d.n_kv_heads * 2 * (d.head_dim / 8 >> shift)), (unsigned)d.n_req);
+  const dim3 grid((unsigned)(d.n_kv_heads * sides * (d.head_dim / 8 >> shift)), (unsigned)d.n_req);
   p->ctx->launches++;
-  return cuda_fail(launch_dependent(compact_kernel, grid, dim3(kThreads), 0, s, d, keep_off, keep_pages, keep_valid, shift,
+  return cuda_fail(launch_dependent(compact_kernel, grid, dim3(kThreads), 0, s, d, keep_off, keep_pages, keep_valid, shift, sides,
                                     reinterpret_cast<uint4 *>(k_pool), reinterpret_cast<uint4 *>(v_pool), new_len, n_pages_kept),
                    "compact_kernel launch");
 }

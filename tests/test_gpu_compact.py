@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 PAGE = 16
 
 
-def _run_and_check(w, n_accept):
+def _run_and_check(w, n_accept, one_pool=False):
     b, t = w.batch, w.tensors
     dev = "cuda:0"
     ctx = B.Context(b.model, 0)
@@ -23,6 +23,8 @@ def _run_and_check(w, n_accept):
     verdict = t.verdict if len(t.verdict) else np.zeros(1, dtype=np.uint8)
     plan.lr_commit(torch.from_numpy(verdict).to(dev), torch.from_numpy(n_accept).to(dev), y.n_steps_accepted, y.survivor,
                    y.committed_len, y.keep_off, y.keep_pages, y.keep_valid, y.free_off, y.free_pages)
+    if one_pool:
+        x.v_pool, t.v_pool = x.k_pool, t.k_pool
     new_len = torch.full((b.n_req,), -7, dtype=torch.int32, device=dev)
     n_kept = torch.full((b.n_req,), -7, dtype=torch.int32, device=dev)
     scratch = plan.compact_scratch()
@@ -75,3 +77,13 @@ def test_long_lists_and_rounds(n_req, heads, head_dim, prefix, segs):
     w = _finish("compact", 6, Model(heads, heads, head_dim, 16), reqs, rng, 0.5, 1.0, False, True, "nan")
     w.tensors.verdict[:] = 1
     _run_and_check(w, np.asarray(w.batch.br_n_draft, dtype=np.int32) - 1)
+
+
+@pytest.mark.parametrize("heads,head_dim,segs", [(1, 64, [3, 40]), (8, 128, [300, 17, 200])])
+def test_one_pool_for_keys_and_values(heads, head_dim, segs):
+    rng = np.random.Generator(np.random.PCG64(heads))
+    reqs = [{"P": 1000 + 3 * r, "segs": segs, "branches": [(n, 9, 9, 8) for n in range(1, len(segs) + 1)]} for r in range(3)]
+    w = _finish("compact", 6, Model(heads, heads, head_dim, 16), reqs, rng, 0.5, 1.0, False, True, "nan")
+    w.tensors.verdict[:] = 1
+    for _ in range(5):
+        _run_and_check(w, np.asarray(w.batch.br_n_draft, dtype=np.int32) - 1, one_pool=True)
