@@ -260,11 +260,18 @@ static int make_side(SideStream &side) {
   return cuda_fail(e, "side stream");
 }
 
-// The plan's side stream: the one the context was made with, that of an earlier plan, or a new one (about 90 us).
+// The plan's side stream: the one the context was made with, that of an earlier plan, or a new one (about 90 us).  Also while
+// the caller's stream is being captured, which making a stream is no part of.
 static int take_side(lr_plan *p) {
   if (p->side.s) return LR_OK;
   std::vector<SideStream> &idle = p->ctx->side_free;
-  if (idle.empty()) return make_side(p->side);
+  if (idle.empty()) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (int rc = cuda_fail(cudaThreadExchangeStreamCaptureMode(&mode), "cudaThreadExchangeStreamCaptureMode")) return rc;
+    const int rc = make_side(p->side);
+    const cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    return rc != LR_OK ? rc : cuda_fail(e, "cudaThreadExchangeStreamCaptureMode");
+  }
   p->side = idle.back();
   idle.pop_back();
   return LR_OK;
@@ -929,23 +936,14 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
     return LR_EINVAL;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), side = reinterpret_cast<cudaStream_t>(side_stream);
-  bool beside = true;
-  if (!p->side.s) {
-    // a stream cannot be made while the caller's is being captured: such a first pass stays on one stream
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (int rc = cuda_fail(cudaStreamIsCapturing(s, &capture), "cudaStreamIsCapturing")) return rc;
-    beside = capture == cudaStreamCaptureStatusNone;
-    if (beside)
-      if (int rc = take_side(p)) return rc;
-  }
+  if (int rc = take_side(p)) return rc;
   // Attention, then acceptance and commit beside it: they fill the SMs while its last CTAs, the merge of its partial results
   // and the gaps between launches leave them idle.  (Which of the two comes first makes no difference.)  One after another
   // and so: the smallest request 22.6 and 19.0 us, one of 4 K tokens 36.9 and 27.2 (head size 64: 28.9 and 22.8), of 32 K
   // 87.7 and 80.2, four of 16 K 102.4 and 91.7, trees 597 and 592.
-  cudaError_t e = beside ? cudaEventRecord(p->side.fork, s) : cudaSuccess;
+  cudaError_t e = cudaEventRecord(p->side.fork, s);
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
   if (int rc = lr_verify_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, stream)) return rc;
-  if (!beside) return pass_accept_commit(ctx, p, io, stream);
   if (!side) side = p->side.s;
   e = cudaStreamWaitEvent(side, p->side.fork, 0);
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");

@@ -4,6 +4,7 @@ do not disturb one another, and a capture as the very first use works."""
 import numpy as np
 import pytest
 import torch
+from cuda.bindings import runtime as cudart
 
 from lr_workloads import make_config, make_random_small
 from oracle import lr_oracle as O
@@ -75,4 +76,29 @@ def test_capture(warm):
     R.run_pass(ctx, plan, x, y)
     assert torch.equal(captured, y.out)
     del graph
+    ctx.close()
+
+
+@pytest.mark.parametrize("given_side", [False, True])
+@pytest.mark.parametrize("n_plans", [1, 3])  # the context has a stream for the first one, the others need new ones
+def test_a_capture_as_first_use_forks(n_plans, given_side):
+    w = make_config(1)
+    ctx = B.Context(w.batch.model, 0)
+    plans, x = [B.Plan(ctx, w.batch) for _ in range(n_plans)], R.DeviceInputs(w.batch, w.tensors)
+    for plan in plans:
+        y = R.PassOutputs(w.batch)
+        torch.cuda.synchronize()
+        graph, side = torch.cuda.CUDAGraph(keep_graph=True), torch.cuda.Stream()
+        with torch.cuda.graph(graph):
+            if given_side:
+                R.run_pass_overlapped(ctx, plan, x, y, side)
+            else:
+                R.run_pass(ctx, plan, x, y)
+        err, _, n_roots = cudart.cudaGraphGetRootNodes(graph.raw_cuda_graph(), 0)
+        assert int(err) == 0 and n_roots == 2  # attention and acceptance, neither behind the other
+        graph.replay()
+        torch.cuda.synchronize()
+        assert plan.lr_poll_status() == 0
+        _same((y.n_accept, y.bonus_id, y.committed_len), _expect(w))
+        del graph
     ctx.close()
