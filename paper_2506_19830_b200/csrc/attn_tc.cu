@@ -396,28 +396,34 @@ __device__ __forceinline__ float max_half(const uint32_t (&v)[64]) {
   }
   return fmaxf(fmaxf(a, b), fmaxf(c, e));
 }
-// The weights of a half as they go to tensor memory, 16 columns (32 weights) at a time, so that no more than these sit in
-// registers beside the scores (which a redo needs again).  Column c of a term holds the weights 2c and 2c + 1.  With three
+// The weights of a half as they go to tensor memory; with several terms 16 columns (32 weights) at a time, so that no more
+// than these sit in registers beside the scores (which a redo needs again).  Column c of a term holds the weights 2c and 2c + 1.  With three
 // terms each is the leading eight bits of what the terms before it leave: cut off, not rounded, which takes one
 // instruction for two weights, and the third has nothing left to cut.
 template <int kTerms>
 struct WeightOut {
-  uint32_t pk[kTerms][16];
+  static constexpr int kCols = kTerms == 1 ? 32 : 16;
+  uint32_t pk[kTerms][kCols];
   uint32_t addr[kTerms];
   __device__ __forceinline__ void add(float2 y, int c) {
     if constexpr (kTerms == 1) {
-      pk[0][c & 15] = pack_bf16(y.x, y.y);
+      pk[0][c] = pack_bf16(y.x, y.y);
     } else {
 #pragma unroll
       for (int t = 0; t < kTerms; ++t) {
         const uint32_t x0 = __float_as_uint(y.x), x1 = __float_as_uint(y.y);
-        pk[t][c & 15] = __byte_perm(x0, x1, 0x7632);
+        pk[t][c % kCols] = __byte_perm(x0, x1, 0x7632);
         if (t + 1 < kTerms) y = fadd2(y, make_float2(-bits_f(x0 & 0xFFFF0000u), -bits_f(x1 & 0xFFFF0000u)));
       }
     }
-    if ((c & 15) == 15)
+    if (c % kCols == kCols - 1) {
+      if constexpr (kTerms == 1) {
+        tmem_st32(addr[0], pk[0]);
+      } else {
 #pragma unroll
-      for (int t = 0; t < kTerms; ++t) tmem_st16(addr[t] + (c & 16), pk[t]);
+        for (int t = 0; t < kTerms; ++t) tmem_st16(addr[t] + (c & 16), pk[t]);
+      }
+    }
   }
 };
 
