@@ -94,7 +94,8 @@ struct Shape {
   static constexpr int kTileBytes = kHalves * kHalfBytes; // [halves][128 rows][128 B] for Q, [16 groups][halves][8 keys][128 B] for K/V
   static constexpr int kGroupBytes = kHalves * kAtomBytes;  // the atoms of one 8-key group
   static constexpr int kStages = kD == 128 ? 5 : 10;
-  static constexpr int kSmemBytes = 2 * kTileBytes + kStages * kTileBytes + 2048;  // tiles, then Ctrl; the base must be 1024-aligned
+  static constexpr int kRedoBytes = kD == 64 ? 8 * kD * 4 : 0;  // a query row for each softmax warp (redo_rows)
+  static constexpr int kSmemBytes = 2 * kTileBytes + kStages * kTileBytes + 2048 + kRedoBytes;  // tiles, Ctrl, rows; the base must be 1024-aligned
   // Head size 64 sends the softmax weights to the tensor core as three bf16 terms, whose sum is the fp32 weight itself:
   // as precise as the CUDA-core kernel that used to serve it.  The two further products are affordable there: their N is
   // 64.  Two terms (2^-17 of a weight lost) put four times as many outputs on the other side of a rounding step as fp32
@@ -454,13 +455,95 @@ __device__ __forceinline__ float exp_half(const uint32_t (&v)[64], WeightOut<kTe
   return acc0.x + acc0.y;
 }
 
+struct RawInputs {  // the tensors behind the tensor maps
+  const uint16_t *q, *k, *v;
+};
+
+// Head size 64: the rows of a warp (lanes `rows`) whose result for a piece is not finite, once more on CUDA cores.  A tile
+// holds keys that some of its rows do not see; their weights are zeros, but a zero times an infinity or a NaN in V is not
+// zero, and another branch's values must not reach a row.  So such a row sums the values of the n_pages pages from `pages`
+// that it does see, with the reference exponent (and for the final output the row sum) it has.  32 keys at a time: a lane
+// scores one, the lanes then share the value rows, two channels each.  sq: 64 floats of this warp's.  Head size 128 does
+// not look.
+__device__ __noinline__ void redo_rows(uint32_t rows, const TcPage *__restrict__ pages, int n_pages, RawInputs in, int64_t n_pool_pages, int n_kv_heads,
+                                       int kv_head, float scale_log2, RowInfo ri, float m_out, float l_out, int slot, int row0,
+                                       uint16_t *__restrict__ out, float *__restrict__ partial_o, float *sq) {
+  constexpr int kD = 64;
+  const int lane = threadIdx.x & 31;
+  for (; rows != 0u; rows &= rows - 1u) {
+    const int src = __ffs(rows) - 1;
+    RowInfo w;
+    w.depth = __shfl_sync(0xFFFFFFFFu, ri.depth, src);
+    w.branch = __shfl_sync(0xFFFFFFFFu, ri.branch, src);
+    w.limit = __shfl_sync(0xFFFFFFFFu, ri.limit, src);
+    w.q_index = __shfl_sync(0xFFFFFFFFu, (long long)ri.q_index, src);
+    const float m = __shfl_sync(0xFFFFFFFFu, m_out, src), l = __shfl_sync(0xFFFFFFFFu, l_out, src);
+    __syncwarp();
+    for (int e = lane; e < kD; e += 32) sq[e] = bits_f((uint32_t)in.q[w.q_index * kD + e] << 16) * scale_log2;
+    __syncwarp();
+    float acc0 = 0.f, acc1 = 0.f;
+    for (int p0 = 0; p0 < n_pages; p0 += 2) {
+      int64_t at = 0;  // of the lane's key, in rows of kD channels
+      bool seen = false;
+      if (p0 + (lane >> 4) < n_pages) {
+        const TcPage pg = pages[p0 + (lane >> 4)];
+        const int64_t id = pg.page >= 0 && pg.page < n_pool_pages ? pg.page : 0;  // as the copies did
+        seen = (lane & 15) < page_n_ok(pg.meta, w);
+        at = (id * n_kv_heads + kv_head) * kPage + (lane & 15);
+      }
+      uint32_t keys = __ballot_sync(0xFFFFFFFFu, seen);
+      if (keys == 0u) continue;
+      float p = 0.f;
+      if (seen) {
+        const uint4 *kp = reinterpret_cast<const uint4 *>(in.k + at * kD);
+        float a = 0.f;
+        for (int c = 0; c < kD / 8; ++c) {
+          const uint4 kk = __ldg(kp + c);
+          const uint32_t x[4] = {kk.x, kk.y, kk.z, kk.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            a = fmaf(sq[c * 8 + 2 * i], bits_f(x[i] << 16), a);
+            a = fmaf(sq[c * 8 + 2 * i + 1], bits_f(x[i] & 0xFFFF0000u), a);
+          }
+        }
+        p = ex2(a - m);
+      }
+      for (; keys != 0u; keys &= keys - 1u) {
+        const int j = __ffs(keys) - 1;
+        const float pj = __shfl_sync(0xFFFFFFFFu, p, j);
+        const int64_t aj = __shfl_sync(0xFFFFFFFFu, (long long)at, j);
+        const uint32_t vv = __ldg(reinterpret_cast<const uint32_t *>(in.v + aj * kD) + lane);
+        acc0 = fmaf(pj, bits_f(vv << 16), acc0);
+        acc1 = fmaf(pj, bits_f(vv & 0xFFFF0000u), acc1);
+      }
+    }
+    if (slot < 0) {
+      const float inv = 1.0f / l;
+      reinterpret_cast<uint32_t *>(out + w.q_index * kD)[lane] = pack_bf16(acc0 * inv, acc1 * inv);
+    } else {
+      const int64_t chunk = (int64_t)slot * (kD / 4) + (lane >> 1);
+      *reinterpret_cast<float2 *>(partial_o + (chunk * 128 + row0 + src) * 4 + (lane & 1) * 2) = make_float2(acc0, acc1);
+    }
+  }
+}
+
 // The store epilogue of a softmax thread: row r of the accumulator at o_addr (and, when the CTA's two streams worked on
 // the same rows, of the other stream's at o_other, weighted) goes out as bf16 (slot < 0) or as an fp32 partial.
-// Not inlined: its two 64-register row buffers must not weigh on the register allocation of the sweep.
+// Not inlined: its two 64-register row buffers must not weigh on the register allocation of the sweep.  Returns the lanes
+// whose row is left to redo_rows.
 template <int kD>
-__device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int slot, bool pair, float w_self, float w_other, float m_out,
+__device__ __noinline__ uint32_t store_rows(uint32_t o_addr, uint32_t o_other, int slot, bool pair, float w_self, float w_other, float m_out,
                                         float l_out, int r, int64_t q_index, uint16_t *__restrict__ out, float *__restrict__ lse,
                                         float *__restrict__ partial_o, float *__restrict__ partial_ml) {
+          bool odd = false;
+          auto look = [&](const uint32_t (&o)[64]) {  // (a row whose sum is not a number sees such a score itself)
+            if constexpr (kD == 64) {
+              float t = 0.f;
+#pragma unroll
+              for (int c = 0; c < 64; ++c) t = fmaf(bits_f(o[c]), 0.f, t);
+              odd = t != t && l_out == l_out && q_index >= 0;
+            }
+          };
           const bool any_other = pair && __any_sync(0xFFFFFFFFu, w_other > 0.f);
           if (slot < 0) {
             const float inv = 1.0f / l_out, a = w_self * inv, b = w_other * inv;
@@ -480,7 +563,8 @@ __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int s
                   for (int c = 0; c < 64; ++c) o[c] = __float_as_uint(fmaf(bits_f(p[c]), b, bits_f(o[c])));
                 }
               }
-              if (q_index >= 0) {
+              look(o);
+              if (q_index >= 0 && !odd) {
                 uint4 *dst = reinterpret_cast<uint4 *>(out + q_index * kD + hf * 64);
 #pragma unroll
                 for (int jj = 0; jj < 8; ++jj)
@@ -509,7 +593,8 @@ __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int s
                   }
                 }
               }
-              if (q_index >= 0) {
+              look(o);
+              if (q_index >= 0 && !odd) {
                 // chunk-major: 16-byte chunk k of row r at [slot][k][r], so a warp's store is 512 contiguous bytes
                 uint4 *dst = reinterpret_cast<uint4 *>(partial_o) + ((int64_t)slot * (kD / 4) + hf * 16) * 128 + r;
 #pragma unroll
@@ -518,12 +603,13 @@ __device__ __noinline__ void store_rows(uint32_t o_addr, uint32_t o_other, int s
             }
             if (q_index >= 0) *reinterpret_cast<float2 *>(partial_ml + prow * 2) = make_float2(m_out, l_out);
           }
+          return kD == 64 ? __ballot_sync(0xFFFFFFFFu, odd) : 0u;
 }
 
 template <int kD>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map,
-               const __grid_constant__ CUtensorMap q_map, DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out,
+               const __grid_constant__ CUtensorMap q_map, DevBatch d, DevTcPlan tc, RawInputs in, uint16_t *__restrict__ out,
                float *__restrict__ lse, float scale_log2) {
   using Sh = Shape<kD>;
   constexpr int kTileBytes = Sh::kTileBytes, kGroupBytes = Sh::kGroupBytes, kStages = Sh::kStages, kHalves = Sh::kHalves;
@@ -1011,9 +1097,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
         if (pair) ++x_cnt;
         if (ok && writer && !idle) {
           tc_fence_after();
-          store_rows<kD>(o_addr, lane_base + 256 + (1 - s) * 128, pi.slot[pair ? 0 : s], pair, w_self, w_other, m_out, l_out, r, ri.q_index, out,
-                     lse, tc.partial_o, tc.partial_ml);
+          const int slot = pi.slot[pair ? 0 : s];
+          const uint32_t odd = store_rows<kD>(o_addr, lane_base + 256 + (1 - s) * 128, slot, pair, w_self, w_other, m_out, l_out, r, ri.q_index, out, lse,
+                                              tc.partial_o, tc.partial_ml);
           tc_fence_before();
+          if constexpr (kD == 64)
+            if (odd != 0u)  // (row_info again: the sweep has no registers to spare for it)
+              redo_rows(odd, tc.pages + rq.page_off + pi.tile_begin * kPagesPerTile, n * kPagesPerTile, in, d.n_pool_pages, d.n_kv_heads, pi.kv_head,
+                        scale_log2, row_info(d, tc, rq, T, mode == 2 ? pi.mtile0 + s : pi.mtile0, r, pi.kv_head), m_out, l_out, slot, quarter * 32, out, tc.partial_o,
+                        reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(ctrl) + kCtrlBytes) + warp * kD);
         }
       }
       // One arrival per thread and piece.  A stream with units in this piece cannot get here before the previous
@@ -1429,9 +1521,9 @@ void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigne
 }
 
 template <int kD>
-static int launch_attn_tc_d(lr_plan *p, const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &qmap, uint16_t *out,
+static int launch_attn_tc_d(lr_plan *p, const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &qmap, const RawInputs &in, uint16_t *out,
                             float *lse, float scale_log2, cudaStream_t s) {
-  attn_tc_kernel<kD><<<p->tc.n_cta, kThreads, Shape<kD>::kSmemBytes, s>>>(kmap, vmap, qmap, p->dev, p->tc, out, lse, scale_log2);
+  attn_tc_kernel<kD><<<p->tc.n_cta, kThreads, Shape<kD>::kSmemBytes, s>>>(kmap, vmap, qmap, p->dev, p->tc, in, out, lse, scale_log2);
   p->ctx->launches++;
   if (int rc = cuda_fail(cudaGetLastError(), "attn_tc_kernel launch")) return rc;
   if (p->tc.n_targets > 0) {  // the merge grid is set up while the attention grid drains
@@ -1452,7 +1544,8 @@ int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void
   if (int rc = get_map(p->ctx, 1, q, p->dev.n_q_rows, &mp)) return rc;
   const CUtensorMap qmap = *mp;
   const float scale_log2 = scale * 1.4426950408889634f;
-  return (p->dev.head_dim == 128 ? launch_attn_tc_d<128> : launch_attn_tc_d<64>)(p, kmap, vmap, qmap, reinterpret_cast<uint16_t *>(out), lse,
+  const RawInputs in = {reinterpret_cast<const uint16_t *>(q), reinterpret_cast<const uint16_t *>(k), reinterpret_cast<const uint16_t *>(v)};
+  return (p->dev.head_dim == 128 ? launch_attn_tc_d<128> : launch_attn_tc_d<64>)(p, kmap, vmap, qmap, in, reinterpret_cast<uint16_t *>(out), lse,
                                                                                 scale_log2, s);
 }
 

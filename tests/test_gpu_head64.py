@@ -96,3 +96,33 @@ def test_a_wait_that_runs_out():
         assert plan.lr_poll_status() == 0
         assert torch.equal(y.out, want)
     ctx.close()
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("args", [(7, 16, 4, 300, 2, 6), (8, 16, 4, 4000, 3, 16), (9, 32, 8, 2000, 3, 16, 12)])
+def test_values_a_row_does_not_see_do_not_reach_it(args, value):
+    """One branch's tail and the deepest step hold values that are not finite: rows that do not see them come out as
+    without them, a row that does shows it in the channels concerned."""
+    w = _chain(*args)
+    b, t = w.batch, w.tensors
+    ctx = B.Context(b.model, 0)
+    plan = B.Plan(ctx, b)
+    x, clean, got = R.DeviceInputs(b, t), R.PassOutputs(b), R.PassOutputs(b)
+    plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, clean.out, clean.lse)
+    rows = np.zeros(b.n_q_rows, dtype=bool)
+    page = int(b.page_ids[int(b.br_own_slot[1])])  # the second branch of the first request, from its third tail token on
+    x.v_pool[page, :, 2, 5:9] = value
+    rows[int(b.cu_q[1]) + max(0, 2 - int(b.br_own_len[1] - (b.cu_q[2] - b.cu_q[1]))): int(b.cu_q[2])] = True
+    deepest = int(b.req_span_off[1]) - 1  # the last step of the first request
+    x.v_pool[int(b.page_ids[int(b.span_slot[deepest])]), :, 1, 5:9] = value
+    bad = [i for i in range(b.n_branch) if b.br_req[i] == 0 and b.br_depth[i] == deepest]
+    for i in bad:
+        rows[int(b.cu_q[i]): int(b.cu_q[i + 1])] = True
+    for _ in range(2):
+        plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, got.out, got.lse)
+        assert plan.lr_poll_status() == 0
+        g, c = got.out.float().cpu().numpy(), clean.out.float().cpu().numpy()
+        assert np.isfinite(g[~rows]).all() and np.abs(g[~rows] - c[~rows]).max() <= 2.0 ** -7 * np.abs(c).max()
+        assert not np.isfinite(g[rows][:, :, 5:9]).any() and np.isfinite(np.delete(g[rows], np.s_[5:9], axis=2)).all()
+        assert torch.equal(got.lse, clean.lse)
+    ctx.close()
