@@ -54,14 +54,14 @@ def check_commit(got: dict, ref: dict):
 
 
 def attention_path_for(model):
-    """The tensor-core path, named explicitly, wherever the head size allows it: a plan that cannot take it then fails
-    with LR_EUNSUPPORTED instead of passing on the CUDA-core kernel."""
-    return B.PATH_TENSOR_CORE if model.head_dim == 128 else B.PATH_GENERIC
+    """The tensor-core path, named explicitly: a plan that cannot take it then fails with LR_EUNSUPPORTED instead of passing
+    on the CUDA-core kernel."""
+    return B.PATH_TENSOR_CORE
 
 
 def run_and_check_pass(w, path=None, check_rows_of_branches=None, rel_large: float = 0.0):
-    """Whole pass through the C ABI on workload w, compared with the oracle.  path None = the tensor-core kernel
-    for head_dim 128 (forced, so a silent fall-back is an error), the CUDA-core kernel otherwise."""
+    """Whole pass through the C ABI on workload w, compared with the oracle.  path None = the tensor-core kernel (forced,
+    so a silent fall-back is an error)."""
     b, t = w.batch, w.tensors
     ctx = B.Context(b.model, 0)
     plan = B.Plan(ctx, b)
