@@ -35,9 +35,9 @@
 //               than one per page half matters: the producer spends about 100
 //               cycles per box, and 32 boxes per tile made it a bottleneck.
 //               Every copy is for this CTA alone.
-//   warps 9, 10 MMA issuers of stream 0 and 1 (warp 11 idles): tcgen05.mma (M=128, N=128, K=16,
-//               bf16 -> fp32) for S = Q K^T (both operands in shared memory) and
-//               O += P V (P read from tensor memory, V from shared memory as the
+//   warps 9, 10 MMA issuers of stream 0 and 1 (warp 11 idles): tcgen05.mma (M=128, K=16, bf16 ->
+//               fp32) for S = Q K^T (N=64 keys, both operands in shared memory) and
+//               O += P V (N = head size, P read from tensor memory, V from shared memory as the
 //               N-major operand).  Issue blocks while the tensor pipe is full, so
 //               one issuer per stream lets the waits of one overlap the MMAs of
 //               the other.  The elected lane comes from elect.sync, so that operands stay in
@@ -1452,7 +1452,6 @@ void tc_plan_tables(const lr_batch *b, const int32_t *req_br_off, const int32_t 
   TcPage *pages = img.add<TcPage>((size_t)h.n_pages, h.o_pages);
   TcRow *rows = img.add<TcRow>((size_t)std::max(1, n_q_rows), h.o_rows);
   h.o_pieces = img.copy(h.pieces.data(), h.pieces.size());
-  h.o_cta_piece_off = img.copy(h.cta_piece_off.data(), h.cta_piece_off.size());
   TcReq *reqs = img.add<TcReq>(h.lists.size(), h.o_reqs);
   TcTarget *targets = img.add<TcTarget>(std::max<size_t>(1, h.targets.size()), h.o_targets);
   if (!img.base) return;
@@ -1508,7 +1507,6 @@ void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigne
   t.pages = reinterpret_cast<const TcPage *>(image_base + h.o_pages);
   t.rows = reinterpret_cast<const TcRow *>(image_base + h.o_rows);
   t.pieces = reinterpret_cast<const TcPiece *>(image_base + h.o_pieces);
-  t.cta_piece_off = reinterpret_cast<const int32_t *>(image_base + h.o_cta_piece_off);
   t.reqs = reinterpret_cast<const TcReq *>(image_base + h.o_reqs);
   t.targets = reinterpret_cast<const TcTarget *>(image_base + h.o_targets);
   t.n_cta = h.n_cta;

@@ -938,9 +938,9 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), side = reinterpret_cast<cudaStream_t>(side_stream);
   if (int rc = take_side(p)) return rc;
   // Attention, then acceptance and commit beside it: they fill the SMs while its last CTAs, the merge of its partial results
-  // and the gaps between launches leave them idle.  (Which of the two comes first makes no difference.)  One after another
-  // and so: the smallest request 22.6 and 19.0 us, one of 4 K tokens 36.9 and 27.2 (head size 64: 28.9 and 22.8), of 32 K
-  // 87.7 and 80.2, four of 16 K 102.4 and 91.7, trees 597 and 592.
+  // and the gaps between launches leave them idle.  (Which of the two comes first makes no difference.)  As three calls one
+  // after another and so: the smallest request 20.6 and 12.5 us, one of 4 K tokens 36.0 and 28.5, of 32 K 93.2 and 86.9, four
+  // of 16 K 110 and 102.
   cudaError_t e = cudaEventRecord(p->side.fork, s);
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
   if (int rc = lr_verify_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, stream)) return rc;

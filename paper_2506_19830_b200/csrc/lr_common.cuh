@@ -98,7 +98,6 @@ struct DevTcPlan {
   const TcPage *pages;
   const TcRow *rows;             // [n_q_rows]
   const TcPiece *pieces;
-  const int32_t *cta_piece_off;  // [n_cta+1]
   const TcReq *reqs;
   const TcTarget *targets;
   int32_t n_cta, n_targets;
@@ -246,7 +245,7 @@ struct TcHostPlan {
   std::vector<TcPiece> pieces;
   std::vector<int32_t> cta_piece_off;
   std::vector<TcTarget> targets;
-  size_t o_heads = 0, o_pages = 0, o_rows = 0, o_pieces = 0, o_cta_piece_off = 0, o_reqs = 0, o_targets = 0;  // image offsets
+  size_t o_heads = 0, o_pages = 0, o_rows = 0, o_pieces = 0, o_reqs = 0, o_targets = 0;  // image offsets
   int n_cta = 0, n_partial_slots = 0, tokens_per_mtile = 0, n_pages = 0;
   // scratch region behind the image: (exponent, sum) pairs, then fp32 partial outputs
   size_t s_ml = 0, s_o = 0, scratch_bytes = 0;
@@ -295,7 +294,7 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 int cuda_fail(cudaError_t e, const char *what);
 
 // kernels (each file exposes launchers)
-int init_kernels(lr_ctx *ctx);  // per-device function attributes; called by lr_create
+// per-device function attributes; called by lr_create
 int init_commit_kernel();
 int init_attn_tc_kernel();
 int init_attn_pair_kernel();
