@@ -42,8 +42,11 @@ constexpr int kChunk = 32 * kVec * 8;  // logits a warp takes at a time
 constexpr int kScanCtasPerSm = 4;
 constexpr int kGroupCap = 1344;     // groups filter_cut_kernel reads again (k_sel + k_sel / 4 + 4 at most, but for ties)
 constexpr int kListCap = 1408;      // candidates of a row
+constexpr int kSortCap = 2048;      // ... padded to a power of two
 constexpr int kListOut = 256;       // kept tokens that go out as a list
-constexpr int kKeyWords = 8;        // words of group maxima a thread of filter_cut_kernel keeps in registers
+constexpr int kManyFrom = 128;      // top_k from which filter_cut_kernel reads many groups at a time and may sort
+constexpr int64_t kManyBytes = 96 << 20;  // ... and the bytes of logits, with top-p alone
+constexpr int kCountMax = 448;      // candidates ranked by counting; more may be sorted
 constexpr int kSelMax = 1024;       // largest top_k the candidates serve
 constexpr int kSelTopP = 128;       // leading tokens to look for when top-k is off
 constexpr int kProbeRows = 16;      // rows the candidates are tried on first when top-k is off
@@ -245,13 +248,14 @@ __host__ __device__ __forceinline__ int slice_len_of(int32_t vocab) { return 256
 // ---- the cut of a row from its candidates -----------------------------------------------------------------
 // A lower bound of the k_sel-th largest logit is any value that k_sel group maxima reach (they are logits of different
 // tokens); it is raised by bisection on the key until little more than k_sel maxima reach it.  Only those groups hold tokens of at least that value: they are read again.  Bound: instructions, a few hundred per warp.
-template <int kGV>
-__global__ void __launch_bounds__(kT)
+template <int kGV, bool kMany>
+__global__ void __launch_bounds__(kT, kMany ? 4 : 0)
 filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2, int32_t top_k, float top_p, int k_sel,
                   int n_chunks, const uint16_t *__restrict__ group_max, const float2 *__restrict__ stats, RowCut *__restrict__ cuts,
                   u64 *__restrict__ lists, int32_t *__restrict__ n_kept_out, int32_t *__restrict__ n_open, int32_t *__restrict__ open_rows,
                   int row0, const int32_t *__restrict__ gave_up) {
-  __shared__ u64 s_cand[kListCap], s_sorted[kListCap], s_cum[kListCap];
+  constexpr int kKeyWords = kGV == 4 || kGV == 2 ? 16 : 8;  // words of group maxima a thread keeps in registers
+  __shared__ u64 s_cand[kMany ? kSortCap : kListCap], s_ranked[kMany ? kCountMax : kListCap], s_cum[kListCap];
   __shared__ int s_grp[kGroupCap];
   __shared__ int s_n, s_n_grp, s_cnt[2][kWarps], s_kept;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -262,8 +266,10 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
   if (tid == 0) s_n = s_n_grp = 0;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the maxima come from the kernel launched just before
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (gave_up != nullptr && *gave_up != 0) {
-    if (tid == 0) open_rows[atomicAdd(n_open, 1)] = (int32_t)row;
+  if (gave_up != nullptr && *gave_up != 0) {  // every row is left to the windows, the tried ones in front of row0 too
+    if (tid == 0) open_rows[row] = (int32_t)row;
+    if (blockIdx.x == 0 && tid < row0) open_rows[tid] = tid;
+    if (blockIdx.x == 0 && tid == 0) *n_open = row0 + (int)gridDim.x;
     return;
   }
   const uint32_t *src = reinterpret_cast<const uint32_t *>(group_max + row * n_chunks * kPerChunk);
@@ -284,6 +290,11 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) z_all += __shfl_xor_sync(0xFFFFFFFFu, z_all, o);
   }
+  // No token weighs more than 1 of z_all: a flat row keeps more than the list of candidates can hold.
+  if (!by_k && __syncthreads_or((double)top_p * z_all > 1.01 * kListCap)) {
+    if (tid == 0) open_rows[atomicAdd(n_open, 1)] = (int32_t)row;
+    return;
+  }
   auto bf2_of = [](int32_t key16) -> __nv_bfloat162 {
     const uint32_t u = f_of_key16(key16) >> 16, uu = u | (u << 16);
     return *reinterpret_cast<const __nv_bfloat162 *>(&uu);
@@ -302,7 +313,7 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
 #pragma unroll
     for (int i = 0; i < kKeyWords; ++i) c2 = __hadd2(c2, __hge2(as_bf2(g2[i]), t));
     int c = (int)(__low2float(c2) + __high2float(c2));
-    for (int i = kKeyWords * kT + tid; i < n_words; i += kT) {  // more than 4096 groups
+    for (int i = kKeyWords * kT + tid; i < n_words; i += kT) {
       const uint32_t w = __ldg(src + i);
       c += __popc(__hge2_mask(as_bf2(w), t)) >> 4;
     }
@@ -340,18 +351,33 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
   if (n_grp <= kGroupCap) {
     const int32_t n_vec = vocab >> 3, rem = vocab & 7;
     const float least_x = __uint_as_float(f_of_key16(least));
-    for (int i = tid; i < n_grp * kGV; i += kT) {
-      const int g = s_grp[i / kGV];
-      const int32_t vi = (g / kPerChunk) * (kChunk / 8) + (g % kPerChunk) + (i % kGV) * 32;
-      if (vi > n_vec || (vi == n_vec && rem == 0)) continue;
-      const uint4 v = vi < n_vec ? __ldg(reinterpret_cast<const uint4 *>(rp) + vi) : ragged_vec(rp, n_vec, rem);
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    constexpr int kFly = kMany ? kGV : 1;  // vectors a thread asks for at a time
+    for (int i0 = tid; i0 < n_grp * kGV; i0 += kFly * kT) {
+      uint4 v[kFly];
+      int32_t at_vec[kFly];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
-        if (__uint_as_float(f) >= least_x) {  // (a NaN is not)
-          const int at = atomicAdd(&s_n, 1);
-          if (at < kListCap) s_cand[at] = cand_of(f, vi * 8 + j);
+      for (int q = 0; q < kFly; ++q) {
+        const int i = i0 + q * kT;
+        v[q] = make_uint4(0x7FC07FC0u, 0x7FC07FC0u, 0x7FC07FC0u, 0x7FC07FC0u);  // NaN: never a candidate
+        at_vec[q] = 0;
+        if (i < n_grp * kGV) {
+          const int g = s_grp[i / kGV];
+          const int32_t vi = (g / kPerChunk) * (kChunk / 8) + (g % kPerChunk) / 32 * (32 * kGV) + g % 32 + (i % kGV) * 32;
+          at_vec[q] = vi;
+          if (vi < n_vec) v[q] = __ldg(reinterpret_cast<const uint4 *>(rp) + vi);
+          else if (vi == n_vec && rem != 0) v[q] = ragged_vec(rp, n_vec, rem);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kFly; ++q) {
+        const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
+          if (__uint_as_float(f) >= least_x) {  // (a NaN is not)
+            const int at = atomicAdd(&s_n, 1);
+            if (at < kListCap) s_cand[at] = cand_of(f, at_vec[q] * 8 + j);
+          }
         }
       }
     }
@@ -359,14 +385,33 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
   __syncthreads();
   const int n = s_n;
   const bool usable = n_grp <= kGroupCap && n >= 1 && n <= kListCap && (!by_k || n >= top_k);
-  if (usable)
+  const bool count = !kMany || n <= kCountMax;
+  const u64 *s_sorted = count ? s_ranked : s_cand;
+  if (usable && count) {
     for (int i = tid; i < n; i += kT) {  // rank by counting: the candidates are all different
       const u64 e = s_cand[i];
       int before = 0;
 #pragma unroll 4
       for (int j = 0; j < n; ++j) before += s_cand[j] > e ? 1 : 0;
-      s_sorted[before] = e;
+      s_ranked[before] = e;
     }
+  } else if (kMany && usable) {  // bitonic, largest first
+    int size = 512;
+    while (size < n) size *= 2;
+    for (int i = n + tid; i < size; i += kT) s_cand[i] = 0;  // behind every candidate
+    for (int run = 2; run <= size; run *= 2)
+      for (int step = run / 2; step > 0; step /= 2) {
+        __syncthreads();
+        for (int i = tid; i < size / 2; i += kT) {
+          const int lo = 2 * i - (i & (step - 1)), hi = lo + step;
+          const u64 x = s_cand[lo], y = s_cand[hi];
+          if ((x < y) == ((lo & run) == 0)) {
+            s_cand[lo] = y;
+            s_cand[hi] = x;
+          }
+        }
+      }
+  }
   __syncthreads();
   // ---- warp 0: the last rank kept.  It is top_k - 1, or the first one at which the mass, itself included, reaches
   //      t = ceil(top_p W), where W is the mass of the leading top_k ranks, or -- to within kMassEps -- of the whole row.
@@ -1033,6 +1078,14 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   if (kC > 1) cluster.sync();  // nobody leaves while its total is being read
 }
 
+// Vectors per group when k_sel leading tokens are looked for: the most, up to 8, that still make many more groups than that.
+// Short rows have few groups anyway and go from 8 to 1.
+int group_vecs(int32_t vocab, int k_sel) {
+  for (const int v : {8, 4, 2})
+    if (vocab / (8 * v) >= 4 * (int64_t)k_sel && (v == 8 || vocab > 65536)) return v;
+  return 1;
+}
+
 struct ScratchLayout {
   size_t cuts, lists, maxima, stats, open, bytes;
   int n_chunks, n_slices;
@@ -1062,19 +1115,24 @@ struct WindowShape {
   bool cached;
   double us;  // estimated time
 };
-// Cluster size for n_rows rows through the windows: the one with the smallest estimate.  Two CTAs fit an SM.  The numbers
-// are us per CTA and per 1000 tokens of its share, fitted to measured rounds of rows with one CTA on every SM and with two
-// (rows of 152064 tokens: 14.5 us for 17 by clusters of eight, 27 for 51 by fours, 38 for 74 by fours, 59 for 136 by pairs, 80
-// for 296 by single CTAs, which have no cluster barriers; of 32000: 15 us for 68 by single CTAs, 23 by pairs, 21 for 296).
-double window_us(const lr_ctx *ctx, int c, int64_t n_rows) {
+// Cluster size for n_rows rows through the windows: the one with the smallest estimate.  Two CTAs fit an SM.  A round of rows
+// takes `two` with two CTAs on every SM and `one` with one, in us and us per 1000 tokens of a CTA's share, fitted to whole calls
+// on flat rows less the 10 us of the draw (single CTAs, pairs, fours: 136 rows of 152064 tokens 63, 52 and 53 us, 340 of them
+// 147, 142 and 158, 408 154, 143 and 198, 612 225, 232 and 316; 340 of 50000 57, 84 and 124; 68 of 20000 11, 21 and 18; eights:
+// 17 of 152064 17 us, 272 223).  136 CTAs in pairs already share SMs, and so count as nearly all.  On other rows all are
+// faster, single CTAs the most.
+double window_us(const lr_ctx *ctx, int c, int64_t n_rows, bool flat) {
   const int64_t clusters = std::max(1, ctx->sm_count * 2 / c);
   const double k = share_of(ctx->model.vocab, c) * 1e-3;
-  const double one = c == 1 ? 6 + 0.42 * k : c == 2 ? 19 + 0.22 * k : c == 4 ? 14 + 0.2 * k : 11 + 0.18 * k;
-  const double two = c == 1 ? 7 + 0.48 * k : c == 2 ? 22 + 0.5 * k : c == 4 ? 20 + 0.47 * k : 17 + 0.55 * k;
-  const double full = std::min(1.0, std::max(0.0, (double)(n_rows * c - ctx->sm_count) / ctx->sm_count));
-  return (double)((n_rows + clusters - 1) / clusters) * (one + full * (two - one));
+  const double one = c == 1 ? 6 + 0.375 * k : c == 2 ? 10 + 0.34 * k : c == 4 ? 7.3 + 0.36 * k : 12 + 0.24 * k;
+  const double two = c == 1 ? 11 + 0.467 * k : c == 2 ? 19.5 + 0.4 * k : c == 4 ? 26 + 0.23 * k : 22.8 + 0.41 * k;
+  const int64_t rounds = n_rows / clusters, rest = n_rows % clusters;
+  const double sms = ctx->sm_count, ctas = (double)(rest * c);
+  const double full = c == 2 && rounds == 0 ? (ctas - 0.7 * sms) / (0.3 * sms) : (ctas - sms) / sms;
+  const double all = (double)rounds * two + (rest ? one + std::min(1.0, std::max(0.0, full)) * (two - one) : 0.0);
+  return c == 1 && !flat ? 0.92 * all : all;
 }
-WindowShape window_shape(const lr_ctx *ctx, int64_t n_rows) {
+WindowShape window_shape(const lr_ctx *ctx, int64_t n_rows, bool flat = false) {
   WindowShape best = {};
   for (const int c : {8, 4, 2, 1}) {
     const size_t fixed = (sizeof(WindowShared) + 15) / 16 * 16, share = (size_t)share_of(ctx->model.vocab, c) * 2;
@@ -1082,7 +1140,7 @@ WindowShape window_shape(const lr_ctx *ctx, int64_t n_rows) {
     w.cluster = c;
     w.cached = fixed + share <= kWindowSmemMax;
     w.smem = fixed + (w.cached ? share : 0);
-    w.us = window_us(ctx, c, n_rows);
+    w.us = window_us(ctx, c, n_rows, flat);
     if (best.cluster == 0 || w.us < best.us) best = w;
   }
   return best;
@@ -1134,33 +1192,45 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
   auto *n_open = reinterpret_cast<int32_t *>(base + L.open);
   const bool by_k = top_k > 0 && top_k < vocab, by_p = top_p < 1.f;
   const int k_sel = by_k ? top_k : kSelTopP;
-  // Groups of 64 tokens when that makes many more of them than k_sel, else of 8.  With too few groups of 8 as well the
-  // bound is too low to be of use, unless the whole row fits the list of candidates.
-  const bool wide = vocab / 64 >= 4 * (int64_t)k_sel;
+  const int gv = group_vecs(vocab, k_sel);
+  // With too few groups of 8 tokens as well the bound is too low to be of use, unless the whole row fits the list of candidates.
   const bool enough = vocab / 8 >= 4 * (int64_t)k_sel || vocab <= kListCap;
-  // Can a few leading tokens decide a row?  With a small top-k always: 17 us against 28 us through the windows for 51 rows
-  // of 152064 tokens and top-k 20, 46 against 213 for 612.  Reading and ranking the groups of a larger one costs about 0.1 us
-  // per k.  With top-p alone they mostly do, but the rows they leave open (taken to be one in five) go through the windows
-  // all the same, and when a kept set is half the vocabulary that is every row.  So they are tried on a few rows first and,
-  // if most of those stay open, on no more.  Rows of 152064 tokens, peaked, as a language model's, flat: 408 of them 89,
-  // 152 and 191 us (tried on all at once 61, 122 and 231; windows alone about 175), 612 of them 105, 175 and 281 (75, 142 and
-  // 340), 136 of them 50, 61 and 62 (42, 61 and 156).
+  // Can a few leading tokens decide a row?  With a small top-k always: 16 us against 37 us through the windows for 51 rows
+  // of 152064 tokens and top-k 20, 46 against 160 and more for 612.  Reading and ranking the groups of a larger one costs
+  // about 10 us and 0.055 per k while every row has an SM, and more behind that (272 rows, top-k 200, 400 and 800: 49, 76 and
+  // 96 us; 612 rows 84, 117 and 147; windows 93 and 184).  With top-p alone they mostly do, but the rows they leave open (taken
+  // to be one in five) go through the windows all the same, and when a kept set is half the vocabulary that is every row.  So
+  // they are tried on a few rows first and, if most of those stay open, on no more.  Rows of 152064 tokens, peaked, as a
+  // language model's, flat: 408 of them 77, 134 and 183 us (windows alone 110, 138 and 153 to 165), 612 of them 106, 170 and
+  // 262 (150, 177 and 236).
   WindowShape w = window_shape(ctx, n_rows);
-  const WindowShape w_open = window_shape(ctx, (n_rows + 4) / 5);
+  const WindowShape w_open = window_shape(ctx, (n_rows + 4) / 5, true);
   const double us_scan = (double)n_rows * vocab * 2 / 5.5e6;
   const int n_probe = !by_k && n_rows >= 4 * kProbeRows ? kProbeRows : 0;
-  const double us_candidates = by_k ? 12.0 + us_scan + (6.0 + 0.1 * top_k) * ((n_rows + 5 * ctx->sm_count - 1) / (5 * ctx->sm_count))
+  const double us_rank = gv == 1 ? (6.0 + 0.1 * top_k) * ((n_rows + 5 * ctx->sm_count - 1) / (5 * ctx->sm_count))
+                                 : (10.0 + 0.055 * top_k) * (1.0 + 0.27 * std::max(0.0, (double)n_rows / ctx->sm_count - 1.0));
+  const double us_candidates = by_k ? 12.0 + us_scan + us_rank
                                     : 24.0 + (n_probe ? 12.0 : 0.0) + us_scan + 0.02 * n_rows + w_open.us;
-  const bool candidates = enough && (by_k ? top_k <= kSelMax : by_p) && ((by_k && top_k <= 128) || us_candidates < w.us);
+  const bool candidates = enough && (by_k ? top_k <= kSelMax : by_p) && ((by_k && top_k <= 128) || us_candidates < window_shape(ctx, n_rows, true).us);
   // The open rows are few or all of them; only the device knows.  Up to n_few rows take the shape for a few.
   WindowShape few = w;
   int n_few = n_rows;
   if (candidates) {
-    auto scan = by_k ? (wide ? filter_scan_kernel<false, kVec> : filter_scan_kernel<false, 1>)
-                     : (wide ? filter_scan_kernel<true, kVec> : filter_scan_kernel<true, 1>);
-    auto cut = wide ? filter_cut_kernel<kVec> : filter_cut_kernel<1>;
+    auto scan = !by_k     ? (gv == 8 ? filter_scan_kernel<true, 8> : filter_scan_kernel<true, 1>)
+                : gv == 8 ? filter_scan_kernel<false, 8>
+                : gv == 4 ? filter_scan_kernel<false, 4>
+                : gv == 2 ? filter_scan_kernel<false, 2>
+                          : filter_scan_kernel<false, 1>;
+    // Many vectors in flight pay where many groups are read (top-k 200, 272 rows of 152064 tokens: 61 and 49 us) or they come
+    // from HBM (top-p, 408 peaked rows of 152064: 88 and 77 us, but 612 of 50000, which L2 holds, 63 and 66).
+    const bool many = by_k ? top_k >= kManyFrom : (int64_t)n_rows * vocab * 2 > kManyBytes;
+    auto cut = gv == 1            ? filter_cut_kernel<1, false>
+               : gv == 8 && !many ? filter_cut_kernel<8, false>
+               : gv == 8          ? filter_cut_kernel<8, true>
+               : gv == 4          ? filter_cut_kernel<4, true>
+                                  : filter_cut_kernel<2, true>;
     int32_t *gave_up = n_open + 1 + n_rows;
-    const int64_t maxima_per_row = (int64_t)L.n_chunks * 32 * kVec / (wide ? kVec : 1);
+    const int64_t maxima_per_row = (int64_t)L.n_chunks * 32 * kVec / gv;
     auto settle = [&](int r0, int n, int32_t *verdict) -> int {
       const uint32_t total = (uint32_t)n * L.n_chunks;
       const unsigned grid = std::min((total + kWarps - 1) / kWarps, (uint32_t)(ctx->sm_count * kScanCtasPerSm));
@@ -1185,11 +1255,12 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
       if (int rc = settle(0, n_probe, nullptr)) return rc;
     if (int rc = settle(n_probe, n_rows - n_probe, n_probe ? gave_up : nullptr)) return rc;
     few = by_k ? window_shape(ctx, 1) : w_open;  // after a top-k hardly ever a row is left
+    if (n_probe) w = window_shape(ctx, n_rows, true);  // rows left open are mostly flat ones
     if (n_probe && few.cluster != w.cluster) {
       int lo = (n_rows + 4) / 5, hi = n_rows;  // `few` is the better one at lo, w at hi
       while (hi - lo > 1) {
         const int mid = lo + (hi - lo) / 2;
-        if (window_us(ctx, few.cluster, mid) <= window_us(ctx, w.cluster, mid)) lo = mid;
+        if (window_us(ctx, few.cluster, mid, true) <= window_us(ctx, w.cluster, mid, true)) lo = mid;
         else hi = mid;
       }
       n_few = lo;
