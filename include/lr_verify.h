@@ -284,7 +284,8 @@ int lr_accept_sample(lr_ctx *ctx, const void *logits_d, int64_t row_stride_elems
  * draft; n_kept_d (nullable, [n_rows]) the size of every row's kept set.
  * Rows, strides and alignment as for lr_accept_greedy; temperature > 0,
  * top_k >= 0, 0 < top_p <= 1, else LR_EINVAL.  scratch_d:
- * lr_accept_sample_filtered_scratch_bytes bytes, 8-byte aligned, no initial
+ * lr_accept_sample_filtered_scratch_bytes bytes (per row about 2 KB and two
+ * bytes for every 8 to 64 tokens, 16 KB at most below 512 K tokens), 8-byte aligned, no initial
  * contents needed; calls sharing it must not overlap on the device.
  */
 int lr_accept_sample_filtered_scratch_bytes(const lr_ctx *ctx, int32_t n_rows, size_t *bytes_out);

@@ -1102,7 +1102,8 @@ ScratchLayout filter_layout(int32_t vocab, int32_t n_rows) {
   };
   s.cuts = take((size_t)n_rows * sizeof(RowCut));
   s.lists = take((size_t)n_rows * kListOut * sizeof(u64));
-  s.maxima = take((size_t)n_rows * s.n_chunks * 32 * kVec * sizeof(uint16_t));
+  // in the smallest groups a top_k can ask for
+  s.maxima = take((size_t)n_rows * s.n_chunks * (32 * kVec / group_vecs(vocab, std::min(vocab, kSelMax))) * sizeof(uint16_t));
   s.stats = take((size_t)n_rows * s.n_chunks * sizeof(float2));
   s.open = take(((size_t)n_rows + 2) * sizeof(int32_t));  // how many, which, and whether the probe gave up
   s.bytes = off;

@@ -147,3 +147,14 @@ def test_routes_agree_on_large_kept_sets(flat, top_k, top_p):
     ua, uf = rng.uniform(0, 1, len(drafts)), rng.uniform(0, 1, nb)
     ua[::3] = 0.0
     _same_in_parts(bf16_round(x), L, 0.6, top_k, top_p, drafts, ua, uf)
+
+
+def test_scratch_does_not_grow_with_groups_nobody_uses():
+    """Per row: the list (2 KB), 32 bytes for the cut, a pair per 2048 tokens and the group maxima, of which there are at most
+    8192 (twice the four times 1024 a top-k can ask for), or one per 64 tokens where that is more, two bytes each."""
+    for vocab in (1000, 32768, 50000, 65536, 65537, 152064, 400003):
+        ctx = B.Context(Model(1, 1, 64, vocab), 0)
+        n_chunks = (vocab + 2047) // 2048
+        groups = min(256 * n_chunks, max(8192 + 256, 32 * n_chunks))
+        assert ctx.accept_sample_filtered_scratch(1000).numel() * 8 <= 1000 * (2048 + 32 + 8 * n_chunks + 2 * groups + 4) + 128, vocab
+        ctx.close()
