@@ -42,7 +42,7 @@ constexpr int kChunk = 32 * kVec * 8;  // logits a warp takes at a time
 constexpr int kScanCtasPerSm = 4;
 constexpr int kGroupCap = 1344;     // groups filter_cut_kernel reads again (k_sel + k_sel / 4 + 4 at most, but for ties)
 constexpr int kListCap = 1408;      // candidates of a row
-constexpr int kSortCap = 2048;      // ... padded to a power of two
+constexpr int kSortCap = 2048;      // ... where many are looked for (a top-k of 1024 finds up to 1284 groups, and ties), to sort
 constexpr int kListOut = 256;       // kept tokens that go out as a list
 constexpr int kManyFrom = 128;      // top_k from which filter_cut_kernel reads many groups at a time and may sort
 constexpr int64_t kManyBytes = 96 << 20;  // ... and the bytes of logits, with top-p alone
@@ -255,7 +255,8 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
                   u64 *__restrict__ lists, int32_t *__restrict__ n_kept_out, int32_t *__restrict__ n_open, int32_t *__restrict__ open_rows,
                   int row0, const int32_t *__restrict__ gave_up) {
   constexpr int kKeyWords = kGV == 4 || kGV == 2 ? 16 : 8;  // words of group maxima a thread keeps in registers
-  __shared__ u64 s_cand[kMany ? kSortCap : kListCap], s_ranked[kMany ? kCountMax : kListCap], s_cum[kListCap];
+  constexpr int kCap = kMany ? kSortCap - 64 : kListCap;
+  __shared__ u64 s_cand[kMany ? kSortCap : kListCap], s_ranked[kMany ? kCountMax : kListCap], s_cum[kCap];
   __shared__ int s_grp[kGroupCap];
   __shared__ int s_n, s_n_grp, s_cnt[2][kWarps], s_kept;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -291,7 +292,7 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
     for (int o = 16; o > 0; o >>= 1) z_all += __shfl_xor_sync(0xFFFFFFFFu, z_all, o);
   }
   // No token weighs more than 1 of z_all: a flat row keeps more than the list of candidates can hold.
-  if (!by_k && __syncthreads_or((double)top_p * z_all > 1.01 * kListCap)) {
+  if (!by_k && __syncthreads_or((double)top_p * z_all > 1.01 * kCap)) {
     if (tid == 0) open_rows[atomicAdd(n_open, 1)] = (int32_t)row;
     return;
   }
@@ -376,7 +377,7 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
           const uint32_t f = (j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16);
           if (__uint_as_float(f) >= least_x) {  // (a NaN is not)
             const int at = atomicAdd(&s_n, 1);
-            if (at < kListCap) s_cand[at] = cand_of(f, at_vec[q] * 8 + j);
+            if (at < kCap) s_cand[at] = cand_of(f, at_vec[q] * 8 + j);
           }
         }
       }
@@ -384,7 +385,7 @@ filter_cut_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32
   }
   __syncthreads();
   const int n = s_n;
-  const bool usable = n_grp <= kGroupCap && n >= 1 && n <= kListCap && (!by_k || n >= top_k);
+  const bool usable = n_grp <= kGroupCap && n >= 1 && n <= kCap && (!by_k || n >= top_k);
   const bool count = !kMany || n <= kCountMax;
   const u64 *s_sorted = count ? s_ranked : s_cand;
   if (usable && count) {

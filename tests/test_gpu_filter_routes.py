@@ -132,7 +132,7 @@ def test_routes_agree(T, offset, top_p):
 
 # The same for a top-k of several hundred (candidates read many at a time, in groups of 64 and of 32, ranked by counting and
 # by sorting, among them many of equal value), and for flat rows, on which the candidates are given up.
-@pytest.mark.parametrize("flat,top_k,top_p", [(0, 130, 0.9131), (0, 200, 1.0), (0, 400, 0.9131), (0, 800, 0.9131), (1, 400, 0.9131), (1, 0, 0.95), (2, 0, 0.95)])
+@pytest.mark.parametrize("flat,top_k,top_p", [(0, 130, 0.9131), (0, 200, 1.0), (0, 400, 0.9131), (0, 800, 0.9131), (0, 1000, 1.0), (1, 400, 0.9131), (1, 0, 0.95), (2, 0, 0.95)])
 def test_routes_agree_on_large_kept_sets(flat, top_k, top_p):
     vocab, nb, L = 152064, 102, 3
     n_rows = nb * (L + 1)
