@@ -1128,8 +1128,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
 // One thread per (query row, 16-byte chunk of channels); a warp holds 32 consecutive rows of one chunk, which
 // is how the partials are laid out ([slot][chunk][row]).  Grid: targets x (head size / 8) CTAs of 256 threads.  The
 // slots are combined in a fixed order.
-template <int kD>
-__global__ void __launch_bounds__(256)
+// What bounds it is the latency of a thread's two trips to memory times the waves of CTAs, not the bytes, which L2 holds: so
+// kBatch = 4 where no M-tile has more slots, which is what a large batch gives (it then has hundreds of M-tiles), with registers
+// for five CTAs on an SM instead of two.  A cycle of 8 ragged requests over four layers 486 -> 477 us, 16 ragged requests
+// 172.9 -> 171.9 (a first pass 225 -> 216), 8 trees 588 -> 586 (674 -> 656); same results.  Where a target has more slots, as few long
+// requests give, eight at a time with three CTAs: one trip to memory instead of two.
+template <int kBatch>
+constexpr int kMergeCtas = kBatch == 4 ? 5 : 3;
+template <int kD, int kBatch>
+__global__ void __launch_bounds__(256, kMergeCtas<kBatch>)
 attn_tc_merge_kernel(DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out, float *__restrict__ lse) {
   const TcTarget g = tc.targets[blockIdx.x];
   const int T = tc.tokens_per_mtile, G = d.group;
@@ -1143,23 +1150,23 @@ attn_tc_merge_kernel(DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out, float
   const int64_t qi = (int64_t)(g.q_row0 + tok) * d.n_q_heads + g.kv_head * G + r % G;
   const float2 *ml = reinterpret_cast<const float2 *>(tc.partial_ml) + (int64_t)g.slot_begin * 128 + r;
   const float4 *po = reinterpret_cast<const float4 *>(tc.partial_o) + ((int64_t)g.slot_begin * (kD / 4) + k) * 128 + r;
-  // Eight slots at a time, the (exponent, sum) pairs and the partial outputs of a batch requested together: one
+  // kBatch slots at a time, the (exponent, sum) pairs and the partial outputs of a batch requested together: one
   // round trip to memory per batch.  The running maximum moves between batches (never within one), in slot order,
   // so the result depends on nothing but the partials.
   float M = -INFINITY, L = 0.f;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int j0 = 0; j0 < g.n_slots; j0 += 8) {
-    float4 o[8];
-    float2 v[8];
+  for (int j0 = 0; j0 < g.n_slots; j0 += kBatch) {
+    float4 o[kBatch];
+    float2 v[kBatch];
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj)
+    for (int jj = 0; jj < kBatch; ++jj)
       if (j0 + jj < g.n_slots) {
         v[jj] = ml[(int64_t)(j0 + jj) * 128];
         o[jj] = po[(int64_t)(j0 + jj) * (kD / 4) * 128];
       }
     float mb = M;
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj)
+    for (int jj = 0; jj < kBatch; ++jj)
       if (j0 + jj < g.n_slots && v[jj].y > 0.f) mb = fmaxf(mb, v[jj].x);  // a stream that saw no key of the row contributes nothing
     if (mb > M) {
       const float a = exp2f(M - mb);  // 0 while nothing has been accumulated (M = -inf)
@@ -1171,7 +1178,7 @@ attn_tc_merge_kernel(DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out, float
       M = mb;
     }
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj)
+    for (int jj = 0; jj < kBatch; ++jj)
       if (j0 + jj < g.n_slots && v[jj].y > 0.f) {
         const float w = exp2f(v[jj].x - M);
         L = fmaf(w, v[jj].y, L);
@@ -1432,6 +1439,7 @@ void tc_plan_structure(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
         memset(&tg, 0, sizeof(tg));
         tg.req = g.list; tg.kv_head = kv; tg.mtile = g.mtile0 + mt;
         tg.slot_begin = n_slots; tg.n_slots = c.n;
+        out.most_slots = std::max(out.most_slots, c.n);
         tg.q_row0 = out.lists[g.list].rq.q_row0; tg.n_q = out.lists[g.list].rq.n_q;
         for (int k = 0; k < c.n; ++k) out.pieces[c.first + k].slot[mt] = n_slots++;
         out.targets.push_back(tg);
@@ -1512,6 +1520,7 @@ void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigne
   t.n_cta = h.n_cta;
   t.n_targets = (int)h.targets.size();
   t.tokens_per_mtile = h.tokens_per_mtile;
+  t.most_slots = h.most_slots;
   t.wait_limit_us = 1000000u;  // one second per wait
   t.phantom_tx_bytes = 0;
   t.partial_ml = reinterpret_cast<float *>(scratch_base + h.s_ml);
@@ -1526,7 +1535,8 @@ static int launch_attn_tc_d(lr_plan *p, const CUtensorMap &kmap, const CUtensorM
   if (int rc = cuda_fail(cudaGetLastError(), "attn_tc_kernel launch")) return rc;
   if (p->tc.n_targets > 0) {  // the merge grid is set up while the attention grid drains
     p->ctx->launches++;
-    return cuda_fail(launch_dependent(attn_tc_merge_kernel<kD>, dim3((unsigned)p->tc.n_targets, kD / 8), dim3(256), 0, s, p->dev, p->tc, out, lse),
+    return cuda_fail(launch_dependent(p->tc.most_slots <= 4 ? attn_tc_merge_kernel<kD, 4> : attn_tc_merge_kernel<kD, 8>,
+                                      dim3((unsigned)p->tc.n_targets, kD / 8), dim3(256), 0, s, p->dev, p->tc, out, lse),
                      "attn_tc_merge_kernel launch");
   }
   return LR_OK;

@@ -101,6 +101,7 @@ struct DevTcPlan {
   const TcReq *reqs;
   const TcTarget *targets;
   int32_t n_cta, n_targets;
+  int32_t most_slots;        // partial slots of the target that has most
   int32_t tokens_per_mtile;  // floor(128 / group)
   uint32_t wait_limit_us;    // bound of every device-side wait (test hook: lr_plan_debug_set_wait_limit)
   uint32_t phantom_tx_bytes; // test hook: bytes CTA 0 expects on its first KV stage beyond what its copies deliver
@@ -246,7 +247,7 @@ struct TcHostPlan {
   std::vector<int32_t> cta_piece_off;
   std::vector<TcTarget> targets;
   size_t o_heads = 0, o_pages = 0, o_rows = 0, o_pieces = 0, o_reqs = 0, o_targets = 0;  // image offsets
-  int n_cta = 0, n_partial_slots = 0, tokens_per_mtile = 0, n_pages = 0;
+  int n_cta = 0, n_partial_slots = 0, most_slots = 0, tokens_per_mtile = 0, n_pages = 0;
   // scratch region behind the image: (exponent, sum) pairs, then fp32 partial outputs
   size_t s_ml = 0, s_o = 0, scratch_bytes = 0;
 };
