@@ -862,16 +862,22 @@ extern "C" int lr_accept_sample_filtered(lr_ctx *ctx, const void *logits, int64_
                                 u_final, n_accept, final_id, p_draft, n_kept, scratch, reinterpret_cast<cudaStream_t>(stream));
 }
 
-extern "C" int lr_commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor,
-                         int32_t *committed, int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid,
-                         int32_t *free_off, int32_t *free_pages, void *stream) {
+static int commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor, int32_t *committed,
+                  int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid, int32_t *free_off, int32_t *free_pages, bool after_accept,
+                  void *stream) {
   if (!p || !n_accept || !n_steps || !survivor || !committed || !keep_off || !keep_pages || !keep_valid || !free_off ||
       !free_pages || (!verdict && p->n_verdicts > 0)) {
     set_error("lr_commit: null argument");
     return LR_EINVAL;
   }
   return launch_commit(p, verdict, n_accept, n_steps, survivor, committed, keep_off, keep_pages, keep_valid, free_off,
-                       free_pages, reinterpret_cast<cudaStream_t>(stream));
+                       free_pages, after_accept, reinterpret_cast<cudaStream_t>(stream));
+}
+
+extern "C" int lr_commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor,
+                         int32_t *committed, int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid,
+                         int32_t *free_off, int32_t *free_pages, void *stream) {
+  return commit(p, verdict, n_accept, n_steps, survivor, committed, keep_off, keep_pages, keep_valid, free_off, free_pages, false, stream);
 }
 
 extern "C" int lr_compact_scratch_bytes(const lr_plan *p, size_t *bytes_out) {
@@ -926,8 +932,8 @@ static int pass_accept_commit(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, voi
   if (int rc = lr_accept_greedy(ctx, io->logits_d, io->logits_stride, io->draft_ids_d, io->cu_draft_d, p->dev.n_branch, io->n_rows,
                                 io->n_accept_d, io->bonus_id_d, io->row_argmax_d, io->accept_scratch_d, stream))
     return rc;
-  return lr_commit(p, io->verdict_d, io->n_accept_d, io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d,
-                   io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d, stream);
+  return commit(p, io->verdict_d, io->n_accept_d, io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d,
+                io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d, true, stream);
 }
 
 extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, float scale, void *side_stream, void *stream) {
@@ -1048,8 +1054,8 @@ static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_
   }
   if (int rc = cuda_fail(cudaStreamWaitEvent(s, p->side.join, 0), "cudaStreamWaitEvent")) return rc;
   if (int rc = accept(b_part, d.n_branch, part_rows, p->n_rows_logits - part_rows)) return rc;
-  if (int rc = lr_commit(p, b + L.verdict, I(L.n_accept), I(L.n_steps), I(L.survivor), I(L.committed), I(L.keep_off),
-                         I(L.keep_pages), I(L.keep_valid), I(L.free_off), I(L.free_pages), stream))
+  if (int rc = commit(p, b + L.verdict, I(L.n_accept), I(L.n_steps), I(L.survivor), I(L.committed), I(L.keep_off), I(L.keep_pages),
+                      I(L.keep_valid), I(L.free_off), I(L.free_pages), true, stream))
     return rc;
   // The ten integer arrays lie next to one another in the staging buffer and leave in one copy, through a pinned buffer the
   // plan keeps, then to the caller's arrays.

@@ -325,8 +325,9 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
                            int32_t *n_kept, void *scratch, cudaStream_t s);
 int launch_compact(lr_plan *p, const int32_t *keep_off, const int32_t *keep_pages, const int32_t *keep_valid, void *k_pool,
                    void *v_pool, int32_t *new_len, int32_t *n_pages_kept, cudaStream_t s);
+// after_accept: the launch before it in the stream is launch_accept's
 int launch_commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor,
                   int32_t *committed, int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid, int32_t *free_off,
-                  int32_t *free_pages, cudaStream_t s);
+                  int32_t *free_pages, bool after_accept, cudaStream_t s);
 
 }  // namespace lr
