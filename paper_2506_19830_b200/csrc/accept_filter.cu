@@ -932,24 +932,48 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int b = blockIdx.x / kC, rank = kC == 1 ? 0 : (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the cuts come from the kernels launched just before
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // Only the cuts come from the kernels launched just before, and the last of those let this one start when everything older
+  // had finished: all else is fetched while it drains (with the commit behind it, 51 rows and top-p alone 35.4 -> 34.9 us, 617
+  // rows with top-k 20 and top-p 0.95 49.6 -> 49.4).
   const int32_t d0 = cu_draft[b], L = cu_draft[b + 1] - d0, r0 = d0 + b;
   const double u_fin = (double)u_final[b];
+  __shared__ int32_t s_draft[kAT];   // the first kAT drafts and their logits
+  __shared__ uint32_t s_logit[kAT];
+  auto draft_of = [&](int i, int32_t &d, uint32_t &f) {
+    d = draft_ids[d0 + i];
+    f = d >= 0 && d < vocab ? (uint32_t)logits[(int64_t)(r0 + i) * row_stride + d] << 16 : 0u;
+  };
+  float u_first = 0.f;
+  if (tid < L) {
+    int32_t d;
+    uint32_t f;
+    draft_of(tid, d, f);
+    s_draft[tid] = d;
+    s_logit[tid] = f;
+    u_first = u_accept[d0 + tid];
+  }
   if (tid == 0) {
     s_n = L;
     s_slice = -1;
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();
 
   // ---- acceptance chain: draft i passes iff u_i < P'_i(d_i); the first one that does not ends it
   for (int i = tid; i < L; i += kAT) {
     const RowCut rc = cuts[r0 + i];
-    const int32_t d = draft_ids[d0 + i];
-    const float u = u_accept[d0 + i];
+    int32_t d;
+    uint32_t f;
+    if (i == tid) {
+      d = s_draft[tid];
+      f = s_logit[tid];
+    } else {
+      draft_of(i, d, f);
+    }
+    const float u = i == tid ? u_first : u_accept[d0 + i];
     float p = 0.f;
     if (d >= 0 && d < vocab && rc.z_fix > 0) {
-      const uint32_t f = (uint32_t)logits[(int64_t)(r0 + i) * row_stride + d] << 16;
       if (is_kept(key32(f), d, rc)) p = (float)wfix_of(f, rc.m, k_log2) / (float)rc.z_fix;
     }
     if (p_draft != nullptr && rank == 0) p_draft[d0 + i] = p;
@@ -967,9 +991,15 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   int32_t dead = -1;
   u64 w_dead = 0;
   if (n < L) {
-    const int32_t d = draft_ids[d0 + n];
+    int32_t d;
+    uint32_t f;
+    if (n < kAT) {
+      d = s_draft[n];
+      f = s_logit[n];
+    } else {
+      draft_of(n, d, f);
+    }
     if (d >= 0 && d < vocab) {
-      const uint32_t f = (uint32_t)rp[d] << 16;
       if (is_kept(key32(f), d, rc)) {
         dead = d;
         w_dead = wfix_of(f, rc.m, k_log2);
