@@ -53,7 +53,7 @@ struct Step {
   int a, surv, drafts, own;        // j*, decisive branch (or -1), its drafts and tail tokens
   int kchain, all, tokens;         // pages of the kept chain spans, of the whole request, tokens of the former
 };
-__device__ __forceinline__ Step decide(const DevBatch &d, const uint8_t *__restrict__ verdict, int r) {
+__device__ __forceinline__ Step decide(const DevBatch &d, const uint8_t *verdict, int r) {
   const int s0 = d.req_span_off[r], s1 = d.req_span_off[r + 1];
   const int b0 = d.req_br_off[r], b1 = d.req_br_off[r + 1];
   const int gamma = s1 - s0 - 1, base = s0 + r;
@@ -124,9 +124,10 @@ __device__ __forceinline__ Slot slot_of(const DevBatch &d, int i) {
 // the decision on a thread's first request too.  Then one trip for n_accept, the scans and the stores are left.  A pass over one request of
 // 4 K tokens 27.9 -> 24.8 us, with head size 64 24.4 -> 23.0; behind the sampled acceptance, plan tables only, 50.3 -> 49.3 and
 // 51.2 -> 49.5 (617 rows without and with filters), 36.0 -> 35.1 (51 rows, top-p).
+// n_accept, and without after_accept the verdicts, may be written while this kernel is resident: neither is __restrict__.
 __global__ void __launch_bounds__(kThreads)
-commit_kernel(DevBatch d, bool after_accept, const uint8_t *__restrict__ verdict,
-              const int32_t *__restrict__ n_accept, int32_t *__restrict__ n_steps_out, int32_t *__restrict__ survivor_out,
+commit_kernel(DevBatch d, bool after_accept, const uint8_t *verdict,
+              const int32_t *n_accept, int32_t *__restrict__ n_steps_out, int32_t *__restrict__ survivor_out,
               int32_t *__restrict__ committed_out, int32_t *__restrict__ keep_off_out, int32_t *__restrict__ keep_pages,
               int32_t *__restrict__ keep_valid, int32_t *__restrict__ free_off_out, int32_t *__restrict__ free_pages) {
   extern __shared__ int32_t sm[];
@@ -152,7 +153,7 @@ commit_kernel(DevBatch d, bool after_accept, const uint8_t *__restrict__ verdict
     const Step st = after_accept && r == tid ? first : decide(d, verdict, r);
     int kept_tail = 0;
     if (st.surv >= 0) {
-      int na = n_accept[st.surv];
+      int na = ld_behind_wait(n_accept + st.surv);
       if (na < 0 || na > st.drafts) {  // not a value the acceptance step can produce
         na = na < 0 ? 0 : st.drafts;
         d.status[0] = kDevBounds;

@@ -276,6 +276,25 @@ void pair_bind_device_plan(const PairHostPlan &h, unsigned char *image_base, uns
 
 void set_error(const char *fmt, ...);
 
+// What the kernel just before wrote, for a kernel that loads other things in front of its griddepcontrol.wait: such words change
+// while this kernel lives, so a load through a `const __restrict__` pointer (which may take the read-only path, or be moved) is
+// not for them, and a line that the early loads brought into L1 can hold some of them.  From L2, in order with the wait.
+template <typename T>
+__device__ __forceinline__ T ld_behind_wait(const T *p) {
+  static_assert(sizeof(T) == 4 || sizeof(T) == 8, "one register or two");
+  T v;
+  if constexpr (sizeof(T) == 4) {
+    uint32_t u;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(u) : "l"(p));
+    memcpy(&v, &u, 4);
+  } else {
+    unsigned long long u;
+    asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(u) : "l"(p));
+    memcpy(&v, &u, 8);
+  }
+  return v;
+}
+
 // Launch as a programmatic dependent of the kernel before it in the stream: the grid is set up while that kernel
 // drains; the kernel itself waits (griddepcontrol.wait) before it touches anything its predecessor wrote.
 template <typename... KArgs, typename... Args>
