@@ -97,6 +97,17 @@ __device__ __forceinline__ u64 wfix_of(uint32_t f, float m, float k_log2) {
   return r;
 }
 
+// a row's cut, behind the wait of a kernel that has loaded other things before (8-byte words: scratch is aligned to no more)
+__device__ __forceinline__ RowCut cut_behind_wait(const RowCut *cut) {
+  static_assert(sizeof(RowCut) == 32 && alignof(RowCut) == 8, "four words");
+  u64 w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w[i] = ld_behind_wait(reinterpret_cast<const u64 *>(cut) + i);
+  RowCut rc;
+  memcpy(&rc, w, sizeof(rc));
+  return rc;
+}
+
 __device__ __forceinline__ bool is_kept(int32_t key, int32_t e, const RowCut &rc) {
   return key > rc.cut_key || (key == rc.cut_key && e <= rc.cut_idx);
 }
@@ -921,7 +932,7 @@ filter_window_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
 template <int kC>
 __global__ void __launch_bounds__(kAT)
 accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2,
-                       const RowCut *__restrict__ cuts, const u64 *__restrict__ lists, int n_slices,
+                       const RowCut * cuts, const u64 * lists, int n_slices,
                        const int32_t *__restrict__ draft_ids, const int32_t *__restrict__ cu_draft,
                        const float *__restrict__ u_accept, const float *__restrict__ u_final, int32_t *__restrict__ n_accept,
                        int32_t *__restrict__ final_id, float *__restrict__ p_draft) {
@@ -939,6 +950,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   const double u_fin = (double)u_final[b];
   __shared__ int32_t s_draft[kAT];   // the first kAT drafts and their logits
   __shared__ uint32_t s_logit[kAT];
+  __shared__ RowCut s_cut[kAT];      // and the cuts of the first kAT rows
   auto draft_of = [&](int i, int32_t &d, uint32_t &f) {
     d = draft_ids[d0 + i];
     f = d >= 0 && d < vocab ? (uint32_t)logits[(int64_t)(r0 + i) * row_stride + d] << 16 : 0u;
@@ -961,8 +973,10 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   __syncthreads();
 
   // ---- acceptance chain: draft i passes iff u_i < P'_i(d_i); the first one that does not ends it
-  for (int i = tid; i < L; i += kAT) {
-    const RowCut rc = cuts[r0 + i];
+  for (int i = tid; i <= L; i += kAT) {
+    const RowCut rc = cut_behind_wait(cuts + r0 + i);
+    if (i < kAT) s_cut[i] = rc;
+    if (i == L) break;  // no draft for the last row
     int32_t d;
     uint32_t f;
     if (i == tid) {
@@ -984,7 +998,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
   if (rank == 0 && tid == 0) n_accept[b] = n;
 
   // ---- the final token: inverse CDF over the kept tokens of the stop row, the rejected one removed
-  const RowCut rc = cuts[r0 + n];
+  const RowCut rc = n < kAT ? s_cut[n] : cut_behind_wait(cuts + r0 + n);
   const bool listed = rc.listed != 0;  // every CTA of the cluster sees the same
   if (listed && rank != 0) return;
   const uint16_t *rp = logits + (int64_t)(r0 + n) * row_stride;
@@ -1014,7 +1028,7 @@ accept_filtered_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, 
     // the smallest index whose cumulative mass exceeds the target: every kept token sums those up to its own index
     const u64 *list = lists + (int64_t)(r0 + n) * kListOut;
     for (int i = tid; i < rc.n_kept; i += kAT) {
-      const u64 e = list[i];
+      const u64 e = ld_behind_wait(list + i);
       s_idx[i] = cand_idx(e);
       s_mass[i] = s_idx[i] == dead ? 0 : wfix_of(f_of_key16(cand_key16(e)), rc.m, k_log2);
     }

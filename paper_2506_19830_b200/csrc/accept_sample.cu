@@ -137,7 +137,7 @@ accept_stats_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int
 
 __global__ void __launch_bounds__(kThreads)
 accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, int32_t vocab, float k_log2,
-                     const float2 *__restrict__ stats, int n_chunks, int chunk, const int32_t *__restrict__ draft_ids,
+                     const float2 *stats, int n_chunks, int chunk, const int32_t *__restrict__ draft_ids,
                      const int32_t *__restrict__ cu_draft, const float *__restrict__ u_accept,
                      const float *__restrict__ u_final, int32_t *__restrict__ n_accept, int32_t *__restrict__ final_id,
                      float *__restrict__ p_draft) {
@@ -182,7 +182,7 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // lr_commit's grid may be set up meanwhile
     const float2 *src = stats + (int64_t)(r0 + i0) * n_chunks;  // consecutive rows are contiguous
-    for (int idx = tid; idx < rows * n_chunks; idx += kThreads) s_st[idx] = src[idx];
+    for (int idx = tid; idx < rows * n_chunks; idx += kThreads) s_st[idx] = ld_behind_wait(src + idx);
     __syncthreads();
     for (int k = warp; k < rows; k += kThreads / 32) {  // one warp per row combines the row's chunk pairs in order
       const float2 *st = s_st + k * n_chunks;

@@ -121,3 +121,52 @@ def test_pass(write_late, n_req, tree):
         assert np.array_equal(late[i].cpu().numpy(), n) and np.array_equal(y.bonus_id.cpu().numpy(), bonus)
         check_commit(y.commit_dict(), O.commit(b, v["verdict"], n))
     ctx.close()
+
+
+@pytest.mark.parametrize("vocab,top_k,top_p", [(20000, None, 1.0), (20000, 20, 1.0), (20000, 300, 0.9), (20000, 0, 0.9), (20000, 5000, 0.7), (4000, 0, 0.9),
+                                               (152064, 0, 0.95)])
+def test_sampled_acceptance(write_late, vocab, top_k, top_p):
+    """Unfiltered (top_k None), through the candidates, through the windows alone, with one and with eight CTAs a branch."""
+    rng = np.random.default_rng(vocab + (top_k or 0))
+    n_branch, n_draft = 5, 62
+    n_rows = n_branch + n_draft
+    model = Model(1, 1, 64, vocab)
+    ctx = B.Context(model, 0)
+    bits = bf16_round((rng.standard_normal((n_rows, vocab)) * 3).astype(np.float32))
+    lg, top = R.bf16_tensor(bits, DEV), O.row_argmax(bits)
+    versions = []
+    for _ in range(3):
+        cu = np.concatenate([[0], np.sort(rng.integers(0, n_draft + 1, n_branch - 1)), [n_draft]]).astype(np.int32)
+        likely = np.concatenate([top[cu[i] + i:cu[i + 1] + i] for i in range(n_branch)])
+        drafts = np.where(rng.random(n_draft) < 0.8, likely, rng.integers(0, vocab, n_draft)).astype(np.int32)
+        versions.append({"n_accept": np.zeros(n_branch, np.int32), "final": np.zeros(n_branch, np.int32), "p_draft": np.zeros(n_draft, np.float32),
+                         "cu": cu, "drafts": drafts, "u_accept": (rng.random(n_draft) * 0.5).astype(np.float32),
+                         "u_final": rng.random(n_branch).astype(np.float32)})
+
+    def call(a, scratch):
+        if top_k is None:
+            ctx.lr_accept_sample(lg, a["drafts"], a["cu"], 0.8, a["u_accept"], a["u_final"], a["n_accept"], a["final"], scratch, a["p_draft"])
+        else:
+            ctx.lr_accept_sample_filtered(lg, a["drafts"], a["cu"], 0.8, top_k, top_p, a["u_accept"], a["u_final"], a["n_accept"], a["final"], scratch,
+                                          a["p_draft"])
+
+    fresh = (lambda: ctx.accept_sample_scratch(n_rows)) if top_k is None else (lambda: ctx.accept_sample_filtered_scratch(n_rows))
+    want = []
+    for v in versions:  # the same call on inputs that have been there for long
+        a = {k: torch.from_numpy(x.copy()).to(DEV) for k, x in v.items()}
+        torch.cuda.synchronize()
+        call(a, fresh())
+        torch.cuda.synchronize()
+        want.append([a[k].cpu() for k in ("n_accept", "final", "p_draft")])
+    mem = Packed(versions, extra=fresh().numel() * 8)
+    mem.buf[:mem.n].copy_(mem.versions[2])
+    got = []
+    torch.cuda.synchronize()
+    for i in range(ROUNDS):
+        write_late(mem.buf, mem.versions[i % 3])
+        call(mem, mem.scratch())
+        got.append([mem[k].clone() for k in ("n_accept", "final", "p_draft")])
+    torch.cuda.synchronize()
+    for i, g in enumerate(got):
+        assert all(torch.equal(x.cpu(), y) for x, y in zip(g, want[i % 3])), i
+    ctx.close()
