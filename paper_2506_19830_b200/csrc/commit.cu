@@ -85,10 +85,11 @@ __device__ __forceinline__ Step decide(const DevBatch &d, const uint8_t *verdict
   return st;
 }
 
-// What the plan says of a page slot: its page, its request and, if it belongs to a span, the span's number in the request
-// (else -1, and the branch), its place in it, what comes before it and the tokens of the span from it on.
+// What the plan says of a page slot that belongs to a span: its page, its request, the span's number in the request (for a
+// tail: ~branch), its place among the pages of that kind, and the tokens of the span from it on (for a tail: its place in the
+// tail).  It stays in registers across the wait, hence few words.
 struct Slot {
-  int pid, r, c, b, idx, before, chain_all, left;
+  int pid, r, part, at, rest;
 };
 __device__ __forceinline__ Slot slot_of(const DevBatch &d, int i) {
   Slot t;
@@ -98,22 +99,17 @@ __device__ __forceinline__ Slot slot_of(const DevBatch &d, int i) {
   t.pid = d.page_ids[i];
   if (item < d.n_span) {
     t.r = d.span_req[item];
-    const int s0 = d.req_span_off[t.r];
-    t.c = item - s0;
-    t.b = -1;
-    t.idx = i - d.span_slot[item];
-    t.before = d.chain_pg[s0 + t.r + t.c];
-    t.chain_all = 0;
-    t.left = d.span_len[item] - t.idx * kPage;
+    const int s0 = d.req_span_off[t.r], idx = i - d.span_slot[item];
+    t.part = item - s0;
+    t.at = d.chain_pg[s0 + t.r + t.part] + idx;
+    t.rest = d.span_len[item] - idx * kPage;
   } else {
-    t.b = item - d.n_span;
-    t.c = -1;
-    t.r = d.br_req[t.b];
+    const int b = item - d.n_span;
+    t.part = ~b;
+    t.r = d.br_req[b];
     const int s0 = d.req_span_off[t.r], s1 = d.req_span_off[t.r + 1], b0 = d.req_br_off[t.r];
-    t.idx = i - d.br_own_slot[t.b];
-    t.before = d.tail_pg[b0 + t.r + (t.b - b0)];
-    t.chain_all = d.chain_pg[s0 + t.r + (s1 - s0)];
-    t.left = 0;
+    t.rest = i - d.br_own_slot[b];
+    t.at = d.chain_pg[s0 + t.r + (s1 - s0)] + d.tail_pg[b0 + t.r + (b - b0)] + t.rest;
   }
   return t;
 }
@@ -194,23 +190,23 @@ commit_kernel(DevBatch d, bool after_accept, const uint8_t *verdict,
     const Slot t = i == slot0 ? first_slot : slot_of(d, i);
     if (t.r < 0) continue;
     const int kchain = s_kchain[t.r];
-    if (t.b < 0) {
-      if (t.c <= s_a[t.r]) {
-        const int dst = s_keep[t.r] + t.before + t.idx;
+    if (t.part >= 0) {
+      if (t.part <= s_a[t.r]) {
+        const int dst = s_keep[t.r] + t.at;
         keep_pages[dst] = t.pid;
-        keep_valid[dst] = min(kPage, t.left);
+        keep_valid[dst] = min(kPage, t.rest);
       } else {
-        free_pages[s_free[t.r] + t.before - kchain + t.idx] = t.pid;
+        free_pages[s_free[t.r] + t.at - kchain] = t.pid;
       }
     } else {
-      const int surv = s_surv[t.r], kp = s_kp[t.r];
-      if (t.b == surv && t.idx < kp) {
-        const int dst = s_keep[t.r] + kchain + t.idx;
+      const int b = ~t.part, surv = s_surv[t.r], kp = s_kp[t.r];
+      if (b == surv && t.rest < kp) {
+        const int dst = s_keep[t.r] + kchain + t.rest;
         keep_pages[dst] = t.pid;
-        keep_valid[dst] = min(kPage, s_kt[t.r] - t.idx * kPage);
+        keep_valid[dst] = min(kPage, s_kt[t.r] - t.rest * kPage);
       } else {
-        const int kept_before = (surv >= 0 && t.b >= surv) ? kp : 0;  // kept pages precede this one in tail order
-        free_pages[s_free[t.r] + t.chain_all - kchain + t.before - kept_before + t.idx] = t.pid;
+        const int kept_before = (surv >= 0 && b >= surv) ? kp : 0;  // kept pages precede this one in tail order
+        free_pages[s_free[t.r] + t.at - kchain - kept_before] = t.pid;
       }
     }
   }
