@@ -24,6 +24,7 @@ constexpr int kStep = 32 * kVec * 8;          // logits a warp takes at a time
 constexpr int kMaxChunks = 160;               // per row: the pairs of kRowBatch rows must fit into 40 KB
 constexpr int kCtasPerSm = 4;
 constexpr int kRowBatch = 32;                 // rows of a branch handled at a time in the chain
+constexpr int kStats = 8;                     // chunk pairs a thread asks for at a time
 
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
@@ -182,7 +183,17 @@ accept_sample_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // lr_commit's grid may be set up meanwhile
     const float2 *src = stats + (int64_t)(r0 + i0) * n_chunks;  // consecutive rows are contiguous
-    for (int idx = tid; idx < rows * n_chunks; idx += kThreads) s_st[idx] = ld_behind_wait(src + idx);
+    for (int at = tid; at < rows * n_chunks; at += kStats * kThreads) {
+      // kStats loads in flight, which is one trip to L2 for 27 rows of 75 chunks; left to a loop of single loads, 617 rows took 49.4 us
+      // with the commit, like this 46.7
+      float2 v[kStats];
+#pragma unroll
+      for (int k = 0; k < kStats; ++k)
+        if (at + k * kThreads < rows * n_chunks) v[k] = ld_behind_wait(src + at + k * kThreads);
+#pragma unroll
+      for (int k = 0; k < kStats; ++k)
+        if (at + k * kThreads < rows * n_chunks) s_st[at + k * kThreads] = v[k];
+    }
     __syncthreads();
     for (int k = warp; k < rows; k += kThreads / 32) {  // one warp per row combines the row's chunk pairs in order
       const float2 *st = s_st + k * n_chunks;
