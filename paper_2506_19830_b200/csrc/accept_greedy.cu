@@ -93,8 +93,10 @@ accept_greedy_kernel(const uint16_t *__restrict__ logits, int64_t row_stride, in
   const int tid = threadIdx.x, lane = tid & 31;
   const int32_t n_vec = vocab >> 3, rem = vocab & 7;
   __shared__ int s_last;
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the logits may come from the kernel launched just before
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // lr_commit's grid may be set up meanwhile
+  // commit_kernel reads the verdicts as soon as this kernel lets it start, so all that is older must have finished by then: that
+  // is why the launch is an ordinary one (which makes the wait a formality), and why the wait comes first.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   for (uint32_t unit = blockIdx.x * (kThreads / 32) + (tid >> 5); unit < total; unit += gridDim.x * (kThreads / 32)) {
     const uint32_t row = unit / n_chunks, c = unit - row * n_chunks;
@@ -241,6 +243,7 @@ int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t
   // a chunk per warp at least, at most kCtasPerSm CTAs per SM
   const uint32_t n_chunks = std::max(1, ((vocab >> 3) + kChunkVecs - 1) / kChunkVecs), total = n_chunks * (uint32_t)n_rows;
   const unsigned grid = std::min((total + kThreads / 32 - 1) / (kThreads / 32), (uint32_t)(ctx->sm_count * kCtasPerSm));
+  // an ordinary launch: see the kernel's first lines
   accept_greedy_kernel<<<grid, kThreads, 0, s>>>(reinterpret_cast<const uint16_t *>(logits), stride, vocab, drafts,
                                                             cu_draft, n_branch, n_rows, first_draft, n_chunks, total, n_accept, bonus, row_argmax,
                                                             reinterpret_cast<unsigned long long *>(scratch));

@@ -115,9 +115,8 @@ __device__ __forceinline__ Slot slot_of(const DevBatch &d, int i) {
 }
 
 // The chain of loads is what this kernel takes, so all of it that does not hang on the kernel just before is gone through while
-// that one drains: what the plan says of a thread's first page slot always, and -- with after_accept, when that kernel is
-// known to be the acceptance, which writes nothing else that is read here and had itself waited for all that came before --
-// the decision on a thread's first request too.  Then one trip for n_accept, the scans and the stores are left.  A pass over one request of
+// that one drains: what the plan says of a thread's first page slot always (its tables come by copies), and -- with after_accept,
+// whose terms stand at launch_commit -- the decision on a thread's first request too.  Then one trip for n_accept, the scans and the stores are left.  A pass over one request of
 // 4 K tokens 27.9 -> 24.8 us, with head size 64 24.4 -> 23.0; behind the sampled acceptance, plan tables only, 50.3 -> 49.3 and
 // 51.2 -> 49.5 (617 rows without and with filters), 36.0 -> 35.1 (51 rows, top-p).
 // n_accept, and without after_accept the verdicts, may be written while this kernel is resident: neither is __restrict__.

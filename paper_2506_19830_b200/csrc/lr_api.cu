@@ -933,7 +933,7 @@ static int pass_accept_commit(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, voi
                                 io->n_accept_d, io->bonus_id_d, io->row_argmax_d, io->accept_scratch_d, stream))
     return rc;
   return commit(p, io->verdict_d, io->n_accept_d, io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d,
-                io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d, true, stream);
+                io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d, /*after_accept=*/p->dev.n_branch > 0, stream);
 }
 
 extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, float scale, void *side_stream, void *stream) {
@@ -1055,7 +1055,7 @@ static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_
   if (int rc = cuda_fail(cudaStreamWaitEvent(s, p->side.join, 0), "cudaStreamWaitEvent")) return rc;
   if (int rc = accept(b_part, d.n_branch, part_rows, p->n_rows_logits - part_rows)) return rc;
   if (int rc = commit(p, b + L.verdict, I(L.n_accept), I(L.n_steps), I(L.survivor), I(L.committed), I(L.keep_off), I(L.keep_pages),
-                      I(L.keep_valid), I(L.free_off), I(L.free_pages), true, stream))
+                      I(L.keep_valid), I(L.free_off), I(L.free_pages), /*after_accept=*/true, stream))
     return rc;
   // The ten integer arrays lie next to one another in the staging buffer and leave in one copy, through a pinned buffer the
   // plan keeps, then to the caller's arrays.

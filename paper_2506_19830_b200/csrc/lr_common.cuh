@@ -296,7 +296,9 @@ __device__ __forceinline__ T ld_behind_wait(const T *p) {
 }
 
 // Launch as a programmatic dependent of the kernel before it in the stream: the grid is set up while that kernel
-// drains; the kernel itself waits (griddepcontrol.wait) before it touches anything its predecessor wrote.
+// drains; the kernel itself waits (griddepcontrol.wait) before it touches anything its predecessor wrote.  Every kernel of this
+// library also waits before it lets its own successor start, so what is older than the predecessor has finished by then: inputs
+// that neither of the two writes may be read in front of the wait, but only behind a predecessor known to be one of these.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -344,7 +346,9 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
                            int32_t *n_kept, void *scratch, cudaStream_t s);
 int launch_compact(lr_plan *p, const int32_t *keep_off, const int32_t *keep_pages, const int32_t *keep_valid, void *k_pool,
                    void *v_pool, int32_t *new_len, int32_t *n_pages_kept, cudaStream_t s);
-// after_accept: the launch before it in the stream is launch_accept's
+// after_accept: the launch before it in the stream is a kernel that does not write the verdicts and that lets its successor start
+// only once everything older has finished -- launch_accept's, which is launched ordinarily.  The verdicts are then read while it
+// still runs (for a chain of steps; the tree kernel reads them behind its wait either way).
 int launch_commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor,
                   int32_t *committed, int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid, int32_t *free_off,
                   int32_t *free_pages, bool after_accept, cudaStream_t s);

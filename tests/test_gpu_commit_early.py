@@ -1,5 +1,5 @@
 """Commit behind the acceptance of the same call: a thread's first request and first page slot are gone through before the
-acceptance counts are there, the others behind.  On both sides of one request a thread, with more page slots than threads."""
+acceptance counts are there, the others behind.  On both sides of one request a thread; the largest batch has more page slots than threads."""
 import numpy as np
 import pytest
 
