@@ -286,3 +286,27 @@ def test_logit_shapes_that_move_the_window(seed):
     ua, uf = rng.uniform(0, 1, nb * L), rng.uniform(0, 1, nb)
     got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, T, top_k, top_p, ua, uf)
     _check(bits, drafts, cu, T, top_k, top_p, ua, uf, got, max_ambiguous_frac=1.0)
+
+
+# With 1000 tokens a token at a top-p of 0.9 holds some 5e-4 of the mass and the two cuts are 4e-5 of it apart: one row in twelve has
+# a heavy token between them, so hardly a branch of 512 rows has none, and none would be compared.  Of 16392 tokens, one there
+# holds about 4e-5.  A top-k has one cut.
+@pytest.mark.parametrize("vocab,top_k,top_p", [(1000, 300, 1.0), (16392, 20, 1.0), (16392, 300, 1.0), (16392, 0, 0.9)])
+def test_branches_longer_than_the_drafts_fetched_ahead(vocab, top_k, top_p):
+    """Branches of 512 drafts and more: the first 512 drafts, logits and cuts of a branch are fetched or kept ahead, the others read
+    where they are needed.  The first rejected draft lies on either side, or there is none."""
+    rng = np.random.default_rng(vocab + top_k)
+    lens, stops = [512, 513, 7, 600, 600], [512, 512, 3, 511, 590]
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    n_rows = int(cu[-1]) + len(lens)
+    bits = bf16_round((rng.standard_normal((n_rows, vocab)) * 2).astype(np.float32))
+    top = O.row_argmax(bits)
+    drafts = np.concatenate([top[cu[b] + b:cu[b + 1] + b] for b in range(len(lens))]).astype(np.int32)
+    ua = np.zeros(len(drafts))  # the most likely token is always kept, and accepted by a uniform of 0 ...
+    for b, (n, stop) in enumerate(zip(lens, stops)):
+        if stop < n:
+            ua[cu[b] + stop] = 0.9999  # ... and rejected by this one, unless it is nearly alone
+    uf = rng.uniform(0, 1, len(lens))
+    got = _run(Model(1, 1, 64, vocab), bits, drafts, cu, 1.0, top_k, top_p, ua, uf)
+    assert got[0].tolist() == stops
+    _check(bits, drafts, cu, 1.0, top_k, top_p, ua, uf, got, max_ambiguous_frac=0.2, rows_to_check=list(range(0, n_rows, 50)))
