@@ -1128,11 +1128,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
 // One thread per (query row, 16-byte chunk of channels); a warp holds 32 consecutive rows of one chunk, which
 // is how the partials are laid out ([slot][chunk][row]).  Grid: targets x (head size / 8) CTAs of 256 threads.  The
 // slots are combined in a fixed order.
-// What bounds it is the latency of a thread's two trips to memory times the waves of CTAs, not the bytes, which L2 holds: so
-// kBatch = 4 where no M-tile has more slots, which is what a large batch gives (it then has hundreds of M-tiles), with registers
-// for five CTAs on an SM instead of two.  A cycle of 8 ragged requests over four layers 486 -> 477 us, 16 ragged requests
-// 172.9 -> 171.9 (a first pass 225 -> 216), 8 trees 588 -> 586 (674 -> 656); same results.  Where a target has more slots, as few long
-// requests give, eight at a time with three CTAs: one trip to memory instead of two.
+// What bounds it is the latency of a thread's two trips to memory times the waves of CTAs, not the bytes, which L2 holds.  Where no
+// M-tile has more than four slots, which is what a large batch gives (it has hundreds of M-tiles), a thread therefore has four in
+// flight, in 43 registers: five CTAs on an SM.  Eight take 70 registers, three CTAs.  With eight for every plan and as it is, in
+// turn: 16 ragged requests 171.8 -> 169.6 us a pass (two runs of one side differ by 0.3 %), a cycle of 8 ragged requests over four
+// layers 483 -> 475 (1 %), 8 trees 588 both; same results.  The rule looks at the target with most slots, so one long
+// request among many short ones takes all of them through the wider form.  Where a target has more slots, as few long requests
+// give, eight at a time make one trip of two.
 template <int kBatch>
 constexpr int kMergeCtas = kBatch == 4 ? 5 : 3;
 template <int kD, int kBatch>
