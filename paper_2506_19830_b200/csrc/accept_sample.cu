@@ -7,9 +7,9 @@
 // the final token by inverse CDF over the stop row with the rejected token removed: first over the chunk weights
 // S_c exp((M_c - m) / T) (no second pass over the row), then inside the one chunk that holds the target, which is read
 // again and prefix-summed.  Every reduction has a fixed order: same inputs, same output.  The second kernel is a chain of
-// latencies (about 10 us behind the first, half of it instruction fetch); what does not depend on the statistics it reads
-// while the first one drains, one butterfly sums a row and one scan finds the chunk: 617 rows, both and the commit 51.7 ->
-// 49.9 us.
+// latencies (some 8 us behind the first); what does not depend on the statistics it reads while the first one drains, the
+// statistics of a branch mostly come in one trip, one butterfly sums a row and one scan finds the chunk: 617 rows, both and the
+// commit 51.7 -> 46.8 us.
 #include <algorithm>
 
 #include "lr_common.cuh"
