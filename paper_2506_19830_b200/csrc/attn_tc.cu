@@ -32,7 +32,7 @@
 //               shared memory as 1024-byte swizzle atoms, the two channel halves of
 //               an 8-key group side by side (groups 2048 bytes apart): the layout
 //               the MMA descriptors read with SBO = 2048.  One box per page rather
-//               than one per page half matters: the producer spends about 70
+//               than one per page half matters: the producer spends about 100
 //               cycles per box, and 32 boxes per tile made it a bottleneck.
 //               Every copy is for this CTA alone.
 //   warps 9, 10 MMA issuers of stream 0 and 1 (warp 11 idles): tcgen05.mma (M=128, K=16, bf16 ->
@@ -630,8 +630,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
   const TcCtaHead *head = tc.heads + blockIdx.x;
   const int piece0 = head->piece0, piece1 = head->piece1;
   // What it takes to start is asked for at once, beside the set-up, and all of this lies in front of the wait for the kernel
-  // before: a CTA's first copies are then issued some hundred cycles behind that wait instead of 3700 behind its entry.  One
-  // request of 256 tokens 12.3 -> 9.5 us, of 4 K 18.8 -> 16.7, with head size 64 18.5 -> 16.2 (attention alone, back to back).
+  // before: a CTA's first copies are then issued 2400 cycles behind that wait instead of 3700 behind its entry.  One request of
+  // 256 tokens 12.3 -> 10.2 us, of 4 K 19.1 -> 17.1, with head size 64 18.5 -> 16.5, 32 of 1200 55.5 -> 53 (attention alone, back to
+  // back).  (One elected lane issuing a tile's boxes, 70 cycles each, gave the short ones another 0.2 us and cost the last 2.5.)
   // The producer and the issuers read the record from shared memory; in the softmax threads, for which nothing waits here, that
   // cost the sweep registers.
   if (warp == 8) {
@@ -696,71 +697,69 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
     // ======================= TMA producer ==========================================
     uint32_t ring = 0, q_count = 0;
     bool ok = true;
-    const uint32_t q_box_bytes = (uint32_t)(64 * G * T * 2), q_addr = smem_u32(q_smem), kv_addr = smem_u32(kv_smem);
-    // a page id as the copies use it: never outside the pool
-    auto checked = [&](int32_t pg, int code) -> int32_t {
-      if (pg >= 0 && pg < d.n_pool_pages) return pg;
-      d.status[0] = kDevBounds;
-      d.status[1] = code;
-      return 0;
-    };
+    const uint32_t q_box_bytes = (uint32_t)(64 * G * T * 2);
     for (int pc = piece0; pc < piece1 && ok; ++pc) {
       const TcPiece pi = pc == piece0 ? head->first : tc.pieces[pc];
       const TcReq rq = pc == piece0 ? head->first_req : tc.reqs[pi.req];
       const int n = pi.tile_end - pi.tile_begin;
-      const RingOrder ord(n, pi.n_mt);
-      // Page ids arrive 32 at a time (one per lane = 4 tiles) and one chunk ahead of their first use; nothing looks at them
-      // before that, so no step of the loop waits for a load it has just issued.  Lanes past the list hold page 0, for
-      // which no copy is issued.
-      auto load_chunk = [&](int c) -> int32_t { return c * 32 + lane < rq.n_pages ? tc.pages[rq.page_off + c * 32 + lane].page : 0; };
-      int c_cur = pi.tile_begin >> 2;
-      int32_t pg_cur, pg_nxt = load_chunk(c_cur + 1);
-      if (pc == piece0) pg_cur = c_cur * 32 + lane < rq.n_pages ? checked(head->first_pages[lane], 201) : 0;  // comes with the CTA head
-      else pg_cur = checked(load_chunk(c_cur), 200);
       // Q tiles of the piece, once the MMAs of the previous piece no longer read the buffers
-      if (q_count > 0) ok = wait_bar(&ctrl->q_empty, (q_count & 1u) ^ 1u, ctrl, d.status, 205);
+      ok = wait_bar(&ctrl->q_empty, (q_count & 1u) ^ 1u, ctrl, d.status, 205);
       if (!ok) break;
-      if (elect_one()) {
-        mbar_arrive_expect_tx(&ctrl->q_full, (uint32_t)(pi.n_mt * kHalves) * q_box_bytes);
-#pragma unroll
-        for (int h = 0; h < 2 * kHalves; ++h)
-          if (h < kHalves * pi.n_mt)
-            tma_load_3d(q_addr + h * kHalfBytes, &q_map, (h % kHalves) * 64, pi.kv_head * G, rq.q_row0 + (pi.mtile0 + h / kHalves) * T, &ctrl->q_full);
-      }
+      if (lane == 0) mbar_arrive_expect_tx(&ctrl->q_full, (uint32_t)(pi.n_mt * kHalves) * q_box_bytes);
       __syncwarp();
+      if (lane < kHalves * pi.n_mt)
+        tma_load_3d(smem_u32(q_smem) + lane * kHalfBytes, &q_map, (lane % kHalves) * 64, pi.kv_head * G,
+                    rq.q_row0 + (pi.mtile0 + lane / kHalves) * T, &ctrl->q_full);
       ++q_count;
+      const RingOrder ord(n, pi.n_mt);
+      // Page ids arrive 32 at a time (one per lane = 4 tiles) and one chunk ahead of their first use,
+      // so no step of the loop waits for a load it has just issued.
+      auto load_chunk = [&](int c) -> int32_t {
+        const int idx = c * 32 + lane;
+        int32_t pg = -1;  // absent page
+        if (idx < rq.n_pages) {
+          pg = tc.pages[rq.page_off + idx].page;
+          if (pg < 0 || pg >= d.n_pool_pages) {  // never fetch outside the pool
+            d.status[0] = kDevBounds;
+            d.status[1] = 200;
+            pg = 0;
+          }
+        }
+        return pg;
+      };
+      int c_cur = pi.tile_begin >> 2;
+      int32_t pg_nxt = load_chunk(c_cur + 1), pg_cur;
+      if (pc == piece0) {  // the first chunk of the first piece comes with the CTA head
+        pg_cur = head->first_pages[lane];
+        if (c_cur * 32 + lane < rq.n_pages && (pg_cur < 0 || pg_cur >= d.n_pool_pages)) {
+          d.status[0] = kDevBounds;
+          d.status[1] = 201;
+          pg_cur = 0;
+        }
+      } else {
+        pg_cur = load_chunk(c_cur);
+      }
       for (int i = 0; i < 2 * n && ok; ++i, ++ring) {
         bool is_v;
         const int t = pi.tile_begin + ord.step(i, is_v);
         if (is_v && (t >> 2) > c_cur) {  // the V index is the oldest tile still needed
           ++c_cur;
-          pg_cur = checked(pg_nxt, 200);
+          pg_cur = pg_nxt;
           pg_nxt = load_chunk(c_cur + 1);
         }
-        // One lane issues the boxes of a tile, four pages at a time: 70 cycles a box, where a copy that every lane issues for
-        // its own page is run lane by lane, 100 cycles each.
-        const int32_t page = (t >> 2) == c_cur ? pg_cur : checked(pg_nxt, 200);
-        const int32_t w = (int32_t)(((int64_t)page * d.n_kv_heads + pi.kv_head) * 2);  // in 8-key groups
+        const int32_t page = __shfl_sync(0xFFFFFFFFu, (t >> 2) == c_cur ? pg_cur : pg_nxt, (t & 3) * 8 + (lane & 7));
         const int npages = min(kPagesPerTile, rq.n_pages - t * kPagesPerTile);
         const uint32_t stage = ring % kStages;
-        if (ring >= (uint32_t)kStages) ok = wait_bar(&ctrl->kv_empty[stage], ((ring / kStages) & 1u) ^ 1u, ctrl, d.status, 210);
+        ok = wait_bar(&ctrl->kv_empty[stage], ((ring / kStages) & 1u) ^ 1u, ctrl, d.status, 210);
         if (!ok) break;
-        const uint32_t dst = kv_addr + stage * kTileBytes;
-        const CUtensorMap *map = is_v ? &v_map : &k_map;
-#pragma unroll
-        for (int p0 = 0; p0 < kPagesPerTile; p0 += 4) {
-          int32_t at[4];
-#pragma unroll
-          for (int p = 0; p < 4; ++p) at[p] = __shfl_sync(0xFFFFFFFFu, w, (t & 3) * 8 + p0 + p);
-          if (elect_one()) {
-            if (p0 == 0)
-              mbar_arrive_expect_tx(&ctrl->kv_full[stage], (uint32_t)(npages * 2 * kGroupBytes) + ((blockIdx.x == 0 && ring == 0) ? tc.phantom_tx_bytes : 0u));
-#pragma unroll
-            for (int p = 0; p < 4; ++p)  // one box per page: two 8-key groups, all channels
-              if (p0 + p < npages) tma_load_4d(dst + (p0 + p) * (2 * kGroupBytes), map, 0, 0, 0, at[p], &ctrl->kv_full[stage]);
-          }
-        }
+        if (lane == 0)
+          mbar_arrive_expect_tx(&ctrl->kv_full[stage], (uint32_t)(npages * 2 * kGroupBytes) + ((blockIdx.x == 0 && ring == 0) ? tc.phantom_tx_bytes : 0u));
         __syncwarp();
+        if (lane < 8 && page >= 0) {  // one box per page: two 8-key groups, all channels
+          const uint32_t dst = smem_u32(kv_smem + stage * kTileBytes) + lane * (2 * kGroupBytes);
+          tma_load_4d(dst, is_v ? &v_map : &k_map, 0, 0, 0, (int32_t)(((int64_t)page * d.n_kv_heads + pi.kv_head) * 2),
+                      &ctrl->kv_full[stage]);
+        }
       }
     }
     if (!ok) {
