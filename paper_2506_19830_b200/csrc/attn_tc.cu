@@ -75,7 +75,7 @@
 
 #include <algorithm>
 
-#include "lr_common.cuh"
+#include "attn_merge.cuh"
 
 namespace lr {
 
@@ -281,11 +281,6 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t *>(&t);
-}
-
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -1142,76 +1137,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant_
   }
 }
 
-// Merge of the partials of one M-tile: O = sum_j 2^(m_j - M) O_j / sum_j 2^(m_j - M) l_j.
-// One thread per (query row, 16-byte chunk of channels); a warp holds 32 consecutive rows of one chunk, which
-// is how the partials are laid out ([slot][chunk][row]).  Grid: targets x (head size / 8) CTAs of 256 threads.  The
-// slots are combined in a fixed order.
-// What bounds it is the latency of a thread's two trips to memory times the waves of CTAs, not the bytes, which L2 holds.  Where no
-// M-tile has more than four slots, which is what a large batch gives (it has hundreds of M-tiles), a thread therefore has four in
-// flight, in 43 registers: five CTAs on an SM.  Eight take 70 registers, three CTAs.  With eight for every plan and as it is, in
-// turn: 16 ragged requests 171.8 -> 169.6 us a pass (two runs of one side differ by 0.3 %), a cycle of 8 ragged requests over four
-// layers 483 -> 475 (1 %), 8 trees 588 both; same results.  The rule looks at the target with most slots, so one long
-// request among many short ones takes all of them through the wider form.  Where a target has more slots, as few long requests
-// give, eight at a time make one trip of two.
-template <int kBatch>
-constexpr int kMergeCtas = kBatch == 4 ? 5 : 3;
 template <int kD, int kBatch>
 __global__ void __launch_bounds__(256, kMergeCtas<kBatch>)
 attn_tc_merge_kernel(DevBatch d, DevTcPlan tc, uint16_t *__restrict__ out, float *__restrict__ lse) {
-  const TcTarget g = tc.targets[blockIdx.x];
-  const int T = tc.tokens_per_mtile, G = d.group;
-  const int item = blockIdx.y * 256 + threadIdx.x;  // 0 .. kD / 4 * 128 - 1
-  const int k = item >> 7, r = item & 127;           // chunk of 4 channels, row
-  const int tok = g.mtile * T + r / G;
-  const bool live = r < T * G && tok < g.n_q;
-  // the partials come from the kernel launched just before this one
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (!live) return;
-  const int64_t qi = (int64_t)(g.q_row0 + tok) * d.n_q_heads + g.kv_head * G + r % G;
-  const float2 *ml = reinterpret_cast<const float2 *>(tc.partial_ml) + (int64_t)g.slot_begin * 128 + r;
-  const float4 *po = reinterpret_cast<const float4 *>(tc.partial_o) + ((int64_t)g.slot_begin * (kD / 4) + k) * 128 + r;
-  // kBatch slots at a time, the (exponent, sum) pairs and the partial outputs of a batch requested together: one
-  // round trip to memory per batch.  The running maximum moves between batches (never within one), in slot order,
-  // so the result depends on nothing but the partials.
-  float M = -INFINITY, L = 0.f;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int j0 = 0; j0 < g.n_slots; j0 += kBatch) {
-    float4 o[kBatch];
-    float2 v[kBatch];
-#pragma unroll
-    for (int jj = 0; jj < kBatch; ++jj)
-      if (j0 + jj < g.n_slots) {
-        v[jj] = ml[(int64_t)(j0 + jj) * 128];
-        o[jj] = po[(int64_t)(j0 + jj) * (kD / 4) * 128];
-      }
-    float mb = M;
-#pragma unroll
-    for (int jj = 0; jj < kBatch; ++jj)
-      if (j0 + jj < g.n_slots && v[jj].y > 0.f) mb = fmaxf(mb, v[jj].x);  // a stream that saw no key of the row contributes nothing
-    if (mb > M) {
-      const float a = exp2f(M - mb);  // 0 while nothing has been accumulated (M = -inf)
-      L *= a;
-      acc.x *= a;
-      acc.y *= a;
-      acc.z *= a;
-      acc.w *= a;
-      M = mb;
-    }
-#pragma unroll
-    for (int jj = 0; jj < kBatch; ++jj)
-      if (j0 + jj < g.n_slots && v[jj].y > 0.f) {
-        const float w = exp2f(v[jj].x - M);
-        L = fmaf(w, v[jj].y, L);
-        acc.x = fmaf(w, o[jj].x, acc.x);
-        acc.y = fmaf(w, o[jj].y, acc.y);
-        acc.z = fmaf(w, o[jj].z, acc.z);
-        acc.w = fmaf(w, o[jj].w, acc.w);
-      }
-  }
-  const float inv = 1.0f / L;
-  uint2 pk = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
-  *reinterpret_cast<uint2 *>(out + qi * kD + k * 4) = pk;
-  if (lse != nullptr && k == 0) lse[qi] = (M + log2f(L)) * 0.6931471805599453f;
+  merge_cta<kD, kBatch>(d, tc, blockIdx.x, blockIdx.y, out, lse);
 }
 
 // ---- tensor maps -------------------------------------------------------------------
@@ -1389,7 +1318,27 @@ void tc_plan_structure(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
     total_tiles += (int64_t)n_kv * g.n_tiles;
     most = std::max<int64_t>(most, (int64_t)(kPieceStartTiles * kDense + kMasked) * g.weight);
   }
-  const int64_t max_cta = std::min<int64_t>(ctx->sm_count, std::max<int64_t>(1, max_ctas_for_tiles(total_tiles)));
+  int64_t max_cta = std::min<int64_t>(ctx->sm_count, std::max<int64_t>(1, max_ctas_for_tiles(total_tiles)));
+  if (m_step == 1) {
+    // A small pass lasts as long as its longest chain of dependent steps, so its acceptance runs beside attention, on SMs left free
+    // for it (pass_tail.cu), if that can be done before attention and the merge are through and costs attention at most a tenth by
+    // the first estimate.  (Fewer CTAs also leave fewer partial results to merge: 144 and 112 both take 16.5 us for one request of
+    // 4 K tokens.)  Where the logits are too many for that all SMs are attention's: eight requests of 350 tokens with 124 MB of
+    // logits take 41 us either way, and their attention alone 16.4 instead of 22.4.  Microseconds on a B200: attention 4.1 and one
+    // for every 50 of load, logits 2 and 45 KB an SM, the merge 4.
+    int64_t rows = b->n_branch;
+    for (int i = 0; i < b->n_branch; ++i) rows += b->br_n_draft[i];
+    const double start = (double)(kPieceStartTiles * kDense) * grps[0].weight, w = (double)total_w - start * n_kv * (double)grps.size();
+    const double bytes = 2.0 * ctx->model.vocab * (double)rows;
+    auto attention = [&](int64_t n) { return 4.1 + (w / (double)n + start) / 50.0; };
+    auto logits = [&](int64_t n) { return 2.0 + bytes / (45e3 * (double)(ctx->sm_count - n)); };
+    const double most_time = 1.1 * attention(max_cta);
+    for (int64_t n = std::min<int64_t>(max_cta, ctx->sm_count - 1); n >= 1 && attention(n) <= most_time && !out.small; --n)
+      if (logits(n) <= attention(n) + 4.0) {
+        out.small = true;
+        max_cta = n;
+      }
+  }
   // walks the partition for limit L; with `emit` it also records the pieces.  A group is a run of dense tiles
   // followed by a run of masked ones, each of uniform cost, so a walk takes O(CTAs + groups) steps.
   struct Contrib { int first, n; };
@@ -1541,6 +1490,7 @@ void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigne
   t.n_targets = (int)h.targets.size();
   t.tokens_per_mtile = h.tokens_per_mtile;
   t.most_slots = h.most_slots;
+  t.small = h.small;
   t.wait_limit_us = 1000000u;  // one second per wait
   t.phantom_tx_bytes = 0;
   t.partial_ml = reinterpret_cast<float *>(scratch_base + h.s_ml);
@@ -1549,14 +1499,14 @@ void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigne
 
 template <int kD>
 static int launch_attn_tc_d(lr_plan *p, const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &qmap, const RawInputs &in, uint16_t *out,
-                            float *lse, float scale_log2, cudaStream_t s) {
+                            float *lse, float scale_log2, bool merge, cudaStream_t s) {
   p->ctx->launches++;
   // set up while the kernel before it drains (a layer's merge, or what is left of the pass before)
   if (int rc = cuda_fail(launch_dependent(attn_tc_kernel<kD>, dim3((unsigned)p->tc.n_cta), dim3(kThreads), Shape<kD>::kSmemBytes, s, kmap, vmap, qmap, p->dev,
                                           p->tc, in, out, lse, scale_log2),
                          "attn_tc_kernel launch"))
     return rc;
-  if (p->tc.n_targets > 0) {  // the merge grid is set up while the attention grid drains
+  if (merge && p->tc.n_targets > 0) {  // the merge grid is set up while the attention grid drains
     p->ctx->launches++;
     return cuda_fail(launch_dependent(p->tc.most_slots <= 4 ? attn_tc_merge_kernel<kD, 4> : attn_tc_merge_kernel<kD, 8>,
                                       dim3((unsigned)p->tc.n_targets, kD / 8), dim3(256), 0, s, p->dev, p->tc, out, lse),
@@ -1565,7 +1515,7 @@ static int launch_attn_tc_d(lr_plan *p, const CUtensorMap &kmap, const CUtensorM
   return LR_OK;
 }
 
-int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
+int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale, bool merge,
                    cudaStream_t s) {
   const CUtensorMap *mp = nullptr;
   if (int rc = get_map(p->ctx, 0, k, p->dev.n_pool_pages, &mp)) return rc;
@@ -1577,7 +1527,7 @@ int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void
   const float scale_log2 = scale * 1.4426950408889634f;
   const RawInputs in = {reinterpret_cast<const uint16_t *>(q), reinterpret_cast<const uint16_t *>(k), reinterpret_cast<const uint16_t *>(v)};
   return (p->dev.head_dim == 128 ? launch_attn_tc_d<128> : launch_attn_tc_d<64>)(p, kmap, vmap, qmap, in, reinterpret_cast<uint16_t *>(out), lse,
-                                                                                scale_log2, s);
+                                                                                scale_log2, merge, s);
 }
 
 }  // namespace lr

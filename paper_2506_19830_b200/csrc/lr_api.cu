@@ -712,8 +712,7 @@ extern "C" int lr_plan_debug_set_page(lr_plan *p, int32_t page_slot, int32_t new
 }
 
 // ---- steps ---------------------------------------------------------------------
-extern "C" int lr_verify_attention(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse,
-                                   float scale, void *stream) {
+static int check_attention(const lr_plan *p, const void *q, const void *k, const void *v, const void *out, const float *lse) {
   if (!p || !q || !k || !v || !out) {
     set_error("lr_verify_attention: null argument");
     return LR_EINVAL;
@@ -722,6 +721,12 @@ extern "C" int lr_verify_attention(lr_plan *p, const void *q, const void *k, con
     set_error("lr_verify_attention: q, pools and out must be 16-byte aligned");
     return LR_EINVAL;
   }
+  return LR_OK;
+}
+
+extern "C" int lr_verify_attention(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse,
+                                   float scale, void *stream) {
+  if (int rc = check_attention(p, q, k, v, out, lse)) return rc;
   if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)p->dev.head_dim);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (p->attention_path == 3) {
@@ -737,7 +742,7 @@ extern "C" int lr_verify_attention(lr_plan *p, const void *q, const void *k, con
       set_error("lr_verify_attention: the tensor-core path does not support this shape");
       return LR_EUNSUPPORTED;
     }
-    return launch_attn_tc(p, q, k, v, out, lse, scale, s);
+    return launch_attn_tc(p, q, k, v, out, lse, scale, true, s);
   }
   return launch_attn_generic(p, q, k, v, out, lse, scale, s);
 }
@@ -751,9 +756,8 @@ extern "C" int lr_accept_scratch_bytes(int32_t n_rows, size_t *bytes_out) {
   return LR_OK;
 }
 
-extern "C" int lr_accept_greedy(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts,
-                                const int32_t *cu_draft, int32_t n_branch, int32_t n_rows, int32_t *n_accept,
-                                int32_t *bonus, int32_t *row_argmax, void *scratch, void *stream) {
+static int check_accept(const lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft, int32_t n_branch,
+                        int32_t n_rows, const int32_t *n_accept, const int32_t *bonus, const void *scratch) {
   if (!ctx || !logits || !cu_draft || !n_accept || !bonus || !scratch || (!drafts && n_rows > n_branch)) {
     set_error("lr_accept_greedy: null argument");
     return LR_EINVAL;
@@ -766,6 +770,13 @@ extern "C" int lr_accept_greedy(lr_ctx *ctx, const void *logits, int64_t stride,
     set_error("lr_accept_greedy: logits must be 16-byte aligned with a row stride that is a multiple of 8 and >= vocab");
     return LR_EINVAL;
   }
+  return LR_OK;
+}
+
+extern "C" int lr_accept_greedy(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts,
+                                const int32_t *cu_draft, int32_t n_branch, int32_t n_rows, int32_t *n_accept,
+                                int32_t *bonus, int32_t *row_argmax, void *scratch, void *stream) {
+  if (int rc = check_accept(ctx, logits, stride, drafts, cu_draft, n_branch, n_rows, n_accept, bonus, scratch)) return rc;
   if (n_branch == 0) return LR_OK;
   return launch_accept(ctx, logits, stride, drafts, cu_draft, n_branch, n_rows, 0, n_accept, bonus, row_argmax, scratch,
                        reinterpret_cast<cudaStream_t>(stream));
@@ -862,22 +873,24 @@ extern "C" int lr_accept_sample_filtered(lr_ctx *ctx, const void *logits, int64_
                                 u_final, n_accept, final_id, p_draft, n_kept, scratch, reinterpret_cast<cudaStream_t>(stream));
 }
 
-static int commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor, int32_t *committed,
-                  int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid, int32_t *free_off, int32_t *free_pages, bool after_accept,
-                  void *stream) {
-  if (!p || !n_accept || !n_steps || !survivor || !committed || !keep_off || !keep_pages || !keep_valid || !free_off ||
-      !free_pages || (!verdict && p->n_verdicts > 0)) {
+static int check_commit(const lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, const CommitOut &o) {
+  if (!p || !n_accept || !o.n_steps || !o.survivor || !o.committed || !o.keep_off || !o.keep_pages || !o.keep_valid || !o.free_off ||
+      !o.free_pages || (!verdict && p->n_verdicts > 0)) {
     set_error("lr_commit: null argument");
     return LR_EINVAL;
   }
-  return launch_commit(p, verdict, n_accept, n_steps, survivor, committed, keep_off, keep_pages, keep_valid, free_off,
-                       free_pages, after_accept, reinterpret_cast<cudaStream_t>(stream));
+  return LR_OK;
+}
+
+static int commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, const CommitOut &o, bool after_accept, void *stream) {
+  if (int rc = check_commit(p, verdict, n_accept, o)) return rc;
+  return launch_commit(p, verdict, n_accept, o, after_accept, reinterpret_cast<cudaStream_t>(stream));
 }
 
 extern "C" int lr_commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor,
                          int32_t *committed, int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid,
                          int32_t *free_off, int32_t *free_pages, void *stream) {
-  return commit(p, verdict, n_accept, n_steps, survivor, committed, keep_off, keep_pages, keep_valid, free_off, free_pages, false, stream);
+  return commit(p, verdict, n_accept, CommitOut{n_steps, survivor, committed, keep_off, keep_pages, keep_valid, free_off, free_pages}, false, stream);
 }
 
 extern "C" int lr_compact_scratch_bytes(const lr_plan *p, size_t *bytes_out) {
@@ -928,12 +941,31 @@ extern "C" int lr_poll_status(lr_plan *p, void *stream, int32_t *detail) {
 }
 
 // ---- whole pass on device buffers ----------------------------------------------------
-static int pass_accept_commit(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, void *stream) {
-  if (int rc = lr_accept_greedy(ctx, io->logits_d, io->logits_stride, io->draft_ids_d, io->cu_draft_d, p->dev.n_branch, io->n_rows,
-                                io->n_accept_d, io->bonus_id_d, io->row_argmax_d, io->accept_scratch_d, stream))
-    return rc;
-  return commit(p, io->verdict_d, io->n_accept_d, io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d,
-                io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d, /*after_accept=*/p->dev.n_branch > 0, stream);
+static CommitOut commit_out(const lr_pass_io *io) {
+  return {io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d, io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d};
+}
+
+// Acceptance and commit on a second stream beside attention: they fill the SMs that it leaves idle.  (Which of the two comes first
+// makes no difference.)  One kernel where the pass is a small one, two else.
+static int pass_side_by_side(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, float scale, bool one_kernel, cudaStream_t side, cudaStream_t s) {
+  if (int rc = take_side(p)) return rc;
+  cudaError_t e = cudaEventRecord(p->side.fork, s);
+  if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
+  if (int rc = lr_verify_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, s)) return rc;
+  if (!side) side = p->side.s;
+  e = cudaStreamWaitEvent(side, p->side.fork, 0);
+  if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
+  int rc;
+  if (one_kernel) {
+    rc = launch_pass_tail(p, io, /*behind_attention=*/false, side);
+  } else {
+    rc = lr_accept_greedy(ctx, io->logits_d, io->logits_stride, io->draft_ids_d, io->cu_draft_d, p->dev.n_branch, (int32_t)io->n_rows, io->n_accept_d,
+                          io->bonus_id_d, io->row_argmax_d, io->accept_scratch_d, side);
+    if (rc == LR_OK) rc = commit(p, io->verdict_d, io->n_accept_d, commit_out(io), /*after_accept=*/p->dev.n_branch > 0, side);
+  }
+  e = cudaEventRecord(p->side.join, side);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->side.join, 0);
+  return rc != LR_OK ? rc : cuda_fail(e, "lr_verify_pass: join");
 }
 
 extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, float scale, void *side_stream, void *stream) {
@@ -942,21 +974,22 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
     return LR_EINVAL;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), side = reinterpret_cast<cudaStream_t>(side_stream);
-  if (int rc = take_side(p)) return rc;
-  // Attention, then acceptance and commit beside it: they fill the SMs while its last CTAs, the merge of its partial results
-  // and the gaps between launches leave them idle.  (Which of the two comes first makes no difference.)  As three calls one
-  // after another and so: the smallest request 20.6 and 12.5 us, one of 4 K tokens 36.0 and 28.5, of 32 K 93.2 and 86.9, four
-  // of 16 K 110 and 102.
-  cudaError_t e = cudaEventRecord(p->side.fork, s);
-  if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
-  if (int rc = lr_verify_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, stream)) return rc;
-  if (!side) side = p->side.s;
-  e = cudaStreamWaitEvent(side, p->side.fork, 0);
-  if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
-  const int rc = pass_accept_commit(ctx, p, io, side);
-  e = cudaEventRecord(p->side.join, side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->side.join, 0);
-  return rc != LR_OK ? rc : cuda_fail(e, "lr_verify_pass: join");
+  const bool tc = p->tc_ok && (p->attention_path == 0 || p->attention_path == 2);
+  if (!tc || !pass_tail_fits(p, io->n_rows)) return pass_side_by_side(ctx, p, io, scale, false, side, s);
+  if (int rc = check_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d)) return rc;
+  if (int rc = check_accept(ctx, io->logits_d, io->logits_stride, io->draft_ids_d, io->cu_draft_d, p->dev.n_branch, (int32_t)io->n_rows, io->n_accept_d,
+                            io->bonus_id_d, io->accept_scratch_d))
+    return rc;
+  if (int rc = check_commit(p, io->verdict_d, io->n_accept_d, commit_out(io))) return rc;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (int rc = cuda_fail(cudaStreamIsCapturing(s, &capture), "cudaStreamIsCapturing")) return rc;
+  // On one stream, two kernels in a row of which the second is set up, and mostly done, while the first runs (pass_tail.cu), there
+  // are no events between two passes, and the next attention is set up early too.  A caller who gives a second stream has a reason
+  // to order work with it.  And in a graph events cost nothing: beside an attention of few CTAs the rest is a root of its own.
+  if (side || (capture != cudaStreamCaptureStatusNone && 2 * p->tc.n_cta <= ctx->sm_count)) return pass_side_by_side(ctx, p, io, scale, true, side, s);
+  if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)p->dev.head_dim);
+  if (int rc = launch_attn_tc(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/false, s)) return rc;
+  return launch_pass_tail(p, io, /*behind_attention=*/true, s);
 }
 
 // ---- whole pass from host buffers --------------------------------------------------
@@ -1054,9 +1087,8 @@ static int issue_pass_host(lr_plan *p, const lr_pass_host_io *io, const void *k_
   }
   if (int rc = cuda_fail(cudaStreamWaitEvent(s, p->side.join, 0), "cudaStreamWaitEvent")) return rc;
   if (int rc = accept(b_part, d.n_branch, part_rows, p->n_rows_logits - part_rows)) return rc;
-  if (int rc = commit(p, b + L.verdict, I(L.n_accept), I(L.n_steps), I(L.survivor), I(L.committed), I(L.keep_off), I(L.keep_pages),
-                      I(L.keep_valid), I(L.free_off), I(L.free_pages), /*after_accept=*/true, stream))
-    return rc;
+  const CommitOut lists = {I(L.n_steps), I(L.survivor), I(L.committed), I(L.keep_off), I(L.keep_pages), I(L.keep_valid), I(L.free_off), I(L.free_pages)};
+  if (int rc = commit(p, b + L.verdict, I(L.n_accept), lists, /*after_accept=*/true, stream)) return rc;
   // The ten integer arrays lie next to one another in the staging buffer and leave in one copy, through a pinned buffer the
   // plan keeps, then to the caller's arrays.
   e = cudaMemcpyAsync(p->results_pinned, b + L.n_accept, L.scratch - L.n_accept, cudaMemcpyDeviceToHost, s);

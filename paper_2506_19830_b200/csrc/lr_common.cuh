@@ -102,6 +102,7 @@ struct DevTcPlan {
   const TcTarget *targets;
   int32_t n_cta, n_targets;
   int32_t most_slots;        // partial slots of the target that has most
+  int32_t small;             // planned with SMs left for the acceptance
   int32_t tokens_per_mtile;  // floor(128 / group)
   uint32_t wait_limit_us;    // bound of every device-side wait (test hook: lr_plan_debug_set_wait_limit)
   uint32_t phantom_tx_bytes; // test hook: bytes CTA 0 expects on its first KV stage beyond what its copies deliver
@@ -248,6 +249,7 @@ struct TcHostPlan {
   std::vector<TcTarget> targets;
   size_t o_heads = 0, o_pages = 0, o_rows = 0, o_pieces = 0, o_reqs = 0, o_targets = 0;  // image offsets
   int n_cta = 0, n_partial_slots = 0, most_slots = 0, tokens_per_mtile = 0, n_pages = 0;
+  bool small = false;
   // scratch region behind the image: (exponent, sum) pairs, then fp32 partial outputs
   size_t s_ml = 0, s_o = 0, scratch_bytes = 0;
 };
@@ -326,8 +328,12 @@ int launch_attn_pair(lr_plan *p, const void *q, const void *k, const void *v, vo
                      cudaStream_t s);
 int launch_attn_generic(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
                         cudaStream_t s);
-int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
+// without `merge` the partial results are left for launch_pass_tail
+int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale, bool merge,
                    cudaStream_t s);
+// The rest of a small pass: acceptance and commit, and behind a launch_attn_tc without merge that too; and whether a pass is one.
+bool pass_tail_fits(const lr_plan *p, int64_t n_rows);
+int launch_pass_tail(lr_plan *p, const lr_pass_io *io, bool behind_attention, cudaStream_t s);
 // first_draft: what cu_draft counts in front of the first branch's rows (a later part of a batch whose rows are given alone)
 int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
                   int32_t n_branch, int32_t n_rows, int32_t first_draft, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,
@@ -348,9 +354,10 @@ int launch_compact(lr_plan *p, const int32_t *keep_off, const int32_t *keep_page
                    void *v_pool, int32_t *new_len, int32_t *n_pages_kept, cudaStream_t s);
 // after_accept: the launch before it in the stream is a kernel that does not write the verdicts and that lets its successor start
 // only once everything older has finished -- launch_accept's, which is launched ordinarily.  The verdicts are then read while it
-// still runs (for a chain of steps; the tree kernel reads them behind its wait either way).
-int launch_commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, int32_t *n_steps, int32_t *survivor,
-                  int32_t *committed, int32_t *keep_off, int32_t *keep_pages, int32_t *keep_valid, int32_t *free_off,
-                  int32_t *free_pages, bool after_accept, cudaStream_t s);
+// still runs.
+struct CommitOut {
+  int32_t *n_steps, *survivor, *committed, *keep_off, *keep_pages, *keep_valid, *free_off, *free_pages;
+};
+int launch_commit(lr_plan *p, const uint8_t *verdict, const int32_t *n_accept, const CommitOut &o, bool after_accept, cudaStream_t s);
 
 }  // namespace lr
