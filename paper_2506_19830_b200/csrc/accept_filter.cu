@@ -1283,15 +1283,12 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
       const uint16_t *from = lg + (int64_t)r0 * stride;
       uint16_t *to = maxima + r0 * maxima_per_row;
       float2 *to_stats = stats + (int64_t)r0 * L.n_chunks;
-      if (verdict) {
-        if (int rc = cuda_fail(launch_dependent(scan, dim3(grid), dim3(kT), 0, s, from, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, to,
-                                                to_stats, n_open, kProbeRows, verdict),
-                               "filter_scan_kernel launch"))
-          return rc;
-      } else {
-        scan<<<grid, kT, 0, s>>>(from, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, to, to_stats, n_open, kProbeRows, verdict);
-        if (int rc = cuda_fail(cudaGetLastError(), "filter_scan_kernel launch")) return rc;
-      }
+      // (also as the first kernel of a call it is set up while whatever is before it drains: 617 rows, top-k 20 and top-p 0.95, with
+      // the commit of the call before 49.3 -> 47.9 us, 45 rows of 1081 tokens 18.6 -> 17.6)
+      if (int rc = cuda_fail(launch_dependent(scan, dim3(grid), dim3(kT), 0, s, from, stride, vocab, k_log2, (uint32_t)L.n_chunks, total, to, to_stats,
+                                              n_open, kProbeRows, verdict),
+                             "filter_scan_kernel launch"))
+        return rc;
       return cuda_fail(launch_dependent(cut, dim3((unsigned)n), dim3(kT), 0, s, lg, stride, vocab, k_log2, top_k, top_p, k_sel, L.n_chunks, maxima,
                                         stats, cuts, lists, n_kept, n_open, n_open + 1, r0, (const int32_t *)verdict),
                        "filter_cut_kernel launch");
