@@ -32,7 +32,7 @@ accept_greedy_kernel(AcceptWork w, const int32_t *__restrict__ draft_ids, const 
   const int tid = threadIdx.x, lane = tid & 31;
   __shared__ int s_last;
   // commit_kernel reads the verdicts as soon as this kernel lets it start, so all that is older must have finished by then: that
-  // is why the launch is an ordinary one (which makes the wait a formality), and why the wait comes first.
+  // is why the wait comes first.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
@@ -106,10 +106,11 @@ int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t
   const AcceptWork w = accept_work(ctx, logits, stride, n_rows, scratch, kVecPerThread);
   // a chunk per warp at least, at most kCtasPerSm CTAs per SM
   const unsigned grid = std::min((w.total + kThreads / 32 - 1) / (kThreads / 32), (uint32_t)(ctx->sm_count * kCtasPerSm));
-  // an ordinary launch: see the kernel's first lines
-  accept_greedy_kernel<<<grid, kThreads, 0, s>>>(w, drafts, cu_draft, n_branch, n_rows, first_draft, n_accept, bonus, row_argmax);
+  // set up while whatever is before it drains; see the kernel's first lines
   ctx->launches++;
-  return cuda_fail(cudaGetLastError(), "accept_greedy_kernel launch");
+  return cuda_fail(launch_dependent(accept_greedy_kernel, dim3(grid), dim3(kThreads), 0, s, w, drafts, cu_draft, n_branch, n_rows, first_draft, n_accept, bonus,
+                                    row_argmax),
+                   "accept_greedy_kernel launch");
 }
 
 }  // namespace lr

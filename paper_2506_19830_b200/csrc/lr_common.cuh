@@ -353,7 +353,7 @@ int launch_accept_filtered(lr_ctx *ctx, const void *logits, int64_t stride, cons
 int launch_compact(lr_plan *p, const int32_t *keep_off, const int32_t *keep_pages, const int32_t *keep_valid, void *k_pool,
                    void *v_pool, int32_t *new_len, int32_t *n_pages_kept, cudaStream_t s);
 // after_accept: the launch before it in the stream is a kernel that does not write the verdicts and that lets its successor start
-// only once everything older has finished -- launch_accept's, which is launched ordinarily.  The verdicts are then read while it
+// only once everything older has finished -- launch_accept's, which waits in its first line.  The verdicts are then read while it
 // still runs.
 struct CommitOut {
   int32_t *n_steps, *survivor, *committed, *keep_off, *keep_pages, *keep_valid, *free_off, *free_pages;
