@@ -69,7 +69,7 @@ __device__ __forceinline__ Best better(Best a, Best b) {
 struct AcceptWork {
   const uint16_t *logits;
   int64_t row_stride;
-  unsigned long long *scratch;  // [0] two counters, [1..] row keys; zeros between calls
+  unsigned long long *scratch;  // [0] counters, [1..] row keys; zeros between calls
   int32_t vocab;
   uint32_t n_chunks, total;
 };

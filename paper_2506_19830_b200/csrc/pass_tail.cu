@@ -7,7 +7,7 @@
 // others run on SMs that the plan has left free (tc_plan_structure): first the CTAs of the commit, which go through their plan
 // tables and then wait for the row keys, then those that stream the logits.  When attention ends, the merge is all that is left.
 // A pass, four kernels and two: 256 tokens 12.7 -> 11.7 us, 4 K tokens 24.6 -> 18.8, with head size 64 22.8 -> 16.9, one of 8 K
-// 29.3 -> 23.6, two of 100 to 400 tokens with 0.1 to 2 MB of logits 18 -> 12.
+// 29.3 -> 23.6, small batches of other shapes by 0 to 40 %.
 //
 // What streams is warps: an SM's rate grows with them and hardly with the loads a lane has in flight (one SM alone: 8 warps 30
 // GB/s, 16 54, 32 80 to 90, with four, eight or sixteen 16-byte loads a lane).  A warp takes consecutive units and publishes once
