@@ -957,7 +957,7 @@ static int pass_side_by_side(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, floa
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
   int rc;
   if (one_kernel) {
-    rc = launch_pass_tail(p, io, /*behind_attention=*/false, side);
+    rc = launch_pass_tail(ctx, p, io, /*behind_attention=*/false, side);
   } else {
     rc = lr_accept_greedy(ctx, io->logits_d, io->logits_stride, io->draft_ids_d, io->cu_draft_d, p->dev.n_branch, (int32_t)io->n_rows, io->n_accept_d,
                           io->bonus_id_d, io->row_argmax_d, io->accept_scratch_d, side);
@@ -975,7 +975,7 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream), side = reinterpret_cast<cudaStream_t>(side_stream);
   const bool tc = p->tc_ok && (p->attention_path == 0 || p->attention_path == 2);
-  if (!tc || !pass_tail_fits(p, io->n_rows)) return pass_side_by_side(ctx, p, io, scale, false, side, s);
+  if (!tc || !pass_tail_fits(ctx, p, io->n_rows)) return pass_side_by_side(ctx, p, io, scale, false, side, s);
   if (int rc = check_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d)) return rc;
   if (int rc = check_accept(ctx, io->logits_d, io->logits_stride, io->draft_ids_d, io->cu_draft_d, p->dev.n_branch, (int32_t)io->n_rows, io->n_accept_d,
                             io->bonus_id_d, io->accept_scratch_d))
@@ -989,7 +989,7 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
   if (side || (capture != cudaStreamCaptureStatusNone && 2 * p->tc.n_cta <= ctx->sm_count)) return pass_side_by_side(ctx, p, io, scale, true, side, s);
   if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)p->dev.head_dim);
   if (int rc = launch_attn_tc(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/false, s)) return rc;
-  return launch_pass_tail(p, io, /*behind_attention=*/true, s);
+  return launch_pass_tail(ctx, p, io, /*behind_attention=*/true, s);
 }
 
 // ---- whole pass from host buffers --------------------------------------------------

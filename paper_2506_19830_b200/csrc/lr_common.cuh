@@ -332,8 +332,9 @@ int launch_attn_generic(lr_plan *p, const void *q, const void *k, const void *v,
 int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale, bool merge,
                    cudaStream_t s);
 // The rest of a small pass: acceptance and commit, and behind a launch_attn_tc without merge that too; and whether a pass is one.
-bool pass_tail_fits(const lr_plan *p, int64_t n_rows);
-int launch_pass_tail(lr_plan *p, const lr_pass_io *io, bool behind_attention, cudaStream_t s);
+// The acceptance goes by the context of the call, which need not be the plan's: its vocabulary may be another.
+bool pass_tail_fits(const lr_ctx *ctx, const lr_plan *p, int64_t n_rows);
+int launch_pass_tail(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, bool behind_attention, cudaStream_t s);
 // first_draft: what cu_draft counts in front of the first branch's rows (a later part of a batch whose rows are given alone)
 int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,
                   int32_t n_branch, int32_t n_rows, int32_t first_draft, int32_t *n_accept, int32_t *bonus, int32_t *row_argmax,

@@ -159,15 +159,15 @@ auto tail_kernel(bool tree) {
 
 }  // namespace
 
-bool pass_tail_fits(const lr_plan *p, int64_t n_rows) {
-  const int vecs = p->ctx->model.vocab >> 3, unit = 32 * kVecPerThread;
+bool pass_tail_fits(const lr_ctx *ctx, const lr_plan *p, int64_t n_rows) {
+  const int vecs = ctx->model.vocab >> 3, unit = 32 * kVecPerThread;
   return p->tc.small && p->dev.n_req <= kMostRequests && p->dev.n_page_slots <= kCommitSlots &&
          n_rows * std::max(1, (vecs + unit - 1) / unit) <= (int64_t)kMostUnits;
 }
 
-int launch_pass_tail(lr_plan *p, const lr_pass_io *io, bool behind_attention, cudaStream_t s) {
+int launch_pass_tail(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, bool behind_attention, cudaStream_t s) {
   const DevBatch &d = p->dev;
-  PassAccept a = {accept_work(p->ctx, io->logits_d, io->logits_stride, (int32_t)io->n_rows, io->accept_scratch_d, kVecPerThread),
+  PassAccept a = {accept_work(ctx, io->logits_d, io->logits_stride, (int32_t)io->n_rows, io->accept_scratch_d, kVecPerThread),
                   io->draft_ids_d, io->cu_draft_d, io->n_accept_d, io->bonus_id_d, io->row_argmax_d, d.n_branch, (int32_t)io->n_rows};
   a.n_commit = std::min(commit_ctas(d), kCommitCtas);
   // a warp's share: what the places beside attention stream in one go (the plan has made sure that they are enough)
@@ -182,7 +182,7 @@ int launch_pass_tail(lr_plan *p, const lr_pass_io *io, bool behind_attention, cu
                                         : (few ? tail_kernel<64, 4>(d.tree) : tail_kernel<64, 8>(d.tree));
   const size_t smem = (size_t)d.n_req * (d.tree ? kCommitSmemPerReq<true> : kCommitSmemPerReq<false>);
   uint16_t *out = reinterpret_cast<uint16_t *>(io->out_d);
-  p->ctx->launches++;
+  ctx->launches++;
   if (!behind_attention) {  // an ordinary launch: most CTAs do not wait for what is just before
     kernel<<<a.n_commit + a.n_stream, kThreads, smem, s>>>(d, p->tc, out, io->lse_d, a, io->verdict_d, o);
     return cuda_fail(cudaGetLastError(), "pass_tail_kernel launch");
