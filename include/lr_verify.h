@@ -188,6 +188,18 @@ typedef struct lr_plan_info {
 } lr_plan_info;
 int lr_plan_describe(const lr_plan *plan, lr_plan_info *info_out);
 
+/* How the attention work of a batch is split on a device of n_sm SMs, worked out on the host without one.  For testing.
+ *   attention   the partition of lr_verify_attention
+ *   pass        that of lr_verify_pass on one stream: another one where a small pass needs SMs for its acceptance
+ *   small_pass  1 if lr_verify_pass may take the form for small passes
+ *   longest_load  what the longest CTA has to do, about a 50th of a microsecond each */
+typedef struct lr_partition_info {
+  int32_t n_cta, n_merge_targets, n_partial_slots;
+  int64_t longest_load;
+} lr_partition_info;
+int lr_debug_partitions(const lr_model *model, const lr_batch *batch, int32_t n_sm, lr_partition_info *attention_out,
+                        lr_partition_info *pass_out, int32_t *small_pass_out);
+
 /* Selects the attention implementation for later lr_verify_attention calls on
  * this plan: 0 = automatic (tensor-core path when the shape allows it), 1 =
  * force the CUDA-core path (every shape), 2 = force the tensor-core path, 3 =

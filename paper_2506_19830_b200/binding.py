@@ -55,6 +55,10 @@ class lr_plan_info(C.Structure):
                                          "n_merge_targets", "n_partial_slots")]
 
 
+class lr_partition_info(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in ("n_cta", "n_merge_targets", "n_partial_slots")] + [("longest_load", C.c_int64)]
+
+
 class lr_pass_host_io(C.Structure):
     _fields_ = [(n, C.c_void_p) for n in (
         "q_h", "logits_h", "draft_ids_h", "verdict_h", "out_h", "n_accept_h", "bonus_id_h", "n_steps_accepted_h",
@@ -86,6 +90,8 @@ def lib() -> C.CDLL:
             "lr_plan_destroy": [vp],
             "lr_plan_set_attention_path": [vp, C.c_int],
             "lr_plan_describe": [vp, C.POINTER(lr_plan_info)],
+            "lr_debug_partitions": [C.POINTER(lr_model), C.POINTER(lr_batch), i32, C.POINTER(lr_partition_info), C.POINTER(lr_partition_info),
+                                    C.POINTER(i32)],
             "lr_plan_debug_set_page": [vp, i32, i32, vp],
             "lr_plan_debug_set_wait_limit": [vp, C.c_uint32],
             "lr_plan_debug_set_phantom_bytes": [vp, C.c_uint32],
@@ -170,6 +176,16 @@ def lr_validate_batch(model, batch) -> None:
     hb = HostBatch(batch)
     m = _model_struct(model)
     _check(lib().lr_validate_batch(C.byref(m), C.byref(hb.c)), "lr_validate_batch")
+
+
+def lr_debug_partitions(model, batch, n_sm: int):
+    """(attention, pass, small): how the attention work of a batch is split on a device of ``n_sm`` SMs."""
+    hb, m, small = HostBatch(batch), _model_struct(model), C.c_int32()
+    parts = [lr_partition_info(), lr_partition_info()]
+    _check(lib().lr_debug_partitions(C.byref(m), C.byref(hb.c), n_sm, C.byref(parts[0]), C.byref(parts[1]), C.byref(small)),
+           "lr_debug_partitions")
+    attention, whole_pass = ({n: int(getattr(p, n)) for n, _ in p._fields_} for p in parts)
+    return attention, whole_pass, bool(small.value)
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

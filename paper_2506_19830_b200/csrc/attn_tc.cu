@@ -74,6 +74,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <numeric>
 
 #include "attn_merge.cuh"
 
@@ -1220,6 +1221,171 @@ int init_attn_tc_kernel() {
 // most CTAs worth using for a number of tiles (tiny problems: not one CTA per tile, their partial results cost more than they save)
 static int64_t max_ctas_for_tiles(int64_t tiles) { return tiles >= 64 ? tiles : tiles / 2; }
 
+namespace {
+
+constexpr double kMostAttention = 1.25;  // of plan_small_pass
+
+struct TcGrp { int list, mtile0, n_mt, n_tiles, n_dense, weight; };  // one per list; every KV head repeats it
+
+// Contiguous partition of the tile sequence (groups in order, tiles in order) over at most max_cta CTAs that
+// minimises the largest CTA load.  A tile costs its group's weight (10 with one M-tile, 16 with two: per-CTA cycle
+// counts on the ragged serving workload gave 2360 and 3790 cycles a tile); every piece -- a CTA's share of one
+// group -- costs kPieceStartTiles tiles more (Q load, pipeline ramp, epilogue: measured 1.7 to 1.8 tiles), so a CTA
+// that spans a group boundary gets fewer tiles; a tile that needs masks (anything past the full prefix pages) costs 8/5 of a dense one (measured: 1.3 to 2.3 times, depending on the workload; 9/5 was no better).  For a load limit L the greedy fill (a CTA takes tiles while it stays within L) needs the fewest
+// CTAs possible; the smallest feasible L is found by bisection.  At most one CTA per two tiles: smaller shares
+// only add partial results to merge.
+class Partitioner {
+ public:
+  Partitioner(const std::vector<TcGrp> &groups, int kv_heads) : grps(groups), n_kv(kv_heads) {
+    for (const TcGrp &g : grps) {
+      total_w += (int64_t)n_kv * g.weight * (kPieceStartTiles * kDense + g.n_dense * kDense + (g.n_tiles - g.n_dense) * kMasked);
+      total_tiles += (int64_t)n_kv * g.n_tiles;
+      most = std::max<int64_t>(most, (int64_t)(kPieceStartTiles * kDense + kMasked) * g.weight);
+      unit = std::gcd(unit, g.weight);
+    }
+  }
+  // what a piece costs before its first tile, and all tiles of the batch
+  int64_t piece_start() const { return (int64_t)kPieceStartTiles * kDense * grps[0].weight; }
+  int64_t tile_load() const { return total_w - piece_start() * n_kv * (int64_t)grps.size(); }
+  int64_t n_tiles() const { return total_tiles; }
+  // the smallest load limit that max_cta CTAs can hold
+  int64_t least_limit(int64_t max_cta) const {
+    // No partition stays below the average load, and a greedy fill does not exceed it by more than a piece start and a tile
+    // per CTA, or nearly so: the bisection starts from there.
+    const int64_t lo = std::max(most, (total_w + max_cta - 1) / max_cta), hi = lo + 2 * most;
+    return least_limit(max_cta, lo, holds(hi, max_cta) ? hi : std::max(hi, total_w));  // one CTA takes everything
+  }
+  // the same from lo on, where hi is known to do.  All loads are multiples of a unit, and so need the limits be.
+  int64_t least_limit(int64_t max_cta, int64_t lo, int64_t hi) const {
+    lo /= unit;
+    hi /= unit;
+    while (lo < hi) {
+      const int64_t mid = lo + (hi - lo) / 2;
+      if (holds(mid * unit, max_cta)) hi = mid; else lo = mid + 1;
+    }
+    return lo * unit;
+  }
+  bool holds(int64_t L, int64_t max_cta) const { return walk(L, max_cta, nullptr, nullptr) <= max_cta; }
+  void fill(int64_t L, const std::vector<TcList> &lists, TcPartition &out) const;
+
+ private:
+  static constexpr int kPieceStartTiles = 2, kDense = 5, kMasked = 8;  // costs in fifths of a dense tile
+  struct Contrib { int first, n; };
+  int64_t walk(int64_t L, int64_t max_cta, TcPartition *out, std::vector<Contrib> *contrib) const;
+
+  const std::vector<TcGrp> &grps;
+  const int n_kv;
+  int64_t total_w = 0, total_tiles = 0, most = 0;
+  int unit = 0;
+};
+
+// Walks the partition for limit L; with `out` it also records the pieces.  A group is a run of dense tiles
+// followed by a run of masked ones, each of uniform cost, so a walk takes O(CTAs + groups) steps.
+int64_t Partitioner::walk(int64_t L, int64_t max_cta, TcPartition *out, std::vector<Contrib> *contrib) const {
+  int64_t n = 0, load = 0;
+  for (const TcGrp &g : grps) {
+    const int64_t start = (int64_t)kPieceStartTiles * kDense * g.weight;
+    for (int kv = 0; kv < n_kv; ++kv) {
+      const int first = out ? (int)out->pieces.size() : 0;
+      bool new_piece = true;
+      int t = 0;
+      while (t < g.n_tiles) {
+        const int run_end = t < g.n_dense ? g.n_dense : g.n_tiles;
+        const int64_t cost = (int64_t)g.weight * (t < g.n_dense ? kDense : kMasked);
+        if (n == 0 || load + cost + (new_piece ? start : 0) > L) {  // open the next CTA: its share of this group is a new piece
+          ++n;
+          load = 0;
+          new_piece = true;
+          if (out) out->cta_piece_off.push_back((int32_t)out->pieces.size());
+          else if (n > max_cta) return n;
+        }
+        if (new_piece) load += start;
+        const int k = (int)std::max<int64_t>(1, std::min<int64_t>(run_end - t, (L - load) / cost));
+        load += (int64_t)k * cost;
+        if (out) {
+          if (new_piece) {
+            TcPiece p;
+            p.req = g.list; p.kv_head = kv; p.mtile0 = g.mtile0; p.n_mt = g.n_mt; p.tile_begin = t; p.tile_end = t + k;
+            p.slot[0] = p.slot[1] = -2;
+            out->pieces.push_back(p);
+          } else {
+            out->pieces.back().tile_end = t + k;
+          }
+          out->longest = std::max(out->longest, load);
+        }
+        new_piece = false;
+        t += k;
+      }
+      if (out) contrib->push_back({first, (int)out->pieces.size() - first});
+    }
+  }
+  return n;
+}
+
+void Partitioner::fill(int64_t L, const std::vector<TcList> &lists, TcPartition &out) const {
+  std::vector<Contrib> contrib;  // the pieces of every (list, KV head), in that order of grps x heads
+  out.n_cta = (int)walk(L, 0, &out, &contrib);
+  out.cta_piece_off.push_back((int32_t)out.pieces.size());
+  // Targets (one M-tile of one group) and the streams that contribute to them, in piece order; the two streams of a
+  // one-M-tile piece are combined inside the CTA.
+  size_t at = 0;
+  for (const TcGrp &g : grps)
+    for (int kv = 0; kv < n_kv; ++kv, ++at)
+      for (int mt = 0; mt < g.n_mt; ++mt) {
+        const Contrib c = contrib[at];
+        if (c.n == 1) {
+          out.pieces[c.first].slot[mt] = -1;
+          continue;
+        }
+        TcTarget tg;
+        memset(&tg, 0, sizeof(tg));
+        tg.req = g.list; tg.kv_head = kv; tg.mtile = g.mtile0 + mt;
+        tg.slot_begin = out.n_partial_slots; tg.n_slots = c.n;
+        out.most_slots = std::max(out.most_slots, c.n);
+        tg.q_row0 = lists[g.list].rq.q_row0; tg.n_q = lists[g.list].rq.n_q;
+        for (int k = 0; k < c.n; ++k) out.pieces[c.first + k].slot[mt] = out.n_partial_slots++;
+        out.targets.push_back(tg);
+      }
+}
+
+// Whether the whole pass on a small plan goes as in pass_tail.cu, and on which partition.
+// A small pass lasts as long as its longest chain of dependent steps, so its acceptance runs beside attention, on SMs left free for
+// it, if that can be done before attention and the merge are through and the average CTA takes at most a tenth more.  Where the
+// partition over all SMs does not leave enough of them, the pass has one of its own: attention by itself, which a serving loop
+// runs once a layer, keeps all SMs (16 requests of 500 tokens, 32 query heads: 16.0 us on 128 CTAs and 25.5 on 110; 16 of 100: 9.3
+// and 17.3).  Shares are whole tiles, so the longest CTA of the narrower one may take more than the average says: up to
+// kMostAttention (four requests of 500 tokens: 1.2, the pass 17.5 us where attention first and acceptance behind it take 21.3; of 100:
+// 1.2, 14.5 and 21), and never a merge that attention did without (those two: 26.6 against 23.9, and 19.7 against 17.0).  Where that
+// rules it out the pass is still one of its kind if what attention leaves free gets through the logits sooner than all SMs do behind
+// it (16 requests of 100 tokens, 5 query heads, 73 MB of logits: 17.5 and 22).  Microseconds on a B200: attention 4.1 and one for every 50 of load, logits 2
+// and 45 KB an SM, the merge 4, commit 2, a second stream's events 3.5.
+void plan_small_pass(const lr_ctx *ctx, const lr_batch *b, const Partitioner &cut, int64_t max_cta, TcHostPlan &out) {
+  int64_t rows = b->n_branch;
+  for (int i = 0; i < b->n_branch; ++i) rows += b->br_n_draft[i];
+  const double start = (double)cut.piece_start(), w = (double)cut.tile_load(), bytes = 2.0 * ctx->model.vocab * (double)rows;
+  const double n_sm = (double)ctx->sm_count;
+  auto load_time = [](double load) { return 4.1 + load / 50.0; };
+  auto attention = [&](int64_t n) { return load_time(w / (double)n + start); };
+  auto logits = [&](int64_t n) { return 2.0 + bytes / (45e3 * (n_sm - (double)n)); };
+  const TcPartition &all = out.all;
+  int64_t n = std::min<int64_t>(max_cta, ctx->sm_count - 1);
+  const double most_time = 1.1 * attention(max_cta);
+  while (n >= 1 && attention(n) <= most_time && logits(n) > attention(n) + 4.0) --n;
+  if (n < 1 || attention(n) > most_time) return;
+  out.small = true;
+  if (n >= all.n_cta) return;  // whole tiles need no more CTAs than leave enough
+  const double alone = load_time((double)all.longest);
+  const int64_t limit = (int64_t)((kMostAttention * alone - load_time(0.0)) * 50.0);
+  if (cut.holds(limit, n)) {
+    cut.fill(cut.least_limit(n, all.longest, limit), out.lists, out.beside);
+    if (!all.targets.empty() || out.beside.targets.empty()) return;
+    out.beside = TcPartition();
+  }
+  out.small = logits(all.n_cta) + 2.0 < alone + 3.5 + bytes / (45e3 * n_sm);
+}
+
+}  // namespace
+
 void tc_plan_structure(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_br_off, const int32_t *span_tin,
                        const int32_t *span_last, TcHostPlan &out) {
   out = TcHostPlan();
@@ -1228,8 +1394,7 @@ void tc_plan_structure(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
   if (m.head_dim != 64 && m.head_dim != 128) return;
   if ((int64_t)b->n_pool_pages * m.n_kv_heads * kPage >= ((int64_t)1 << 31)) return;  // tensor-map coordinates are 32-bit
   const int T = 128 / G;
-  struct Grp { int list, mtile0, n_mt, n_tiles, n_dense, weight; };  // one per list; every KV head repeats it
-  std::vector<Grp> grps;
+  std::vector<TcGrp> grps;
   // Two M-tiles per group read every KV tile once for both, which is what a large pass needs.  A small pass --
   // a few tiles per SM -- is dominated by the partial results of its key split instead; there every M-tile is a
   // group of its own: a CTA then spends its two streams on the even and odd tiles of one M-tile, combines them
@@ -1298,125 +1463,19 @@ void tc_plan_structure(const lr_ctx *ctx, const lr_batch *b, const int32_t *req_
       list.run1 = (int)out.runs.size();
       const int n_tiles = (list.rq.n_pages + kPagesPerTile - 1) / kPagesPerTile;
       out.n_pages += n_tiles * kPagesPerTile;  // absent pages of the last tile: nothing valid
-      grps.push_back(Grp{(int)out.lists.size(), m0, mts, n_tiles, std::min(n_tiles, list.rq.n_dense_tiles), mts == 2 ? 16 : 10});
+      grps.push_back(TcGrp{(int)out.lists.size(), m0, mts, n_tiles, std::min(n_tiles, list.rq.n_dense_tiles), mts == 2 ? 16 : 10});
       out.lists.push_back(list);
     }
   }
   if (grps.empty()) return;
-  // Contiguous partition of the tile sequence (groups in order, tiles in order) over at most max_cta CTAs that
-  // minimises the largest CTA load.  A tile costs its group's weight (10 with one M-tile, 16 with two: per-CTA cycle
-  // counts on the ragged serving workload gave 2360 and 3790 cycles a tile); every piece -- a CTA's share of one
-  // group -- costs kPieceStartTiles tiles more (Q load, pipeline ramp, epilogue: measured 1.7 to 1.8 tiles), so a CTA
-  // that spans a group boundary gets fewer tiles; a tile that needs masks (anything past the full prefix pages) costs 8/5 of a dense one (measured: 1.3 to 2.3 times, depending on the workload; 9/5 was no better).  For a load limit L the greedy fill (a CTA takes tiles while it stays within L) needs the fewest
-  // CTAs possible; the smallest feasible L is found by bisection.  At most one CTA per two tiles: smaller shares
-  // only add partial results to merge.
-  constexpr int kPieceStartTiles = 2, kDense = 5, kMasked = 8;  // costs in fifths of a dense tile
-  const int n_kv = m.n_kv_heads;
-  int64_t total_w = 0, total_tiles = 0, most = 0;
-  for (const Grp &g : grps) {
-    total_w += (int64_t)n_kv * g.weight * (kPieceStartTiles * kDense + g.n_dense * kDense + (g.n_tiles - g.n_dense) * kMasked);
-    total_tiles += (int64_t)n_kv * g.n_tiles;
-    most = std::max<int64_t>(most, (int64_t)(kPieceStartTiles * kDense + kMasked) * g.weight);
-  }
-  int64_t max_cta = std::min<int64_t>(ctx->sm_count, std::max<int64_t>(1, max_ctas_for_tiles(total_tiles)));
-  if (m_step == 1) {
-    // A small pass lasts as long as its longest chain of dependent steps, so its acceptance runs beside attention, on SMs left free
-    // for it (pass_tail.cu), if that can be done before attention and the merge are through and costs attention at most a tenth by
-    // the first estimate.  (Fewer CTAs also leave fewer partial results to merge: 144 and 112 both take 16.5 us for one request of
-    // 4 K tokens.)  Where the logits are too many for that all SMs are attention's: eight requests of 350 tokens with 124 MB of
-    // logits take 41 us either way, and their attention alone 16.4 instead of 22.4.  Microseconds on a B200: attention 4.1 and one
-    // for every 50 of load, logits 2 and 45 KB an SM, the merge 4.
-    int64_t rows = b->n_branch;
-    for (int i = 0; i < b->n_branch; ++i) rows += b->br_n_draft[i];
-    const double start = (double)(kPieceStartTiles * kDense) * grps[0].weight, w = (double)total_w - start * n_kv * (double)grps.size();
-    const double bytes = 2.0 * ctx->model.vocab * (double)rows;
-    auto attention = [&](int64_t n) { return 4.1 + (w / (double)n + start) / 50.0; };
-    auto logits = [&](int64_t n) { return 2.0 + bytes / (45e3 * (double)(ctx->sm_count - n)); };
-    const double most_time = 1.1 * attention(max_cta);
-    for (int64_t n = std::min<int64_t>(max_cta, ctx->sm_count - 1); n >= 1 && attention(n) <= most_time && !out.small; --n)
-      if (logits(n) <= attention(n) + 4.0) {
-        out.small = true;
-        max_cta = n;
-      }
-  }
-  // walks the partition for limit L; with `emit` it also records the pieces.  A group is a run of dense tiles
-  // followed by a run of masked ones, each of uniform cost, so a walk takes O(CTAs + groups) steps.
-  struct Contrib { int first, n; };
-  std::vector<Contrib> contrib;  // the pieces of every (list, KV head), in that order of grps x heads
-  auto walk = [&](int64_t L, bool emit) -> int64_t {
-    int64_t n = 0, load = 0;
-    for (const Grp &g : grps) {
-      const int64_t start = (int64_t)kPieceStartTiles * kDense * g.weight;
-      for (int kv = 0; kv < n_kv; ++kv) {
-        const int first = (int)out.pieces.size();
-        bool new_piece = true;
-        int t = 0;
-        while (t < g.n_tiles) {
-          const int run_end = t < g.n_dense ? g.n_dense : g.n_tiles;
-          const int64_t cost = (int64_t)g.weight * (t < g.n_dense ? kDense : kMasked);
-          if (n == 0 || load + cost + (new_piece ? start : 0) > L) {  // open the next CTA: its share of this group is a new piece
-            ++n;
-            load = 0;
-            new_piece = true;
-            if (emit) out.cta_piece_off.push_back((int32_t)out.pieces.size());
-            else if (n > max_cta) return n;
-          }
-          if (new_piece) load += start;
-          const int k = (int)std::max<int64_t>(1, std::min<int64_t>(run_end - t, (L - load) / cost));
-          load += (int64_t)k * cost;
-          if (emit) {
-            if (new_piece) {
-              TcPiece p;
-              p.req = g.list; p.kv_head = kv; p.mtile0 = g.mtile0; p.n_mt = g.n_mt; p.tile_begin = t; p.tile_end = t + k;
-              p.slot[0] = p.slot[1] = -2;
-              out.pieces.push_back(p);
-            } else {
-              out.pieces.back().tile_end = t + k;
-            }
-          }
-          new_piece = false;
-          t += k;
-        }
-        if (emit) contrib.push_back({first, (int)out.pieces.size() - first});
-      }
-    }
-    return n;
-  };
-  // No partition stays below the average load, and a greedy fill does not exceed it by more than a piece start and a tile
-  // per CTA, or nearly so: the bisection starts from there.
-  int64_t lo = std::max(most, (total_w + max_cta - 1) / max_cta), hi = lo + 2 * most;
-  if (walk(hi, false) > max_cta) hi = std::max(hi, total_w);  // one CTA takes everything
-  while (lo < hi) {
-    const int64_t mid = lo + (hi - lo) / 2;
-    if (walk(mid, false) <= max_cta) hi = mid; else lo = mid + 1;
-  }
-  out.n_cta = (int)walk(lo, true);
-  out.cta_piece_off.push_back((int32_t)out.pieces.size());
-  // Targets (one M-tile of one group) and the streams that contribute to them, in piece order; the two streams of a
-  // one-M-tile piece are combined inside the CTA.
-  int n_slots = 0;
-  size_t at = 0;
-  for (const Grp &g : grps)
-    for (int kv = 0; kv < n_kv; ++kv, ++at)
-      for (int mt = 0; mt < g.n_mt; ++mt) {
-        const Contrib c = contrib[at];
-        if (c.n == 1) {
-          out.pieces[c.first].slot[mt] = -1;
-          continue;
-        }
-        TcTarget tg;
-        memset(&tg, 0, sizeof(tg));
-        tg.req = g.list; tg.kv_head = kv; tg.mtile = g.mtile0 + mt;
-        tg.slot_begin = n_slots; tg.n_slots = c.n;
-        out.most_slots = std::max(out.most_slots, c.n);
-        tg.q_row0 = out.lists[g.list].rq.q_row0; tg.n_q = out.lists[g.list].rq.n_q;
-        for (int k = 0; k < c.n; ++k) out.pieces[c.first + k].slot[mt] = n_slots++;
-        out.targets.push_back(tg);
-      }
+  const Partitioner cut(grps, m.n_kv_heads);
+  const int64_t max_cta = std::min<int64_t>(ctx->sm_count, std::max<int64_t>(1, max_ctas_for_tiles(cut.n_tiles())));
+  cut.fill(cut.least_limit(max_cta), out.lists, out.all);
+  if (m_step == 1) plan_small_pass(ctx, b, cut, max_cta, out);
   out.ok = true;
-  out.n_partial_slots = n_slots;
   out.tokens_per_mtile = T;
   out.s_ml = 0;
+  const int n_slots = std::max(out.all.n_partial_slots, out.beside.n_partial_slots);  // the two never run at the same time
   out.s_o = ((size_t)n_slots * 128 * 2 * sizeof(float) + 255) / 256 * 256;
   out.scratch_bytes = out.s_o + (size_t)n_slots * 128 * m.head_dim * sizeof(float);
 }
@@ -1425,15 +1484,18 @@ void tc_plan_tables(const lr_batch *b, const int32_t *req_br_off, const int32_t 
   if (!h.ok) return;
   static_assert(sizeof(TcCtaHead) == 256, "one CTA head = 256 bytes");
   const int n_q_rows = b->cu_q[b->n_branch];
-  TcCtaHead *heads = img.add<TcCtaHead>((size_t)h.n_cta, h.o_heads);
   TcPage *pages = img.add<TcPage>((size_t)h.n_pages, h.o_pages);
   TcRow *rows = img.add<TcRow>((size_t)std::max(1, n_q_rows), h.o_rows);
-  h.o_pieces = img.copy(h.pieces.data(), h.pieces.size());
   TcReq *reqs = img.add<TcReq>(h.lists.size(), h.o_reqs);
-  TcTarget *targets = img.add<TcTarget>(std::max<size_t>(1, h.targets.size()), h.o_targets);
+  TcCtaHead *heads[2];
+  TcPartition *const parts[2] = {&h.all, &h.beside};
+  for (int k = 0; k < 2; ++k) {
+    TcPartition &part = *parts[k];
+    heads[k] = img.add<TcCtaHead>((size_t)part.n_cta, part.o_heads);
+    part.o_pieces = img.copy(part.pieces.data(), part.pieces.size());
+    part.o_targets = img.copy(part.targets.data(), part.targets.size());
+  }
   if (!img.base) return;
-  if (!h.targets.empty()) memcpy(targets, h.targets.data(), h.targets.size() * sizeof(TcTarget));
-  else memset(targets, 0, sizeof(TcTarget));  // keep the section non-empty
   for (size_t l = 0; l < h.lists.size(); ++l) {
     const TcList &list = h.lists[l];
     reqs[l] = list.rq;
@@ -1455,67 +1517,78 @@ void tc_plan_tables(const lr_batch *b, const int32_t *req_br_off, const int32_t 
       const int q0 = b->cu_q[i], q_len = b->cu_q[i + 1] - q0;
       for (int k = 0; k < q_len; ++k) rows[q0 + k] = TcRow{depth_branch, b->br_own_len[i] - q_len + k};
     }
-  memset(heads, 0, (size_t)h.n_cta * sizeof(TcCtaHead));
-  for (int c = 0; c < h.n_cta; ++c) {
-    TcCtaHead &hd = heads[c];
-    hd.piece0 = h.cta_piece_off[c];
-    hd.piece1 = h.cta_piece_off[c + 1];
-    if (hd.piece1 > hd.piece0) {
-      hd.first = h.pieces[hd.piece0];
-      hd.first_req = h.lists[hd.first.req].rq;
-      const int first = (hd.first.tile_begin >> 2) * 32;
-      for (int k = 0; k < 32; ++k) hd.first_pages[k] = first + k < hd.first_req.n_pages ? pages[hd.first_req.page_off + first + k].page : -1;
+  for (int k = 0; k < 2; ++k) {
+    const TcPartition &part = *parts[k];
+    memset(heads[k], 0, (size_t)part.n_cta * sizeof(TcCtaHead));
+    for (int c = 0; c < part.n_cta; ++c) {
+      TcCtaHead &hd = heads[k][c];
+      hd.piece0 = part.cta_piece_off[c];
+      hd.piece1 = part.cta_piece_off[c + 1];
+      if (hd.piece1 > hd.piece0) {
+        hd.first = part.pieces[hd.piece0];
+        hd.first_req = h.lists[hd.first.req].rq;
+        const int first = (hd.first.tile_begin >> 2) * 32;
+        for (int i = 0; i < 32; ++i) hd.first_pages[i] = first + i < hd.first_req.n_pages ? pages[hd.first_req.page_off + first + i].page : -1;
+      }
     }
   }
 }
 
 void tc_bind_device_plan(const TcHostPlan &h, unsigned char *image_base, unsigned char *scratch_base, lr_plan *p) {
   p->tc_ok = h.ok;
-  p->tc_pieces = (int)h.pieces.size();
+  p->tc_pieces = (int)h.all.pieces.size();
   p->o_tc_pages = h.o_pages;
-  p->o_tc_heads = h.o_heads;
+  p->o_tc_heads[0] = h.all.o_heads;
+  p->o_tc_heads[1] = h.beside.o_heads;
   p->n_tc_pages = h.ok ? h.n_pages : 0;
-  p->n_tc_heads = h.ok ? h.n_cta : 0;
-  p->tc_partial_slots = h.n_partial_slots;
+  p->n_tc_heads[0] = h.all.n_cta;
+  p->n_tc_heads[1] = h.beside.n_cta;
+  p->tc_partial_slots = h.all.n_partial_slots;
+  p->small = h.small;
   memset(&p->tc, 0, sizeof(p->tc));
+  memset(&p->tc_pass, 0, sizeof(p->tc_pass));
   if (!h.ok) return;
   DevTcPlan &t = p->tc;
-  t.heads = reinterpret_cast<const TcCtaHead *>(image_base + h.o_heads);
   t.pages = reinterpret_cast<const TcPage *>(image_base + h.o_pages);
   t.rows = reinterpret_cast<const TcRow *>(image_base + h.o_rows);
-  t.pieces = reinterpret_cast<const TcPiece *>(image_base + h.o_pieces);
   t.reqs = reinterpret_cast<const TcReq *>(image_base + h.o_reqs);
-  t.targets = reinterpret_cast<const TcTarget *>(image_base + h.o_targets);
-  t.n_cta = h.n_cta;
-  t.n_targets = (int)h.targets.size();
   t.tokens_per_mtile = h.tokens_per_mtile;
-  t.most_slots = h.most_slots;
-  t.small = h.small;
   t.wait_limit_us = 1000000u;  // one second per wait
   t.phantom_tx_bytes = 0;
   t.partial_ml = reinterpret_cast<float *>(scratch_base + h.s_ml);
   t.partial_o = reinterpret_cast<float *>(scratch_base + h.s_o);
+  p->tc_pass = t;
+  auto bind = [&](const TcPartition &part, DevTcPlan &to) {
+    to.heads = reinterpret_cast<const TcCtaHead *>(image_base + part.o_heads);
+    to.pieces = reinterpret_cast<const TcPiece *>(image_base + part.o_pieces);
+    to.targets = reinterpret_cast<const TcTarget *>(image_base + part.o_targets);
+    to.n_cta = part.n_cta;
+    to.n_targets = (int)part.targets.size();
+    to.most_slots = part.most_slots;
+  };
+  bind(h.all, t);
+  bind(h.beside.n_cta > 0 ? h.beside : h.all, p->tc_pass);
 }
 
 template <int kD>
-static int launch_attn_tc_d(lr_plan *p, const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &qmap, const RawInputs &in, uint16_t *out,
+static int launch_attn_tc_d(lr_plan *p, const DevTcPlan &tc, const CUtensorMap &kmap, const CUtensorMap &vmap, const CUtensorMap &qmap, const RawInputs &in, uint16_t *out,
                             float *lse, float scale_log2, bool merge, cudaStream_t s) {
   p->ctx->launches++;
   // set up while the kernel before it drains (a layer's merge, or what is left of the pass before)
-  if (int rc = cuda_fail(launch_dependent(attn_tc_kernel<kD>, dim3((unsigned)p->tc.n_cta), dim3(kThreads), Shape<kD>::kSmemBytes, s, kmap, vmap, qmap, p->dev,
-                                          p->tc, in, out, lse, scale_log2),
+  if (int rc = cuda_fail(launch_dependent(attn_tc_kernel<kD>, dim3((unsigned)tc.n_cta), dim3(kThreads), Shape<kD>::kSmemBytes, s, kmap, vmap, qmap, p->dev,
+                                          tc, in, out, lse, scale_log2),
                          "attn_tc_kernel launch"))
     return rc;
-  if (merge && p->tc.n_targets > 0) {  // the merge grid is set up while the attention grid drains
+  if (merge && tc.n_targets > 0) {  // the merge grid is set up while the attention grid drains
     p->ctx->launches++;
-    return cuda_fail(launch_dependent(p->tc.most_slots <= 4 ? attn_tc_merge_kernel<kD, 4> : attn_tc_merge_kernel<kD, 8>,
-                                      dim3((unsigned)p->tc.n_targets, kD / 8), dim3(256), 0, s, p->dev, p->tc, out, lse),
+    return cuda_fail(launch_dependent(tc.most_slots <= 4 ? attn_tc_merge_kernel<kD, 4> : attn_tc_merge_kernel<kD, 8>,
+                                      dim3((unsigned)tc.n_targets, kD / 8), dim3(256), 0, s, p->dev, tc, out, lse),
                      "attn_tc_merge_kernel launch");
   }
   return LR_OK;
 }
 
-int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale, bool merge,
+int launch_attn_tc(lr_plan *p, const DevTcPlan &tc, const void *q, const void *k, const void *v, void *out, float *lse, float scale, bool merge,
                    cudaStream_t s) {
   const CUtensorMap *mp = nullptr;
   if (int rc = get_map(p->ctx, 0, k, p->dev.n_pool_pages, &mp)) return rc;
@@ -1526,7 +1599,7 @@ int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void
   const CUtensorMap qmap = *mp;
   const float scale_log2 = scale * 1.4426950408889634f;
   const RawInputs in = {reinterpret_cast<const uint16_t *>(q), reinterpret_cast<const uint16_t *>(k), reinterpret_cast<const uint16_t *>(v)};
-  return (p->dev.head_dim == 128 ? launch_attn_tc_d<128> : launch_attn_tc_d<64>)(p, kmap, vmap, qmap, in, reinterpret_cast<uint16_t *>(out), lse,
+  return (p->dev.head_dim == 128 ? launch_attn_tc_d<128> : launch_attn_tc_d<64>)(p, tc, kmap, vmap, qmap, in, reinterpret_cast<uint16_t *>(out), lse,
                                                                                 scale_log2, merge, s);
 }
 

@@ -523,7 +523,7 @@ static int plan_build(lr_ctx *ctx, const lr_batch *b, Layout &L, void *ws, size_
   tc_bind_device_plan(L.tc, base, base + p->scratch_off, p);
   p->pair_ok = p->pair_built = false;
   memset(&p->pr, 0, sizeof(p->pr));
-  p->pr.wait_limit_us = p->tc.wait_limit_us = 1000000u;  // one second per wait
+  p->pr.wait_limit_us = p->tc.wait_limit_us = p->tc_pass.wait_limit_us = 1000000u;  // one second per wait
   p->o_req_span_off = L.o_req_span_off;
   p->o_span_len = L.o_span_len;
   p->o_span_slot = L.o_span_slot;
@@ -662,12 +662,31 @@ extern "C" int lr_plan_describe(const lr_plan *p, lr_plan_info *info) {
   return LR_OK;
 }
 
+extern "C" int lr_debug_partitions(const lr_model *m, const lr_batch *b, int32_t n_sm, lr_partition_info *attention, lr_partition_info *pass,
+                                   int32_t *small_pass) {
+  if (!m || !attention || !pass || !small_pass || n_sm < 1) {
+    set_error("lr_debug_partitions: bad argument");
+    return LR_EINVAL;
+  }
+  if (int rc = check_model(m, "lr_debug_partitions")) return rc;
+  lr_ctx ctx = {};
+  ctx.model = *m;
+  ctx.sm_count = n_sm;
+  Layout L;
+  if (int rc = layout(&ctx, b, L)) return rc;
+  auto info = [](const TcPartition &p) { return lr_partition_info{p.n_cta, (int32_t)p.targets.size(), p.n_partial_slots, p.longest}; };
+  *attention = info(L.tc.all);
+  *pass = info(L.tc.beside.n_cta > 0 ? L.tc.beside : L.tc.all);
+  *small_pass = L.tc.small;
+  return LR_OK;
+}
+
 extern "C" int lr_plan_debug_set_wait_limit(lr_plan *p, uint32_t microseconds) {
   if (!p || microseconds == 0) {
     set_error("lr_plan_debug_set_wait_limit: bad argument");
     return LR_EINVAL;
   }
-  p->tc.wait_limit_us = microseconds;
+  p->tc.wait_limit_us = p->tc_pass.wait_limit_us = microseconds;
   p->pr.wait_limit_us = microseconds;
   return LR_OK;
 }
@@ -677,7 +696,7 @@ extern "C" int lr_plan_debug_set_phantom_bytes(lr_plan *p, uint32_t bytes) {
     set_error("lr_plan_debug_set_phantom_bytes: null plan");
     return LR_EINVAL;
   }
-  p->tc.phantom_tx_bytes = bytes;
+  p->tc.phantom_tx_bytes = p->tc_pass.phantom_tx_bytes = bytes;
   p->pr.phantom_tx_bytes = bytes;
   return LR_OK;
 }
@@ -698,10 +717,12 @@ extern "C" int lr_plan_debug_set_page(lr_plan *p, int32_t page_slot, int32_t new
   TcPage *pages = reinterpret_cast<TcPage *>(img + p->o_tc_pages);
   for (int i = 0; i < p->n_tc_pages; ++i)
     if (pages[i].page == old_id && (pages[i].meta & 31u) != 0u) pages[i].page = new_id;
-  TcCtaHead *heads = reinterpret_cast<TcCtaHead *>(img + p->o_tc_heads);
-  for (int c = 0; c < p->n_tc_heads; ++c)
-    for (int k = 0; k < 32; ++k)
-      if (heads[c].first_pages[k] == old_id && heads[c].piece1 > heads[c].piece0) heads[c].first_pages[k] = new_id;
+  for (int part = 0; part < 2; ++part) {
+    TcCtaHead *heads = reinterpret_cast<TcCtaHead *>(img + p->o_tc_heads[part]);
+    for (int c = 0; c < p->n_tc_heads[part]; ++c)
+      for (int k = 0; k < 32; ++k)
+        if (heads[c].first_pages[k] == old_id && heads[c].piece1 > heads[c].piece0) heads[c].first_pages[k] = new_id;
+  }
   cudaError_t e = cudaMemcpyAsync(p->workspace_d, p->pinned, p->image_bytes, cudaMemcpyHostToDevice, s);
   if (p->pair_built) {
     if (int rc = build_pair(p)) return rc;
@@ -742,7 +763,7 @@ extern "C" int lr_verify_attention(lr_plan *p, const void *q, const void *k, con
       set_error("lr_verify_attention: the tensor-core path does not support this shape");
       return LR_EUNSUPPORTED;
     }
-    return launch_attn_tc(p, q, k, v, out, lse, scale, true, s);
+    return launch_attn_tc(p, p->tc, q, k, v, out, lse, scale, true, s);
   }
   return launch_attn_generic(p, q, k, v, out, lse, scale, s);
 }
@@ -951,7 +972,11 @@ static int pass_side_by_side(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, floa
   if (int rc = take_side(p)) return rc;
   cudaError_t e = cudaEventRecord(p->side.fork, s);
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
-  if (int rc = lr_verify_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, s)) return rc;
+  if (one_kernel) {  // (its arguments have been checked)
+    if (int rc = launch_attn_tc(p, p->tc_pass, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/true, s)) return rc;
+  } else if (int rc = lr_verify_attention(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, s)) {
+    return rc;
+  }
   if (!side) side = p->side.s;
   e = cudaStreamWaitEvent(side, p->side.fork, 0);
   if (e != cudaSuccess) return cuda_fail(e, "lr_verify_pass: fork");
@@ -981,14 +1006,14 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
                             io->bonus_id_d, io->accept_scratch_d))
     return rc;
   if (int rc = check_commit(p, io->verdict_d, io->n_accept_d, commit_out(io))) return rc;
+  if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)p->dev.head_dim);
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (int rc = cuda_fail(cudaStreamIsCapturing(s, &capture), "cudaStreamIsCapturing")) return rc;
   // On one stream, two kernels in a row of which the second is set up, and mostly done, while the first runs (pass_tail.cu), there
   // are no events between two passes, and the next attention is set up early too.  A caller who gives a second stream has a reason
   // to order work with it.  And in a graph events cost nothing: beside an attention of few CTAs the rest is a root of its own.
-  if (side || (capture != cudaStreamCaptureStatusNone && 2 * p->tc.n_cta <= ctx->sm_count)) return pass_side_by_side(ctx, p, io, scale, true, side, s);
-  if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)p->dev.head_dim);
-  if (int rc = launch_attn_tc(p, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/false, s)) return rc;
+  if (side || (capture != cudaStreamCaptureStatusNone && 2 * p->tc_pass.n_cta <= p->ctx->sm_count)) return pass_side_by_side(ctx, p, io, scale, true, side, s);
+  if (int rc = launch_attn_tc(p, p->tc_pass, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/false, s)) return rc;
   return launch_pass_tail(ctx, p, io, /*behind_attention=*/true, s);
 }
 

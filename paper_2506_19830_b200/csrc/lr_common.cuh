@@ -102,7 +102,6 @@ struct DevTcPlan {
   const TcTarget *targets;
   int32_t n_cta, n_targets;
   int32_t most_slots;        // partial slots of the target that has most
-  int32_t small;             // planned with SMs left for the acceptance
   int32_t tokens_per_mtile;  // floor(128 / group)
   uint32_t wait_limit_us;    // bound of every device-side wait (test hook: lr_plan_debug_set_wait_limit)
   uint32_t phantom_tx_bytes; // test hook: bytes CTA 0 expects on its first KV stage beyond what its copies deliver
@@ -175,6 +174,8 @@ struct lr_plan {
   lr_ctx *ctx;
   lr::DevBatch dev;
   lr::DevTcPlan tc;
+  lr::DevTcPlan tc_pass;  // of a small pass: the same, or the partition that leaves SMs free
+  bool small;             // the whole pass as in pass_tail.cu
   lr::DevPairPlan pr;
   bool tc_ok;             // shape allows the tensor-core path
   // The CTA-pair plan is built and uploaded when its path is first selected.  Its tables have a part of the workspace to
@@ -190,8 +191,8 @@ struct lr_plan {
   int attention_path;     // 0 auto, 1 generic, 2 tensor core (single CTA), 3 tensor core (CTA pairs)
   int tc_pieces, tc_partial_slots;  // for lr_plan_describe
   // where the physical page ids sit in the image (lr_plan_debug_set_page)
-  size_t o_page_ids, o_tc_pages, o_tc_heads;
-  int n_tc_pages, n_tc_heads;
+  size_t o_page_ids, o_tc_pages, o_tc_heads[2];
+  int n_tc_pages, n_tc_heads[2];
   void *pinned;           // pinned host image
   size_t pinned_cap;
   void *results_pinned;   // pinned bounce buffer for the integer results of lr_verify_pass_host (taken on first use)
@@ -240,16 +241,23 @@ struct TcList {        // the page list of one (request, group of M-tiles)
   TcReq rq;
   int run0, run1;
 };
+struct TcPartition {   // the tiles over CTAs
+  std::vector<TcPiece> pieces;
+  std::vector<int32_t> cta_piece_off;
+  std::vector<TcTarget> targets;
+  size_t o_heads = 0, o_pieces = 0, o_targets = 0;  // image offsets
+  int n_cta = 0, n_partial_slots = 0, most_slots = 0;
+  int64_t longest = 0;  // load of the CTA that has most
+};
 struct TcHostPlan {
   bool ok = false;  // shape supported by the tensor-core path
   std::vector<TcRun> runs;
   std::vector<TcList> lists;
-  std::vector<TcPiece> pieces;
-  std::vector<int32_t> cta_piece_off;
-  std::vector<TcTarget> targets;
-  size_t o_heads = 0, o_pages = 0, o_rows = 0, o_pieces = 0, o_reqs = 0, o_targets = 0;  // image offsets
-  int n_cta = 0, n_partial_slots = 0, most_slots = 0, tokens_per_mtile = 0, n_pages = 0;
-  bool small = false;
+  TcPartition all;     // over all SMs: of lr_verify_attention, whoever calls it
+  TcPartition beside;  // of a small pass whose acceptance needs SMs that `all` does not leave; else empty
+  bool small = false;  // lr_verify_pass may go as in pass_tail.cu
+  size_t o_pages = 0, o_rows = 0, o_reqs = 0;  // image offsets
+  int tokens_per_mtile = 0, n_pages = 0;
   // scratch region behind the image: (exponent, sum) pairs, then fp32 partial outputs
   size_t s_ml = 0, s_o = 0, scratch_bytes = 0;
 };
@@ -329,7 +337,7 @@ int launch_attn_pair(lr_plan *p, const void *q, const void *k, const void *v, vo
 int launch_attn_generic(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale,
                         cudaStream_t s);
 // without `merge` the partial results are left for launch_pass_tail
-int launch_attn_tc(lr_plan *p, const void *q, const void *k, const void *v, void *out, float *lse, float scale, bool merge,
+int launch_attn_tc(lr_plan *p, const DevTcPlan &tc, const void *q, const void *k, const void *v, void *out, float *lse, float scale, bool merge,
                    cudaStream_t s);
 // The rest of a small pass: acceptance and commit, and behind a launch_attn_tc without merge that too; and whether a pass is one.
 // The acceptance goes by the context of the call, which need not be the plan's: its vocabulary may be another.

@@ -161,7 +161,7 @@ auto tail_kernel(bool tree) {
 
 bool pass_tail_fits(const lr_ctx *ctx, const lr_plan *p, int64_t n_rows) {
   const int vecs = ctx->model.vocab >> 3, unit = 32 * kVecPerThread;
-  return p->tc.small && p->dev.n_req <= kMostRequests && p->dev.n_page_slots <= kCommitSlots &&
+  return p->small && p->dev.n_req <= kMostRequests && p->dev.n_page_slots <= kCommitSlots &&
          n_rows * std::max(1, (vecs + unit - 1) / unit) <= (int64_t)kMostUnits;
 }
 
@@ -171,11 +171,12 @@ int launch_pass_tail(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, bool behind_
                   io->draft_ids_d, io->cu_draft_d, io->n_accept_d, io->bonus_id_d, io->row_argmax_d, d.n_branch, (int32_t)io->n_rows};
   a.n_commit = std::min(commit_ctas(d), kCommitCtas);
   // a warp's share: what the places beside attention stream in one go (the plan has made sure that they are enough)
-  const bool few = p->tc.most_slots <= kFewSlots;
-  const uint32_t places = (uint32_t)std::max(1, tail_ctas(few ? 4 : 8) * (p->ctx->sm_count - p->tc.n_cta) - a.n_commit);
+  const DevTcPlan &tc = p->tc_pass;
+  const bool few = tc.most_slots <= kFewSlots;
+  const uint32_t places = (uint32_t)std::max(1, tail_ctas(few ? 4 : 8) * (p->ctx->sm_count - tc.n_cta) - a.n_commit);
   a.share = (a.w.total + places * (kThreads / 32) - 1) / (places * (kThreads / 32));
   a.n_stream = (int)((a.w.total + a.share * (kThreads / 32) - 1) / (a.share * (kThreads / 32)));
-  a.wait_limit_ns = 1000ull * kPatience * p->tc.wait_limit_us;
+  a.wait_limit_ns = 1000ull * kPatience * tc.wait_limit_us;
   const CommitOut o = {io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d,
                        io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d};
   const auto kernel = d.head_dim == 128 ? (few ? tail_kernel<128, 4>(d.tree) : tail_kernel<128, 8>(d.tree))
@@ -184,10 +185,10 @@ int launch_pass_tail(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, bool behind_
   uint16_t *out = reinterpret_cast<uint16_t *>(io->out_d);
   ctx->launches++;
   if (!behind_attention) {  // an ordinary launch: most CTAs do not wait for what is just before
-    kernel<<<a.n_commit + a.n_stream, kThreads, smem, s>>>(d, p->tc, out, io->lse_d, a, io->verdict_d, o);
+    kernel<<<a.n_commit + a.n_stream, kThreads, smem, s>>>(d, tc, out, io->lse_d, a, io->verdict_d, o);
     return cuda_fail(cudaGetLastError(), "pass_tail_kernel launch");
   }
-  return cuda_fail(launch_dependent(kernel, dim3((unsigned)(a.n_commit + a.n_stream + p->tc.n_targets * (d.head_dim / 8))), dim3(kThreads), smem, s, d, p->tc,
+  return cuda_fail(launch_dependent(kernel, dim3((unsigned)(a.n_commit + a.n_stream + tc.n_targets * (d.head_dim / 8))), dim3(kThreads), smem, s, d, tc,
                                     out, io->lse_d, a, io->verdict_d, o),
                    "pass_tail_kernel launch");
 }

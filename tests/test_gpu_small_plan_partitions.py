@@ -1,0 +1,68 @@
+"""A small plan serves lr_verify_attention, which has all SMs, and lr_verify_pass, which may leave some to the acceptance: the
+former's partition, launches and bits do not hang on the vocabulary, both are right, and both see a page id that is changed."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import REL_LARGE, check_attention
+from lr_workloads import Model
+from lr_workloads.gen import _finish
+from oracle import lr_oracle as O
+from paper_2506_19830_b200 import binding as B
+from paper_2506_19830_b200 import runner as R
+
+pytestmark = pytest.mark.gpu
+
+
+def _work(heads, head_dim, vocab, n_req, prefix, steps, drafts, with_logits):
+    rng = np.random.Generator(np.random.PCG64(n_req + prefix))
+    reqs = [{"P": prefix, "segs": [32] * steps, "branches": [(n, drafts, drafts, drafts) for n in range(1, steps + 1)]} for _ in range(n_req)]
+    return _finish("plans", 3, Model(*heads, head_dim, vocab), reqs, rng, 0.3, 0.7, with_logits, True, "nan")
+
+
+@pytest.mark.parametrize("heads,head_dim,vocab,n_req,prefix,steps,drafts,own", [
+    ((5, 1), 128, 152064, 16, 100, 3, 4, False), ((40, 8), 128, 32000, 4, 500, 3, 16, True), ((40, 8), 128, 152064, 4, 100, 5, 4, True),
+    ((40, 8), 128, 152064, 1, 1500, 3, 16, True), ((32, 8), 64, 152064, 1, 1500, 3, 16, True)])
+def test_two_partitions(heads, head_dim, vocab, n_req, prefix, steps, drafts, own):
+    w = _work(heads, head_dim, 8, n_req, prefix, steps, drafts, False)
+    b, t = w.batch, w.tensors
+    got = []
+    for v in (8, vocab):
+        ctx = B.Context(Model(*heads, head_dim, v), 0)
+        plan, x, y = B.Plan(ctx, b), R.DeviceInputs(b, t, with_logits=False), R.PassOutputs(b)
+        n = ctx.launch_count
+        plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out, y.lse)
+        got.append((plan.lr_plan_describe(), ctx.launch_count - n, y.out, y.lse))
+        assert plan.lr_poll_status() == 0
+        plan.close()
+        ctx.close()
+    assert got[0][:2] == got[1][:2] and all(torch.equal(p, q) for p, q in zip(got[0][2:], got[1][2:]))
+    assert got[0][1] == (2 if got[0][0]["n_merge_targets"] else 1)
+    o_ref, l_ref = O.verify_attention(b, t.q, t.k_pool, t.v_pool)
+    check_attention(got[0][2], got[0][3], o_ref, l_ref, rel_large=REL_LARGE)
+    # the pass of the large vocabulary, on its own partition
+    ctx = B.Context(Model(*heads, head_dim, vocab), 0)
+    attention, of_pass, _ = B.lr_debug_partitions(ctx.model, b, torch.cuda.get_device_properties(0).multi_processor_count)
+    assert attention["n_cta"] == got[0][0]["n_cta"] and (of_pass != attention) == own
+    plan, x, y = B.Plan(ctx, b), R.DeviceInputs(b, t, with_logits=False), R.PassOutputs(b)
+    x.logits = torch.randn((b.n_logit_rows, vocab), device="cuda:0", dtype=torch.bfloat16)
+    x.draft_ids = torch.zeros(max(1, int(b.cu_draft[-1])), dtype=torch.int32, device="cuda:0")
+    n = ctx.launch_count
+    R.run_pass(ctx, plan, x, y)
+    assert ctx.launch_count - n == 2
+    assert plan.lr_poll_status() == 0
+    check_attention(y.out, y.lse, o_ref, l_ref, rel_large=REL_LARGE)
+    # an id outside the pool, in every table of the plan
+    for k in range(2):
+        call = (lambda: R.run_pass(ctx, plan, x, y)) if k == 0 else (lambda: plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out, y.lse))
+        slot = int(b.span_slot[0])
+        plan.lr_plan_debug_set_page(slot, b.n_pool_pages + 7)
+        call()
+        with pytest.raises(B.LrError):
+            plan.lr_poll_status()
+        plan.lr_plan_debug_set_page(slot, int(b.page_ids[slot]))
+        call()
+        assert plan.lr_poll_status() == 0
+        check_attention(y.out, y.lse, o_ref, l_ref, rel_large=REL_LARGE)
+    plan.close()
+    ctx.close()
