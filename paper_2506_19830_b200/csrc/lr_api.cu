@@ -967,7 +967,7 @@ static CommitOut commit_out(const lr_pass_io *io) {
 }
 
 // Acceptance and commit on a second stream beside attention: they fill the SMs that it leaves idle.  (Which of the two comes first
-// makes no difference.)  One kernel where the pass is a small one, two else.
+// makes no difference.)  As one kernel they run on the few SMs that a small pass leaves them, so they have to start with attention.
 static int pass_side_by_side(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, float scale, bool one_kernel, cudaStream_t side, cudaStream_t s) {
   if (int rc = take_side(p)) return rc;
   cudaError_t e = cudaEventRecord(p->side.fork, s);
@@ -1011,8 +1011,13 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
   if (int rc = cuda_fail(cudaStreamIsCapturing(s, &capture), "cudaStreamIsCapturing")) return rc;
   // On one stream, two kernels in a row of which the second is set up, and mostly done, while the first runs (pass_tail.cu), there
   // are no events between two passes, and the next attention is set up early too.  A caller who gives a second stream has a reason
-  // to order work with it.  And in a graph events cost nothing: beside an attention of few CTAs the rest is a root of its own.
-  if (side || (capture != cudaStreamCaptureStatusNone && 2 * p->tc_pass.n_cta <= p->ctx->sm_count)) return pass_side_by_side(ctx, p, io, scale, true, side, s);
+  // to order work with it.  In a graph events cost nothing and both streams' kernels start together: acceptance and commit are one
+  // kernel there (one request of 4 K tokens 19.0 -> 16.2 us), and beside an attention of few CTAs they are a root of their own.
+  // Launched one by one, the second stream's kernel often comes when CTAs of the merge, which wait for attention, already sit on
+  // the SMs left free, and then runs behind all of it on a few SMs: a pass by itself 31.5 us with acceptance and commit as two
+  // kernels and 34.8 with one, of 8 K tokens 37.1 and 44.8, 13 ragged requests of up to 900 tokens 48.6 and 61.
+  const bool captured = capture != cudaStreamCaptureStatusNone;
+  if (side || (captured && 2 * p->tc_pass.n_cta <= p->ctx->sm_count)) return pass_side_by_side(ctx, p, io, scale, captured, side, s);
   if (int rc = launch_attn_tc(p, p->tc_pass, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/false, s)) return rc;
   return launch_pass_tail(ctx, p, io, /*behind_attention=*/true, s);
 }

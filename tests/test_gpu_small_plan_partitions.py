@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_util import REL_LARGE, check_attention
+from gpu_util import REL_LARGE, check_attention, check_commit
 from lr_workloads import Model
 from lr_workloads.gen import _finish
 from oracle import lr_oracle as O
@@ -64,5 +64,38 @@ def test_two_partitions(heads, head_dim, vocab, n_req, prefix, steps, drafts, ow
         call()
         assert plan.lr_poll_status() == 0
         check_attention(y.out, y.lse, o_ref, l_ref, rel_large=REL_LARGE)
+    plan.close()
+    ctx.close()
+
+
+def test_a_second_stream():
+    """Launched, the pass is attention on all SMs with acceptance and commit as two kernels beside it; in a graph they are one."""
+    w = _work((40, 8), 128, 5000, 1, 1500, 3, 16, True)
+    b, t = w.batch, w.tensors
+    ctx = B.Context(b.model, 0)
+    plan, x, y, side = B.Plan(ctx, b), R.DeviceInputs(b, t), R.PassOutputs(b), torch.cuda.Stream()
+    plan.lr_verify_attention(x.q, x.k_pool, x.v_pool, y.out)
+    want = y.out.clone()
+    n_ref, bonus_ref, _ = O.accept_greedy(t.logits, t.draft_ids, b.cu_draft)
+    o_ref, _ = O.verify_attention(b, t.q, t.k_pool, t.v_pool)
+    for _ in range(3):
+        n = ctx.launch_count
+        R.run_pass_overlapped(ctx, plan, x, y, side)
+        assert ctx.launch_count - n == 4
+        assert plan.lr_poll_status() == 0 and torch.equal(y.out, want)
+        assert np.array_equal(y.n_accept.cpu().numpy(), n_ref) and np.array_equal(y.bonus_id.cpu().numpy(), bonus_ref)
+        check_commit(y.commit_dict(), O.commit(b, t.verdict, n_ref))
+        y.n_accept.zero_(), y.keep_pages.zero_(), y.out.zero_()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        n = ctx.launch_count
+        R.run_pass_overlapped(ctx, plan, x, y, side)
+        assert ctx.launch_count - n == 3
+    graph.replay()
+    assert plan.lr_poll_status() == 0
+    check_attention(y.out, None, o_ref, None, rel_large=REL_LARGE)
+    assert np.array_equal(y.n_accept.cpu().numpy(), n_ref) and np.array_equal(y.bonus_id.cpu().numpy(), bonus_ref)
+    check_commit(y.commit_dict(), O.commit(b, t.verdict, n_ref))
+    del graph
     plan.close()
     ctx.close()
