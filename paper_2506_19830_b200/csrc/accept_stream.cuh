@@ -160,7 +160,7 @@ __device__ __forceinline__ int accept_branch(const unsigned long long *keys, con
       t[k] = 0;
       dr[k] = -1;
       if (i <= L) t[k] = (int32_t)(0xFFFFFFFFu - (uint32_t)ld_behind_wait(keys + i));
-      if (i < L) dr[k] = draft_ids[d0 + i];
+      if (i < L) dr[k] = ld_behind_wait(draft_ids + d0 + i);
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -174,25 +174,6 @@ __device__ __forceinline__ int accept_branch(const unsigned long long *keys, con
     }
   }
   return n;
-}
-
-// What a CTA of kThreads that knows all keys to be there makes of them: one thread per branch, so that hundreds of branches cost
-// one pass.  Branch b's rows start at cu_draft[b] - first_draft + b.  Leaves the keys zeroed.
-template <int kThreads>
-__device__ __forceinline__ void accept_finish(unsigned long long *scratch, const int32_t *draft_ids, const int32_t *cu_draft, int32_t n_branch,
-                                              int32_t n_rows, int32_t first_draft, int32_t *n_accept, int32_t *bonus_id, int32_t *row_argmax) {
-  unsigned long long *row_key = scratch + 1;
-  const int tid = threadIdx.x;
-  for (int b = tid; b < n_branch; b += kThreads) {
-    const int32_t d0 = cu_draft[b], L = cu_draft[b + 1] - d0;
-    int32_t bonus;
-    n_accept[b] = accept_branch(row_key + (d0 - first_draft + b), draft_ids, d0, L, bonus);
-    bonus_id[b] = bonus;
-  }
-  if (row_argmax != nullptr)
-    for (int r = tid; r < n_rows; r += kThreads) row_argmax[r] = (int32_t)(0xFFFFFFFFu - (uint32_t)ld_behind_wait(row_key + r));
-  __syncthreads();
-  for (int r = tid; r < n_rows; r += kThreads) row_key[r] = 0ull;
 }
 
 inline AcceptWork accept_work(const lr_ctx *ctx, const void *logits, int64_t row_stride, int32_t n_rows, void *scratch, int vecs) {
