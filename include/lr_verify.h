@@ -190,8 +190,9 @@ int lr_plan_describe(const lr_plan *plan, lr_plan_info *info_out);
 
 /* How the attention work of a batch is split on a device of n_sm SMs, worked out on the host without one.  For testing.
  *   attention   the partition of lr_verify_attention
- *   pass        that of lr_verify_pass on one stream: another one where a small pass needs SMs for its acceptance
- *   small_pass  1 if lr_verify_pass may take the form for small passes
+ *   pass        that of lr_verify_pass on one stream: another one where a small pass with head size 64 needs SMs for its acceptance
+ *   small_pass  whether lr_verify_pass may take the form for small passes: 1 with the acceptance beside attention, 2 with the
+ *               acceptance on all SMs behind it
  *   longest_load  what the longest CTA has to do, about a 50th of a microsecond each */
 typedef struct lr_partition_info {
   int32_t n_cta, n_merge_targets, n_partial_slots;

@@ -179,13 +179,13 @@ def lr_validate_batch(model, batch) -> None:
 
 
 def lr_debug_partitions(model, batch, n_sm: int):
-    """(attention, pass, small): how the attention work of a batch is split on a device of ``n_sm`` SMs."""
+    """(attention, pass, form of a small pass): how the attention work of a batch is split on a device of ``n_sm`` SMs."""
     hb, m, small = HostBatch(batch), _model_struct(model), C.c_int32()
     parts = [lr_partition_info(), lr_partition_info()]
     _check(lib().lr_debug_partitions(C.byref(m), C.byref(hb.c), n_sm, C.byref(parts[0]), C.byref(parts[1]), C.byref(small)),
            "lr_debug_partitions")
     attention, whole_pass = ({n: int(getattr(p, n)) for n, _ in p._fields_} for p in parts)
-    return attention, whole_pass, bool(small.value)
+    return attention, whole_pass, small.value
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

@@ -1348,17 +1348,23 @@ void Partitioner::fill(int64_t L, const std::vector<TcList> &lists, TcPartition 
       }
 }
 
-// Whether the whole pass on a small plan goes as in pass_tail.cu, and on which partition.
+// Whether the whole pass on a small plan goes as in pass_tail.cu, and how.
 // A small pass lasts as long as its longest chain of dependent steps, so its acceptance runs beside attention, on SMs left free for
 // it, if that can be done before attention and the merge are through and the average CTA takes at most a tenth more.  Where the
-// partition over all SMs does not leave enough of them, the pass has one of its own: attention by itself, which a serving loop
-// runs once a layer, keeps all SMs (16 requests of 500 tokens, 32 query heads: 16.0 us on 128 CTAs and 25.5 on 110; 16 of 100: 9.3
-// and 17.3).  Shares are whole tiles, so the longest CTA of the narrower one may take more than the average says: up to
-// kMostAttention (four requests of 500 tokens: 1.2, the pass 17.5 us where attention first and acceptance behind it take 21.3; of 100:
-// 1.2, 14.5 and 21), and never a merge that attention did without (those two: 26.6 against 23.9, and 19.7 against 17.0).  Where that
-// rules it out the pass is still one of its kind if what attention leaves free gets through the logits sooner than all SMs do behind
-// it (16 requests of 100 tokens, 5 query heads, 73 MB of logits: 17.5 and 22).  Microseconds on a B200: attention 4.1 and one for every 50 of load, logits 2
-// and 45 KB an SM, the merge 4, commit 2, a second stream's events 3.5.
+// partition over all SMs does not leave enough of them:
+// - With head size 64 the pass has a partition of its own: attention by itself, which a serving loop runs once a layer, keeps all SMs.
+//   Shares are whole tiles, so the longest CTA of the narrower one may take more than the average says, up to kMostAttention; and it
+//   never brings a merge that attention did without.  One request of 4 K tokens 16.9 us, with attention first and acceptance behind it 22.4.
+// - With head size 128 a result hangs on how the keys are split: the weights are rounded to bf16 against the largest score of their
+//   piece, and fewer pieces round more of the large weights.  Against 64 bits a narrower partition is 0.26 % further off in the mean
+//   over 22 batches, 1.2 % at most (head size 64 has the fp32 weights: not at all).  So the pass keeps attention's partition, and its
+//   acceptance streams on all SMs as attention's CTAs leave them: one request of 4 K tokens 19.9 us (22.5 with a second stream's events,
+//   16.7 on a narrower partition), 8 K 25.4 (27.3, 22.4), four of 500 17.6 (22.1, 17.4).  Without a merge to carry that gains nothing
+//   (16 of 500: 25.0 and 24.5).
+// - Where the logits are many and attention's CTAs few, the SMs left free get through them sooner than all of them do behind attention
+//   (16 requests of 100 tokens, 5 query heads, 73 MB of logits: 17.2 us and 22.3).
+// Microseconds on a B200: attention 4.1 and one for every 50 of load, logits 2 and 45 KB an SM, the merge 4, commit 2, a second
+// stream's events 3.5.
 void plan_small_pass(const lr_ctx *ctx, const lr_batch *b, const Partitioner &cut, int64_t max_cta, TcHostPlan &out) {
   int64_t rows = b->n_branch;
   for (int i = 0; i < b->n_branch; ++i) rows += b->br_n_draft[i];
@@ -1368,20 +1374,21 @@ void plan_small_pass(const lr_ctx *ctx, const lr_batch *b, const Partitioner &cu
   auto attention = [&](int64_t n) { return load_time(w / (double)n + start); };
   auto logits = [&](int64_t n) { return 2.0 + bytes / (45e3 * (n_sm - (double)n)); };
   const TcPartition &all = out.all;
+  const bool merges = !all.targets.empty();
   int64_t n = std::min<int64_t>(max_cta, ctx->sm_count - 1);
   const double most_time = 1.1 * attention(max_cta);
   while (n >= 1 && attention(n) <= most_time && logits(n) > attention(n) + 4.0) --n;
   if (n < 1 || attention(n) > most_time) return;
-  out.small = true;
+  out.small = kBesideAttention;
   if (n >= all.n_cta) return;  // whole tiles need no more CTAs than leave enough
   const double alone = load_time((double)all.longest);
   const int64_t limit = (int64_t)((kMostAttention * alone - load_time(0.0)) * 50.0);
-  if (cut.holds(limit, n)) {
+  if (ctx->model.head_dim == 64 && cut.holds(limit, n)) {
     cut.fill(cut.least_limit(n, all.longest, limit), out.lists, out.beside);
-    if (!all.targets.empty() || out.beside.targets.empty()) return;
+    if (merges || out.beside.targets.empty()) return;
     out.beside = TcPartition();
   }
-  out.small = logits(all.n_cta) + 2.0 < alone + 3.5 + bytes / (45e3 * n_sm);
+  if (logits(all.n_cta) + 2.0 >= alone + 3.5 + bytes / (45e3 * n_sm)) out.small = merges ? kBehindAttention : kNotSmall;
 }
 
 }  // namespace

@@ -677,7 +677,7 @@ extern "C" int lr_debug_partitions(const lr_model *m, const lr_batch *b, int32_t
   auto info = [](const TcPartition &p) { return lr_partition_info{p.n_cta, (int32_t)p.targets.size(), p.n_partial_slots, p.longest}; };
   *attention = info(L.tc.all);
   *pass = info(L.tc.beside.n_cta > 0 ? L.tc.beside : L.tc.all);
-  *small_pass = L.tc.small;
+  *small_pass = (int32_t)L.tc.small;
   return LR_OK;
 }
 
@@ -1011,13 +1011,16 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
   if (int rc = cuda_fail(cudaStreamIsCapturing(s, &capture), "cudaStreamIsCapturing")) return rc;
   // On one stream, two kernels in a row of which the second is set up, and mostly done, while the first runs (pass_tail.cu), there
   // are no events between two passes, and the next attention is set up early too.  A caller who gives a second stream has a reason
-  // to order work with it.  In a graph events cost nothing and both streams' kernels start together: acceptance and commit are one
-  // kernel there (one request of 4 K tokens 19.0 -> 16.2 us), and beside an attention of few CTAs they are a root of their own.
+  // to order work with it.  In a graph events cost nothing and both streams' kernels start together: where the acceptance has SMs
+  // of its own it is one kernel with the commit there (one request of 4 K tokens, head size 64, 18.9 -> 16.6 us), and beside an
+  // attention of few CTAs a root of its own; where it has not, two kernels on a second stream are as good (4 K tokens, head size 128,
+  // 19.2 us and 19.6).
   // Launched one by one, the second stream's kernel often comes when CTAs of the merge, which wait for attention, already sit on
-  // the SMs left free, and then runs behind all of it on a few SMs: a pass by itself 31.5 us with acceptance and commit as two
-  // kernels and 34.8 with one, of 8 K tokens 37.1 and 44.8, 13 ragged requests of up to 900 tokens 48.6 and 61.
-  const bool captured = capture != cudaStreamCaptureStatusNone;
-  if (side || (captured && 2 * p->tc_pass.n_cta <= p->ctx->sm_count)) return pass_side_by_side(ctx, p, io, scale, captured, side, s);
+  // the SMs left free, and then runs behind all of it on a few SMs: a pass by itself, head size 64, 32.2 us with acceptance and commit
+  // as two kernels and 35.2 with one.
+  const bool captured = capture != cudaStreamCaptureStatusNone, beside = p->small == kBesideAttention;
+  if (side || (captured && (!beside || 2 * p->tc_pass.n_cta <= p->ctx->sm_count)))
+    return pass_side_by_side(ctx, p, io, scale, /*one_kernel=*/captured && beside, side, s);
   if (int rc = launch_attn_tc(p, p->tc_pass, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/false, s)) return rc;
   return launch_pass_tail(ctx, p, io, /*behind_attention=*/true, s);
 }

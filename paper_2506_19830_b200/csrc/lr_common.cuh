@@ -109,6 +109,9 @@ struct DevTcPlan {
   float *partial_ml;         // [n_slots][128][2] (reference exponent in log2 units, sum)
 };
 
+// Whether a pass may go as in pass_tail.cu, and whether its acceptance has SMs of its own or all of them behind attention.
+enum SmallPass : int32_t { kNotSmall = 0, kBesideAttention = 1, kBehindAttention = 2 };
+
 // ---- CTA-pair attention plan (device side) -----------------------------------
 // Two CTAs on neighbouring SMs work as one unit: CTA c of the pair owns M-tile mtile0 + c of a piece (its query
 // rows, scores, probabilities and output accumulator) and supplies half of every KV tile; one tcgen05.mma with
@@ -175,7 +178,7 @@ struct lr_plan {
   lr::DevBatch dev;
   lr::DevTcPlan tc;
   lr::DevTcPlan tc_pass;  // of a small pass: the same, or the partition that leaves SMs free
-  bool small;             // the whole pass as in pass_tail.cu
+  lr::SmallPass small;
   lr::DevPairPlan pr;
   bool tc_ok;             // shape allows the tensor-core path
   // The CTA-pair plan is built and uploaded when its path is first selected.  Its tables have a part of the workspace to
@@ -255,7 +258,7 @@ struct TcHostPlan {
   std::vector<TcList> lists;
   TcPartition all;     // over all SMs: of lr_verify_attention, whoever calls it
   TcPartition beside;  // of a small pass whose acceptance needs SMs that `all` does not leave; else empty
-  bool small = false;  // lr_verify_pass may go as in pass_tail.cu
+  SmallPass small = kNotSmall;
   size_t o_pages = 0, o_rows = 0, o_reqs = 0;  // image offsets
   int tokens_per_mtile = 0, n_pages = 0;
   // scratch region behind the image: (exponent, sum) pairs, then fp32 partial outputs

@@ -1,5 +1,6 @@
 """How the attention work of a batch is split (host side of the planner): lr_verify_attention's partition knows nothing of the
-logits, and a small pass that has one of its own keeps to its bounds."""
+logits, a small pass with head size 64 that has one of its own keeps to its bounds, and one with head size 128, whose results hang
+on the split of the keys, has attention's."""
 import numpy as np
 import pytest
 
@@ -32,14 +33,14 @@ def test_bounds(geometry, n_sm):
                     attention, own, small = B.lr_debug_partitions(b.model, b, n_sm)
                     seen.add(tuple(attention.values()))
                     assert 1 <= own["n_cta"] <= attention["n_cta"] <= n_sm
+                    assert small != 2 or (own == attention and attention["n_merge_targets"] > 0)
                     if own != attention:
                         narrow += 1
-                        assert small and own["n_cta"] < attention["n_cta"]
+                        assert geometry[2] == 64 and small == 1 and own["n_cta"] < attention["n_cta"]
                         assert _time(own) <= 1.25 * _time(attention)
                         assert attention["n_merge_targets"] > 0 or own["n_merge_targets"] == 0
                 assert len(seen) == 1  # whatever the vocabulary
-    if geometry[1] == 8 and n_sm == 148:
-        assert narrow > 0
+    assert geometry != (32, 8, 64) or narrow > 0
 
 
 # (geometry, vocabulary, requests, prefix, steps, drafts): the CTAs of attention, and its merge targets
