@@ -415,9 +415,9 @@ typedef struct lr_pass_io {
 
 /* lr_verify_attention, lr_accept_greedy and lr_commit in one call: everything they
  * write is ready in the order of `stream`.  `ctx` is the acceptance's, as in
- * lr_accept_greedy; its vocabulary may be another than the plan's.  Acceptance and commit need nothing
- * from attention and may run beside it, on side_stream if one is given, else on
- * `stream` (small passes) or a stream of the plan. */
+ * lr_accept_greedy; its vocabulary may be another than the plan's.  Acceptance
+ * and commit need nothing from attention and may run beside it, on side_stream if
+ * one is given, else on `stream` or a stream of the plan. */
 int lr_verify_pass(lr_ctx *ctx, lr_plan *plan, const lr_pass_io *io, float softmax_scale, void *side_stream, void *stream);
 
 /* ---- whole pass with host buffers ---------------------------------------- */

@@ -163,8 +163,9 @@ struct CountsGiven {
 // One CTA of the commit.  The chain of loads is what it takes, so all of it that does not hang on the kernel just before is gone
 // through while that one drains: what the plan says of a thread's first page slot always (its tables come by copies), and -- with
 // `early`, whose terms stand at launch_commit -- the decision on a thread's first request too.  Then one trip for the counts, the
-// scans and the stores are left.  A pass over one request of 4 K tokens 27.9 -> 24.8 us, with head size 64 24.4 -> 23.0; behind the
-// sampled acceptance, plan tables only, 50.3 -> 49.3 and 51.2 -> 49.5 (617 rows without and with filters), 36.0 -> 35.1 (51 rows, top-p).
+// scans and the stores are left.  Behind the sampled acceptance, plan tables only: 50.3 -> 49.3 and 51.2 -> 49.5 us (617 rows without and
+// with filters), 36.0 -> 35.1 (51 rows, top-p).  As a kernel of its own behind the greedy one, the decision too: 27.9 -> 24.8 us for a pass over
+// one request of 4 K tokens when such passes had it.
 // The counts, and without `early` the verdicts, may be written while this kernel is resident: neither is __restrict__.
 template <bool kTree, class Counts>
 __device__ __forceinline__ void commit_cta(const DevBatch &d, int cta, int n_cta, bool early, const uint8_t *verdict, Counts counts, const CommitOut &o) {

@@ -4,15 +4,23 @@
 // A small pass is a chain of latencies: as four kernels on two streams it was attention (13 us for one request of 4 K tokens),
 // acceptance behind it because an attention CTA leaves no registers for another on its SM (8), and commit (2), with events at
 // both ends.  Here the launch is a programmatic dependent of the attention kernel, and only the CTAs that merge wait for it.  The
-// others run on SMs that the plan has left free (tc_plan_structure): first the CTAs of the commit, which go through their plan
-// tables and then wait for the row keys, then those that stream the logits.  When attention ends, the merge is all that is left.
-// A pass, four kernels and two: 256 tokens 12.7 -> 11.7 us, 4 K tokens 24.6 -> 18.8, with head size 64 22.8 -> 16.9, one of 8 K
-// 29.3 -> 23.6, small batches of other shapes by 0 to 40 %.
+// others run on SMs that attention leaves free, or behind it where it leaves too few (plan_small_pass): first the CTAs of the
+// commit, which go through their plan tables and then wait for the row keys, then those that stream the logits.
+// As four kernels and as two, with the same attention, one after another on the same buffers: 256 tokens 13.6 -> 12.1 us; 4 K tokens with
+// head size 64, beside a narrower attention, 22.4 -> 16.9; with head size 128, behind it, 22.5 -> 19.9; 8 K so 27.3 -> 25.4.  Some of that is
+// the set-up of the next pass's attention while this one ends: passes that are waited for one by one take 20.0 and 20.5, 32.1 and
+// 26.1, 33.2 and 29.5, 38.4 and 34.8.
 //
 // What streams is warps: an SM's rate grows with them and hardly with the loads a lane has in flight (one SM alone: 8 warps 30
 // GB/s, 16 54, 32 80 to 90, with four, eight or sixteen 16-byte loads a lane).  A warp takes consecutive units and publishes once
 // a row: handing units out by a counter, or an atomic for each of them, cost more than the reading (one address takes about one
-// atomic a nanosecond).  A CTA that waits, waits for CTAs of the grid that wait for nothing, and those that wait do not fill one SM.
+// atomic a nanosecond).
+//
+// Every wait ends: the CTAs of the commit are the first of the grid and wait for those that stream, which wait for nothing and need only
+// places; those that merge are the last and wait for an attention whose CTAs all run by then.  At most two CTAs of a pass hold places
+// while they wait for others to get some, and at most 128 grids run on a GPU at a time: 256 of the 444 places and more that it has, so
+// passes on other streams cannot take the last ones either.  (Attention CTAs that wait for the kernel before them are launched when all of
+// that kernel's streaming CTAs have ended.)  And the wait gives up after a limit.
 #include <algorithm>
 
 #include "accept_stream.cuh"
@@ -29,7 +37,7 @@ constexpr int kVecPerThread = 6;     // eight spill
 // CTAs an SM: 64 registers a thread, or 72 where the merge has eight slots in flight.
 constexpr int kFewSlots = 4;         // partial slots an M-tile up to which the merge takes the narrower form, as when it is alone
 constexpr int tail_ctas(int batch) { return batch <= kFewSlots ? 4 : 3; }
-// CTAs of the commit.  They wait for others of the grid, so they are too few to fill even one SM.
+// CTAs of the commit: they wait for others of the grid, so they are few.
 constexpr int kCommitCtas = tail_ctas(8) - 1;
 constexpr int kCommitSlots = 2048;   // page slots that so few write: four a thread
 constexpr int kMostRequests = 512;   // every CTA has shared memory for the decisions of so many, 18 KB
