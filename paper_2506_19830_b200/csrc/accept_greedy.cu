@@ -125,10 +125,11 @@ int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t
   // a chunk per warp at least, at most kCtasPerSm CTAs per SM
   const unsigned grid = std::min((w.total + kThreads / 32 - 1) / (kThreads / 32), (uint32_t)(ctx->sm_count * kCtasPerSm));
   // Set up while whatever is before it drains; see the kernel's first lines.  Behind a fill of 64 values, the attention of one request
-  // of 4 K tokens, and that of 4 ragged ones, 51 to 2268 rows of 152064 are ready 1.1 to 2.8 us sooner than with an ordinary launch
-  // (411 rows: 32.1 -> 29.8, 44.7 -> 42.5, 59.0 -> 57.0; 2268: 110.5 -> 108.2, 124.9 -> 123.2, 140.3 -> 138.6), in a graph 0.2 us.  Behind
-  // another acceptance of the same size, which no program does, it goes either way: 411 rows 29.0 and 27.0, in a graph 26.3 and 26.5;
-  // 500 rows 33.2 and 34.1, in a graph 30.4 and 33.7.
+  // of 4 K tokens, and that of 4 ragged ones, 51 to 2268 rows of 152064 are ready 0.3 to 2.8 us sooner than with an ordinary launch
+  // (411 rows: 32.1 -> 29.8, 44.7 -> 42.5, 59.0 -> 57.0; 2268: 110.5 -> 108.2, 124.9 -> 123.2, 140.3 -> 138.6), in a graph 0.2.  Behind
+  // another acceptance of the same size, as a benchmark of the kernel alone has it and no program, an ordinary launch is the faster one
+  // from 300 rows on in a graph (411 rows 25.1 and 29.0, 500 28.4 and 31.1, 2268 105.4 and 107.0) and at some sizes without (411 rows
+  // 27.9 and 29.4, 500 30.6 and 31.5; 206 17.7 and 17.6, 1000 53.5 and 53.3); starting CTAs or warps apart from one another changes nothing.
   ctx->launches++;
   return cuda_fail(launch_dependent(accept_greedy_kernel, dim3(grid), dim3(kThreads), 0, s, w, drafts, cu_draft, n_branch, n_rows, first_draft, n_accept, bonus,
                                     row_argmax),
