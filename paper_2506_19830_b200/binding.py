@@ -10,7 +10,6 @@ from __future__ import annotations
 import ctypes as C
 import os
 import struct
-import weakref
 from typing import Optional
 
 import numpy as np
@@ -207,12 +206,14 @@ class Context:
         m = _model_struct(model)
         _check(lib().lr_create(C.byref(h), C.byref(m), device), "lr_create")
         self.handle = h
-        self._plans = weakref.WeakSet()  # plans must be destroyed before their context
+        # Handles of the plans that are left: plans are destroyed before their context, also where the collector finalises both in
+        # whatever order (weak references to them are dead by then).
+        self._open = set()
 
     def close(self):
         if self.handle:
-            for p in list(self._plans):
-                p.close()
+            while self._open:
+                lib().lr_plan_destroy(self._open.pop())
             lib().lr_destroy(self.handle)
             self.handle = None
 
@@ -303,15 +304,17 @@ class Plan:
             lib().lr_plan_drop(draft)
             raise
         _check(lib().lr_plan_finish(draft, self._ws_ptr, n.value, stream, C.byref(h)), "lr_plan_finish")
-        self.handle = h
-        ctx._plans.add(self)
+        self.handle, self._open = h, ctx._open
+        self._open.add(h.value)
         self.n_req = self.host.c.n_req
         self.n_branch = self.host.c.n_branch
         self.n_page_slots = self.host.c.n_page_slots
 
     def close(self):
         if self.handle:
-            lib().lr_plan_destroy(self.handle)
+            if self.handle.value in self._open:  # else its context has destroyed it
+                self._open.remove(self.handle.value)
+                lib().lr_plan_destroy(self.handle)
             self.handle = None
 
     def __del__(self):
