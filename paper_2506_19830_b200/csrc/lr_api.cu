@@ -1017,10 +1017,10 @@ extern "C" int lr_verify_pass(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, flo
   // 19.2 us and 19.6).
   // Launched one by one, the second stream's kernel often comes when CTAs of the merge, which wait for attention, already sit on
   // the SMs left free, and then runs behind all of it on a few SMs: a pass by itself, head size 64, 32.2 us with acceptance and commit
-  // as two kernels and 35.2 with one.
+  // as two kernels and 35.2 with one.  So they are two there, unless there is no merge and few logits.
   const bool captured = capture != cudaStreamCaptureStatusNone, beside = p->small == kBesideAttention;
   if (side || (captured && (!beside || 2 * p->tc_pass.n_cta <= p->ctx->sm_count)))
-    return pass_side_by_side(ctx, p, io, scale, /*one_kernel=*/captured && beside, side, s);
+    return pass_side_by_side(ctx, p, io, scale, /*one_kernel=*/captured ? beside : pass_tail_apart(ctx, p, (int32_t)io->n_rows), side, s);
   if (int rc = launch_attn_tc(p, p->tc_pass, io->q_d, io->k_pool_d, io->v_pool_d, io->out_d, io->lse_d, scale, /*merge=*/false, s)) return rc;
   return launch_pass_tail(ctx, p, io, /*behind_attention=*/true, s);
 }

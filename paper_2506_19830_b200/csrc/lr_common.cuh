@@ -345,6 +345,9 @@ int launch_attn_tc(lr_plan *p, const DevTcPlan &tc, const void *q, const void *k
 // The rest of a small pass: acceptance and commit, and behind a launch_attn_tc without merge that too; and whether a pass is one.
 // The acceptance goes by the context of the call, which need not be the plan's: its vocabulary may be another.
 bool pass_tail_fits(const lr_ctx *ctx, const lr_plan *p, int64_t n_rows);
+// Whether that kernel, on a second stream, and attention cannot be in each other's way, whichever comes first: no CTAs of a merge that
+// wait on the SMs left free, and no more CTAs than there are such SMs, so that attention finds whole SMs all the same.
+bool pass_tail_apart(const lr_ctx *ctx, const lr_plan *p, int32_t n_rows);
 int launch_pass_tail(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, bool behind_attention, cudaStream_t s);
 // first_draft: what cu_draft counts in front of the first branch's rows (a later part of a batch whose rows are given alone)
 int launch_accept(lr_ctx *ctx, const void *logits, int64_t stride, const int32_t *drafts, const int32_t *cu_draft,

@@ -168,7 +168,28 @@ auto tail_kernel(bool tree) {
   return tree ? pass_tail_kernel<kD, kBatch, true> : pass_tail_kernel<kD, kBatch, false>;
 }
 
+// CTAs of the commit and those that stream; a warp's share is what the places beside attention, or behind it, stream in one go.
+struct TailGrid {
+  int n_commit, n_stream;
+  uint32_t share;
+};
+TailGrid tail_grid(const lr_plan *p, uint32_t total) {
+  const DevTcPlan &tc = p->tc_pass;
+  TailGrid g;
+  g.n_commit = std::min(commit_ctas(p->dev), kCommitCtas);
+  const int n_sm = p->ctx->sm_count, most = p->small == kBehindAttention ? kStreamCtas * n_sm : tail_ctas(tc.most_slots) * (n_sm - tc.n_cta);
+  const uint32_t warps = (uint32_t)std::max(1, most - g.n_commit) * (kThreads / 32);
+  g.share = (total + warps - 1) / warps;
+  g.n_stream = (int)((total + g.share * (kThreads / 32) - 1) / (g.share * (kThreads / 32)));
+  return g;
+}
+
 }  // namespace
+
+bool pass_tail_apart(const lr_ctx *ctx, const lr_plan *p, int32_t n_rows) {
+  const TailGrid g = tail_grid(p, accept_work(ctx, nullptr, 0, n_rows, nullptr, kVecPerThread).total);
+  return p->small == kBesideAttention && p->tc_pass.n_targets == 0 && g.n_commit + g.n_stream <= p->ctx->sm_count - p->tc_pass.n_cta;
+}
 
 bool pass_tail_fits(const lr_ctx *ctx, const lr_plan *p, int64_t n_rows) {
   const int vecs = ctx->model.vocab >> 3, unit = 32 * kVecPerThread;
@@ -180,15 +201,12 @@ int launch_pass_tail(lr_ctx *ctx, lr_plan *p, const lr_pass_io *io, bool behind_
   const DevBatch &d = p->dev;
   PassAccept a = {accept_work(ctx, io->logits_d, io->logits_stride, (int32_t)io->n_rows, io->accept_scratch_d, kVecPerThread),
                   io->draft_ids_d, io->cu_draft_d, io->n_accept_d, io->bonus_id_d, io->row_argmax_d, d.n_branch, (int32_t)io->n_rows};
-  a.n_commit = std::min(commit_ctas(d), kCommitCtas);
-  // a warp's share: what the places beside attention, or behind it, stream in one go
   const DevTcPlan &tc = p->tc_pass;
   const bool few = tc.most_slots <= kFewSlots;
-  const int n_sm = p->ctx->sm_count;
-  const uint32_t places =
-      (uint32_t)std::max(1, (p->small == kBehindAttention ? kStreamCtas * n_sm : tail_ctas(few ? 4 : 8) * (n_sm - tc.n_cta)) - a.n_commit);
-  a.share = (a.w.total + places * (kThreads / 32) - 1) / (places * (kThreads / 32));
-  a.n_stream = (int)((a.w.total + a.share * (kThreads / 32) - 1) / (a.share * (kThreads / 32)));
+  const TailGrid grid = tail_grid(p, a.w.total);
+  a.n_commit = grid.n_commit;
+  a.n_stream = grid.n_stream;
+  a.share = grid.share;
   a.wait_limit_ns = 1000ull * kPatience * tc.wait_limit_us;
   const CommitOut o = {io->n_steps_accepted_d, io->survivor_d, io->committed_len_d, io->keep_off_d,
                        io->keep_pages_d, io->keep_valid_d, io->free_off_d, io->free_pages_d};

@@ -112,3 +112,27 @@ def test_a_second_stream(heads, head_dim, vocab, form):
         del graph
     plan.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("n_req,vocab,n", [(8, 5748, 2), (8, 152064, 3)])
+def test_a_second_stream_without_a_merge(n_req, vocab, n):
+    """Few logits and no merge: acceptance and commit are one kernel, which fits the SMs that attention leaves; many: two."""
+    w = _work((32, 8), 64, vocab, n_req, 60, 1, 4, True)
+    b, t = w.batch, w.tensors
+    ctx = B.Context(b.model, 0)
+    plan, x, y, side = B.Plan(ctx, b), R.DeviceInputs(b, t), R.PassOutputs(b), torch.cuda.Stream()
+    n_ref, bonus_ref, _ = O.accept_greedy(t.logits, t.draft_ids, b.cu_draft)
+    o_ref, _ = O.verify_attention(b, t.q, t.k_pool, t.v_pool)
+    assert plan.lr_plan_describe()["n_merge_targets"] == 0
+    for _ in range(3):
+        before = ctx.launch_count
+        R.run_pass_overlapped(ctx, plan, x, y, side)
+        assert ctx.launch_count - before == n
+        assert plan.lr_poll_status() == 0
+        check_attention(y.out, None, o_ref, None, rel_large=REL_LARGE)
+        assert np.array_equal(y.n_accept.cpu().numpy(), n_ref) and np.array_equal(y.bonus_id.cpu().numpy(), bonus_ref)
+        check_commit(y.commit_dict(), O.commit(b, t.verdict, n_ref))
+        assert int(y.scratch.abs().sum().item()) == 0
+        y.n_accept.zero_(), y.keep_pages.zero_(), y.out.zero_()
+    plan.close()
+    ctx.close()
